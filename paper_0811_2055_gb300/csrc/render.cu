@@ -59,7 +59,7 @@ void kernel_table_host(int kernel, int32_t *K)
     }
 }
 
-void set_splat_smem_limits();
+void set_splat_smem();
 
 // once per device: the kernel tables, and the dynamic shared-memory limit of the splat kernels
 // (a device setting, so it is made before any launch that a stream capture could record)
@@ -76,7 +76,7 @@ void ensure_tables()
     kernel_table_host(GBLOD_KERNEL_GAUSSIAN, K[0]);
     kernel_table_host(GBLOD_KERNEL_CUBIC, K[1]);
     GB_CUDA(cudaMemcpyToSymbol(g_ktab, K, sizeof(K)));
-    set_splat_smem_limits();
+    set_splat_smem();
     done[dev] = 1;
 }
 
@@ -964,10 +964,12 @@ __global__ void k_tile_items(uint32_t ntiles, const uint32_t *tile_cnt, uint32_t
     if (t < ntiles) item_cnt[t] = (tile_cnt[t] + ITEM - 1) / ITEM;
 }
 
+// also clears the unit counter of the splat launch that follows
 __global__ void k_fill_items(uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
-                             const uint32_t *item_off, uint4 *items)
+                             const uint32_t *item_off, uint4 *items, unsigned *next)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) *next = 0u;
     if (t >= ntiles) return;
     const uint32_t c = tile_cnt[t], o = tile_off[t];
     uint32_t k = item_off[t];
@@ -975,52 +977,52 @@ __global__ void k_fill_items(uint32_t ntiles, const uint32_t *tile_cnt, const ui
 }
 
 // ------------------------------------------------------------------ R3
-// One block per work item (a tile and up to ITEM of its records).  The tile is cut into 8 x 4
-// pixel blocks, one lane per pixel; each warp owns up to SPLAT_SLOTS blocks of one block column
-// (see strip_height).  Records are staged through shared memory STAGE at a time and listed per
-// block column; each warp compacts, by ballot, its column's records whose support reaches one of
-// its blocks, evaluates only those for its pixels and keeps the sums in registers.
-// Exact integer shortcuts of the per-pixel rule, all identities:
-//   (q S) >> 37 < 1024  <=>  q < QL = floor((2^47 - 1) / S) + 1     (one compare per miss)
-//   floor(Wq K / 2^16)   =   Wh K + floor(Wl K / 2^16),  Wq = Wh 2^16 + Wl, Wl < 2^16
-// Wh K goes to a 64-bit sum and floor(Wl K / 2^16) < 2^16 to a 32-bit one (at most ITEM = 2048
-// records per block keeps it below 2^27).  Each pixel's sum is added to the image once.
+// The tile is cut into 8 x 4 pixel blocks, one lane per pixel; a warp owns up to SPLAT_SLOTS blocks of
+// one block column (see strip_height) and works on its own: a unit of work is (item, strip), an item
+// a tile and up to ITEM of its records, and the warps of a persistent grid take units from a
+// counter.  No barrier, no staging by other warps: a warp reads its item's records 32 at a time, one
+// per lane, tests each against its two pairs of blocks, and compacts the ones that reach them into
+// lists of its own in shared memory, by the arithmetic they need; a list of 16 or more is walked with one
+// pixel per lane and block, without branches, the sums in registers.  Each pixel's sum is added to
+// the image once per unit.
+//
+// What bounds the walk: a (record, pixel) pair takes one table read (about 2.6 shared-memory
+// wavefronts for 32 lanes, of one a cycle for the four schedulers: 10.6 cycles), one high-word
+// multiply (4.2 cycles of the multiplier) and about seven other instructions, 12.8 cycles in all for
+// 32 pairs of a faint record, 15 of a light one.  Measured (GB300): 16.8M particles at 1080p, 8.4e9
+// pairs, 4.37 ms (6.74 with block-wide staging, barriers and a 64-bit sum per pair); 150M particles,
+// 4.7e10 pairs, 28.4 ms (41.1).  Reading and listing the records, walks skipped, is 0.9 and 6.2 ms of
+// that.  The forms used, all identities of the rule:
+//   index  (q S) >> 37, q < 2^32: the high word of q S, shifted by 5; q of the warp's blocks from one
+//          square each in x and y and one three-input addition a block; indices from 1024 on (outside
+//          the support) are clamped to a zero entry, so no pixel is tested.
+//   amplitude, Wq < 2^23 (most of the pixel work: wide blobs are faint): floor(Wq K / 2^16) + 2^23 is one
+//          fp32 multiply-add rounded towards zero (exact product, unit spacing in [2^23, 2^24)); its
+//          bits are summed as integers, the constant taken off once per list.
+//   amplitude, Wq < 2^32: Wh K + floor(Wl K / 2^16), Wq = Wh 2^16 + Wl, both below 2^16 (Wh + 1), in one
+//          32-bit sum that is emptied after every `chunk` records, chunk (largest Wh + 1) <= 2^16.
 constexpr int SPLAT_SLOTS = 4; // 8 warps x 4 blocks of 32 pixels: tiles up to 1024 pixels
-static_assert(ITEM <= (1u << 15), "32-bit partial sums need at most 2^15 records per item");
+constexpr int LIST_MIN = 16;   // a list is walked when it holds this many records
+constexpr int LIST = LIST_MIN - 1 + 32;
 
-constexpr int STAGE = 512; // records staged in shared memory at a time (record index: 9 bits)
+// A warp's lists.  FAINT: Wq < 2^23; LIGHT: Wq < 2^32; either with a narrow support (QL = 2^47 / S <= 2^30:
+// every pixel of a strip the support reaches lies within 2^15 + 32 px, in 1/256 px, of the centre, so
+// q < 2^32), by the pairs of blocks reached: both, only the upper, only the lower.  WIDE: Wq < 2^23 with a
+// wider support.  HEAVY: the rest.
+enum { L_FAINT, L_FAINT_UP, L_FAINT_LOW, L_LIGHT, L_LIGHT_UP, L_LIGHT_LOW, L_WIDE, L_HEAVY, L_COUNT };
 
 struct SplatSmem {
-    int32_t K[1024];
-    uint4 raw[STAGE];             // records of the next stage, copied asynchronously
-    int4 A[STAGE];                // U, V, S, Wh = Wq >> 16
-    uint4 B[STAGE];               // QL low, Wl = Wq & 0xFFFF, QL high, unused
-    uint16_t list[RT / 32][STAGE]; // per warp: record | touched blocks of its column << 9; small records
-                                   // touching all four blocks from the front, other small ones from the back
-    uint16_t large[RT / 32][STAGE]; // per warp: the same for records with QL > 2^30
-    uint16_t cand[8][STAGE];       // per block column: records whose support may reach it
-    uint32_t ncand[2][8];          // candidate counts, two sets used on alternate stages
+    uint32_t K[1025];                   // the kernel table and a zero entry
+    float Kf[1025];                     // K 2^-16
+    uint32_t count[RT / 32][L_COUNT];   // records in each list
+    uint4 list[RT / 32][L_COUNT][LIST]; // {U, V, S, Wq}; Wq as a float in FAINT, WIDE and HEAVY
 };
 // dynamic shared memory: four CTAs per SM fit in its 228 KB with the 1 KB each CTA reserves
 static_assert(4 * (sizeof(SplatSmem) + 1024) <= 228 * 1024, "four splat CTAs per SM");
 
-// 16-byte global -> shared copy that bypasses registers and L1 (completes at cp_async_wait_all)
-__device__ __forceinline__ void cp_async16(uint32_t smem_addr, const uint4 *g)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// A record is "small" when QL <= 2^30: every pixel of a block its support reaches then lies
-// within 2^15 + 8 px of its centre on each axis (in 1/256 px), so dx^2 + dy^2 < 2^32 and the
-// table index (q S) >> 37 is the high word of a 32 x 32 product shifted by 5.
-constexpr unsigned long long QL_SMALL = 1ull << 30;
-
 // Each warp owns up to SPLAT_SLOTS blocks of 8 x 4 pixels in one block column: with the tile's
-// nbx x nby blocks, sh = the smallest count with nbx ceil(nby / sh) <= 8 warps, warp w takes column
-// w % nbx and the block rows g, g + ng, g + 2 ng, ... (g = w / nbx, ng = ceil(nby / sh)), so the
-// rows of a column are interleaved between its warps and their work stays balanced.
+// nbx x nby blocks, sh = the smallest count with nbx ceil(nby / sh) <= 8 strips, strip w takes column
+// w % nbx and the sh consecutive block rows from (w / nbx) sh on.
 __host__ __device__ __forceinline__ int strip_height(int nbx, int nby)
 {
     int sh = 1;
@@ -1028,206 +1030,253 @@ __host__ __device__ __forceinline__ int strip_height(int nbx, int nby)
     return sh;
 }
 
-// Splats records [it.y, it.z) of tile `tile` (index inside the view) of view P into img; COUNT
-// adds the pixel updates to `hits`.  Each
-// lane owns one pixel column position of its warp's strip and one pixel in every block of it;
-// a record's centre offset in x and its square are computed once per strip, not once per block.
+// strips of a TW x TH tile (at most 8)
+__host__ __device__ __forceinline__ uint32_t strips_of(int TW, int TH)
+{
+    const int nbx = (TW + 7) >> 3, nby = (TH + 3) >> 2, sh = strip_height(nbx, nby);
+    return (uint32_t)(nbx * ((nby + sh - 1) / sh));
+}
+
+constexpr int BLOCK_DY = 4 * 256; // y offset between consecutive blocks, 1/256 px
+
+// Table indices (1024: outside) of blocks FIRST .. FIRST + N - 1 at this lane's pixel (px, py)
+template <int FIRST, int N> __device__ __forceinline__ void block_idx(const uint4 &A, int px, int py, uint32_t (&idx)[N])
+{
+    const uint32_t dx = (uint32_t)px - A.x, dy = (uint32_t)(py + FIRST * BLOCK_DY) - A.y;
+    const uint32_t g = 2u * BLOCK_DY * dy; // (dy + BLOCK_DY)^2 = dy^2 + g + BLOCK_DY^2
+    uint32_t q = dx * dx + dy * dy;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        idx[k] = min(__umulhi(q, A.z) >> 5, 1024u);
+        q += g + (uint32_t)((2 * k + 1) * BLOCK_DY * BLOCK_DY);
+    }
+}
+
+// The same for any support: q in 64 bits, (q S) >> 32 = S (q >> 32) + the high word of S and q's low word
+// (a pixel of a strip the support reaches has q S < 2^52, so nothing is lost)
+__device__ __forceinline__ void block_idx_wide(const uint4 &A, int px, int py, uint32_t (&idx)[SPLAT_SLOTS])
+{
+    const int dx = px - (int)A.x, dy = py - (int)A.y;
+    const long long g = 2ll * BLOCK_DY * dy;
+    unsigned long long q = (unsigned long long)((long long)dx * dx + (long long)dy * dy);
+#pragma unroll
+    for (int k = 0; k < SPLAT_SLOTS; ++k) {
+        idx[k] = min((__umulhi((uint32_t)q, A.z) + (uint32_t)(q >> 32) * A.z) >> 5, 1024u);
+        q += (unsigned long long)(g + (2 * k + 1) * BLOCK_DY * BLOCK_DY);
+    }
+}
+
+struct StripSums {
+    unsigned long long acc[SPLAT_SLOTS] = {0ull, 0ull, 0ull, 0ull};
+    unsigned hits[SPLAT_SLOTS] = {0u, 0u, 0u, 0u};
+};
+
+// Walks a list of n faint records over blocks FIRST .. FIRST + N - 1 (N even)
+template <int FIRST, int N, bool WIDE, bool COUNT>
+__device__ __forceinline__ void walk_faint(const uint4 *__restrict__ list, int n, int px, int py, const float *Kf,
+                                           StripSums &a)
+{
+    uint32_t sum[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) sum[k] = 0u - (uint32_t)n * 0x4B000000u; // n times the bits of 2^23
+#pragma unroll 2
+    for (int i = 0; i < n; ++i) {
+        const uint4 A = list[i];
+        uint32_t idx[N];
+        if constexpr (WIDE) block_idx_wide(A, px, py, idx);
+        else block_idx<FIRST, N>(A, px, py, idx);
+        float k[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            k[j] = Kf[idx[j]];
+            if (COUNT) a.hits[FIRST + j] += idx[j] < 1024u ? 1u : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < N; j += 2) // two products an instruction
+            asm("{.reg .b64 w, k, c, r;\n\tmov.b64 w, {%4, %4};\n\tmov.b64 k, {%2, %3};\n\tmov.b64 c, {%5, %5};\n\t"
+                "fma.rz.f32x2 r, w, k, c;\n\tmov.b64 {%0, %1}, r;}"
+                : "=f"(k[j]), "=f"(k[j + 1])
+                : "f"(k[j]), "f"(k[j + 1]), "f"(__uint_as_float(A.w)), "f"(0x1p23f));
+#pragma unroll
+        for (int j = 0; j < N; ++j) sum[j] += __float_as_uint(k[j]);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) a.acc[FIRST + k] += sum[k]; // below 2^23 LIST
+}
+
+// records a 32-bit sum takes between flushes: a power of two with chunk (Wh + 1) <= 2^16 for Wh <= wmax < 2^16
+__device__ __forceinline__ int flush_chunk(uint32_t wmax) { return 1 << (16 - (32 - __clz((int)wmax))); }
+
+// Walks a list of n light records
+template <int FIRST, int N, bool COUNT>
+__device__ __forceinline__ void walk_light(const uint4 *__restrict__ list, int n, int px, int py, const uint32_t *K,
+                                           StripSums &a)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t wmax = lane < n ? list[lane].w >> 16 : 0u;
+    if (32 + lane < n) wmax = max(wmax, list[32 + lane].w >> 16);
+    const int chunk = flush_chunk(__reduce_max_sync(0xffffffffu, wmax));
+    for (int i0 = 0; i0 < n; i0 += chunk) {
+        const int i1 = min(n, i0 + chunk);
+        uint32_t sum[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) sum[k] = 0u;
+#pragma unroll 2
+        for (int i = i0; i < i1; ++i) {
+            const uint4 A = list[i];
+            const uint32_t Wh = A.w >> 16, Wl = A.w & 0xFFFFu;
+            uint32_t idx[N];
+            block_idx<FIRST, N>(A, px, py, idx);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                const uint32_t kv = K[idx[k]];
+                sum[k] += Wh * kv;
+                sum[k] += (Wl * kv) >> 16;
+                if (COUNT) a.hits[FIRST + k] += idx[k] < 1024u ? 1u : 0u;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < N; ++k) a.acc[FIRST + k] += sum[k];
+    }
+}
+
 template <bool COUNT>
-__device__ __forceinline__ void splat_item(const uint4 *__restrict__ rec, const uint4 it, const uint32_t tile,
+__device__ __forceinline__ void walk_heavy(const uint4 *__restrict__ list, int n, int px, int py, const uint32_t *K,
+                                           StripSums &a)
+{
+    for (int i = 0; i < n; ++i) {
+        const uint4 A = list[i];
+        const unsigned long long Wq = __float2ull_rn(__uint_as_float(A.w));
+        const uint32_t Wh = (uint32_t)(Wq >> 16), Wl = (uint32_t)Wq & 0xFFFFu;
+        uint32_t idx[SPLAT_SLOTS];
+        block_idx_wide(A, px, py, idx);
+#pragma unroll
+        for (int k = 0; k < SPLAT_SLOTS; ++k) {
+            const uint32_t kv = K[idx[k]];
+            a.acc[k] += (unsigned long long)Wh * kv + ((Wl * kv) >> 16);
+            if (COUNT) a.hits[k] += idx[k] < 1024u ? 1u : 0u;
+        }
+    }
+}
+
+// Splats records [it.y, it.z) of tile it.x (index inside the view) of view P into the pixels of strip
+// `strip`; COUNT adds the pixel updates to `hits`.  Every lane of the warp calls it.
+template <bool COUNT>
+__device__ __forceinline__ void splat_unit(const uint4 *__restrict__ rec, const uint4 it, const int strip,
                                            const Proj &P, unsigned long long *__restrict__ img, SplatSmem &sm,
                                            unsigned &hits)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = gbd::lanemask_lt();
-    const int tx = (int)(tile % (uint32_t)P.tiles_x), ty = (int)(tile / (uint32_t)P.tiles_x);
-    const int X0 = tx * P.TW, Y0 = ty * P.TH;
-    const int TWc = min(P.TW, P.W - X0), THc = min(P.TH, P.H - Y0); // tile clipped to the image
     const int nbx = (P.TW + 7) >> 3, nby = (P.TH + 3) >> 2;
     const int sh = strip_height(nbx, nby);
-    const int ng = (nby + sh - 1) / sh;                    // row groups
-    const int scol = warp % nbx, srow = warp / nbx;         // block column, first block row
-    const bool active = warp < nbx * ng;                    // warp-uniform
-    const int bx0 = scol * 8;
-    const int pxl = bx0 + (lane & 7), pyl0 = srow * 4 + (lane >> 3);
-    const int pxv = (X0 + pxl) * 256 + 128, pyv0 = (Y0 + pyl0) * 256 + 128;
-    // blocks k of the strip that exist inside the clipped tile; their pixel-centre rectangles
-    unsigned kvalid = 0;
-#pragma unroll
-    for (int k = 0; k < SPLAT_SLOTS; ++k)
-        if (k < sh && srow + k * ng < nby && bx0 < TWc && (srow + k * ng) * 4 < THc) kvalid |= 1u << k;
-    if (!active) kvalid = 0;
-    const int cx0 = (X0 + bx0) * 256 + 128, cx1 = (X0 + min(bx0 + 7, TWc - 1)) * 256 + 128;
-    unsigned long long acc[SPLAT_SLOTS];
-    uint32_t acc_lo[SPLAT_SLOTS];
-    unsigned hk[SPLAT_SLOTS];
-#pragma unroll
-    for (int k = 0; k < SPLAT_SLOTS; ++k) {
-        acc[k] = 0ull;
-        acc_lo[k] = 0u;
-        hk[k] = 0u;
-    }
-    const int dstep = ng * 1024; // y offset between the warp's consecutive blocks, 1/256 px
-    uint16_t *lst = sm.list[warp], *lrg = sm.large[warp];
-    // records reach shared memory through `raw`, copied (cp.async) one stage ahead of their use
-    const uint32_t raw_addr = (uint32_t)__cvta_generic_to_shared(&sm.raw[threadIdx.x]);
-    for (int t = threadIdx.x; t < STAGE; t += RT)
-        if (it.y + t < it.z) cp_async16(raw_addr + 16u * (uint32_t)(t - threadIdx.x), rec + it.y + t);
-    cp_async_commit();
-    if (threadIdx.x < 16) sm.ncand[threadIdx.x >> 3][threadIdx.x & 7] = 0u;
-    int par = 0;
-    for (uint32_t base = it.y; base < it.z; base += STAGE, par ^= 1) {
-        cp_async_wait_all();
-        __syncthreads();
-        // the other set of counts was last read two stages ago: clear it for the next stage
-        if (threadIdx.x < 8) sm.ncand[par ^ 1][threadIdx.x] = 0u;
-        const int nb = (int)min((uint32_t)STAGE, it.z - base);
-        for (int t = threadIdx.x; t < nb; t += RT) {
-            const uint4 R = sm.raw[t];
-            const unsigned long long Wq = __float2ull_rn(__uint_as_float(R.w));
-            const unsigned long long QL = 140737488355327ull / (unsigned long long)R.z + 1ull;
-            sm.A[t] = make_int4((int)R.x, (int)R.y, (int)R.z, (int)(uint32_t)(Wq >> 16));
-            sm.B[t] = make_uint4((uint32_t)QL, (uint32_t)(Wq & 0xFFFFull), (uint32_t)(QL >> 32), 0u);
-            // block columns whose pixel centres may lie inside the support (|x - U| < sqrt(QL),
-            // rounded up): a superset of the columns the exact per-block test can accept
-            const int rq = (int)sqrtf((float)QL) + 2;
-            const int lx0 = ((int)R.x - 128 - rq) >> 8, lx1 = ((int)R.x - 128 + rq) >> 8; // floor
-            const int c0 = max(0, lx0 - X0) >> 3, c1 = min(TWc - 1, lx1 - X0) >> 3;
-            if (lx1 - X0 >= 0)
-                for (int c = c0; c <= c1; ++c) sm.cand[c][atomicAdd(&sm.ncand[par][c], 1u)] = (uint16_t)t;
+    const int tx = (int)(it.x % (uint32_t)P.tiles_x), ty = (int)(it.x / (uint32_t)P.tiles_x);
+    const int X1 = min((tx + 1) * P.TW, P.W), Y1 = min((ty + 1) * P.TH, P.H); // tile clipped to the image
+    const int xs = tx * P.TW + (strip % nbx) * 8, ys = ty * P.TH + (strip / nbx) * sh * 4; // the strip's first pixel
+    if (xs >= X1 || ys >= Y1) return;
+    const int ye = min(ys + sh * 4, Y1); // its end
+    const int px = (xs + (lane & 7)) * 256 + 128, py = (ys + (lane >> 3)) * 256 + 128;
+    // pixel-centre rectangles of the two pairs of blocks (there may be no lower pair)
+    const float cx0 = (float)(xs * 256 + 128), cx1 = (float)((min(xs + 8, X1) - 1) * 256 + 128);
+    const float cy0 = (float)(ys * 256 + 128), cy1 = (float)((min(ys + 8, ye) - 1) * 256 + 128);
+    const float cy2 = (float)((ys + 8) * 256 + 128), cy3 = (float)((ye - 1) * 256 + 128);
+    const bool two = ys + 8 < ye;
+    StripSums a;
+    uint4(*list)[LIST] = sm.list[warp];
+    uint32_t *count = sm.count[warp];
+    if (lane < L_COUNT) count[lane] = 0u;
+    for (uint32_t base = it.y; base < it.z; base += 32) {
+        uint4 R = make_uint4(0u, 0u, 1u, 0u);
+        bool up = false, low = false;
+        float ql = 0.0f;
+        if (base + lane < it.z) {
+            R = __ldg(&rec[base + lane]);
+            // Pairs the support may reach: |centre - pixel-centre rectangle|^2 < QL, QL rounded up (2^-18
+            // covers the reciprocal's and the sums' rounding); a pair more only costs time, the clamped
+            // table index decides every pixel.
+            ql = __fdividef(0x1p47f, __uint2float_rn(R.z)) * (1.0f + 0x1p-18f) + 2.0f;
+            const float u = (float)(int)R.x, v = (float)(int)R.y;
+            const float ex = fmaxf(fmaxf(cx0 - u, u - cx1), 0.0f), ex2 = ex * ex;
+            const float eu = fmaxf(fmaxf(cy0 - v, v - cy1), 0.0f), el = fmaxf(fmaxf(cy2 - v, v - cy3), 0.0f);
+            up = fmaf(eu, eu, ex2) < ql;
+            low = two && fmaf(el, el, ex2) < ql;
         }
-        __syncthreads();
-        for (int t = threadIdx.x; t < STAGE; t += RT)
-            if (base + STAGE + t < it.z)
-                cp_async16(raw_addr + 16u * (uint32_t)(t - threadIdx.x), rec + base + STAGE + t);
-        cp_async_commit();
-        if (!kvalid) continue; // warp-uniform
-        // records whose support reaches a pixel centre of a block of this strip: exact test
-        // q_min < QL against each block's pixel-centre rectangle
-        int nf = 0, np = 0, nl = 0;
-        const int nc = (int)sm.ncand[par][scol];
-        for (int j0 = 0; j0 < nc; j0 += 32) {
-            const int j = j0 + lane < nc ? sm.cand[scol][j0 + lane] : 0;
-            unsigned m = 0;
-            bool small = false;
-            if (j0 + lane < nc) {
-                const int4 A = sm.A[j];
-                const uint4 B = sm.B[j];
-                const unsigned long long QL = ((unsigned long long)B.z << 32) | B.x;
-                small = QL <= QL_SMALL;
-                const long long ex = (long long)A.x - (long long)min(max(A.x, cx0), cx1);
-                const unsigned long long ex2 = (unsigned long long)(ex * ex);
-#pragma unroll
-                for (int k = 0; k < SPLAT_SLOTS; ++k) {
-                    if (!(kvalid >> k & 1u)) continue;
-                    const int by = (srow + k * ng) * 4;
-                    const int cy0 = (Y0 + by) * 256 + 128, cy1 = (Y0 + min(by + 3, THc - 1)) * 256 + 128;
-                    const long long ey = (long long)A.y - (long long)min(max(A.y, cy0), cy1);
-                    if (ex2 + (unsigned long long)(ey * ey) < QL) m |= 1u << k;
-                }
-            }
-            const bool tf = m == 0xFu && small, tp = m && m != 0xFu && small, tl = m && !small;
-            const uint32_t mf = __ballot_sync(0xffffffffu, tf), mp = __ballot_sync(0xffffffffu, tp),
-                           ml = __ballot_sync(0xffffffffu, tl);
-            const uint16_t e = (uint16_t)(j | (m << 9));
-            if (tf) lst[nf + __popc(mf & lt)] = e;
-            if (tp) lst[STAGE - 1 - (np + __popc(mp & lt))] = e;
-            if (tl) lrg[nl + __popc(ml & lt)] = e;
-            nf += __popc(mf);
-            np += __popc(mp);
-            nl += __popc(ml);
+        const bool in = up || low;
+        const uint32_t any = __ballot_sync(0xffffffffu, in);
+        __syncwarp(); // the counters and the walks of the round before
+        if (in) {
+            const float W = __uint_as_float(R.w);
+            const bool narrow = ql < 0x1p30f * 0.999f, faint = W < 0x1p23f - 1.0f;
+            int l = up && low ? 0 : (up ? 1 : 2);
+            if (!faint) l += L_LIGHT;
+            if (!narrow) l = L_WIDE;
+            if (!(W < 0x1p32f) || (!narrow && !faint)) l = L_HEAVY;
+            R.w = l >= L_LIGHT && l <= L_LIGHT_LOW ? __float2uint_rn(W) : __float_as_uint(rintf(W));
+            const uint32_t peers = __match_any_sync(any, l), rank = __popc(peers & lt);
+            const uint32_t at = count[l] + rank;
+            list[l][at] = R;
+            __syncwarp(any);
+            if (rank == 0) count[l] = at + __popc(peers);
         }
         __syncwarp();
-        // small records touching all four blocks: no per-block test, four independent chains
-#pragma unroll 4
-        for (int i = 0; i < nf; ++i) {
-            const int j = lst[i] & 511;
-            const int4 A = sm.A[j];
-            const uint2 B = *reinterpret_cast<const uint2 *>(&sm.B[j]); // QL, Wl
-            const int dx = pxv - A.x;
-            const uint32_t dx2 = (uint32_t)(dx * dx);
-            const int dy0 = pyv0 - A.y;
-#pragma unroll
-            for (int k = 0; k < SPLAT_SLOTS; ++k) {
-                const int dy = dy0 + k * dstep;
-                const uint32_t q = dx2 + (uint32_t)(dy * dy);
-                if (q < B.x) {
-                    const uint32_t idx = __umulhi(q, (uint32_t)A.z) >> 5;
-                    const uint32_t kv = (uint32_t)sm.K[idx];
-                    acc[k] += (unsigned long long)(uint32_t)A.w * kv;
-                    acc_lo[k] += (B.y * kv) >> 16;
-                    if (COUNT) ++hk[k];
-                }
+        // lists to walk: the full ones, and after the last round every one that holds a record
+        const uint32_t n = lane < L_COUNT ? count[lane] : 0u;
+        uint32_t todo = __ballot_sync(0xffffffffu, n >= (base + 32 >= it.z ? 1u : (uint32_t)LIST_MIN));
+        while (todo) {
+            const int l = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int m = (int)__shfl_sync(0xffffffffu, n, l);
+            const uint4 *t = list[l];
+            switch (l) {
+            case L_FAINT: walk_faint<0, 4, false, COUNT>(t, m, px, py, sm.Kf, a); break;
+            case L_FAINT_UP: walk_faint<0, 2, false, COUNT>(t, m, px, py, sm.Kf, a); break;
+            case L_FAINT_LOW: walk_faint<2, 2, false, COUNT>(t, m, px, py, sm.Kf, a); break;
+            case L_LIGHT: walk_light<0, 4, COUNT>(t, m, px, py, sm.K, a); break;
+            case L_LIGHT_UP: walk_light<0, 2, COUNT>(t, m, px, py, sm.K, a); break;
+            case L_LIGHT_LOW: walk_light<2, 2, COUNT>(t, m, px, py, sm.K, a); break;
+            case L_WIDE: walk_faint<0, 4, true, COUNT>(t, m, px, py, sm.Kf, a); break;
+            default: walk_heavy<COUNT>(t, m, px, py, sm.K, a); break;
             }
-        }
-        // lanes whose pixel lies outside the tile compute too; their sums are never stored
-#pragma unroll 2
-        for (int i = STAGE - np; i < STAGE; ++i) {
-            const uint32_t e = lst[i];
-            const int j = e & 511;
-            const int4 A = sm.A[j];
-            const uint2 B = *reinterpret_cast<const uint2 *>(&sm.B[j]); // QL, Wl
-            const int dx = pxv - A.x;
-            const uint32_t dx2 = (uint32_t)(dx * dx);
-            const int dy0 = pyv0 - A.y;
-#pragma unroll
-            for (int k = 0; k < SPLAT_SLOTS; ++k) {
-                if (!(e >> (9 + k) & 1u)) continue; // warp-uniform
-                const int dy = dy0 + k * dstep;
-                const uint32_t q = dx2 + (uint32_t)(dy * dy);
-                if (q < B.x) {
-                    const uint32_t idx = __umulhi(q, (uint32_t)A.z) >> 5;
-                    const uint32_t kv = (uint32_t)sm.K[idx];
-                    acc[k] += (unsigned long long)(uint32_t)A.w * kv;
-                    acc_lo[k] += (B.y * kv) >> 16;
-                    if (COUNT) ++hk[k];
-                }
-            }
-        }
-        for (int i = 0; i < nl; ++i) {
-            const uint32_t e = lrg[i];
-            const int j = e & 511;
-            const int4 A = sm.A[j];
-            const uint4 B = sm.B[j];
-            const unsigned long long QL = ((unsigned long long)B.z << 32) | B.x;
-            const int dx = pxv - A.x;
-            const long long dx2 = (long long)dx * dx;
-            const int dy0 = pyv0 - A.y;
-#pragma unroll
-            for (int k = 0; k < SPLAT_SLOTS; ++k) {
-                if (!(e >> (9 + k) & 1u)) continue;
-                const int dy = dy0 + k * dstep;
-                const unsigned long long q = (unsigned long long)(dx2 + (long long)dy * dy);
-                if (q < QL) {
-                    const uint32_t idx = (uint32_t)((q * (unsigned long long)(uint32_t)A.z) >> 37);
-                    const uint32_t kv = (uint32_t)sm.K[idx];
-                    acc[k] += (unsigned long long)(uint32_t)A.w * kv;
-                    acc_lo[k] += (B.y * kv) >> 16;
-                    if (COUNT) ++hk[k];
-                }
-            }
+            if (lane == 0) count[l] = 0u;
         }
     }
 #pragma unroll
     for (int k = 0; k < SPLAT_SLOTS; ++k) {
-        const int pyl = pyl0 + 4 * ng * k;
-        if (!(kvalid >> k & 1u) || pxl >= TWc || pyl >= THc) continue;
-        if (COUNT) hits += hk[k];
-        const unsigned long long v = acc[k] + acc_lo[k];
-        if (v) atomicAdd(&img[(size_t)(Y0 + pyl) * P.W + (X0 + pxl)], v);
+        const int x = xs + (lane & 7), y = ys + (lane >> 3) + 4 * k;
+        if (x >= X1 || y >= ye) continue;
+        if (COUNT) hits += a.hits[k];
+        if (a.acc[k]) atomicAdd(&img[(size_t)y * P.W + x], a.acc[k]);
     }
+}
+
+__device__ __forceinline__ void splat_table(SplatSmem &sm, int kernel)
+{
+    for (int i = threadIdx.x; i <= 1024; i += RT) {
+        sm.K[i] = i < 1024 ? (uint32_t)g_ktab[kernel][i] : 0u;
+        sm.Kf[i] = (float)sm.K[i] * 0x1p-16f;
+    }
+    __syncthreads();
+}
+
+// the next unit of a persistent grid's warp
+__device__ __forceinline__ uint32_t next_unit(unsigned *counter)
+{
+    uint32_t u = 0;
+    if ((threadIdx.x & 31) == 0) u = atomicAdd(counter, 1u);
+    return __shfl_sync(0xffffffffu, u, 0);
 }
 
 template <bool COUNT>
 __global__ void __launch_bounds__(RT, 4) k_splat_tiles(const uint4 *__restrict__ rec, const uint4 *__restrict__ items,
-                                                       Proj P, unsigned long long *__restrict__ img,
-                                                       FrameStatsDev *stats)
+                                                       uint32_t nunits, uint32_t strips, unsigned *next, Proj P,
+                                                       unsigned long long *__restrict__ img, FrameStatsDev *stats)
 {
     extern __shared__ __align__(16) unsigned char splat_smem[];
     SplatSmem &sm = *reinterpret_cast<SplatSmem *>(splat_smem);
-    for (int i = threadIdx.x; i < 1024; i += RT) sm.K[i] = g_ktab[P.kernel][i];
+    splat_table(sm, P.kernel);
     unsigned hits = 0;
-    const uint4 it = items[blockIdx.x];
-    splat_item<COUNT>(rec, it, it.x, P, img, sm, hits);
+    for (uint32_t u = next_unit(next); u < nunits; u = next_unit(next))
+        splat_unit<COUNT>(rec, items[u / strips], (int)(u % strips), P, img, sm, hits);
     if (COUNT) count_hits(hits, stats);
 }
 
@@ -1373,6 +1422,19 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
                       (uint32_t)(h[3] & 0xFFFFFFFFull)};
 }
 
+// R3 over `items` work items: a persistent grid, no more CTAs than the units need
+void launch_splat(bool count, const uint4 *rec, const uint4 *items, uint32_t nitems, unsigned *next, const Proj &P,
+                  unsigned long long *img, FrameStatsDev *stats, cudaStream_t s)
+{
+    const uint32_t strips = strips_of(P.TW, P.TH);
+    const unsigned long long units = (unsigned long long)nitems * strips;
+    if (units > 0xFFFF0000ull) fail(GBLOD_ERR_RANGE, "too many splat work units");
+    const unsigned grid = (unsigned)std::min<unsigned long long>((units + RT / 32 - 1) / (RT / 32),
+                                                                (unsigned long long)persistent_blocks(4));
+    launch(GBLOD_K_SPLAT, count ? k_splat_tiles<true> : k_splat_tiles<false>, dim3(grid), dim3(RT), sizeof(SplatSmem), s, rec,
+           items, (uint32_t)units, strips, next, P, img, stats);
+}
+
 template <class Src>
 void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long long lo, unsigned long long hi,
                const PassCounts &pc, unsigned long long *img, cudaStream_t s)
@@ -1398,9 +1460,8 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
     }
     launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
            (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p, (const uint32_t *)r->item_off.p,
-           r->items.p);
-    launch(GBLOD_K_SPLAT, r->count_updates ? k_splat_tiles<true> : k_splat_tiles<false>, dim3(pc.items), dim3(RT),
-           sizeof(SplatSmem), s, (const uint4 *)r->records.p, (const uint4 *)r->items.p, P, img, r->stats);
+           r->items.p, r->status + 1);
+    launch_splat(r->count_updates, r->records.p, r->items.p, pc.items, r->status + 1, P, img, r->stats, s);
 }
 
 template <class Src>
@@ -1776,32 +1837,18 @@ __global__ void k_bfill_items(uint32_t ntiles, const ViewDev *__restrict__ views
 
 template <bool COUNT>
 __global__ void __launch_bounds__(RT, 4) k_bsplat(const uint4 *__restrict__ rec, const uint4 *__restrict__ items,
-                                                  const uint32_t *nitems_p, uint32_t items_cap,
-                                                  const ViewDev *__restrict__ views, unsigned *next_item,
+                                                  const uint32_t *nitems_p, uint32_t items_cap, uint32_t strips,
+                                                  int kernel, const ViewDev *__restrict__ views, unsigned *next,
                                                   FrameStatsDev *stats)
 {
     extern __shared__ __align__(16) unsigned char splat_smem[];
     SplatSmem &sm = *reinterpret_cast<SplatSmem *>(splat_smem);
-    __shared__ Proj sP;
-    __shared__ uint32_t s_item;
-    int kernel_loaded = -1;
+    splat_table(sm, kernel);
     unsigned hits = 0;
-    const uint32_t nitems = min(*nitems_p, items_cap);
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(next_item, 1u);
-        __syncthreads();
-        const uint32_t i = s_item;
-        if (i >= nitems) break;
-        const uint4 it = items[i];
-        if (threadIdx.x == 0) sP = views[it.w].P;
-        __syncthreads();
-        const Proj P = sP;
-        if (P.kernel != kernel_loaded) {
-            for (int j = threadIdx.x; j < 1024; j += RT) sm.K[j] = g_ktab[P.kernel][j];
-            kernel_loaded = P.kernel;
-        }
-        splat_item<COUNT>(rec, it, it.x, P, views[it.w].accum, sm, hits);
+    const uint32_t nunits = min(*nitems_p, items_cap) * strips;
+    for (uint32_t u = next_unit(next); u < nunits; u = next_unit(next)) {
+        const uint4 it = items[u / strips];
+        splat_unit<COUNT>(rec, it, (int)(u % strips), views[it.w].P, views[it.w].accum, sm, hits);
     }
     if (COUNT) count_hits(hits, stats);
 }
@@ -1904,8 +1951,8 @@ BatchPlan plan_batch(const gblod_view *views, int n, const gblod_render_params &
     return b;
 }
 
-// the splat kernels stage SplatSmem (above the 48 KB a launch may take without opting in)
-void set_splat_smem_limits()
+// the splat kernels' SplatSmem is above the 48 KB a launch may take without opting in
+void set_splat_smem()
 {
     const int bytes = (int)sizeof(SplatSmem);
     GB_CUDA(cudaFuncSetAttribute(k_splat_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
@@ -2014,7 +2061,8 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     // R3: persistent over the items of all views
     launch(GBLOD_K_SPLAT, (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? k_bsplat<true> : k_bsplat<false>, dim3(G), dim3(RT),
            sizeof(SplatSmem), s, (const uint4 *)r->records.p, (const uint4 *)r->items.p,
-           (const uint32_t *)(r->item_off.p + b.ntiles), (uint32_t)items_cap, (const ViewDev *)dv,
+           (const uint32_t *)(r->item_off.p + b.ntiles),
+           (uint32_t)items_cap, strips_of(b.host[0].P.TW, b.host[0].P.TH), b.host[0].P.kernel, (const ViewDev *)dv,
            r->lvl_cnt.p + b.max_levels + 2, r->stats);
     // R4
     if (rp.tone_auto) {
@@ -2031,9 +2079,9 @@ namespace {
 void renderer_init(gblod_renderer *r, cudaStream_t s)
 {
     ensure_tables();
-    r->status = static_cast<unsigned *>(r->A.get(sizeof(unsigned), s));
+    r->status = static_cast<unsigned *>(r->A.get(2 * sizeof(unsigned), s)); // and the splat's unit counter
     r->stats = static_cast<FrameStatsDev *>(r->A.get(sizeof(FrameStatsDev), s));
-    GB_CUDA(cudaMemsetAsync(r->status, 0, sizeof(unsigned), s));
+    GB_CUDA(cudaMemsetAsync(r->status, 0, 2 * sizeof(unsigned), s));
     GB_CUDA(cudaMemsetAsync(r->stats, 0, sizeof(FrameStatsDev), s));
     GB_CUDA(cudaStreamSynchronize(s));
 }
@@ -2043,7 +2091,7 @@ void renderer_release(gblod_renderer *r)
     cudaStream_t s = r->last_stream;
     const Allocator &A = r->A;
     if (s) (void)cudaStreamSynchronize(s);
-    A.put(r->status, sizeof(unsigned), s);
+    A.put(r->status, 2 * sizeof(unsigned), s);
     A.put(r->stats, sizeof(FrameStatsDev), s);
     r->frontA.release(A, s); r->frontB.release(A, s); r->sel.release(A, s); r->lvl_cnt.release(A, s);
     r->sel_pfx.release(A, s); r->sel_base.release(A, s);
@@ -2198,7 +2246,7 @@ constexpr size_t NA_OFF_ITEM_OFF = NA_OFF_ITEM_CNT + na_align(NA_TILES * 4);
 constexpr size_t NA_OFF_SCAN = NA_OFF_ITEM_OFF + na_align((NA_TILES + 1) * 4);
 constexpr size_t NA_OFF_STATS = NA_OFF_SCAN + na_align(NA_SCAN_BYTES);
 constexpr size_t NA_OFF_STATUS = NA_OFF_STATS + na_align(sizeof(FrameStatsDev));
-constexpr size_t NA_OFF_MAXV = NA_OFF_STATUS + na_align(sizeof(unsigned));
+constexpr size_t NA_OFF_MAXV = NA_OFF_STATUS + na_align(2 * sizeof(unsigned)); // status, the splat's unit counter
 constexpr size_t NA_BYTES = NA_OFF_MAXV + na_align(sizeof(unsigned long long));
 static_assert(NA_BYTES == GBLOD_NOALLOC_SCRATCH_BYTES, "GBLOD_NOALLOC_SCRATCH_BYTES must match the layout");
 // the two scans of NA_TILES counts find their temp space large enough and never allocate
@@ -2293,9 +2341,8 @@ gblod_status render_brute_noalloc(const float *xyz, const float *mass, const flo
            tile_cur, records, img,
            (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? stats : (FrameStatsDev *)nullptr);
     launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((nt + 255) / 256), dim3(256), 0, s, nt,
-           (const uint32_t *)tile_cnt, (const uint32_t *)tile_off, (const uint32_t *)item_off, items);
-    launch(GBLOD_K_SPLAT, (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? k_splat_tiles<true> : k_splat_tiles<false>,
-           dim3(nitems), dim3(RT), sizeof(SplatSmem), s, (const uint4 *)records, (const uint4 *)items, P, img, stats);
+           (const uint32_t *)tile_cnt, (const uint32_t *)tile_off, (const uint32_t *)item_off, items, status + 1);
+    launch_splat((rp.flags & GBLOD_RENDER_COUNT_UPDATES) != 0, records, items, nitems, status + 1, P, img, stats, s);
     if (image) {
         double lo = 0.0, hi = 0.0;
         if (rp.tone_auto) {
