@@ -42,18 +42,30 @@ __global__ void k_mass_check(const float *mass, size_t n, unsigned *minb, unsign
     }
 }
 
-// pow2: the root cube starts at 0 and scale is a power of two in fp32 range (the fp32 product is exact)
-__global__ void k_morton(const float *__restrict__ xyz, const uint32_t *__restrict__ order, size_t n, double lx,
-                         double ly, double lz, double scale, uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
-                         int pow2)
+// Keys, the particles packed for the gather by sorted position (one aligned 16-byte read each instead
+// of 12 + 4 bytes from two arrays), and the OR of every key's difference from particle 0's (which
+// digits the sort must pass over).  pow2: the root cube starts at 0 and scale is a power of two in fp32
+// range (the fp32 product is exact)
+__global__ void k_morton(const float *__restrict__ xyz, const float *__restrict__ h,
+                         const uint32_t *__restrict__ order, size_t n, double lx, double ly, double lz, double scale,
+                         uint64_t *__restrict__ keys, uint32_t *__restrict__ vals, float4 *__restrict__ pack,
+                         unsigned long long *diff, int pow2)
 {
     const float sf = (float)scale;
+    const uint64_t key0 = pow2 ? gbd::morton_key_pow2(xyz[0], xyz[1], xyz[2], sf)
+                               : gbd::morton_key(xyz[0], xyz[1], xyz[2], lx, ly, lz, scale);
+    uint64_t acc = 0;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const size_t src = order ? (size_t)order[i] : i;
         const float x = xyz[3 * src], y = xyz[3 * src + 1], z = xyz[3 * src + 2];
-        keys[i] = pow2 ? gbd::morton_key_pow2(x, y, z, sf) : gbd::morton_key(x, y, z, lx, ly, lz, scale);
+        const uint64_t key = pow2 ? gbd::morton_key_pow2(x, y, z, sf) : gbd::morton_key(x, y, z, lx, ly, lz, scale);
+        keys[i] = key;
+        acc |= key ^ key0;
         if (!order) vals[i] = (uint32_t)i;
+        pack[src] = make_float4(x, y, z, h[src]);
     }
+    for (int d = 16; d > 0; d >>= 1) acc |= __shfl_xor_sync(0xffffffffu, acc, d);
+    if ((threadIdx.x & 31) == 0 && acc) atomicOr(diff, (unsigned long long)acc);
 }
 
 __global__ void k_id_keys(const uint32_t *ids, size_t n, uint64_t *keys, uint32_t *vals)
@@ -64,46 +76,38 @@ __global__ void k_id_keys(const uint32_t *ids, size_t n, uint64_t *keys, uint32_
     }
 }
 
-// Particles in sorted order: s4 = (x, y, z, m), sh = h, sid = the caller's id (written only when
-// the caller gave ids: otherwise it equals perm), mfix = the fixed-point mass (written only for
-// unequal masses: with one mass m0 for all, a node's exact mass is its count times m0's, and the
-// mass array is not read).
-__global__ void k_gather_sorted(const float *__restrict__ xyz, const float *__restrict__ mass,
-                                const float *__restrict__ h, const uint32_t *__restrict__ ids,
-                                const uint32_t *__restrict__ perm, size_t n, float4 *__restrict__ s4,
-                                float *__restrict__ sh, uint32_t *__restrict__ sid, U128 *__restrict__ mfix,
-                                int equal_mass, float m0)
+// Particles in sorted order: s4 = (x, y, z, h), sm = mass (written only for unequal masses: with one
+// mass m0 for all the mass array is not read), sid = the caller's id (written only when the caller gave
+// ids: otherwise it equals perm), mfix = the fixed-point mass (unequal masses only: else a node's
+// exact mass is its count times m0's).  Bound by random 16-byte reads (150M: 7.2 ms from the
+// caller's arrays, 36 ms of build + frame; 3.6 ms from the packed ones).
+__global__ void k_gather_sorted(const float4 *__restrict__ pack, const float *__restrict__ mass,
+                                const uint32_t *__restrict__ ids, const uint32_t *__restrict__ perm, size_t n,
+                                float4 *__restrict__ s4, float *__restrict__ sm, uint32_t *__restrict__ sid,
+                                U128 *__restrict__ mfix)
 {
     // four independent elements per thread and iteration (each a coalesced sweep of the sorted
     // order), so that four random reads of the particle arrays are in flight at a time
     constexpr int GU = 4;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t j0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j0 < n; j0 += stride * GU) {
-        size_t i[GU];
-        float x[GU], y[GU], z[GU], m[GU], hh[GU];
+        uint32_t i[GU];
+        float4 p[GU];
 #pragma unroll
-        for (int u = 0; u < GU; ++u) {
-            const size_t j = j0 + u * stride;
-            i[u] = j < n ? (size_t)perm[j] : 0;
-        }
+        for (int u = 0; u < GU; ++u) i[u] = j0 + u * stride < n ? perm[j0 + u * stride] : 0u;
 #pragma unroll
-        for (int u = 0; u < GU; ++u) {
-            if (j0 + u * stride < n) {
-                x[u] = xyz[3 * i[u]];
-                y[u] = xyz[3 * i[u] + 1];
-                z[u] = xyz[3 * i[u] + 2];
-                m[u] = equal_mass ? m0 : mass[i[u]];
-                hh[u] = h[i[u]];
-            }
-        }
+        for (int u = 0; u < GU; ++u) p[u] = pack[i[u]];
 #pragma unroll
         for (int u = 0; u < GU; ++u) {
             const size_t j = j0 + u * stride;
             if (j < n) {
-                s4[j] = make_float4(x[u], y[u], z[u], m[u]);
-                sh[j] = hh[u];
+                s4[j] = p[u];
                 if (sid) sid[j] = ids[i[u]];
-                if (mfix) mfix[j] = gbd::mass_fixed(m[u]);
+                if (mfix) {
+                    const float m = mass[i[u]];
+                    sm[j] = m;
+                    mfix[j] = gbd::mass_fixed(m);
+                }
             }
         }
     }
@@ -240,7 +244,7 @@ __global__ void k_node_mass(size_t nn, size_t n, const uint32_t *first, const ui
 // bounds; leaves: largest h.  One block per node (grid-stride), NaN coordinates are skipped.
 __global__ void k_leaf_nodes(size_t nn, const uint32_t *__restrict__ flags, const uint32_t *__restrict__ first,
                              const uint32_t *__restrict__ count, const uint64_t *__restrict__ pfirst,
-                             const float4 *__restrict__ s4, const float *__restrict__ sh, float4 *__restrict__ pts4,
+                             const float4 *__restrict__ s4, const float *__restrict__ sm, float m0, float4 *__restrict__ pts4,
                              float *__restrict__ hs, uint32_t *__restrict__ pt_src, float *__restrict__ bmin,
                              float *__restrict__ bmax, unsigned *__restrict__ hmax_bits)
 {
@@ -263,8 +267,8 @@ __global__ void k_leaf_nodes(size_t nn, const uint32_t *__restrict__ flags, cons
             mx1 = fmaxf(mx1, p.y);
             mx2 = fmaxf(mx2, p.z);
             if (leaf) {
-                const float h = sh[b + k];
-                pts4[pf + k] = p;
+                const float h = p.w;
+                pts4[pf + k] = make_float4(p.x, p.y, p.z, sm ? sm[b + k] : m0);
                 hs[pf + k] = h;
                 pt_src[pf + k] = b + k;
                 hm = h > hm ? h : hm;
@@ -457,24 +461,32 @@ struct BuildTemps {
 
 static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const float *mass, const float *h,
                                        const uint32_t *ids, uint64_t n, const gblod_build_params &p,
-                                       const Allocator &A, cudaStream_t s);
+                                       const Allocator &A, cudaStream_t s, bool roomy);
 
 gblod_octree *build_octree(const float *xyz, const float *mass, const float *h, const uint32_t *ids, uint64_t n,
                            const gblod_build_params &p, const Allocator &A, cudaStream_t s)
 {
-    gblod_octree *o = new gblod_octree();
-    try {
-        return build_octree_impl(o, xyz, mass, h, ids, n, p, A, s);
-    } catch (...) {
-        (void)cudaStreamSynchronize(s);
-        free_octree(o);
-        throw;
+    // A roomy build's work arrays peak at about 94 bytes a particle, a lean one's at 66.  Memory from a
+    // caller's allocator is spent leanly; from the library's pool leanly only when roomy does not fit.
+    for (bool roomy = !A.has_hook;; roomy = false) {
+        gblod_octree *o = new gblod_octree();
+        try {
+            return build_octree_impl(o, xyz, mass, h, ids, n, p, A, s, roomy);
+        } catch (const Error &e) {
+            (void)cudaStreamSynchronize(s);
+            free_octree(o);
+            if (e.st != GBLOD_ERR_OOM || !roomy) throw;
+        } catch (...) {
+            (void)cudaStreamSynchronize(s);
+            free_octree(o);
+            throw;
+        }
     }
 }
 
 static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const float *mass, const float *h,
                                        const uint32_t *ids, uint64_t n, const gblod_build_params &p,
-                                       const Allocator &A, cudaStream_t s)
+                                       const Allocator &A, cudaStream_t s, bool roomy)
 {
     HostStage hs;
     BuildTemps tmp(A, s);
@@ -509,31 +521,49 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
         std::memcpy(&m0, &hm[0], sizeof(float));
     }
 
-    // A1 + A2: keys in (key, id) order
-    Scratch<uint64_t> keyA(A, n, s), keyB(A, n, s);
-    Scratch<uint32_t> valA(A, n, s), valB(A, n, s);
+    // A1 + A2: keys in (key, id) order.  Roomy builds hold all work arrays of the sort and the sorted
+    // particles in one block: the pool then finds the same few sizes free in every build (with an array
+    // each, the next build's requests split the freed blocks and the pool maps memory anew: 5 ms at 150M).
+    const size_t n16 = (n + 3) / 4 * 4; // keeps the parts of the block 16-byte aligned
+    Scratch<float4> block(A, roomy ? 2 * n16 + n16 / 2 + n16 / 4 : 0, s);
+    Scratch<uint64_t> keyA(A, n, s), keyB(A, roomy ? 0 : n, s);
+    Scratch<uint32_t> valA(A, n, s), valB(A, roomy ? 0 : n, s);
+    Scratch<float4> own_pack(A, roomy ? 0 : n, s);
+    float4 *pack = roomy ? block.p + n16 : own_pack.p;
+    uint64_t *kalt = roomy ? reinterpret_cast<uint64_t *>(block.p + 2 * n16) : keyB.p;
+    uint32_t *valt = roomy ? reinterpret_cast<uint32_t *>(block.p + 2 * n16 + n16 / 2) : valB.p;
     uint64_t *keys = keyA.p;
     uint32_t *vals = valA.p;
+    auto other_key = [&] { return keys == keyA.p ? kalt : keyA.p; };
+    auto other_val = [&] { return vals == valA.p ? valt : valA.p; };
     const double scale = 2097152.0 / p.root_side;
     int sexp = 0;
     const int pow2 = p.root_lo[0] == 0.0 && p.root_lo[1] == 0.0 && p.root_lo[2] == 0.0 &&
                      std::frexp(scale, &sexp) == 0.5 && sexp > -120 && sexp < 120 ? 1 : 0;
+    Scratch<unsigned long long> diff(A, 1, s);
+    GB_CUDA(cudaMemsetAsync(diff.p, 0, sizeof(unsigned long long), s));
     if (ids) {
         launch(GBLOD_K_BUILD_OTHER, k_id_keys, dim3(G), dim3(T), 0, s, ids, (size_t)n, keys, vals);
-        radix_sort_pairs(A, sort, &keys, &vals, keys == keyA.p ? keyB.p : keyA.p, vals == valA.p ? valB.p : valA.p,
-                         n, 32, s, hs);
+        radix_sort_pairs(A, sort, &keys, &vals, other_key(), other_val(), n, 32, s, hs);
         // vals = input indices in id order; keys in that order
-        uint64_t *kdst = keys == keyA.p ? keyB.p : keyA.p;
-        launch(GBLOD_K_MORTON, k_morton, dim3(G), dim3(T), 0, s, xyz, (const uint32_t *)vals, (size_t)n, p.root_lo[0],
-               p.root_lo[1], p.root_lo[2], scale, kdst, (uint32_t *)nullptr, pow2);
+        uint64_t *kdst = other_key();
+        launch(GBLOD_K_MORTON, k_morton, dim3(G), dim3(T), 0, s, xyz, h, (const uint32_t *)vals, (size_t)n,
+               p.root_lo[0], p.root_lo[1], p.root_lo[2], scale, kdst, (uint32_t *)nullptr, pack, diff.p, pow2);
         keys = kdst;
     } else {
-        launch(GBLOD_K_MORTON, k_morton, dim3(G), dim3(T), 0, s, xyz, (const uint32_t *)nullptr, (size_t)n,
-               p.root_lo[0], p.root_lo[1], p.root_lo[2], scale, keys, vals, pow2);
+        launch(GBLOD_K_MORTON, k_morton, dim3(G), dim3(T), 0, s, xyz, h, (const uint32_t *)nullptr, (size_t)n,
+               p.root_lo[0], p.root_lo[1], p.root_lo[2], scale, keys, vals, pack, diff.p, pow2);
     }
-    radix_sort_pairs(A, sort, &keys, &vals, keys == keyA.p ? keyB.p : keyA.p, vals == valA.p ? valB.p : valA.p, n, 63,
-                     s, hs);
+    radix_sort_pairs(A, sort, &keys, &vals, other_key(), other_val(), n, 63, s, hs, diff.p);
     // keep the sorted keys and permutation in the octree
+    if (keys == kalt && roomy) {
+        GB_CUDA(cudaMemcpyAsync(keyA.p, keys, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
+        keys = keyA.p;
+    }
+    if (vals == valt && roomy) {
+        GB_CUDA(cudaMemcpyAsync(valA.p, vals, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+        vals = valA.p;
+    }
     uint64_t *skey = keys;
     uint32_t *sidx = vals;
     if (skey == keyA.p) keyA.release_ptr(); else keyB.release_ptr();
@@ -543,14 +573,16 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
     keyA.reset(); keyB.reset(); valA.reset(); valB.reset();
 
     // sorted particle arrays and fixed-point masses (with no caller ids the sorted ids are sidx;
-    // with equal masses no prefix of masses is needed)
-    Scratch<float4> s4(A, n, s);
-    Scratch<float> sh(A, n, s);
+    // with equal masses no sorted masses and no prefix of them are needed)
+    Scratch<float4> own_s4(A, roomy ? 0 : n, s);
+    float4 *s4 = roomy ? block.p : own_s4.p;
+    Scratch<float> sm(A, o->equal_mass ? 1 : n, s);
     Scratch<uint32_t> sid(A, ids ? n : 1, s);
     Scratch<U128> mpre(A, o->equal_mass ? 1 : n, s), mtot(A, 1, s);
-    launch(GBLOD_K_BUILD_OTHER, k_gather_sorted, dim3(G), dim3(T), 0, s, xyz, mass, h, ids, (const uint32_t *)sidx,
-           (size_t)n, s4.p, sh.p, ids ? sid.p : (uint32_t *)nullptr, o->equal_mass ? (U128 *)nullptr : mpre.p,
-           o->equal_mass, m0);
+    launch(GBLOD_K_BUILD_OTHER, k_gather_sorted, dim3(G), dim3(T), 0, s, (const float4 *)pack, mass, ids,
+           (const uint32_t *)sidx, (size_t)n, s4, sm.p, ids ? sid.p : (uint32_t *)nullptr,
+           o->equal_mass ? (U128 *)nullptr : mpre.p);
+    own_pack.reset();
     if (!o->equal_mass) scan_exclusive_u128(A, scan, mpre.p, mpre.p, n, mtot.p, s);
     const uint32_t *sorted_ids = ids ? sid.p : sidx;
 
@@ -614,7 +646,7 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
         Scratch<uint32_t> reps(A, n_rep, s);
         launch(GBLOD_K_BUILD_OTHER, k_compact_reps, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn,
                (const uint32_t *)isrep.p, (const uint32_t *)reppos.p, reps.p);
-        SelectIn in{s4.p, sh.p, sorted_ids, N.code.p, N.first.p, N.count.p, pfirst.p, w.p, sc.p, hmax.p,
+        SelectIn in{s4, sm.p, sorted_ids, N.code.p, N.first.p, N.count.p, pfirst.p, w.p, sc.p, hmax.p,
                     o->pts4, o->hs, o->pt_src, p.n_max};
         select_representatives(A, s, hs, scan, in, reps.p, n_rep, p.n_max, p.seed, o->equal_mass);
     }
@@ -622,8 +654,8 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
     // leaves, bounds, cull radii
     launch(GBLOD_K_BUILD_OTHER, k_leaf_nodes, dim3((unsigned)std::min<size_t>(nn, 65535 * 4)), dim3(T), 0, s, nn,
            (const uint32_t *)flags.p, (const uint32_t *)N.first.p, (const uint32_t *)N.count.p,
-           (const uint64_t *)pfirst.p, (const float4 *)s4.p, (const float *)sh.p, o->pts4, o->hs, o->pt_src, bmin.p,
-           bmax.p, hmax.p);
+           (const uint64_t *)pfirst.p, (const float4 *)s4, o->equal_mass ? (const float *)nullptr : (const float *)sm.p,
+           m0, o->pts4, o->hs, o->pt_src, bmin.p, bmax.p, hmax.p);
     for (int d = o->depth_max; d >= 0; --d) {
         const uint64_t L = level_first[d];
         const uint32_t nd = (uint32_t)(level_first[d + 1] - L);

@@ -176,9 +176,11 @@ struct SortTmp {
 };
 // Stable LSD radix sort of (keys, vals) ascending by bits [0, key_bits) of the key.  On return
 // the sorted data is in (*keys, *vals), which point either to the input or to the alternate
-// buffers.  Digits that are constant over all keys are skipped.
+// buffers.  Digits that are constant over all keys are skipped: varying_bits (device), if given, holds
+// the OR of key ^ (any one key) over all keys.
 void radix_sort_pairs(const Allocator &A, SortTmp &t, uint64_t **keys, uint32_t **vals, uint64_t *keys_alt,
-                      uint32_t *vals_alt, size_t n, int key_bits, cudaStream_t s, HostStage &hs);
+                      uint32_t *vals_alt, size_t n, int key_bits, cudaStream_t s, HostStage &hs,
+                      const unsigned long long *varying_bits = nullptr);
 
 } // namespace gb
 

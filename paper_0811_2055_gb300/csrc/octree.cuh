@@ -61,8 +61,8 @@ __device__ __forceinline__ void block_decode(const ushort4 q, uint32_t cw, const
 
 // Work arrays the subselection reads and writes (all device pointers).
 struct SelectIn {
-    const float4 *s4;        // sorted particles (x, y, z, mass)
-    const float *sh;         // sorted smoothing lengths
+    const float4 *s4;        // sorted particles (x, y, z, h)
+    const float *sm;         // sorted masses (read for unequal masses only)
     const uint32_t *sid;     // sorted ids
     const uint64_t *ncode;   // per node
     const uint32_t *nfirst;  // per node

@@ -75,7 +75,7 @@ __device__ __forceinline__ uint64_t sel_key(const SelectIn &in, uint32_t j, uint
     id = in.sid[j];
     const uint64_t u = gbd::node_draw(seed, code, id);
     if (equal_mass) return u;
-    const double k = __ddiv_rn(gbd::neg_log_unit(u), (double)in.s4[j].w);
+    const double k = __ddiv_rn(gbd::neg_log_unit(u), (double)in.sm[j]);
     return (uint64_t)__double_as_longlong(k);
 }
 
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(ST) k_sel_write(SelectIn in, RepInfo R, uint32
             const uint64_t idx = pf + rank;
             const uint32_t j = C.first + C.start + wi * 32 + lane;
             const float4 p = in.s4[j];
-            const float h = __fmul_rn(in.sh[j], sr);
+            const float h = __fmul_rn(p.w, sr);
             in.pts4[idx] = make_float4(p.x, p.y, p.z, wr);
             in.hs[idx] = h;
             in.pt_src[idx] = j;
