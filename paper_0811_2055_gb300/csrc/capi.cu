@@ -406,8 +406,7 @@ gblod_status gblod_diff_render(gblod_renderer *r, const float *d_xyz, const floa
         if (n > 0 && (!d_xyz || !d_w || !d_logh)) fail(GBLOD_ERR_INVALID_ARG, "point arrays must not be NULL");
         const gblod_render_params p = check_params(params);
         for (int i = 0; i < n_views; ++i) check_camera(&cams[i]);
-        diff_pass(r, d_xyz, d_w, d_logh, n, cams, n_views, p, d_images, nullptr, nullptr, nullptr, nullptr,
-                  (cudaStream_t)stream);
+        diff_forward(r, d_xyz, d_w, d_logh, n, cams, n_views, p, d_images, (cudaStream_t)stream);
     });
 }
 
@@ -422,8 +421,8 @@ gblod_status gblod_diff_backward(gblod_renderer *r, const float *d_xyz, const fl
             fail(GBLOD_ERR_INVALID_ARG, "point and gradient arrays must not be NULL");
         const gblod_render_params p = check_params(params);
         for (int i = 0; i < n_views; ++i) check_camera(&cams[i]);
-        diff_pass(r, d_xyz, d_w, d_logh, n, cams, n_views, p, nullptr, d_grad_images, d_grad_xyz, d_grad_w,
-                  d_grad_logh, (cudaStream_t)stream);
+        diff_backward(r, d_xyz, d_w, d_logh, n, cams, n_views, p, d_grad_images, d_grad_xyz, d_grad_w, d_grad_logh,
+                      (cudaStream_t)stream);
     });
 }
 

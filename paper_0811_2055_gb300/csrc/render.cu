@@ -2103,8 +2103,8 @@ void renderer_release(gblod_renderer *r)
     r->pass_stats.release(A, s);
     r->b_views.release(A, s); r->b_frontA.release(A, s); r->b_frontB.release(A, s); r->b_sel.release(A, s);
     r->b_counts.release(A, s); r->b_pfx.release(A, s); r->b_base.release(A, s);
-    r->d_cams.release(A, s); r->d_rec.release(A, s); r->d_cnt.release(A, s); r->d_off.release(A, s);
-    r->d_cur.release(A, s); r->d_icnt.release(A, s); r->d_ioff.release(A, s); r->d_items.release(A, s);
+    r->d_cams.release(A, s); r->d_rec.release(A, s); r->d_hist.release(A, s); r->d_off.release(A, s);
+    r->d_cnt.release(A, s); r->d_items.release(A, s); r->d_big.release(A, s);
     r->scan.buf.release(A, s);
 }
 
