@@ -239,7 +239,7 @@ __device__ __forceinline__ unsigned walk_boxes(const BoxWalk &b, uint32_t tag, T
     }
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
     const uint32_t excl = incl - b.n;
-    __shared__ uint8_t owner_at[RT / 32][32];
+    __shared__ uint8_t owner_at[32][32]; // blocks of up to 1024 threads
     uint8_t *own = owner_at[threadIdx.x >> 5];
     unsigned hits = 0;
     int carry = 0; // owner of the previous window's last pair
@@ -278,6 +278,101 @@ __device__ __forceinline__ unsigned walk_boxes(const BoxWalk &b, uint32_t tag, T
                 ++hits;
             }
         }
+    }
+    return hits;
+}
+
+// The per-pixel rule over boxes of at most 8 x 8 pixels, four points at a time: a group of eight lanes
+// takes one point of the warp's (on: this lane has one), a column per lane, row by row.  A round of 32
+// (point, pixel) pairs is about 14 instructions, where walk_boxes spends some 66 more on finding each
+// pair's point and shuffling its operands; columns and rows a box does not have idle.  Distances in 32
+// bits and Wq < 2^32 (group_box decides; walk_boxes takes the rest).  K has a zero entry 1024.  add(x, y, c)
+// receives every nonzero contribution c < 2^32.  Returns this lane's pixel updates (COUNT).  Every lane of the
+// warp calls it.  Small boxes of 150M particles, the whole box in view (k_splat_small): 7.9 ms walked, 8.1 ms with
+// this alone, 6.6 ms with the smallest boxes in lane_boxes (the shuffles and lookups of idle lanes bind
+// here: the additions alone are 0.8 ms).  LOD scatter of 16.8M particles 0.59 -> 0.43 ms.
+__device__ __forceinline__ bool group_box(int r, float Wf) { return r <= R_NARROW && Wf < 0x1p32f; }
+
+template <bool COUNT, class Add>
+__device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t S, float Wf, int x0, int x1, int y0,
+                                                int y1, const int32_t *K, Add add)
+{
+    static_assert(DIRECT_BOX <= 8, "a group's lanes are the columns of a box");
+    const uint32_t m = __ballot_sync(0xffffffffu, on);
+    if (!m) return 0u;
+    const int lane = threadIdx.x & 31, col = lane & 7;
+    __shared__ uint8_t nth[32][32]; // lanes that have a point, in order
+    uint8_t *own = nth[threadIdx.x >> 5];
+    __syncwarp();
+    if (on) own[__popc(m & gbd::lanemask_lt())] = (uint8_t)lane;
+    __syncwarp();
+    const uint32_t Wq = on ? __float2uint_rn(Wf) : 0u, xy = (uint32_t)x0 | (uint32_t)y0 << 16;
+    const uint32_t ext = (uint32_t)(x1 - x0) | (uint32_t)(y1 - y0) << 8;
+    const int n = __popc(m);
+    unsigned hits = 0;
+    for (int r = 0; r < n; r += 4) {
+        const int k = r + (lane >> 3);
+        const int src = own[min(k, n - 1)];
+        const uint32_t qxy = __shfl_sync(0xffffffffu, xy, src), qext = __shfl_sync(0xffffffffu, ext, src);
+        const int qU = __shfl_sync(0xffffffffu, U, src), qV = __shfl_sync(0xffffffffu, V, src);
+        const uint32_t qS = __shfl_sync(0xffffffffu, S, src), qW = __shfl_sync(0xffffffffu, Wq, src);
+        const uint32_t Wh = qW >> 16, Wl = qW & 0xFFFFu;
+        const bool act = k < n && col <= (int)(qext & 0xFFu);
+        const int rows = act ? (int)(qext >> 8) + 1 : 0;
+        const int x = (int)(qxy & 0xFFFFu) + col, y = (int)(qxy >> 16);
+        const int dx = x * 256 + 128 - qU;
+        const uint32_t dx2 = (uint32_t)(dx * dx);
+        const int dy = y * 256 + 128 - qV;
+        const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)rows);
+        for (int j0 = 0; j0 < most; j0 += 4) { // four rows' lookups in flight, no branch but the additions
+            uint32_t c[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int d = dy + (j0 + j) * 256;
+                const uint32_t idx = j0 + j < rows ? min(__umulhi(dx2 + (uint32_t)(d * d), qS) >> 5, 1024u) : 1024u;
+                const uint32_t kv = (uint32_t)K[idx];
+                c[j] = Wh * kv + ((Wl * kv) >> 16);
+                if (COUNT) hits += idx < 1024u ? 1u : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c[j]) add(x, y + j0 + j, c[j]);
+        }
+    }
+    return hits;
+}
+
+// The same for boxes of at most LANE_BOX x LANE_BOX pixels, one per lane: nothing is shuffled, and 32
+// different points' table reads and additions go out together.
+constexpr int LANE_BOX = 4;
+template <bool COUNT, class Add>
+__device__ __forceinline__ unsigned lane_boxes(bool on, int U, int V, uint32_t S, float Wf, int x0, int x1, int y0,
+                                               int y1, const int32_t *K, Add add)
+{
+    const int bw = on ? x1 - x0 + 1 : 0, bh = on ? y1 - y0 + 1 : 0;
+    const int mh = (int)__reduce_max_sync(0xffffffffu, (unsigned)bh);
+    const uint32_t Wq = on ? __float2uint_rn(Wf) : 0u, Wh = Wq >> 16, Wl = Wq & 0xFFFFu;
+    uint32_t dx2[LANE_BOX];
+#pragma unroll
+    for (int c = 0; c < LANE_BOX; ++c) {
+        const int dx = (x0 + c) * 256 + 128 - U;
+        dx2[c] = (uint32_t)(dx * dx);
+    }
+    unsigned hits = 0;
+    for (int j = 0; j < mh; ++j) {
+        const int dy = (y0 + j) * 256 + 128 - V;
+        const uint32_t dy2 = (uint32_t)(dy * dy);
+        uint32_t v[LANE_BOX];
+#pragma unroll
+        for (int c = 0; c < LANE_BOX; ++c) {
+            const uint32_t idx = c < bw && j < bh ? min(__umulhi(dx2[c] + dy2, S) >> 5, 1024u) : 1024u;
+            const uint32_t kv = (uint32_t)K[idx];
+            v[c] = Wh * kv + ((Wl * kv) >> 16);
+            if (COUNT) hits += idx < 1024u ? 1u : 0u;
+        }
+#pragma unroll
+        for (int c = 0; c < LANE_BOX; ++c)
+            if (v[c]) add(x0 + c, y0 + j, v[c]);
     }
     return hits;
 }
@@ -477,6 +572,7 @@ struct SrcLOD {
     const int64_t *base;
     const uint32_t *nsel;
     const unsigned long long *total;
+    unsigned long long bound; // host: at least the number of points
 };
 
 // selected nodes' 16-bit block codes (decoded on load)
@@ -489,7 +585,7 @@ struct SrcLODQ : SrcLOD {
 
 struct SrcFlat {
     const float *xyz, *mass, *h;
-    unsigned long long n;
+    unsigned long long n, bound;
 };
 
 __device__ __forceinline__ unsigned long long src_total(const SrcLOD &s) { return *s.total; }
@@ -744,40 +840,48 @@ __global__ void __launch_bounds__(RT, 4) k_project_scatter(Src src, Proj P, unsi
     if (cstats) count_hits(hits, cstats);
 }
 
-// Partitioned binning for point sources in no spatial order (the caller's particle arrays): the
-// warp-level aggregation of the per-tile counters above finds few equal tiles in a warp there, so
-// every (splat, tile) pair would be one global atomic on one of a few thousand counters.  Instead
-// each CTA of the persistent grid counts its own points per tile in shared memory and writes one
-// histogram, tile-major: hist[t * G + cta].  An exclusive scan of the histograms gives every CTA
+// Partitioned binning.  Each CTA of the grid counts its own points per tile in shared memory and writes
+// one histogram, tile-major: hist[t * G + cta].  An exclusive scan of the histograms gives every CTA
 // its own base in every tile, so the scatter pass places records with shared-memory atomics only,
 // and the records of a tile keep the order of the CTAs.  Both passes walk the same chunks (the same
-// grid G and chunk stride), so they see the same points.  Points whose pixel box is at most
-// DIRECT_BOX on a side are binned too, into a second record stream (their own histograms, after the
-// binned points' in the same scan), and splatted by k_splat_small into a shared-memory tile image:
-// in no spatial order, adding them straight to the image would be one global atomic per pixel at
-// random addresses.
-constexpr uint32_t PART_MAX_TILES = 4096; // two shared-memory histograms: 32 KB
-constexpr uint32_t ITEM_SMALL = 4096;     // small records per k_splat_small work item
+// grid G and chunk stride), so they see the same points.  (Global counters need the pairs of a warp
+// grouped by tile: __match_any_sync loops over the distinct tiles, up to 260 cycles a round.  LOD frames,
+// count + scatter: 16.8M particles 1080p 2.07 ms with it, 0.58 ms so; 150M near view 5.4, 2.1 ms.)
+//
+// Points whose pixel box is at most DIRECT_BOX on a side: of an octree's nodes (SMALL false), the scatter
+// pass adds their contributions straight to the image (neighbours in the order are neighbours in
+// space); of a caller's arrays in no spatial order (SMALL true) they are binned too, into a second
+// record stream (their own histograms, after the binned points' in the same scan), and splatted by
+// k_splat_small into a shared-memory tile image: added straight to the image, every pixel would be a
+// global atomic at a random address.
+// One CTA of 1024 threads per SM for unordered points: every CTA writes into all tiles' records, and a
+// quarter of the CTAs leaves a quarter of the half-written lines open in L2 (16.8M particles, scatter 1.00 ->
+// 0.64 ms); an octree's points reach few tiles at a time, and four CTAs of 256 overlap better (0.59
+// against 0.66).
+template <bool SMALL> constexpr int PART_THREADS = SMALL ? 1024 : 256;
+constexpr size_t PART_MAX_SMEM = 200 * 1024; // shared-memory histograms: frames of more tiles take the global counters
+constexpr uint32_t ITEM_SMALL = 4096;        // small records per k_splat_small work item
 
-template <class Src>
-__global__ void __launch_bounds__(RT, 4) k_project_hist(Src src, Proj P, unsigned long long e_lo,
-                                                     unsigned long long e_hi, uint32_t *__restrict__ hist,
-                                                     unsigned *status, FrameStatsDev *stats)
+template <class Src, bool SMALL>
+__global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL>) k_project_hist(Src src, Proj P, unsigned long long e_lo,
+                                                     unsigned long long e_hi, uint32_t chunk,
+                                                     uint32_t *__restrict__ hist, unsigned *status, FrameStatsDev *stats)
 {
-    extern __shared__ uint32_t sh_cnt[]; // [ntiles] binned points, then [ntiles] small boxes
-    const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y);
-    for (uint32_t t = threadIdx.x; t < 2 * ntiles; t += RT) sh_cnt[t] = 0u;
+    constexpr int NT = PART_THREADS<SMALL>;
+    extern __shared__ uint32_t sh_cnt[]; // [ntiles] binned points, then (SMALL) [ntiles] small boxes
+    const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y), ncnt = SMALL ? 2 * ntiles : ntiles;
+    for (uint32_t t = threadIdx.x; t < ncnt; t += NT) sh_cnt[t] = 0u;
     __syncthreads();
     const unsigned long long total = min(src_total(src), e_hi);
     const int lane = threadIdx.x & 31;
     unsigned long long splats = 0, pairs = 0;
     AmpSum amp;
-    for (unsigned long long a = e_lo + (unsigned long long)blockIdx.x * CHUNK; a < total;
-         a += (unsigned long long)gridDim.x * CHUNK) {
-        const unsigned long long b = min(total, a + CHUNK);
+    for (unsigned long long a = e_lo + (unsigned long long)blockIdx.x * chunk; a < total;
+         a += (unsigned long long)gridDim.x * chunk) {
+        const unsigned long long b = min(total, a + chunk);
         uint32_t j0, j1;
         src_range(src, a, b, j0, j1);
-        for (unsigned long long e0 = a; e0 < b; e0 += RT) {
+        for (unsigned long long e0 = a; e0 < b; e0 += NT) {
             const unsigned long long e = e0 + threadIdx.x;
             int res = 0;
             Splat s;
@@ -792,8 +896,8 @@ __global__ void __launch_bounds__(RT, 4) k_project_hist(Src src, Proj P, unsigne
                 ++splats;
                 int x0, x1, y0, y1;
                 splat_box(s.U, s.V, s.S, P.W, P.H, x0, x1, y0, y1);
-                if (x0 <= x1 && y0 <= y1) {
-                    const bool small = direct_box(x0, x1, y0, y1);
+                const bool small = direct_box(x0, x1, y0, y1);
+                if (x0 <= x1 && y0 <= y1 && (SMALL || !small)) {
                     uint32_t *cnt = small ? sh_cnt + ntiles : sh_cnt;
                     const int tx0 = x0 / P.TW, tx1 = x1 / P.TW, ty0 = y0 / P.TH, ty1 = y1 / P.TH;
                     if (!small) pairs += (unsigned long long)(tx1 - tx0 + 1) * (unsigned long long)(ty1 - ty0 + 1);
@@ -811,39 +915,48 @@ __global__ void __launch_bounds__(RT, 4) k_project_hist(Src src, Proj P, unsigne
     if (lane == 0 && pairs) atomicAdd(&stats->pairs, pairs);
     amp.flush(stats);
     __syncthreads();
-    for (uint32_t t = threadIdx.x; t < 2 * ntiles; t += RT) hist[(size_t)t * gridDim.x + blockIdx.x] = sh_cnt[t];
+    for (uint32_t t = threadIdx.x; t < ncnt; t += NT) hist[(size_t)t * gridDim.x + blockIdx.x] = sh_cnt[t];
 }
 
-// tile counts and offsets from the scanned (tile, CTA) histogram
-__global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, const uint32_t *__restrict__ off,
-                                  const uint32_t *total, uint32_t *tile_cnt, uint32_t *tile_off)
+// tile counts, offsets and work items (of per_item records) from the scanned (tile, CTA) histogram
+__global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, uint32_t per_item, const uint32_t *__restrict__ off,
+                                  const uint32_t *total, uint32_t *tile_cnt, uint32_t *tile_off, uint32_t *item_cnt)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ntiles) return;
     const uint32_t a = off[(size_t)t * G], b = t + 1 < ntiles ? off[(size_t)(t + 1) * G] : *total;
     tile_off[t] = a;
     tile_cnt[t] = b - a;
+    item_cnt[t] = (b - a + per_item - 1) / per_item;
 }
 
-// Writes the (tile, point) records of the binned points at this CTA's bases and splats the points
-// with small boxes into img (cstats, if not null, receives the latter's pixel updates).
-template <class Src>
-__global__ void __launch_bounds__(RT, 4) k_project_scatter_part(Src src, Proj P, unsigned long long e_lo,
-                                                             unsigned long long e_hi, const uint32_t *__restrict__ off,
+// Writes the (tile, point) records of the binned points (SMALL: and of the small boxes) at this CTA's
+// bases; without SMALL the points with small boxes are splatted into img (cstats, if not null,
+// receives their pixel updates).
+template <class Src, bool SMALL>
+__global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL>) k_project_scatter_part(Src src, Proj P, unsigned long long e_lo,
+                                                             unsigned long long e_hi, uint32_t chunk,
+                                                             const uint32_t *__restrict__ off,
                                                              uint4 *__restrict__ rec, unsigned long long *img,
                                                              FrameStatsDev *cstats)
 {
-    extern __shared__ uint32_t sh_cur[]; // [ntiles] binned points, then [ntiles] small boxes
-    const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y);
-    for (uint32_t t = threadIdx.x; t < 2 * ntiles; t += RT) sh_cur[t] = off[(size_t)t * gridDim.x + blockIdx.x];
-    __syncthreads();
+    constexpr int NT = PART_THREADS<SMALL>;
+    __shared__ int32_t K[SMALL ? 1 : 1025];
+    extern __shared__ uint32_t sh_cur[]; // [ntiles] binned points, then (SMALL) [ntiles] small boxes
+    const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y), ncnt = SMALL ? 2 * ntiles : ntiles;
     const unsigned long long total = min(src_total(src), e_hi);
-    for (unsigned long long a = e_lo + (unsigned long long)blockIdx.x * CHUNK; a < total;
-         a += (unsigned long long)gridDim.x * CHUNK) {
-        const unsigned long long b = min(total, a + CHUNK);
+    unsigned hits = 0;
+    if (e_lo + (unsigned long long)blockIdx.x * chunk < total)
+        for (uint32_t t = threadIdx.x; t < ncnt; t += NT) sh_cur[t] = off[(size_t)t * gridDim.x + blockIdx.x];
+    if (!SMALL)
+        for (int t = threadIdx.x; t <= 1024; t += NT) K[t] = t < 1024 ? g_ktab[P.kernel][t] : 0;
+    __syncthreads();
+    for (unsigned long long a = e_lo + (unsigned long long)blockIdx.x * chunk; a < total;
+         a += (unsigned long long)gridDim.x * chunk) {
+        const unsigned long long b = min(total, a + chunk);
         uint32_t j0, j1;
         src_range(src, a, b, j0, j1);
-        for (unsigned long long e0 = a; e0 < b; e0 += RT) {
+        for (unsigned long long e0 = a; e0 < b; e0 += NT) {
             const unsigned long long e = e0 + threadIdx.x;
             int res = 0;
             Splat s;
@@ -852,27 +965,36 @@ __global__ void __launch_bounds__(RT, 4) k_project_scatter_part(Src src, Proj P,
                 src_load(src, e, j0, j1, x, y, z, w, h);
                 res = project(P, x, y, z, w, h, s);
             }
+            BoxWalk direct;
+            int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
+            bool mine = false;
             if (res == 1) {
-                int x0, x1, y0, y1;
-                splat_box(s.U, s.V, s.S, P.W, P.H, x0, x1, y0, y1);
+                const int rad = splat_box(s.U, s.V, s.S, P.W, P.H, x0, x1, y0, y1);
                 if (x0 <= x1 && y0 <= y1) {
-                    uint32_t *cur = direct_box(x0, x1, y0, y1) ? sh_cur + ntiles : sh_cur;
-                    const uint4 r = make_uint4((uint32_t)s.U, (uint32_t)s.V, s.S, __float_as_uint(s.Wf));
-                    const int tx0 = x0 / P.TW, tx1 = x1 / P.TW, ty0 = y0 / P.TH, ty1 = y1 / P.TH;
-                    for (int ty = ty0; ty <= ty1; ++ty)
-                        for (int tx = tx0; tx <= tx1; ++tx) rec[atomicAdd(&cur[ty * P.tiles_x + tx], 1u)] = r;
+                    const bool small = direct_box(x0, x1, y0, y1);
+                    if (!SMALL && small) {
+                        mine = group_box(rad, s.Wf);
+                        if (!mine) direct = box_walk(s.U, s.V, s.S, __float2ull_rn(s.Wf), rad, x0, x1, y0, y1);
+                    } else {
+                        uint32_t *cur = small ? sh_cur + ntiles : sh_cur;
+                        const uint4 r = make_uint4((uint32_t)s.U, (uint32_t)s.V, s.S, __float_as_uint(s.Wf));
+                        const int tx0 = x0 / P.TW, tx1 = x1 / P.TW, ty0 = y0 / P.TH, ty1 = y1 / P.TH;
+                        for (int ty = ty0; ty <= ty1; ++ty)
+                            for (int tx = tx0; tx <= tx1; ++tx) rec[atomicAdd(&cur[ty * P.tiles_x + tx], 1u)] = r;
+                    }
                 }
+            }
+            if (!SMALL) {
+                hits += group_boxes<true>(
+                    mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K,
+                    [&](int x, int y, uint32_t c) { atomicAdd(&img[(size_t)y * P.W + x], (unsigned long long)c); });
+                hits += walk_boxes<false>(
+                    direct, 0u, [&](uint32_t, uint32_t i) { return K[i]; },
+                    [&](uint32_t, int x, int y, unsigned long long c) { atomicAdd(&img[(size_t)y * P.W + x], c); });
             }
         }
     }
-    (void)img;
-    (void)cstats;
-}
-
-__global__ void k_tile_items_n(uint32_t ntiles, const uint32_t *tile_cnt, uint32_t per_item, uint32_t *item_cnt)
-{
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < ntiles) item_cnt[t] = (tile_cnt[t] + per_item - 1) / per_item;
+    if (!SMALL && cstats) count_hits(hits, cstats);
 }
 
 __global__ void k_fill_items_n(uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
@@ -886,12 +1008,13 @@ __global__ void k_fill_items_n(uint32_t ntiles, const uint32_t *tile_cnt, const 
 }
 
 // Small-box records of one work item (a tile and up to ITEM_SMALL of its records): each warp takes
-// 32 records at a time and walks their pixel boxes, clipped to the tile, with walk_boxes, adding the
+// 32 records at a time and takes their pixel boxes, clipped to the tile, four at a time (group_boxes) or, for
+// wide supports and the largest amplitudes, together (walk_boxes), adding the
 // per-pixel rule's contributions to a shared tile image.  A contribution c < 2^49 is added as three
 // fields, c = lo + mid 2^16 + hi 2^32 with lo, mid < 2^16, to 32-bit words by fire-and-forget
 // 32-bit shared atomics (hi, rarely nonzero, only when it is): a pixel receives at most one
 // contribution per record, so at most ITEM_SMALL = 2^12 per item, and no word can overflow
-// (lo and mid sums < 2^28, hi sums < 2^29).  The lo and mid words have four copies, one per group
+// (mid sums < 2^28, lo sums < 2^32, hi sums < 2^29).  The lo and mid words have four copies, one per group
 // of two warps, so that warps adding to the same pixel -- points pile up in dense halo cores --
 // mostly meet only in the final sum; the fields are then recombined in 64 bits and added to the
 // image once per pixel.  A box is small once clipped to the image, so its pixels can lie far from a
@@ -899,11 +1022,12 @@ __global__ void k_fill_items_n(uint32_t ntiles, const uint32_t *tile_cnt, const 
 // for those.
 static_assert(ITEM_SMALL <= (1u << 12), "32-bit field sums of the small-box tile image");
 template <bool COUNT>
-__global__ void __launch_bounds__(RT, 5) k_splat_small(const uint4 *__restrict__ rec, const uint4 *__restrict__ items,
+__global__ void __launch_bounds__(RT, 4) k_splat_small(const uint4 *__restrict__ rec, const uint4 *__restrict__ items,
                                                       Proj P, unsigned long long *__restrict__ img, FrameStatsDev *stats)
 {
     __shared__ uint32_t tlo[4][1024], tmid[4][1024], thi[1024]; // TW x TH <= 1024 (checked on the host)
-    __shared__ int32_t K[1024];
+    __shared__ int32_t K[1025];
+    if (threadIdx.x == 0) K[1024] = 0;
     for (int i = threadIdx.x; i < 1024; i += RT) {
         K[i] = g_ktab[P.kernel][i];
         thi[i] = 0u;
@@ -924,18 +1048,32 @@ __global__ void __launch_bounds__(RT, 5) k_splat_small(const uint4 *__restrict__
     for (uint32_t base = it.y + (threadIdx.x & ~31u); base < it.z; base += RT) { // uniform per warp
         const uint32_t r = base + (threadIdx.x & 31u);
         BoxWalk b;
+        uint4 R = make_uint4(0u, 0u, 0u, 0u);
+        int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
+        bool mine = false;
         if (r < it.z) {
-            const uint4 R = rec[r];
+            R = rec[r];
             const int U = (int)R.x, V = (int)R.y;
-            int x0, x1, y0, y1;
             const int rad = splat_box(U, V, R.z, P.W, P.H, x0, x1, y0, y1);
             x0 = max(x0, X0);
             x1 = min(x1, X1);
             y0 = max(y0, Y0);
             y1 = min(y1, Y1);
-            if (x0 <= x1 && y0 <= y1)
-                b = box_walk(U, V, R.z, __float2ull_rn(__uint_as_float(R.w)), rad, x0, x1, y0, y1);
+            if (x0 <= x1 && y0 <= y1) {
+                mine = group_box(rad, __uint_as_float(R.w));
+                if (!mine) b = box_walk(U, V, R.z, __float2ull_rn(__uint_as_float(R.w)), rad, x0, x1, y0, y1);
+            }
         }
+        // a contribution below 2^32 as 20 low bits and, where it has more, the rest in the middle word
+        // (2^12 contributions of less than 2^20 stay below 2^32)
+        auto add = [&](int x, int y, uint32_t c) {
+            const int p = (y - Y0) * TW + (x - X0);
+            atomicAdd(&lo[p], c & 0xFFFFFu);
+            if (c >> 20) atomicAdd(&mid[p], (c >> 20) << 4);
+        };
+        const bool tiny = mine && x1 - x0 < LANE_BOX && y1 - y0 < LANE_BOX;
+        hits += lane_boxes<COUNT>(tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K, add);
+        hits += group_boxes<COUNT>(mine && !tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K, add);
         hits += walk_boxes<false>(b, 0u, [&](uint32_t, uint32_t i) { return K[i]; },
                                   [&](uint32_t, int x, int y, unsigned long long c) {
             const int p = (y - Y0) * TW + (x - X0);
@@ -1359,14 +1497,35 @@ struct PassCounts {
     uint32_t items, small_items;      // splat work items, small-box work items (partitioned only)
 };
 
-// The caller's particle arrays are in no spatial order: they are binned by the partitioned passes
-// (one shared-memory histogram per CTA) whenever the tile count fits shared memory.
+// The caller's particle arrays are in no spatial order (a stream of its own for small boxes).
 template <class Src> constexpr bool unordered_source() { return false; }
 template <> constexpr bool unordered_source<SrcFlat>() { return true; }
 
-template <class Src> bool partitioned(const Proj &P)
+// How a frame is binned: in parts (shared-memory histograms) whenever they fit, with `grid` CTAs over
+// chunks of `chunk` points -- about four CTAs per SM, fewer when the points or the histograms do not
+// allow -- or through the global tile counters.
+struct Binning {
+    bool part;
+    unsigned grid;
+    uint32_t chunk;
+    size_t smem;
+};
+
+template <class Src> Binning binning(const Src &src, const Proj &P)
 {
-    return unordered_source<Src>() && (uint32_t)(P.tiles_x * P.tiles_y) <= PART_MAX_TILES;
+    Binning b;
+    b.smem = (size_t)P.tiles_x * P.tiles_y * (unordered_source<Src>() ? 8 : 4);
+    b.part = b.smem <= PART_MAX_SMEM;
+    const unsigned nt = (unsigned)PART_THREADS<unordered_source<Src>()>;
+    const unsigned full = (unsigned)persistent_blocks(
+        b.part ? (int)std::min<size_t>(1024 / nt, std::max<size_t>(1, 216 * 1024 / (b.smem + 6 * 1024))) : 4);
+    // at least one point a thread; the bound is all that is known here of an octree frame's points
+    const unsigned long long per = (src.bound + full - 1) / full;
+    b.chunk = b.part ? (uint32_t)std::min<unsigned long long>(CHUNK, std::max<unsigned long long>(nt, (per + nt - 1) / nt * nt))
+                     : CHUNK;
+    b.grid = b.part ? (unsigned)std::max<unsigned long long>(1, std::min<unsigned long long>(full, (src.bound + b.chunk - 1) / b.chunk))
+                    : full;
+    return b;
 }
 
 template <class Src>
@@ -1375,50 +1534,50 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
 {
     const Allocator &A = r->A;
     const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y);
-    const unsigned G = (unsigned)persistent_blocks(4);
-    if (partitioned<Src>(P)) {
-        const size_t nh = (size_t)ntiles * G;
-        r->cta_hist.ensure(A, 2 * nh, s);
-        r->cta_off.ensure(A, 2 * nh + 1, s);
-        r->tile_cnt_s.ensure(A, ntiles, s);
-        r->tile_off_s.ensure(A, ntiles + 1, s);
-        r->item_cnt_s.ensure(A, ntiles, s);
-        r->item_off_s.ensure(A, ntiles + 1, s);
-        launch(GBLOD_K_PROJECT_COUNT, k_project_hist<Src>, dim3(G), dim3(RT), (size_t)ntiles * 8, s, src, P, lo, hi,
-               r->cta_hist.p, r->status, stats);
-        scan_exclusive_u32(A, r->scan, r->cta_hist.p, r->cta_off.p, 2 * nh, r->cta_off.p + 2 * nh, s);
+    const Binning bn = binning(src, P);
+    constexpr bool SMALL = unordered_source<Src>();
+    const size_t nh = (size_t)ntiles * bn.grid, nall = SMALL ? 2 * nh : nh;
+    if (bn.part) {
+        r->cta_hist.ensure(A, nall, s);
+        r->cta_off.ensure(A, nall + 1, s);
+        launch(GBLOD_K_PROJECT_COUNT, k_project_hist<Src, SMALL>, dim3(bn.grid), dim3(PART_THREADS<SMALL>), bn.smem, s, src, P, lo, hi,
+               bn.chunk, r->cta_hist.p, r->status, stats);
+        scan_exclusive_u32(A, r->scan, r->cta_hist.p, r->cta_off.p, nall, r->cta_off.p + nall, s);
         const dim3 tg((ntiles + 255) / 256);
-        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, ntiles, G, (const uint32_t *)r->cta_off.p,
-               (const uint32_t *)(r->cta_off.p + nh), r->tile_cnt.p, r->tile_off.p);
-        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, ntiles, G,
-               (const uint32_t *)(r->cta_off.p + nh), (const uint32_t *)(r->cta_off.p + 2 * nh), r->tile_cnt_s.p,
-               r->tile_off_s.p);
-        GB_CUDA(cudaMemcpyAsync(r->tile_off.p + ntiles, r->cta_off.p + nh, 4, cudaMemcpyDeviceToDevice, s));
-        launch(GBLOD_K_RENDER_OTHER, k_tile_items_n, tg, dim3(256), 0, s, ntiles, (const uint32_t *)r->tile_cnt_s.p,
-               ITEM_SMALL, r->item_cnt_s.p);
-        scan_exclusive_u32(A, r->scan, r->item_cnt_s.p, r->item_off_s.p, ntiles, r->item_off_s.p + ntiles, s);
+        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, ntiles, (uint32_t)bn.grid, ITEM,
+               (const uint32_t *)r->cta_off.p, (const uint32_t *)(r->cta_off.p + nh), r->tile_cnt.p, r->tile_off.p,
+               r->item_cnt.p);
+        if (SMALL) {
+            r->tile_cnt_s.ensure(A, ntiles, s);
+            r->tile_off_s.ensure(A, ntiles + 1, s);
+            r->item_cnt_s.ensure(A, ntiles, s);
+            r->item_off_s.ensure(A, ntiles + 1, s);
+            launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, ntiles, (uint32_t)bn.grid, ITEM_SMALL,
+                   (const uint32_t *)(r->cta_off.p + nh), (const uint32_t *)(r->cta_off.p + 2 * nh), r->tile_cnt_s.p,
+                   r->tile_off_s.p, r->item_cnt_s.p);
+            scan_exclusive_u32(A, r->scan, r->item_cnt_s.p, r->item_off_s.p, ntiles, r->item_off_s.p + ntiles, s);
+        }
     } else {
         GB_CUDA(cudaMemsetAsync(r->tile_cnt.p, 0, (size_t)ntiles * 4, s));
-        launch(GBLOD_K_PROJECT_COUNT, k_project_count<Src>, dim3(G), dim3(RT), 0, s, src, P, lo, hi, r->tile_cnt.p,
+        launch(GBLOD_K_PROJECT_COUNT, k_project_count<Src>, dim3(bn.grid), dim3(RT), 0, s, src, P, lo, hi, r->tile_cnt.p,
                r->status, stats);
         scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, ntiles, r->tile_off.p + ntiles, s);
+        launch(GBLOD_K_RENDER_OTHER, k_tile_items, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
+               (const uint32_t *)r->tile_cnt.p, r->item_cnt.p);
     }
-    launch(GBLOD_K_RENDER_OTHER, k_tile_items, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
-           (const uint32_t *)r->tile_cnt.p, r->item_cnt.p);
     scan_exclusive_u32(A, r->scan, r->item_cnt.p, r->item_off.p, ntiles, r->item_off.p + ntiles, s);
     unsigned long long *h = static_cast<unsigned long long *>(r->hs.get(40));
     h[2] = h[3] = h[4] = 0;
     GB_CUDA(cudaMemcpyAsync(h, &stats->pairs, 8, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaMemcpyAsync(h + 1, &stats->points, 8, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaMemcpyAsync(h + 2, r->item_off.p + ntiles, 4, cudaMemcpyDeviceToHost, s));
-    if (partitioned<Src>(P)) {
-        const size_t nh = (size_t)ntiles * G;
+    const bool streams = bn.part && SMALL;
+    if (streams) {
         GB_CUDA(cudaMemcpyAsync(h + 3, r->item_off_s.p + ntiles, 4, cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaMemcpyAsync(h + 4, r->cta_off.p + 2 * nh, 4, cudaMemcpyDeviceToHost, s));
     }
     GB_CUDA(cudaStreamSynchronize(s));
-    const bool part = partitioned<Src>(P);
-    return PassCounts{part ? (h[4] & 0xFFFFFFFFull) : h[0], h[1], (uint32_t)(h[2] & 0xFFFFFFFFull),
+    return PassCounts{streams ? (h[4] & 0xFFFFFFFFull) : h[0], h[1], (uint32_t)(h[2] & 0xFFFFFFFFull),
                       (uint32_t)(h[3] & 0xFFFFFFFFull)};
 }
 
@@ -1441,22 +1600,25 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
 {
     const Allocator &A = r->A;
     const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y);
+    const Binning bn = binning(src, P);
+    constexpr bool SMALL = unordered_source<Src>();
+    FrameStatsDev *cstats = r->count_updates ? r->stats : (FrameStatsDev *)nullptr;
     r->records.ensure(A, pc.pairs, s);
     r->items.ensure(A, (size_t)pc.items + pc.small_items, s);
-    if (partitioned<Src>(P)) {
-        launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter_part<Src>, dim3((unsigned)persistent_blocks(4)), dim3(RT),
-               (size_t)ntiles * 8, s, src, P, lo, hi, (const uint32_t *)r->cta_off.p, r->records.p, img,
-               r->count_updates ? r->stats : (FrameStatsDev *)nullptr);
-        launch(GBLOD_K_RENDER_OTHER, k_fill_items_n, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
-               (const uint32_t *)r->tile_cnt_s.p, (const uint32_t *)r->tile_off_s.p, (const uint32_t *)r->item_off_s.p,
-               ITEM_SMALL, r->items.p + pc.items);
-        launch(GBLOD_K_SPLAT, r->count_updates ? k_splat_small<true> : k_splat_small<false>, dim3(pc.small_items),
-               dim3(RT), 0, s, (const uint4 *)r->records.p, (const uint4 *)(r->items.p + pc.items), P, img, r->stats);
+    if (bn.part) {
+        launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter_part<Src, SMALL>, dim3(bn.grid), dim3(PART_THREADS<SMALL>), bn.smem, s,
+               src, P, lo, hi, bn.chunk, (const uint32_t *)r->cta_off.p, r->records.p, img, cstats);
+        if (SMALL) {
+            launch(GBLOD_K_RENDER_OTHER, k_fill_items_n, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
+                   (const uint32_t *)r->tile_cnt_s.p, (const uint32_t *)r->tile_off_s.p,
+                   (const uint32_t *)r->item_off_s.p, ITEM_SMALL, r->items.p + pc.items);
+            launch(GBLOD_K_SPLAT, r->count_updates ? k_splat_small<true> : k_splat_small<false>, dim3(pc.small_items),
+                   dim3(RT), 0, s, (const uint4 *)r->records.p, (const uint4 *)(r->items.p + pc.items), P, img, r->stats);
+        }
     } else {
         GB_CUDA(cudaMemcpyAsync(r->tile_cur.p, r->tile_off.p, (size_t)ntiles * 4, cudaMemcpyDeviceToDevice, s));
-        launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter<Src>, dim3((unsigned)persistent_blocks(4)), dim3(RT), 0, s,
-               src, P, lo, hi, r->tile_cur.p, r->records.p, img,
-               r->count_updates ? r->stats : (FrameStatsDev *)nullptr);
+        launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter<Src>, dim3(bn.grid), dim3(RT), 0, s, src, P, lo, hi,
+               r->tile_cur.p, r->records.p, img, cstats);
     }
     launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
            (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p, (const uint32_t *)r->item_off.p,
@@ -1951,9 +2113,16 @@ BatchPlan plan_batch(const gblod_view *views, int n, const gblod_render_params &
     return b;
 }
 
-// the splat kernels' SplatSmem is above the 48 KB a launch may take without opting in
+// the splat kernels' SplatSmem and the binning histograms of frames with many tiles are above the 48 KB
+// a launch may take without opting in
 void set_splat_smem()
 {
+    const void *part[] = {(const void *)k_project_hist<SrcLOD, false>, (const void *)k_project_hist<SrcLODQ, false>,
+                          (const void *)k_project_hist<SrcFlat, true>, (const void *)k_project_scatter_part<SrcLOD, false>,
+                          (const void *)k_project_scatter_part<SrcLODQ, false>,
+                          (const void *)k_project_scatter_part<SrcFlat, true>};
+    for (const void *f : part)
+        GB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PART_MAX_SMEM));
     const int bytes = (int)sizeof(SplatSmem);
     GB_CUDA(cudaFuncSetAttribute(k_splat_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     GB_CUDA(cudaFuncSetAttribute(k_splat_tiles<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
@@ -2158,7 +2327,7 @@ void render_lod(gblod_renderer *r, const gblod_octree *o, const gblod_camera &ca
     }
     launch(GBLOD_K_SELECT_NODES, k_sel_prefix, dim3(1), dim3(1024), 0, s, nodes, (const uint32_t *)r->sel.p,
            (const uint32_t *)nsel, r->sel_pfx.p, r->sel_base.p, r->stats);
-    SrcLOD src{o->pts4, o->hs, r->sel_pfx.p, r->sel_base.p, nsel, &r->stats->points};
+    SrcLOD src{o->pts4, o->hs, r->sel_pfx.p, r->sel_base.p, nsel, &r->stats->points, o->n_points};
     if (q) {
         SrcLODQ sq;
         static_cast<SrcLOD &>(sq) = src;
@@ -2202,7 +2371,7 @@ void render_brute(gblod_renderer *r, const float *xyz, const float *mass, const 
     GB_CUDA(cudaMemsetAsync(r->stats, 0, offsetof(FrameStatsDev, pixel_updates_total), s));
     const unsigned long long pts[1] = {n};
     GB_CUDA(cudaMemcpyAsync(&r->stats->points, pts, 8, cudaMemcpyHostToDevice, s));
-    SrcFlat src{xyz, mass, h, n};
+    SrcFlat src{xyz, mass, h, n, n};
     frame_common(r, src, P, rp, image, accum, s);
 }
 
@@ -2307,7 +2476,7 @@ gblod_status render_brute_noalloc(const float *xyz, const float *mass, const flo
     GB_CUDA(cudaMemsetAsync(tile_cnt, 0, ntiles * 4, s));
     GB_CUDA(cudaMemsetAsync(stats, 0, sizeof(FrameStatsDev), s));
     GB_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned), s));
-    const SrcFlat src{xyz, mass, h, n};
+    const SrcFlat src{xyz, mass, h, n, n};
     const unsigned G = (unsigned)persistent_blocks(4);
     const uint32_t nt = (uint32_t)ntiles;
     launch(GBLOD_K_PROJECT_COUNT, k_project_count<SrcFlat>, dim3(G), dim3(RT), 0, s, src, P, 0ull, ~0ull, tile_cnt,

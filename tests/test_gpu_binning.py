@@ -1,0 +1,43 @@
+"""Frames binned in parts (shared-memory histograms) and through the global tile counters, against the oracle
+bit for bit: tile counts below and above the shared-memory limit of each point source, fewer points
+than one chunk, chunks that end in the middle of a node, record-budget pieces, an octree's fp32 points
+and its 16-bit codes, and the caller's unordered arrays."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_0811_2055_gb300 import synth
+
+from gpu_helpers import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 255, 257, 30011])
+@pytest.mark.parametrize("W,H,tw,th", [(96, 50, 64, 16), (1800, 1000, 32, 32), (1800, 1000, 8, 8), (1500, 1200, 8, 4)])
+@pytest.mark.parametrize("budget", [0, 3000])
+def test_binning_equals_the_oracle(n, W, H, tw, th, budget):
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    p = synth.tiny(n, seed=n)
+    d = to_dev(p.xyz, p.mass, p.h)
+    cam = synth.look_at((0.4, 0.6, -0.7), (0.5, 0.5, 0.5), width=W, height=H)
+    ot = O.build_tree(p.xyz, p.mass, p.h, seed=1, n_max=700)
+    t = G.build_lod(*d, n_max=700, seed=1)
+    r = G.Renderer()
+    kw = dict(lambda_px=9.0, tile_w=tw, tile_h=th, record_budget=budget)
+    want, st, nd, _ = O.render_lod(ot, cam, O.rparams(lambda_px=9.0))
+    _, acc = r.render(t, cam, G.make_params(**kw))
+    assert st == 0 and r.status() == G.OK and np.array_equal(G.u64(acc), want)
+    assert r.stats()["splats"] == nd
+    want, st, nd = O.splat_particles(p.xyz, p.mass, p.h, cam, O.rparams())
+    _, acc = r.render_bruteforce(*d, cam, G.make_params(**kw))
+    assert st == 0 and r.status() == G.OK and np.array_equal(G.u64(acc), want)
+    t.quantize()
+    _, _, decoded = O.block_quantize(ot)
+    want, st, nd, _ = O.render_lod(decoded, cam, O.rparams(lambda_px=9.0))
+    _, acc = r.render(t, cam, G.make_params(point_format=G.POINTS_BLOCK16, **kw))
+    assert st == 0 and r.status() == G.OK and np.array_equal(G.u64(acc), want)
+    t.free()
+    r.close()
