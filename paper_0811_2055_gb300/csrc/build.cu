@@ -648,7 +648,9 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
                (const uint32_t *)isrep.p, (const uint32_t *)reppos.p, reps.p);
         SelectIn in{s4, sm.p, sorted_ids, N.code.p, N.first.p, N.count.p, pfirst.p, w.p, sc.p, hmax.p,
                     o->pts4, o->hs, o->pt_src, p.n_max};
-        select_representatives(A, s, hs, scan, in, reps.p, n_rep, p.n_max, p.seed, o->equal_mass);
+        // the packed particles and the sort's buffers are done with: 28 bytes a particle for the codes
+        select_representatives(A, s, hs, scan, in, reps.p, n_rep, p.n_max, p.seed, o->equal_mass,
+                               roomy ? block.p + n16 : nullptr, roomy ? (n16 + n16 / 2 + n16 / 4) * sizeof(float4) : 0);
     }
 
     // leaves, bounds, cull radii

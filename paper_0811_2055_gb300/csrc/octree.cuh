@@ -77,9 +77,10 @@ struct SelectIn {
     uint32_t n_max;
 };
 
-// A4 + A5 for every node whose index is listed in rep_nodes (device, n_rep entries).
+// A4 + A5 for every node whose index is listed in rep_nodes (device, n_rep entries).  `spare` (may be
+// null): 16-byte aligned device memory to use for the elements' codes if they fit.
 void select_representatives(const Allocator &A, cudaStream_t s, HostStage &hs, ScanTmp &scan, const SelectIn &in,
                             const uint32_t *rep_nodes, uint32_t n_rep, uint32_t n_max, uint64_t seed,
-                            int equal_mass);
+                            int equal_mass, void *spare, size_t spare_bytes);
 
 } // namespace gb

@@ -5,16 +5,24 @@
 // Every particle i of node c gets the key k_i = u_i (all masses equal) or the bits of
 // E(u_i)/m_i (exponential race), u_i = Philox(seed; id_i, code_c); the node keeps the n_max
 // smallest (k_i, id_i).  Per node this is a segmented radix select, all nodes at once:
-//   hist     4096-element chunks histogram the top log2(B) key bits (B ~ count/1024 bins, at
-//            most 4096: a shared-memory histogram per chunk)
-//   find     per node, the bin b that holds rank n_max
-//   mark     keys below bin b set their bit in a per-node bitmap (warp ballots, no atomics);
-//            keys in bin b become candidates (k, id, position)
-//   resolve  per node, 8-bit radix rounds over the candidates' remaining (k, id) bits decide
-//            the last `need` members
-//   count/write  a per-chunk popcount, a scan, and a stable compaction of the bitmap write
-//            the representatives in ascending (Morton key, id) order.
-// Keys are recomputed from the ids (counter-based generator) instead of being stored.
+//   hist     4096-element chunks histogram the elements' bins (shared memory); equal masses: the top
+//            log2(B) key bits (B ~ count/128 bins, at most 4096).  Unequal masses: B logarithmic bins
+//            around the expected threshold, of the key computed in fp32 -- FP64 runs at 1/64 of the fp32
+//            rate, and the key's series takes some 50 FP64 operations.  Each element's bin goes to a
+//            16-bit code, with a mark if the key's error could put it into the next bin.
+//   find     per node, the bin b that holds rank n_max (an fp32 key errs by a factor below 1 + 2^-16, and so
+//            does the threshold: an element whose bins, error included, all lie below b is kept, above b
+//            dropped)
+//   mark     from the codes alone: elements below set their bit in a per-node bitmap, the others of bin b
+//            become candidates, with their exact key
+//   resolve  per node, 8-bit radix rounds over the candidates' remaining (k, id) bits decide the last
+//            n_max - kept members
+//   write    a stable compaction of the bitmap writes the representatives in ascending (Morton
+//            key, id) order.
+// Keys are recomputed from the ids (counter-based generator) instead of being stored; where there is no
+// memory for the codes, mark recomputes them too (Philox is the cost of either pass: 150M equal masses, mark
+// 3.4 ms recomputed, 0.72 ms from codes; 1M unequal masses, hist + mark + resolve 1.73 ms in
+// FP64, now 0.11).
 #include <algorithm>
 
 #include "lodmath.cuh"
@@ -38,18 +46,35 @@ struct RepInfo {
     const uint32_t *chunk_off; // first chunk of each rep slot (n_rep + 1 entries)
     const uint32_t *hoff;      // first histogram bin of each rep slot
     const uint8_t *logb;       // log2 bins
+    const int16_t *bin0;       // unequal masses: the bits above bin_shift of the first bin's lower edge
+    const float *rmean;        // unequal masses: 1 / mean mass
     const uint64_t *woff;      // first bitmap word of each rep slot
 };
 
-__global__ void k_sel_setup(uint32_t n_rep, const uint32_t *nodes, const uint32_t *ncount, uint32_t *nchunks,
-                            uint32_t *nbins, uint8_t *logb, uint64_t *nwords)
+// log2 of the bins per octave for 2^logb logarithmic bins: 16 octaves in all
+__device__ __forceinline__ int bin_shift(int logb) { return 23 - (logb - 4); }
+
+__global__ void k_sel_setup(uint32_t n_rep, const uint32_t *nodes, const uint32_t *ncount, const float *nw,
+                            uint32_t n_max, int equal_mass, uint32_t *nchunks, uint32_t *nbins, uint8_t *logb,
+                            int16_t *bin0, float *rmean, uint64_t *nwords)
 {
     const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n_rep) return;
     const uint32_t c = ncount[nodes[r]];
     nchunks[r] = (c + CH - 1) / CH;
-    uint32_t want = (c + 1023) / 1024, lb = 0;
-    while (lb < 12 && (1u << lb) < want) ++lb; // at most 4096 bins: the chunk histogram stays in shared memory
+    uint32_t lb = 0;
+    if (equal_mass) {
+        const uint32_t want = (c + 127) / 128;
+        while (lb < 12 && (1u << lb) < want) ++lb; // at most 4096 bins: the chunk histogram stays in shared memory
+    } else {
+        // 16, 4 or 1 bins an octave of E m_mean / m_i.  The expected threshold x of equal masses has
+        // n_max / c = 1 - exp(-x); unequal masses move it up, 16 octaves leave room (the first and the last bin take
+        // what lies outside).
+        lb = c >= 4096 ? 8 : (c >= 64 ? 6 : 4);
+        const float part = (float)n_max / (float)c;
+        rmean[r] = 1.0f / (nw[nodes[r]] * part);
+        bin0[r] = (int16_t)((int)(__float_as_uint(-log1pf(-fminf(part, 0.9999f))) >> bin_shift((int)lb)) - (1 << (lb - 1)));
+    }
     logb[r] = (uint8_t)lb;
     nbins[r] = 1u << lb;
     nwords[r] = (c + 31) / 32;
@@ -69,6 +94,48 @@ __device__ __forceinline__ uint32_t find_slot(const uint32_t *chunk_off, uint32_
     return lo;
 }
 
+// What a block needs to know of its chunk, laid out once (blocks that looked it up through the node arrays,
+// four dependent loads: 150M, mark 0.93 -> 0.72 ms, write 1.52 -> 1.43)
+struct __align__(16) Chunk {
+    uint32_t j0, len, start, r; // first element; elements; the first one's position in the node; rep slot
+    uint64_t code, words;       // node code; first bitmap word
+    int logb, bin0;
+    float rmean;
+    uint32_t node;
+};
+
+__global__ void k_sel_chunks(uint32_t n_chunks, uint32_t n_rep, SelectIn in, RepInfo R, Chunk *__restrict__ chunks)
+{
+    const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= n_chunks) return;
+    const uint32_t r = find_slot(R.chunk_off, n_rep, c), node = R.nodes[r], start = (c - R.chunk_off[r]) * CH;
+    Chunk C;
+    C.j0 = in.nfirst[node] + start;
+    C.len = min(CH, in.ncount[node] - start);
+    C.start = start;
+    C.r = r;
+    C.code = in.ncode[node];
+    C.words = R.woff[r] + start / 32;
+    C.logb = R.logb[r];
+    C.bin0 = R.bin0[r];
+    C.rmean = R.rmean[r];
+    C.node = node;
+    chunks[c] = C;
+}
+
+__device__ __forceinline__ Chunk load_chunk(const Chunk *chunks)
+{
+    static_assert(sizeof(Chunk) == 48, "three 16-byte loads");
+    const uint4 *p = reinterpret_cast<const uint4 *>(chunks + blockIdx.x);
+    union {
+        uint4 q[3];
+        Chunk c;
+    } u;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u.q[i] = __ldg(p + i);
+    return u.c;
+}
+
 __device__ __forceinline__ uint64_t sel_key(const SelectIn &in, uint32_t j, uint64_t code, uint64_t seed,
                                             int equal_mass, uint32_t &id)
 {
@@ -79,50 +146,62 @@ __device__ __forceinline__ uint64_t sel_key(const SelectIn &in, uint32_t j, uint
     return (uint64_t)__double_as_longlong(k);
 }
 
-struct ChunkCtx {
-    uint32_t r, node, first, count, start;
-    uint64_t code;
-    int logb;
-};
+// An element's code: its bin, and bit 15 if the exact key may lie in the next one.  `mid` is the bin that
+// counts it in the histogram.
+constexpr uint32_t CODE_NEXT = 0x8000u, CODE_NONE = 0x7FFFu; // CODE_NONE: past the node's end, above every bin
 
-__device__ __forceinline__ void load_chunk(ChunkCtx &C, const SelectIn &in, const RepInfo &R, uint32_t n_rep)
+// E(u) / m in fp32, m the mass over the node's mean, within a factor 1 + 2^-18 of the exact key: 1 - U is
+// exact where U is near 1 (the smallest keys), so both forms keep their relative error (logf, log1pf: 2 ulp;
+// four roundings more).  Masses lie in [2^-24, 2^24], so m and E / m are normal numbers, and __fdividef is
+// good to 2 ulp.
+__device__ __forceinline__ float fast_key(uint64_t u, float m)
 {
-    __shared__ ChunkCtx sc;
-    if (threadIdx.x == 0) {
-        const uint32_t c = blockIdx.x;
-        const uint32_t r = find_slot(R.chunk_off, n_rep, c);
-        const uint32_t node = R.nodes[r];
-        sc.r = r;
-        sc.node = node;
-        sc.first = in.nfirst[node];
-        sc.count = in.ncount[node];
-        sc.start = (c - R.chunk_off[r]) * CH;
-        sc.code = in.ncode[node];
-        sc.logb = R.logb[r];
-    }
-    __syncthreads();
-    C = sc;
+    const uint64_t v = u >> 12;                                                   // U = (v + 1/2) 2^-52
+    const float U = __ull2float_rn(2 * v + 1) * 0x1p-53f, V = __ull2float_rn((1ull << 53) - (2 * v + 1)) * 0x1p-53f;
+    const float E = v >= (1ull << 51) ? -log1pf(-V) : -logf(U);
+    return __fdividef(E, m);
 }
 
-__global__ void __launch_bounds__(ST) k_sel_hist(SelectIn in, RepInfo R, uint32_t n_rep, uint64_t seed,
-                                                 int equal_mass, uint32_t *hist)
+__device__ __forceinline__ uint32_t log_bin(float a, const Chunk &C)
+{
+    const int v = (int)(__float_as_uint(a) >> bin_shift(C.logb)) - C.bin0;
+    return (uint32_t)min(max(v, 0), (1 << C.logb) - 1);
+}
+
+__device__ __forceinline__ uint32_t sel_code(const SelectIn &in, uint32_t j, const Chunk &C, uint64_t seed,
+                                             int equal_mass, uint32_t &mid)
+{
+    const uint64_t u = gbd::node_draw(seed, C.code, in.sid[j]);
+    if (equal_mass) {
+        mid = C.logb ? (uint32_t)(u >> (64 - C.logb)) : 0u;
+        return mid;
+    }
+    const float a = fast_key(u, in.sm[j] * C.rmean);
+    mid = log_bin(a, C);
+    const uint32_t low = log_bin(a * (1.0f - 0x1p-16f), C), high = log_bin(a * (1.0f + 0x1p-16f), C);
+    return low | (high != low ? CODE_NEXT : 0u);
+}
+
+// codes (may be null): n_chunks x CH
+__global__ void __launch_bounds__(ST) k_sel_hist(SelectIn in, RepInfo R, const Chunk *chunks, uint64_t seed,
+                                                 int equal_mass, uint32_t *hist, uint16_t *__restrict__ codes)
 {
     __shared__ uint32_t sh[4096];
-    ChunkCtx C;
-    load_chunk(C, in, R, n_rep);
+    const Chunk C = load_chunk(chunks);
     const int nb = 1 << C.logb; // <= 4096
     for (int i = threadIdx.x; i < nb; i += ST) sh[i] = 0u;
     __syncthreads();
     uint32_t *gh = hist + R.hoff[C.r];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint16_t *co = codes ? codes + (size_t)blockIdx.x * CH : nullptr;
     for (int k = 0; k < ROUNDS; ++k) {
-        const uint32_t rel = C.start + (uint32_t)warp * (ROUNDS * 32) + (uint32_t)k * 32 + lane;
-        if (rel < C.count) {
-            uint32_t id;
-            const uint64_t key = sel_key(in, C.first + rel, C.code, seed, equal_mass, id);
-            const uint32_t d = C.logb ? (uint32_t)(key >> (64 - C.logb)) : 0u;
-            atomicAdd(&sh[d], 1u);
+        const uint32_t at = (uint32_t)k * ST + threadIdx.x;
+        uint32_t code = CODE_NONE;
+        if (at < C.len) {
+            uint32_t mid;
+            code = sel_code(in, C.j0 + at, C, seed, equal_mass, mid);
+            atomicAdd(&sh[mid], 1u);
         }
+        if (co) co[at] = (uint16_t)code;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nb; i += ST)
@@ -154,59 +233,84 @@ __device__ __forceinline__ uint32_t block_scan_u32(uint32_t v, uint32_t &tot)
     return before + incl - v;
 }
 
-__global__ void __launch_bounds__(ST) k_sel_find(RepInfo R, uint32_t n_max, const uint32_t *hist, uint32_t *tb,
-                                                 uint32_t *need, uint64_t *ccount)
+// the threshold's bin, and at most how many candidates there are: its elements, and with fp32 keys those
+// of the two bins beside it whose error reaches it
+__global__ void __launch_bounds__(ST) k_sel_find(RepInfo R, uint32_t n_max, int equal_mass, const uint32_t *hist,
+                                                 uint32_t *tb, uint64_t *ccap)
 {
     const uint32_t r = blockIdx.x;
     const uint32_t nb = 1u << R.logb[r];
     const uint32_t *h = hist + R.hoff[r];
     uint32_t run = 0;
     for (uint32_t base = 0; base < nb; base += ST) {
-        const uint32_t hv = base + threadIdx.x < nb ? h[base + threadIdx.x] : 0u;
+        const uint32_t i = base + threadIdx.x;
+        const uint32_t hv = i < nb ? h[i] : 0u;
         uint32_t tot;
         const uint32_t ex = block_scan_u32(hv, tot);
         const uint32_t cum = run + ex;
         if (cum < n_max && n_max <= cum + hv) {
-            tb[r] = base + threadIdx.x;
-            need[r] = n_max - cum;
-            ccount[r] = hv;
+            tb[r] = i;
+            ccap[r] = (uint64_t)hv + (equal_mass || i == 0 ? 0u : h[i - 1]) + (equal_mass || i + 1 >= nb ? 0u : h[i + 1]);
         }
         run += tot;
     }
 }
 
-__global__ void __launch_bounds__(ST) k_sel_mark(SelectIn in, RepInfo R, uint32_t n_rep, uint64_t seed,
-                                                 int equal_mass, const uint32_t *tb, const uint64_t *cand_off,
-                                                 uint32_t *cursor, Cand *cand, uint32_t *bitmap)
+// A thread takes 16 consecutive elements of the chunk: from their codes (two 16-byte loads), or computed
+// (CODES false).  kept[r] counts a node's elements below the threshold's bin, chunk_sel a chunk's.
+template <bool CODES>
+__global__ void __launch_bounds__(ST) k_sel_mark(SelectIn in, const Chunk *chunks, uint64_t seed, int equal_mass,
+                                                 const uint16_t *__restrict__ codes, const uint32_t *tb,
+                                                 const uint64_t *cand_off, uint32_t *cursor, uint32_t *kept,
+                                                 uint32_t *chunk_sel, Cand *cand, uint32_t *bitmap)
 {
-    ChunkCtx C;
-    load_chunk(C, in, R, n_rep);
-    const uint32_t b = tb[C.r];
-    uint32_t *words = bitmap + R.woff[C.r];
-    Cand *cb = cand + cand_off[C.r];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t lt = gbd::lanemask_lt();
-    for (int k = 0; k < ROUNDS; ++k) {
-        const uint32_t rel0 = C.start + (uint32_t)warp * (ROUNDS * 32) + (uint32_t)k * 32;
-        if (rel0 >= C.count) break; // warp-uniform
-        const uint32_t rel = rel0 + lane;
-        const bool ok = rel < C.count;
-        uint64_t key = 0;
-        uint32_t id = 0, d = 0xFFFFFFFFu;
-        if (ok) {
-            key = sel_key(in, C.first + rel, C.code, seed, equal_mass, id);
-            d = C.logb ? (uint32_t)(key >> (64 - C.logb)) : 0u;
+    static_assert(CH == ST * 16, "16 elements a thread");
+    __shared__ uint32_t sum;
+    if (threadIdx.x == 0) sum = 0u;
+    const Chunk C = load_chunk(chunks);
+    __syncthreads();
+    const uint32_t b = tb[C.r], at = threadIdx.x * 16;
+    uint32_t code[16];
+    if (CODES) {
+        const uint4 *p = reinterpret_cast<const uint4 *>(codes + (size_t)blockIdx.x * CH + at);
+        const uint4 q0 = __ldg(p), q1 = __ldg(p + 1);
+        const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+        for (int k = 0; k < 16; ++k) code[k] = k & 1 ? w[k >> 1] >> 16 : w[k >> 1] & 0xFFFFu;
+    } else {
+#pragma unroll 4
+        for (int k = 0; k < 16; ++k) {
+            uint32_t mid;
+            code[k] = at + k < C.len ? sel_code(in, C.j0 + at + k, C, seed, equal_mass, mid) : CODE_NONE;
         }
-        const uint32_t below = __ballot_sync(0xffffffffu, ok && d < b);
-        if (lane == 0) words[rel0 >> 5] = below;
-        const uint32_t eq = __ballot_sync(0xffffffffu, ok && d == b);
-        if (eq) {
-            const int leader = __ffs(eq) - 1;
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(&cursor[C.r], (uint32_t)__popc(eq));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (ok && d == b) cb[base + __popc(eq & lt)] = Cand{key, id, rel};
+    }
+    uint32_t below = 0, eq = 0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const uint32_t low = code[k] & CODE_NONE, high = low + (code[k] >> 15);
+        below |= high < b ? 1u << k : 0u;
+        eq |= low <= b && b <= high ? 1u << k : 0u;
+    }
+    // two threads' 16 bits are a bitmap word (the last may lie past the node's words)
+    const uint32_t other = __shfl_down_sync(0xffffffffu, below, 1);
+    if (!(threadIdx.x & 1) && at < C.len) bitmap[C.words + (at >> 5)] = below | other << 16;
+    const uint32_t nk = __reduce_add_sync(0xffffffffu, __popc(below));
+    if ((threadIdx.x & 31) == 0 && nk) atomicAdd(&sum, nk);
+    if (eq) {
+        Cand *cb = cand + cand_off[C.r];
+        uint32_t to = atomicAdd(&cursor[C.r], (uint32_t)__popc(eq));
+        while (eq) {
+            const uint32_t i = at + (uint32_t)(__ffs(eq) - 1);
+            eq &= eq - 1u;
+            uint32_t id;
+            const uint64_t key = sel_key(in, C.j0 + i, C.code, seed, equal_mass, id);
+            cb[to++] = Cand{key, id, C.start + i};
         }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        chunk_sel[blockIdx.x] = sum;
+        if (sum) atomicAdd(&kept[C.r], sum);
     }
 }
 
@@ -221,18 +325,25 @@ __device__ __forceinline__ uint32_t digit96(const Cand &c, int sh, int nbits)
     return (uint32_t)(v & ((1ull << nbits) - 1ull));
 }
 
-__global__ void __launch_bounds__(ST) k_sel_resolve(RepInfo R, const uint32_t *need_in, const uint64_t *ccount,
-                                                    const uint64_t *cand_off, uint64_t cand_total, Cand *cand,
-                                                    uint32_t *bitmap)
+// The candidates' members: their n_max - kept smallest (key, id).  Equal-mass candidates share their top
+// logb key bits; keys of unequal masses start at the sign bit.
+__global__ void __launch_bounds__(ST) k_sel_resolve(RepInfo R, uint32_t n_max, int equal_mass, const uint32_t *kept,
+                                                    const uint32_t *ncand, const uint64_t *cand_off,
+                                                    uint64_t cand_total, Cand *cand, uint32_t *bitmap,
+                                                    uint32_t *chunk_sel)
 {
     __shared__ uint32_t hist[256];
     __shared__ uint32_t s_b, s_cum, s_hb, s_cnt;
     const uint32_t r = blockIdx.x;
-    uint32_t m = (uint32_t)ccount[r], need = need_in[r];
+    uint32_t m = ncand[r], need = n_max - kept[r];
     Cand *A = cand + cand_off[r];
     Cand *B = cand + cand_total + cand_off[r];
-    uint32_t *words = bitmap + R.woff[r];
-    int top = 96 - R.logb[r];
+    uint32_t *words = bitmap + R.woff[r], *sel = chunk_sel + R.chunk_off[r];
+    auto keep = [&](uint32_t rel) {
+        atomicOr(&words[rel >> 5], 1u << (rel & 31));
+        atomicAdd(&sel[rel / CH], 1u);
+    };
+    int top = 96 - (equal_mass ? R.logb[r] : 0);
     while (need < m && top > 0) {
         const int nbits = top < 8 ? top : 8;
         const int sh = top - nbits;
@@ -241,87 +352,70 @@ __global__ void __launch_bounds__(ST) k_sel_resolve(RepInfo R, const uint32_t *n
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < m; i += ST) atomicAdd(&hist[digit96(A[i], sh, nbits)], 1u);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t cum = 0, q = 0;
-            for (; q < (1u << nbits); ++q) {
-                if (cum + hist[q] >= need) break;
-                cum += hist[q];
-            }
-            s_b = q;
+        // the digit that holds rank `need`
+        uint32_t tot;
+        const uint32_t hv = hist[threadIdx.x], cum = block_scan_u32(hv, tot);
+        if (cum < need && need <= cum + hv) {
+            s_b = threadIdx.x;
             s_cum = cum;
-            s_hb = hist[q];
+            s_hb = hv;
         }
         __syncthreads();
         const uint32_t b = s_b;
-        for (uint32_t i = threadIdx.x; i < m; i += ST) {
-            const Cand c = A[i];
-            const uint32_t d = digit96(c, sh, nbits);
-            if (d < b)
-                atomicOr(&words[c.rel >> 5], 1u << (c.rel & 31));
-            else if (d == b)
-                B[atomicAdd(&s_cnt, 1u)] = c;
+        if (s_hb < m) { // else every candidate has this digit
+            for (uint32_t i = threadIdx.x; i < m; i += ST) {
+                const Cand c = A[i];
+                const uint32_t d = digit96(c, sh, nbits);
+                if (d < b)
+                    keep(c.rel);
+                else if (d == b)
+                    B[atomicAdd(&s_cnt, 1u)] = c;
+            }
+            Cand *t = A;
+            A = B;
+            B = t;
         }
         __syncthreads();
         need -= s_cum;
         m = s_hb;
-        Cand *t = A;
-        A = B;
-        B = t;
         top = sh;
         __syncthreads();
     }
     // the remaining candidates are all kept (need == m), or, only possible with duplicate ids,
     // the first `need` of them
-    for (uint32_t i = threadIdx.x; i < m && i < need; i += ST) atomicOr(&words[A[i].rel >> 5], 1u << (A[i].rel & 31));
+    for (uint32_t i = threadIdx.x; i < m && i < need; i += ST) keep(A[i].rel);
 }
+static_assert(ST == 256, "one thread per digit");
 
-__global__ void __launch_bounds__(ST) k_sel_count(SelectIn in, RepInfo R, uint32_t n_rep, const uint32_t *bitmap,
-                                                  uint32_t *chunk_sel)
-{
-    ChunkCtx C;
-    load_chunk(C, in, R, n_rep);
-    const uint32_t len = min(CH, C.count - C.start);
-    const uint32_t nw = (len + 31) / 32;
-    const uint32_t *words = bitmap + R.woff[C.r] + C.start / 32;
-    uint32_t v = 0;
-    for (uint32_t i = threadIdx.x; i < nw; i += ST) v += __popc(words[i]);
-    uint32_t tot;
-    (void)block_scan_u32(v, tot);
-    if (threadIdx.x == 0) chunk_sel[blockIdx.x] = tot;
-}
-
-__global__ void __launch_bounds__(ST) k_sel_write(SelectIn in, RepInfo R, uint32_t n_rep, const uint32_t *bitmap,
+__global__ void __launch_bounds__(ST) k_sel_write(SelectIn in, const Chunk *chunks, const uint32_t *bitmap,
                                                   const uint32_t *chunk_pos)
 {
     __shared__ uint32_t woff[ST / 32];
-    ChunkCtx C;
-    load_chunk(C, in, R, n_rep);
+    const Chunk C = load_chunk(chunks);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t len = min(CH, C.count - C.start);
-    const uint32_t nw = (len + 31) / 32;
-    const uint32_t *words = bitmap + R.woff[C.r] + C.start / 32;
+    const uint32_t nw = (C.len + 31) / 32;
+    const uint32_t *words = bitmap + C.words;
     const uint32_t w0 = (uint32_t)warp * ROUNDS;
-    uint32_t mine = 0;
-    for (int q = lane; q < ROUNDS; q += 32)
-        if (w0 + q < nw) mine += __popc(words[w0 + q]);
-    for (int d = 16; d > 0; d >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, d);
+    const uint32_t mw = lane < ROUNDS && w0 + lane < nw ? words[w0 + lane] : 0u; // the warp's words, one a lane
+    const uint32_t mine = __reduce_add_sync(0xffffffffu, __popc(mw));
     if (lane == 0) woff[warp] = mine;
     __syncthreads();
-    uint32_t base = chunk_pos[blockIdx.x] - chunk_pos[R.chunk_off[C.r]];
+    uint32_t base = chunk_pos[blockIdx.x] - C.r * in.n_max; // every node before it keeps n_max
     for (int w = 0; w < warp; ++w) base += woff[w];
+    if (!mine) return;
     const uint64_t pf = in.npfirst[C.node];
     const float wr = in.nw[C.node], sr = in.ns[C.node];
     const uint32_t lt = gbd::lanemask_lt();
     float hm = 0.0f;
+    const uint32_t j0 = C.j0 + w0 * 32 + lane;
+#pragma unroll 4
     for (int q = 0; q < ROUNDS; ++q) {
-        const uint32_t wi = w0 + q;
-        if (wi >= nw) break;
-        const uint32_t W = words[wi];
+        const uint32_t W = __shfl_sync(0xffffffffu, mw, q);
         const uint32_t rank = base + __popc(W & lt);
         if (((W >> lane) & 1u) && rank < in.n_max) {
             const uint64_t idx = pf + rank;
-            const uint32_t j = C.first + C.start + wi * 32 + lane;
-            const float4 p = in.s4[j];
+            const uint32_t j = j0 + q * 32;
+            const float4 p = __ldg(&in.s4[j]);
             const float h = __fmul_rn(p.w, sr);
             in.pts4[idx] = make_float4(p.x, p.y, p.z, wr);
             in.hs[idx] = h;
@@ -349,53 +443,60 @@ template <class T> T readback(const T *d, cudaStream_t s, HostStage &hs)
 
 void select_representatives(const Allocator &A, cudaStream_t s, HostStage &hs, ScanTmp &scan, const SelectIn &in,
                             const uint32_t *rep_nodes, uint32_t n_rep, uint32_t n_max, uint64_t seed,
-                            int equal_mass)
+                            int equal_mass, void *spare, size_t spare_bytes)
 {
     Scratch<uint32_t> nchunks(A, n_rep + 1, s), chunk_off(A, n_rep + 1, s), nbins(A, n_rep, s), hoff(A, n_rep, s);
     Scratch<uint64_t> nwords(A, n_rep, s), woff(A, n_rep, s);
     Scratch<uint8_t> logb(A, n_rep, s);
+    Scratch<int16_t> bin0(A, n_rep, s);
+    Scratch<float> rmean(A, n_rep, s);
     Scratch<uint32_t> tot32(A, 2, s);
     Scratch<uint64_t> tot64(A, 1, s);
     launch(GBLOD_K_BUILD_OTHER, k_sel_setup, dim3((n_rep + 255) / 256), dim3(256), 0, s, n_rep, rep_nodes, in.ncount,
-           nchunks.p, nbins.p, logb.p, nwords.p);
+           in.nw, n_max, equal_mass, nchunks.p, nbins.p, logb.p, bin0.p, rmean.p,
+           nwords.p);
     scan_exclusive_u32(A, scan, nchunks.p, chunk_off.p, n_rep, chunk_off.p + n_rep, s);
     scan_exclusive_u32(A, scan, nbins.p, hoff.p, n_rep, tot32.p, s);
     scan_exclusive_u64(A, scan, nwords.p, woff.p, n_rep, tot64.p, s);
-    uint32_t totals[2];
-    GB_CUDA(cudaMemcpyAsync(static_cast<uint32_t *>(hs.get(16)), chunk_off.p + n_rep, 4, cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(static_cast<uint32_t *>(hs.get(16)) + 1, tot32.p, 4, cudaMemcpyDeviceToHost, s));
+    uint32_t *h32 = static_cast<uint32_t *>(hs.get(16));
+    uint64_t *h64 = reinterpret_cast<uint64_t *>(h32 + 2);
+    GB_CUDA(cudaMemcpyAsync(h32, chunk_off.p + n_rep, 4, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(h32 + 1, tot32.p, 4, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(h64, tot64.p, 8, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
-    totals[0] = static_cast<uint32_t *>(hs.get(16))[0];
-    totals[1] = static_cast<uint32_t *>(hs.get(16))[1];
-    const uint64_t total_words = readback(tot64.p, s, hs);
-    const uint32_t n_chunks = totals[0], n_bins = totals[1];
+    const uint32_t n_chunks = h32[0], n_bins = h32[1];
+    const uint64_t total_words = *h64;
 
-    RepInfo R{rep_nodes, chunk_off.p, hoff.p, logb.p, woff.p};
-    Scratch<uint32_t> hist(A, n_bins, s), tb(A, n_rep, s), need(A, n_rep, s);
-    Scratch<uint64_t> ccount(A, n_rep, s), cand_off(A, n_rep, s);
+    RepInfo R{rep_nodes, chunk_off.p, hoff.p, logb.p, bin0.p, rmean.p, woff.p};
+    Scratch<Chunk> chunks(A, n_chunks, s);
+    launch(GBLOD_K_BUILD_OTHER, k_sel_chunks, dim3((n_chunks + 255) / 256), dim3(256), 0, s, n_chunks, n_rep, in, R,
+           chunks.p);
+    uint16_t *codes = (size_t)n_chunks * CH * sizeof(uint16_t) <= spare_bytes ? static_cast<uint16_t *>(spare) : nullptr;
+    Scratch<uint32_t> hist(A, n_bins, s), tb(A, n_rep, s), counters(A, 2 * (size_t)n_rep, s);
+    Scratch<uint64_t> ccap(A, n_rep, s), cand_off(A, n_rep, s);
     Scratch<uint32_t> bitmap(A, total_words, s);
+    uint32_t *cursor = counters.p, *kept = counters.p + n_rep;
     GB_CUDA(cudaMemsetAsync(hist.p, 0, (size_t)n_bins * 4, s));
-    launch(GBLOD_K_SEL_HIST, k_sel_hist, dim3(n_chunks), dim3(ST), 0, s, in, R, n_rep, seed, equal_mass, hist.p);
-    launch(GBLOD_K_BUILD_OTHER, k_sel_find, dim3(n_rep), dim3(ST), 0, s, R, n_max, (const uint32_t *)hist.p, tb.p,
-           need.p, ccount.p);
-    scan_exclusive_u64(A, scan, ccount.p, cand_off.p, n_rep, tot64.p, s);
+    GB_CUDA(cudaMemsetAsync(counters.p, 0, 2 * (size_t)n_rep * 4, s));
+    launch(GBLOD_K_SEL_HIST, k_sel_hist, dim3(n_chunks), dim3(ST), 0, s, in, R, (const Chunk *)chunks.p, seed,
+           equal_mass, hist.p, codes);
+    launch(GBLOD_K_BUILD_OTHER, k_sel_find, dim3(n_rep), dim3(ST), 0, s, R, n_max, equal_mass, (const uint32_t *)hist.p,
+           tb.p, ccap.p);
+    scan_exclusive_u64(A, scan, ccap.p, cand_off.p, n_rep, tot64.p, s);
     const uint64_t cand_total = readback(tot64.p, s, hs);
     Scratch<Cand> cand(A, 2 * (size_t)cand_total + 2, s);
-    Scratch<uint32_t> cursor(A, n_rep, s);
-    GB_CUDA(cudaMemsetAsync(cursor.p, 0, (size_t)n_rep * 4, s));
-    launch(GBLOD_K_SEL_MARK, k_sel_mark, dim3(n_chunks), dim3(ST), 0, s, in, R, n_rep, seed, equal_mass,
-           (const uint32_t *)tb.p, (const uint64_t *)cand_off.p, cursor.p, cand.p, bitmap.p);
-    launch(GBLOD_K_BUILD_OTHER, k_sel_resolve, dim3(n_rep), dim3(ST), 0, s, R, (const uint32_t *)need.p,
-           (const uint64_t *)ccount.p, (const uint64_t *)cand_off.p, cand_total, cand.p, bitmap.p);
     Scratch<uint32_t> chunk_sel(A, n_chunks, s), chunk_pos(A, n_chunks, s);
-    launch(GBLOD_K_BUILD_OTHER, k_sel_count, dim3(n_chunks), dim3(ST), 0, s, in, R, n_rep, (const uint32_t *)bitmap.p,
-           chunk_sel.p);
+    launch(GBLOD_K_SEL_MARK, codes ? k_sel_mark<true> : k_sel_mark<false>, dim3(n_chunks), dim3(ST), 0, s, in,
+           (const Chunk *)chunks.p, seed, equal_mass, (const uint16_t *)codes, (const uint32_t *)tb.p, (const uint64_t *)cand_off.p, cursor, kept,
+           chunk_sel.p, cand.p, bitmap.p);
+    launch(GBLOD_K_BUILD_OTHER, k_sel_resolve, dim3(n_rep), dim3(ST), 0, s, R, n_max, equal_mass, (const uint32_t *)kept,
+           (const uint32_t *)cursor, (const uint64_t *)cand_off.p, cand_total, cand.p, bitmap.p, chunk_sel.p);
     scan_exclusive_u32(A, scan, chunk_sel.p, chunk_pos.p, n_chunks, tot32.p, s);
-    launch(GBLOD_K_SEL_WRITE, k_sel_write, dim3(n_chunks), dim3(ST), 0, s, in, R, n_rep, (const uint32_t *)bitmap.p,
+    launch(GBLOD_K_SEL_WRITE, k_sel_write, dim3(n_chunks), dim3(ST), 0, s, in, (const Chunk *)chunks.p, (const uint32_t *)bitmap.p,
            (const uint32_t *)chunk_pos.p);
-    const uint32_t kept = readback(tot32.p, s, hs); // modulo 2^32, like the positions it sums
-    if (kept != (uint32_t)((uint64_t)n_rep * n_max))
-        fail(GBLOD_ERR_CUDA, "subselection kept " + std::to_string(kept) + " points, expected " +
+    const uint32_t n_kept = readback(tot32.p, s, hs); // modulo 2^32, like the positions it sums
+    if (n_kept != (uint32_t)((uint64_t)n_rep * n_max))
+        fail(GBLOD_ERR_CUDA, "subselection kept " + std::to_string(n_kept) + " points, expected " +
                                  std::to_string((uint64_t)n_rep * n_max));
 }
 
