@@ -190,9 +190,8 @@ __device__ __forceinline__ bool direct_box(int x0, int x1, int y0, int y1)
 constexpr int R_NARROW = 46340;
 
 // One point's clipped pixel box for walk_boxes: n pixels (0: none) from origin xy = x0 | y0 << 16,
-// meta = ceil(2^8 / bw) | bw << 9 | wide << 13 | kernel << 14 | Wl << 16 for box width bw <=
-// DIRECT_BOX and the radial kernel's table (0 Gaussian, 1 cubic), and the rule's other operands U,
-// V, S and Wh (Wq = Wh 2^16 + Wl).
+// meta = ceil(2^8 / bw) | bw << 9 | wide << 13 | Wl << 16 for box width bw <= DIRECT_BOX, and the
+// rule's other operands U, V, S and Wh (Wq = Wh 2^16 + Wl).
 struct BoxWalk {
     uint32_t n = 0, xy = 0, meta = 0;
     int U = 0, V = 0;
@@ -200,13 +199,13 @@ struct BoxWalk {
 };
 
 __device__ __forceinline__ BoxWalk box_walk(int U, int V, uint32_t S, unsigned long long Wq, int r, int x0, int x1,
-                                            int y0, int y1, int kernel = 0)
+                                            int y0, int y1)
 {
     BoxWalk b;
     const uint32_t bw = (uint32_t)(x1 - x0 + 1);
     b.n = bw * (uint32_t)(y1 - y0 + 1);
     b.xy = (uint32_t)x0 | ((uint32_t)y0 << 16);
-    b.meta = ((256u + bw - 1u) / bw) | (bw << 9) | (r > R_NARROW ? 1u << 13 : 0u) | ((uint32_t)kernel << 14) |
+    b.meta = ((256u + bw - 1u) / bw) | (bw << 9) | (r > R_NARROW ? 1u << 13 : 0u) |
              ((uint32_t)(Wq & 0xFFFFull) << 16);
     b.U = U;
     b.V = V;
@@ -286,16 +285,17 @@ __device__ __forceinline__ unsigned walk_boxes(const BoxWalk &b, uint32_t tag, T
 // takes one point of the warp's (on: this lane has one), a column per lane, row by row.  A round of 32
 // (point, pixel) pairs is about 14 instructions, where walk_boxes spends some 66 more on finding each
 // pair's point and shuffling its operands; columns and rows a box does not have idle.  Distances in 32
-// bits and Wq < 2^32 (group_box decides; walk_boxes takes the rest).  K has a zero entry 1024.  add(x, y, c)
-// receives every nonzero contribution c < 2^32.  Returns this lane's pixel updates (COUNT).  Every lane of the
+// bits and Wq < 2^32 (group_box decides; walk_boxes takes the rest).  K has a zero entry 1024.  at(t, x, y) gives,
+// for a box's column x from row y (t: the point's tag if TAGGED, else 0), the function (j, c) that receives every
+// nonzero contribution c < 2^32 to row y + j.  Returns this lane's pixel updates (COUNT).  Every lane of the
 // warp calls it.  Small boxes of 150M particles, the whole box in view (k_splat_small): 7.9 ms walked, 8.1 ms with
 // this alone, 6.6 ms with the smallest boxes in lane_boxes (the shuffles and lookups of idle lanes bind
 // here: the additions alone are 0.8 ms).  LOD scatter of 16.8M particles 0.59 -> 0.43 ms.
 __device__ __forceinline__ bool group_box(int r, float Wf) { return r <= R_NARROW && Wf < 0x1p32f; }
 
-template <bool COUNT, class Add>
+template <bool COUNT, bool TAGGED = false, class At>
 __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t S, float Wf, int x0, int x1, int y0,
-                                                int y1, const int32_t *K, Add add)
+                                                int y1, const int32_t *K, At at, uint32_t tag = 0u)
 {
     static_assert(DIRECT_BOX <= 8, "a group's lanes are the columns of a box");
     const uint32_t m = __ballot_sync(0xffffffffu, on);
@@ -316,13 +316,14 @@ __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t 
         const uint32_t qxy = __shfl_sync(0xffffffffu, xy, src), qext = __shfl_sync(0xffffffffu, ext, src);
         const int qU = __shfl_sync(0xffffffffu, U, src), qV = __shfl_sync(0xffffffffu, V, src);
         const uint32_t qS = __shfl_sync(0xffffffffu, S, src), qW = __shfl_sync(0xffffffffu, Wq, src);
+        const uint32_t t = TAGGED ? __shfl_sync(0xffffffffu, tag, src) : 0u;
         const uint32_t Wh = qW >> 16, Wl = qW & 0xFFFFu;
+        const auto add = at(t, (int)(qxy & 0xFFFFu) + col, (int)(qxy >> 16));
         const bool act = k < n && col <= (int)(qext & 0xFFu);
         const int rows = act ? (int)(qext >> 8) + 1 : 0;
-        const int x = (int)(qxy & 0xFFFFu) + col, y = (int)(qxy >> 16);
-        const int dx = x * 256 + 128 - qU;
+        const int dx = ((int)(qxy & 0xFFFFu) + col) * 256 + 128 - qU;
         const uint32_t dx2 = (uint32_t)(dx * dx);
-        const int dy = y * 256 + 128 - qV;
+        const int dy = (int)(qxy >> 16) * 256 + 128 - qV;
         const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)rows);
         for (int j0 = 0; j0 < most; j0 += 4) { // four rows' lookups in flight, no branch but the additions
             uint32_t c[4];
@@ -336,7 +337,7 @@ __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t 
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (c[j]) add(x, y + j0 + j, c[j]);
+                if (c[j]) add(j0 + j, c[j]);
         }
     }
     return hits;
@@ -987,7 +988,10 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
             if (!SMALL) {
                 hits += group_boxes<true>(
                     mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K,
-                    [&](int x, int y, uint32_t c) { atomicAdd(&img[(size_t)y * P.W + x], (unsigned long long)c); });
+                    [&](uint32_t, int x, int y) {
+                        unsigned long long *p = img + (size_t)y * P.W + x;
+                        return [p, &P](int j, uint32_t c) { atomicAdd(&p[(size_t)j * P.W], (unsigned long long)c); };
+                    });
                 hits += walk_boxes<false>(
                     direct, 0u, [&](uint32_t, uint32_t i) { return K[i]; },
                     [&](uint32_t, int x, int y, unsigned long long c) { atomicAdd(&img[(size_t)y * P.W + x], c); });
@@ -1066,14 +1070,17 @@ __global__ void __launch_bounds__(RT, 4) k_splat_small(const uint4 *__restrict__
         }
         // a contribution below 2^32 as 20 low bits and, where it has more, the rest in the middle word
         // (2^12 contributions of less than 2^20 stay below 2^32)
-        auto add = [&](int x, int y, uint32_t c) {
+        auto at = [&](uint32_t, int x, int y) {
             const int p = (y - Y0) * TW + (x - X0);
-            atomicAdd(&lo[p], c & 0xFFFFFu);
-            if (c >> 20) atomicAdd(&mid[p], (c >> 20) << 4);
+            return [=](int j, uint32_t c) {
+                atomicAdd(&lo[p + j * TW], c & 0xFFFFFu);
+                if (c >> 20) atomicAdd(&mid[p + j * TW], (c >> 20) << 4);
+            };
         };
         const bool tiny = mine && x1 - x0 < LANE_BOX && y1 - y0 < LANE_BOX;
-        hits += lane_boxes<COUNT>(tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K, add);
-        hits += group_boxes<COUNT>(mine && !tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K, add);
+        hits += lane_boxes<COUNT>(tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K,
+                                  [&](int x, int y, uint32_t c) { at(0u, x, y)(0, c); });
+        hits += group_boxes<COUNT>(mine && !tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K, at);
         hits += walk_boxes<false>(b, 0u, [&](uint32_t, uint32_t i) { return K[i]; },
                                   [&](uint32_t, int x, int y, unsigned long long c) {
             const int p = (y - Y0) * TW + (x - X0);
@@ -1419,49 +1426,95 @@ __global__ void __launch_bounds__(RT, 4) k_splat_tiles(const uint4 *__restrict__
 }
 
 // ------------------------------------------------------------------ R4
-__global__ void k_image_max(const unsigned long long *img, size_t n, unsigned long long *out)
+// Both passes over an image keep eight pixels' loads in flight per thread; they read 8 bytes a pixel, and with
+// one load a thread they waited for memory (eight views, 20.7M pixels: maximum 0.193 -> 0.036 ms, tone map
+// 0.249 -> 0.054 ms).
+constexpr int PX = 8;
+
+__device__ __forceinline__ unsigned long long pixels_max(const unsigned long long *__restrict__ img, size_t n)
 {
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
     unsigned long long m = 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        m = img[i] > m ? img[i] : m;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += PX * stride) {
+        unsigned long long a[PX];
+#pragma unroll
+        for (int k = 0; k < PX; ++k) a[k] = i + k * stride < n ? __ldg(&img[i + k * stride]) : 0ull;
+#pragma unroll
+        for (int k = 0; k < PX; ++k) m = a[k] > m ? a[k] : m;
+    }
     for (int d = 16; d > 0; d >>= 1) {
         const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, d);
         m = o > m ? o : m;
     }
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+    return m;
 }
 
 // out = 0 if I <= lo, else min(255, rne(255 ln(I/lo) / ln(hi/lo))), I = acc 2^-32
-__global__ void k_tonemap(const unsigned long long *img, size_t n, const unsigned long long *maxv, int auto_range,
-                          double lo_acc_fixed, double hi_acc_fixed, uint8_t *out)
+__device__ __forceinline__ void pixels_tone(const unsigned long long *__restrict__ img, size_t n, double lo, double hi,
+                                            uint8_t *__restrict__ out)
 {
-    __shared__ double s_lo;
+    __shared__ unsigned long long s_low;
     __shared__ float s_l2lo, s_scale;
-    __shared__ int s_ok;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long a[PX];
+    auto load = [&] {
+#pragma unroll
+        for (int k = 0; k < PX; ++k) a[k] = i + k * stride < n ? __ldg(&img[i + k * stride]) : 0ull;
+    };
+    load(); // under the range's logarithms
     if (threadIdx.x == 0) {
-        double hi = hi_acc_fixed, lo = lo_acc_fixed;
-        if (auto_range) {
-            hi = (double)*maxv;
-            lo = hi * 1e-4;
+        const bool ok = hi > 0.0 && lo > 0.0 && hi > lo;
+        // the largest accumulator a with !((double)a > lo): a compare of integers per pixel, where FP64
+        // runs at 1/64 of the integer rate.  From 2^53 on, (double)a rounds to nearest even.
+        unsigned long long low = ~0ull;
+        if (ok && lo < 0x1p64) {
+            low = (unsigned long long)lo;
+            if (lo >= 0x1p53) {
+                low += (1ull << (63 - __clzll((long long)low) - 52)) / 2; // half a step above
+                if ((double)low > lo) --low;
+            }
         }
-        s_ok = (hi > 0.0 && lo > 0.0 && hi > lo) ? 1 : 0;
-        s_lo = lo;
-        s_l2lo = s_ok ? (float)log2(lo) : 0.0f;
-        s_scale = s_ok ? (float)(255.0 / log2(hi / lo)) : 0.0f;
+        s_low = low;
+        s_l2lo = ok ? (float)log2(lo) : 0.0f;
+        s_scale = ok ? (float)(255.0 / log2(hi / lo)) : 0.0f;
     }
     __syncthreads();
-    const double lo = s_lo;
+    const unsigned long long low = s_low;
     const float l2lo = s_l2lo, scale = s_scale;
-    const int ok = s_ok;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const unsigned long long a = img[i];
-        uint8_t o = 0;
-        if (ok && (double)a > lo) {
-            const float t = rintf((log2f((float)a) - l2lo) * scale);
-            o = (uint8_t)(t > 255.0f ? 255.0f : (t < 0.0f ? 0.0f : t));
+    while (i < n) {
+#pragma unroll
+        for (int k = 0; k < PX; ++k) {
+            const float t = rintf((log2f((float)a[k]) - l2lo) * scale);
+            const uint8_t o = a[k] > low ? (uint8_t)(t > 255.0f ? 255.0f : (t < 0.0f ? 0.0f : t)) : (uint8_t)0;
+            if (i + k * stride < n) out[i + k * stride] = o;
         }
-        out[i] = o;
+        i += PX * stride;
+        load();
     }
+}
+
+__global__ void __launch_bounds__(256) k_image_max(const unsigned long long *img, size_t n, unsigned long long *out)
+{
+    const unsigned long long m = pixels_max(img, n);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+}
+
+__global__ void __launch_bounds__(256) k_tonemap(const unsigned long long *img, size_t n, const unsigned long long *maxv,
+                                                 int auto_range, double lo_acc_fixed, double hi_acc_fixed, uint8_t *out)
+{
+    double hi = hi_acc_fixed, lo = lo_acc_fixed;
+    if (auto_range) {
+        hi = (double)*maxv;
+        lo = hi * 1e-4;
+    }
+    pixels_tone(img, n, lo, hi, out);
+}
+
+// blocks for R4 over npix pixels in all: a thread's eight pixels or more
+unsigned tone_blocks(unsigned long long npix)
+{
+    return (unsigned)std::max<unsigned long long>(1, std::min<unsigned long long>((unsigned long long)persistent_blocks(8), npix / (256 * PX)));
 }
 
 __global__ void k_project_debug(const float4 *pts4, const float *h, size_t n, Proj P, long long *out)
@@ -1684,13 +1737,13 @@ void frame_common(gblod_renderer *r, const Src &src, const Proj &P, const gblod_
         double lo = 0.0, hi = 0.0;
         if (rp.tone_auto) {
             GB_CUDA(cudaMemsetAsync(r->maxv.p, 0, 8, s));
-            launch(GBLOD_K_TONEMAP, k_image_max, dim3(persistent_blocks(2)), dim3(256), 0, s,
+            launch(GBLOD_K_TONEMAP, k_image_max, dim3(tone_blocks(npix)), dim3(256), 0, s,
                    (const unsigned long long *)img, npix, r->maxv.p);
         } else {
             lo = std::ldexp(rp.tone_lo, 32);
             hi = std::ldexp(rp.tone_hi, 32);
         }
-        launch(GBLOD_K_TONEMAP, k_tonemap, dim3(persistent_blocks(2)), dim3(256), 0, s,
+        launch(GBLOD_K_TONEMAP, k_tonemap, dim3(tone_blocks(npix)), dim3(256), 0, s,
                (const unsigned long long *)img, npix, (const unsigned long long *)r->maxv.p, rp.tone_auto ? 1 : 0,
                lo, hi, image);
     }
@@ -1874,17 +1927,27 @@ __device__ __forceinline__ int bsrc_load(const SrcBatch &s, unsigned long long e
 
 // Counting pass (SCATTER false) or record pass (true) over the flat point space of a batch; the
 // record pass also splats the points with small boxes into their view's image, and counts their
-// pixel updates when count_updates is set.
-template <bool SCATTER>
-__global__ void __launch_bounds__(RT) k_bproject(SrcBatch src, uint32_t *__restrict__ tile_cnt,
-                                                 uint32_t *__restrict__ cursor, uint4 *__restrict__ rec,
+// pixel updates when count_updates is set.  PART: binned in parts like an octree frame, the tiles of all
+// views in one shared-memory histogram; `tiles` is the (tile, CTA) histogram (counting) or its scan (records).
+// Else it is the tiles' counts or cursors.  (Eight views, 1080p, count + records: 4.5 ms with global counters
+// and walked boxes, 2.3 ms in parts and with group_boxes.)
+template <bool SCATTER, bool PART>
+__global__ void __launch_bounds__(RT, 4) k_bproject(SrcBatch src, uint32_t *__restrict__ tiles,
+                                                 uint32_t ntiles, int kernel, uint4 *__restrict__ rec,
                                                  unsigned long long rec_cap, unsigned *status, FrameStatsDev *stats,
                                                  int count_updates)
 {
+    extern __shared__ uint32_t sh_tiles[]; // PART: [ntiles] counts or next record positions
+    __shared__ int32_t K[SCATTER ? 1025 : 1];
+    if (PART)
+        for (uint32_t t = threadIdx.x; t < ntiles; t += RT)
+            sh_tiles[t] = SCATTER ? tiles[(size_t)t * gridDim.x + blockIdx.x] : 0u;
+    if (SCATTER)
+        for (int t = threadIdx.x; t <= 1024; t += RT) K[t] = t < 1024 ? g_ktab[kernel][t] : 0;
+    __syncthreads();
     const unsigned long long total = *src.total;
     unsigned hits = 0;
     const int lane = threadIdx.x & 31;
-    const uint32_t lt = gbd::lanemask_lt();
     unsigned long long splats = 0, pairs = 0;
     AmpSum amp;
     __shared__ Proj sP[2];
@@ -1919,16 +1982,19 @@ __global__ void __launch_bounds__(RT) k_bproject(SrcBatch src, uint32_t *__restr
             int tw = 1, tiles_x = 1;
             uint4 r = make_uint4(0u, 0u, 0u, 0u);
             BoxWalk direct;
+            bool mine = false;
+            int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
             if (res == 1) {
                 const Proj &P = v == sV[0] ? sP[0] : (v == sV[1] ? sP[1] : src.views[v].P);
                 const uint32_t tb = src.views[v].tile_base;
                 if (!SCATTER) ++splats;
-                int x0, x1, y0, y1;
                 const int rad = splat_box(s.U, s.V, s.S, P.W, P.H, x0, x1, y0, y1);
                 if (x0 <= x1 && y0 <= y1) {
                     if (direct_box(x0, x1, y0, y1)) {
-                        if (SCATTER)
-                            direct = box_walk(s.U, s.V, s.S, __float2ull_rn(s.Wf), rad, x0, x1, y0, y1, P.kernel);
+                        if (SCATTER) {
+                            mine = group_box(rad, s.Wf);
+                            if (!mine) direct = box_walk(s.U, s.V, s.S, __float2ull_rn(s.Wf), rad, x0, x1, y0, y1);
+                        }
                     } else {
                         const int tx0 = x0 / P.TW, tx1 = x1 / P.TW, ty0 = y0 / P.TH, ty1 = y1 / P.TH;
                         tw = tx1 - tx0 + 1;
@@ -1941,26 +2007,44 @@ __global__ void __launch_bounds__(RT) k_bproject(SrcBatch src, uint32_t *__restr
                 }
             }
             if (SCATTER) {
-                scatter_pairs(n, t00, tw, tiles_x, r, cursor, rec, rec_cap);
-                hits += walk_boxes<true>(
-                    direct, (uint32_t)v, [&](uint32_t meta, uint32_t i) { return g_ktab[(meta >> 14) & 1u][i]; },
-                    [&](uint32_t t, int x, int y, unsigned long long c) {
-                        atomicAdd(&src.views[t].accum[(size_t)y * src.views[t].P.W + x], c);
-                    });
-            } else if (n) {
-                // counting: fire-and-forget atomics, so the per-lane loop is cheaper than the
-                // warp-cooperative walk
-                for (uint32_t m = 0; m < n; ++m) {
-                    const uint32_t row = m / (uint32_t)tw;
-                    const uint32_t t = t00 + row * (uint32_t)tiles_x + (m - row * (uint32_t)tw);
-                    const uint32_t peers = __match_any_sync(__activemask(), t);
-                    if (lane == __ffs(peers) - 1) atomicAdd(&tile_cnt[t], (uint32_t)__popc(peers));
+                if (PART) {
+                    const uint32_t th = n / (uint32_t)tw;
+                    for (uint32_t ty = 0; ty < th; ++ty)
+                        for (uint32_t tx = 0; tx < (uint32_t)tw; ++tx) {
+                            const uint32_t pos = atomicAdd(&sh_tiles[t00 + ty * (uint32_t)tiles_x + tx], 1u);
+                            if (pos < rec_cap) rec[pos] = r;
+                        }
+                } else {
+                    scatter_pairs(n, t00, tw, tiles_x, r, tiles, rec, rec_cap);
                 }
+                auto at = [&](uint32_t t, int x, int y) {
+                    const ViewDev &V = src.views[t];
+                    const int W = V.P.W;
+                    unsigned long long *p = V.accum + (size_t)y * W + x;
+                    return [p, W](int j, unsigned long long c) { atomicAdd(&p[(size_t)j * W], c); };
+                };
+                hits += group_boxes<true, true>(mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at, (uint32_t)v);
+                hits += walk_boxes<true>(direct, (uint32_t)v, [&](uint32_t, uint32_t i) { return K[i]; },
+                                         [&](uint32_t t, int x, int y, unsigned long long c) { at(t, x, y)(0, c); });
+            } else if (n) {
+                const uint32_t th = n / (uint32_t)tw;
+                for (uint32_t ty = 0; ty < th; ++ty)
+                    for (uint32_t tx = 0; tx < (uint32_t)tw; ++tx) {
+                        const uint32_t t = t00 + ty * (uint32_t)tiles_x + tx;
+                        if (PART) {
+                            atomicAdd(&sh_tiles[t], 1u);
+                        } else {
+                            const uint32_t peers = __match_any_sync(__activemask(), t);
+                            if (lane == __ffs(peers) - 1) atomicAdd(&tiles[t], (uint32_t)__popc(peers));
+                        }
+                    }
             }
         }
         __syncthreads();
     }
     if (!SCATTER) {
+        if (PART) // the loop ends in a barrier, or has not run
+            for (uint32_t t = threadIdx.x; t < ntiles; t += RT) tiles[(size_t)t * gridDim.x + blockIdx.x] = sh_tiles[t];
         for (int d = 16; d > 0; d >>= 1) {
             splats += __shfl_xor_sync(0xffffffffu, splats, d);
             pairs += __shfl_xor_sync(0xffffffffu, pairs, d);
@@ -2015,52 +2099,44 @@ __global__ void __launch_bounds__(RT, 4) k_bsplat(const uint4 *__restrict__ rec,
     if (COUNT) count_hits(hits, stats);
 }
 
-// R4 over the views of a batch: blockIdx.y = view, grid-stride over that view's pixels
-__global__ void k_bmax(const ViewDev *__restrict__ views, unsigned long long *maxv)
+// R4 over the views of a batch: blockIdx.y = view
+__global__ void __launch_bounds__(256) k_bmax(const ViewDev *__restrict__ views, unsigned long long *maxv)
 {
     const ViewDev &V = views[blockIdx.y];
-    const size_t n = (size_t)V.P.W * V.P.H;
-    unsigned long long m = 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        m = V.accum[i] > m ? V.accum[i] : m;
-    for (int d = 16; d > 0; d >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, d);
-        m = o > m ? o : m;
-    }
+    const unsigned long long m = pixels_max(V.accum, (size_t)V.P.W * V.P.H);
     if ((threadIdx.x & 31) == 0 && m) atomicMax(&maxv[blockIdx.y], m);
 }
-__global__ void k_btonemap(const ViewDev *__restrict__ views, const unsigned long long *maxv, int auto_range)
+
+__global__ void __launch_bounds__(256) k_btonemap(const ViewDev *__restrict__ views, const unsigned long long *maxv,
+                                                  int auto_range)
 {
     const ViewDev &V = views[blockIdx.y];
     if (!V.image) return;
-    __shared__ double s_lo;
-    __shared__ float s_l2lo, s_scale;
-    __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        double hi = V.hi_acc, lo = V.lo_acc;
-        if (auto_range) {
-            hi = (double)maxv[blockIdx.y];
-            lo = hi * 1e-4;
-        }
-        s_ok = (hi > 0.0 && lo > 0.0 && hi > lo) ? 1 : 0;
-        s_lo = lo;
-        s_l2lo = s_ok ? (float)log2(lo) : 0.0f;
-        s_scale = s_ok ? (float)(255.0 / log2(hi / lo)) : 0.0f;
+    double hi = V.hi_acc, lo = V.lo_acc;
+    if (auto_range) {
+        hi = (double)maxv[blockIdx.y];
+        lo = hi * 1e-4;
     }
-    __syncthreads();
-    const double lo = s_lo;
-    const float l2lo = s_l2lo, scale = s_scale;
-    const int ok = s_ok;
-    const size_t n = (size_t)V.P.W * V.P.H;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const unsigned long long a = V.accum[i];
-        uint8_t o = 0;
-        if (ok && (double)a > lo) {
-            const float t = rintf((log2f((float)a) - l2lo) * scale);
-            o = (uint8_t)(t > 255.0f ? 255.0f : (t < 0.0f ? 0.0f : t));
-        }
-        V.image[i] = o;
+    pixels_tone(V.accum, (size_t)V.P.W * V.P.H, lo, hi, V.image);
+}
+
+// A batch is binned in parts if its tiles fit a shared-memory histogram: CTAs per SM, 0 if not
+int batch_part(uint32_t ntiles)
+{
+    const size_t smem = (size_t)ntiles * 4;
+    if (smem > PART_MAX_SMEM) return 0;
+    return (int)std::min<size_t>(4, std::max<size_t>(1, 216 * 1024 / (smem + 6 * 1024)));
+}
+
+// histogram entries of a batch of up to ntiles tiles
+size_t batch_hist(uint32_t ntiles)
+{
+    size_t m = 0;
+    for (int k = 1; k <= 4; ++k) { // the most tiles with k CTAs per SM
+        const size_t most = std::min<size_t>(PART_MAX_SMEM / 4, (216 * 1024 / (size_t)k - 6 * 1024) / 4);
+        m = std::max(m, std::min<size_t>(ntiles, most) * (size_t)persistent_blocks(k));
     }
+    return m;
 }
 
 struct BatchPlan {
@@ -2120,7 +2196,8 @@ void set_splat_smem()
     const void *part[] = {(const void *)k_project_hist<SrcLOD, false>, (const void *)k_project_hist<SrcLODQ, false>,
                           (const void *)k_project_hist<SrcFlat, true>, (const void *)k_project_scatter_part<SrcLOD, false>,
                           (const void *)k_project_scatter_part<SrcLODQ, false>,
-                          (const void *)k_project_scatter_part<SrcFlat, true>};
+                          (const void *)k_project_scatter_part<SrcFlat, true>, (const void *)k_bproject<false, true>,
+                          (const void *)k_bproject<true, true>};
     for (const void *f : part)
         GB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PART_MAX_SMEM));
     const int bytes = (int)sizeof(SplatSmem);
@@ -2156,10 +2233,12 @@ void reserve_batch(gblod_renderer *r, const gblod_view *views, int n, const gblo
     r->records.ensure(A, rec_cap, s);
     r->items.ensure(A, b.ntiles + rec_cap / ITEM + 1, s);
     r->maxv.ensure(A, n, s);
+    r->b_hist.ensure(A, batch_hist(b.ntiles) + 1, s);
     // scan temp for the largest scans of this batch
     scan_exclusive_u64(A, r->scan, reinterpret_cast<const uint64_t *>(r->b_counts.p),
                        reinterpret_cast<uint64_t *>(r->b_pfx.p), b.nodes + 1, nullptr, s);
     scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, b.ntiles, nullptr, s);
+    scan_exclusive_u32(A, r->scan, r->b_hist.p, r->b_hist.p, batch_hist(b.ntiles), nullptr, s);
     r->b_rec_cap = rec_cap;
     GB_CUDA(cudaStreamSynchronize(s));
 }
@@ -2174,7 +2253,8 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     if (r->b_views.cap < (size_t)n * sizeof(ViewDev) || r->b_frontA.cap < b.nodes + 1 || r->b_sel.cap < b.nodes + 1 ||
         r->b_pfx.cap < b.nodes + 2 || r->lvl_cnt.cap < b.max_levels + 3 || r->tile_cnt.cap < b.ntiles ||
         r->tile_off.cap < b.ntiles + 1 || r->item_off.cap < b.ntiles + 1 || r->records.cap < r->b_rec_cap ||
-        r->items.cap < items_cap || r->maxv.cap < (size_t)n || r->b_rec_cap == 0)
+        r->items.cap < items_cap || r->maxv.cap < (size_t)n || r->b_hist.cap < batch_hist(b.ntiles) + 1 ||
+        r->b_rec_cap == 0)
         fail(GBLOD_ERR_INVALID_ARG, "gblod_render_batch: call gblod_renderer_reserve_batch for this batch first");
     r->last_stream = s;
     r->last_was_lod = false;
@@ -2189,7 +2269,6 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     const unsigned G = (unsigned)persistent_blocks(4);
     GB_CUDA(cudaMemsetAsync(r->stats, 0, offsetof(FrameStatsDev, pixel_updates_total), s));
     GB_CUDA(cudaMemsetAsync(r->lvl_cnt.p, 0, (size_t)(b.max_levels + 3) * 4, s));
-    GB_CUDA(cudaMemsetAsync(r->tile_cnt.p, 0, (size_t)b.ntiles * 4, s));
     const dim3 GV((unsigned)std::max(1, (int)G / n), (unsigned)n); // (blocks per view, views)
     launch(GBLOD_K_RENDER_OTHER, k_bzero, GV, dim3(256), 0, s, (const ViewDev *)dv);
     // R1 over (view, node) pairs
@@ -2213,16 +2292,32 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
            r->b_base.p, r->stats);
     // R2: count, offsets, scatter
     const SrcBatch src{dv, r->b_sel.p, r->b_pfx.p, r->b_base.p, nsel, &r->stats->points};
-    launch(GBLOD_K_PROJECT_COUNT, k_bproject<false>, dim3(G), dim3(RT), 0, s, src, r->tile_cnt.p,
-           (uint32_t *)nullptr, (uint4 *)nullptr, 0ull, r->status, r->stats, 0);
-    scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, b.ntiles, r->tile_off.p + b.ntiles, s);
-    launch(GBLOD_K_RENDER_OTHER, k_tile_items, dim3((b.ntiles + 255) / 256), dim3(256), 0, s, b.ntiles,
-           (const uint32_t *)r->tile_cnt.p, r->item_cnt.p);
+    const int per_sm = batch_part(b.ntiles), kernel = b.host[0].P.kernel, count = (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? 1 : 0;
+    const unsigned long long rec_cap = r->b_rec_cap;
+    const dim3 tg((b.ntiles + 255) / 256);
+    if (per_sm) {
+        const unsigned GP = (unsigned)persistent_blocks(per_sm);
+        const size_t smem = (size_t)b.ntiles * 4, nh = (size_t)b.ntiles * GP;
+        launch(GBLOD_K_PROJECT_COUNT, k_bproject<false, true>, dim3(GP), dim3(RT), smem, s, src, r->b_hist.p, b.ntiles, kernel,
+               (uint4 *)nullptr, 0ull, r->status, r->stats, 0);
+        scan_exclusive_u32(A, r->scan, r->b_hist.p, r->b_hist.p, nh, r->b_hist.p + nh, s);
+        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, b.ntiles, (uint32_t)GP, ITEM,
+               (const uint32_t *)r->b_hist.p, (const uint32_t *)(r->b_hist.p + nh), r->tile_cnt.p, r->tile_off.p,
+               r->item_cnt.p);
+        launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, true>, dim3(GP), dim3(RT), smem, s, src, r->b_hist.p, b.ntiles, kernel,
+               r->records.p, rec_cap, r->status, r->stats, count);
+    } else {
+        GB_CUDA(cudaMemsetAsync(r->tile_cnt.p, 0, (size_t)b.ntiles * 4, s));
+        launch(GBLOD_K_PROJECT_COUNT, k_bproject<false, false>, dim3(G), dim3(RT), 0, s, src, r->tile_cnt.p, b.ntiles, kernel,
+               (uint4 *)nullptr, 0ull, r->status, r->stats, 0);
+        scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, b.ntiles, r->tile_off.p + b.ntiles, s);
+        launch(GBLOD_K_RENDER_OTHER, k_tile_items, tg, dim3(256), 0, s, b.ntiles, (const uint32_t *)r->tile_cnt.p,
+               r->item_cnt.p);
+        GB_CUDA(cudaMemcpyAsync(r->tile_cur.p, r->tile_off.p, (size_t)b.ntiles * 4, cudaMemcpyDeviceToDevice, s));
+        launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, false>, dim3(G), dim3(RT), 0, s, src, r->tile_cur.p, b.ntiles, kernel,
+               r->records.p, rec_cap, r->status, r->stats, count);
+    }
     scan_exclusive_u32(A, r->scan, r->item_cnt.p, r->item_off.p, b.ntiles, r->item_off.p + b.ntiles, s);
-    GB_CUDA(cudaMemcpyAsync(r->tile_cur.p, r->tile_off.p, (size_t)b.ntiles * 4, cudaMemcpyDeviceToDevice, s));
-    launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true>, dim3(G), dim3(RT), 0, s, src, (uint32_t *)nullptr,
-           r->tile_cur.p, r->records.p, (unsigned long long)r->b_rec_cap, r->status, r->stats,
-           (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? 1 : 0);
     launch(GBLOD_K_RENDER_OTHER, k_bfill_items, dim3((b.ntiles + 255) / 256), dim3(256), 0, s, b.ntiles,
            (const ViewDev *)dv, n, (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p,
            (const uint32_t *)r->item_off.p, r->items.p, (uint32_t)items_cap, (unsigned long long)r->b_rec_cap,
@@ -2234,16 +2329,14 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
            (uint32_t)items_cap, strips_of(b.host[0].P.TW, b.host[0].P.TH), b.host[0].P.kernel, (const ViewDev *)dv,
            r->lvl_cnt.p + b.max_levels + 2, r->stats);
     // R4
+    const dim3 GT((tone_blocks(b.npix) + (unsigned)n - 1) / (unsigned)n, (unsigned)n);
     if (rp.tone_auto) {
         GB_CUDA(cudaMemsetAsync(r->maxv.p, 0, (size_t)n * 8, s));
-        launch(GBLOD_K_TONEMAP, k_bmax, GV, dim3(256), 0, s, (const ViewDev *)dv, r->maxv.p);
+        launch(GBLOD_K_TONEMAP, k_bmax, GT, dim3(256), 0, s, (const ViewDev *)dv, r->maxv.p);
     }
-    launch(GBLOD_K_TONEMAP, k_btonemap, GV, dim3(256), 0, s, (const ViewDev *)dv,
+    launch(GBLOD_K_TONEMAP, k_btonemap, GT, dim3(256), 0, s, (const ViewDev *)dv,
            (const unsigned long long *)r->maxv.p, rp.tone_auto ? 1 : 0);
 }
-
-namespace {
-} // namespace
 
 void renderer_init(gblod_renderer *r, cudaStream_t s)
 {
@@ -2265,7 +2358,7 @@ void renderer_release(gblod_renderer *r)
     r->frontA.release(A, s); r->frontB.release(A, s); r->sel.release(A, s); r->lvl_cnt.release(A, s);
     r->sel_pfx.release(A, s); r->sel_base.release(A, s);
     r->tile_cnt.release(A, s); r->tile_off.release(A, s); r->tile_cur.release(A, s);
-    r->cta_hist.release(A, s); r->cta_off.release(A, s);
+    r->cta_hist.release(A, s); r->cta_off.release(A, s); r->b_hist.release(A, s);
     r->tile_cnt_s.release(A, s); r->tile_off_s.release(A, s); r->item_cnt_s.release(A, s); r->item_off_s.release(A, s);
     r->item_cnt.release(A, s); r->item_off.release(A, s);
     r->records.release(A, s); r->items.release(A, s); r->accum.release(A, s); r->maxv.release(A, s);
@@ -2350,13 +2443,13 @@ void tonemap_image(gblod_renderer *r, const uint64_t *accum, int W, int H, const
     double lo = 0.0, hi = 0.0;
     if (rp.tone_auto) {
         GB_CUDA(cudaMemsetAsync(r->maxv.p, 0, 8, s));
-        launch(GBLOD_K_TONEMAP, k_image_max, dim3(persistent_blocks(2)), dim3(256), 0, s,
+        launch(GBLOD_K_TONEMAP, k_image_max, dim3(tone_blocks(npix)), dim3(256), 0, s,
                (const unsigned long long *)accum, npix, r->maxv.p);
     } else {
         lo = std::ldexp(rp.tone_lo, 32);
         hi = std::ldexp(rp.tone_hi, 32);
     }
-    launch(GBLOD_K_TONEMAP, k_tonemap, dim3(persistent_blocks(2)), dim3(256), 0, s, (const unsigned long long *)accum,
+    launch(GBLOD_K_TONEMAP, k_tonemap, dim3(tone_blocks(npix)), dim3(256), 0, s, (const unsigned long long *)accum,
            npix, (const unsigned long long *)r->maxv.p, rp.tone_auto ? 1 : 0, lo, hi, image);
 }
 
@@ -2516,13 +2609,13 @@ gblod_status render_brute_noalloc(const float *xyz, const float *mass, const flo
         double lo = 0.0, hi = 0.0;
         if (rp.tone_auto) {
             GB_CUDA(cudaMemsetAsync(maxv, 0, 8, s));
-            launch(GBLOD_K_TONEMAP, k_image_max, dim3(persistent_blocks(2)), dim3(256), 0, s,
+            launch(GBLOD_K_TONEMAP, k_image_max, dim3(tone_blocks(npix)), dim3(256), 0, s,
                    (const unsigned long long *)img, npix, maxv);
         } else {
             lo = std::ldexp(rp.tone_lo, 32);
             hi = std::ldexp(rp.tone_hi, 32);
         }
-        launch(GBLOD_K_TONEMAP, k_tonemap, dim3(persistent_blocks(2)), dim3(256), 0, s,
+        launch(GBLOD_K_TONEMAP, k_tonemap, dim3(tone_blocks(npix)), dim3(256), 0, s,
                (const unsigned long long *)img, npix, (const unsigned long long *)maxv, rp.tone_auto ? 1 : 0, lo, hi,
                image);
     }

@@ -24,6 +24,7 @@ struct gblod_renderer {
     gb::DBuf<int64_t> sel_base;
     // R2 / R3
     gb::DBuf<uint32_t> tile_cnt, tile_off, tile_cur, item_cnt, item_off;
+    gb::DBuf<uint32_t> b_hist;            // batches: the same, scanned in place
     gb::DBuf<uint32_t> cta_hist, cta_off; // partitioned binning: (tile, CTA) counts and their offsets
     gb::DBuf<uint32_t> tile_cnt_s, tile_off_s, item_cnt_s, item_off_s; // its small-box record stream
     gb::DBuf<uint4> records, items;
