@@ -843,8 +843,9 @@ __global__ void __launch_bounds__(RT, 4) k_project_scatter(Src src, Proj P, unsi
 
 // Partitioned binning.  Each CTA of the grid counts its own points per tile in shared memory and writes
 // one histogram, tile-major: hist[t * G + cta].  An exclusive scan of the histograms gives every CTA
-// its own base in every tile, so the scatter pass places records with shared-memory atomics only,
-// and the records of a tile keep the order of the CTAs.  Both passes walk the same chunks (the same
+// its own base in every tile, so the scatter pass places records with shared-memory atomics only.  The CTAs
+// may be split in groups of gs, each with its own tile-major histogram and so its own region of the
+// records, where a tile has one run per group (see binning).  Both passes walk the same chunks (the same
 // grid G and chunk stride), so they see the same points.  (Global counters need the pairs of a warp
 // grouped by tile: __match_any_sync loops over the distinct tiles, up to 260 cycles a round.  LOD frames,
 // count + scatter: 16.8M particles 1080p 2.07 ms with it, 0.58 ms so; 150M near view 5.4, 2.1 ms.)
@@ -863,9 +864,19 @@ template <bool SMALL> constexpr int PART_THREADS = SMALL ? 1024 : 256;
 constexpr size_t PART_MAX_SMEM = 200 * 1024; // shared-memory histograms: frames of more tiles take the global counters
 constexpr uint32_t ITEM_SMALL = 4096;        // small records per k_splat_small work item
 
+// where CTA `cta` keeps tile t's count
+__device__ __forceinline__ size_t hist_at(uint32_t t, uint32_t ntiles, uint32_t cta, uint32_t gs)
+{
+    return ((size_t)(cta / gs) * ntiles + t) * gs + cta % gs;
+}
+
+struct PointIn {
+    float x, y, z, w, h;
+};
+
 template <class Src, bool SMALL>
 __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL>) k_project_hist(Src src, Proj P, unsigned long long e_lo,
-                                                     unsigned long long e_hi, uint32_t chunk,
+                                                     unsigned long long e_hi, uint32_t chunk, uint32_t gs,
                                                      uint32_t *__restrict__ hist, unsigned *status, FrameStatsDev *stats)
 {
     constexpr int NT = PART_THREADS<SMALL>;
@@ -877,6 +888,11 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
     const int lane = threadIdx.x & 31;
     unsigned long long splats = 0, pairs = 0;
     AmpSum amp;
+    PointIn ahead; // SMALL: the thread's next point, read before this one's arithmetic
+    if constexpr (SMALL) {
+        const unsigned long long e = e_lo + (unsigned long long)blockIdx.x * chunk + threadIdx.x;
+        if (e < total) src_load(src, e, 0u, 0u, ahead.x, ahead.y, ahead.z, ahead.w, ahead.h);
+    }
     for (unsigned long long a = e_lo + (unsigned long long)blockIdx.x * chunk; a < total;
          a += (unsigned long long)gridDim.x * chunk) {
         const unsigned long long b = min(total, a + chunk);
@@ -886,7 +902,12 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
             const unsigned long long e = e0 + threadIdx.x;
             int res = 0;
             Splat s;
-            if (e < b) {
+            if constexpr (SMALL) {
+                const PointIn q = ahead;
+                const unsigned long long en = e0 + NT < b ? e + NT : a + (unsigned long long)gridDim.x * chunk + threadIdx.x;
+                if (en < total) src_load(src, en, 0u, 0u, ahead.x, ahead.y, ahead.z, ahead.w, ahead.h);
+                if (e < b) res = project(P, q.x, q.y, q.z, q.w, q.h, s);
+            } else if (e < b) {
                 float x, y, z, w, h;
                 src_load(src, e, j0, j1, x, y, z, w, h);
                 res = project(P, x, y, z, w, h, s);
@@ -916,10 +937,15 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
     if (lane == 0 && pairs) atomicAdd(&stats->pairs, pairs);
     amp.flush(stats);
     __syncthreads();
-    for (uint32_t t = threadIdx.x; t < ncnt; t += NT) hist[(size_t)t * gridDim.x + blockIdx.x] = sh_cnt[t];
+    for (uint32_t t = threadIdx.x; t < ntiles; t += NT) {
+        const size_t at = hist_at(t, ntiles, blockIdx.x, gs);
+        hist[at] = sh_cnt[t];
+        if (SMALL) hist[(size_t)ntiles * gridDim.x + at] = sh_cnt[ntiles + t];
+    }
 }
 
-// tile counts, offsets and work items (of per_item records) from the scanned (tile, CTA) histogram
+// counts, offsets and work items (of per_item records) of the tiles' runs from the scanned (tile, CTA) histogram
+// of CTA groups of G
 __global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, uint32_t per_item, const uint32_t *__restrict__ off,
                                   const uint32_t *total, uint32_t *tile_cnt, uint32_t *tile_off, uint32_t *item_cnt)
 {
@@ -936,7 +962,7 @@ __global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, uint32_t per_item
 // receives their pixel updates).
 template <class Src, bool SMALL>
 __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL>) k_project_scatter_part(Src src, Proj P, unsigned long long e_lo,
-                                                             unsigned long long e_hi, uint32_t chunk,
+                                                             unsigned long long e_hi, uint32_t chunk, uint32_t gs,
                                                              const uint32_t *__restrict__ off,
                                                              uint4 *__restrict__ rec, unsigned long long *img,
                                                              FrameStatsDev *cstats)
@@ -944,14 +970,23 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
     constexpr int NT = PART_THREADS<SMALL>;
     __shared__ int32_t K[SMALL ? 1 : 1025];
     extern __shared__ uint32_t sh_cur[]; // [ntiles] binned points, then (SMALL) [ntiles] small boxes
-    const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y), ncnt = SMALL ? 2 * ntiles : ntiles;
+    const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y);
     const unsigned long long total = min(src_total(src), e_hi);
     unsigned hits = 0;
     if (e_lo + (unsigned long long)blockIdx.x * chunk < total)
-        for (uint32_t t = threadIdx.x; t < ncnt; t += NT) sh_cur[t] = off[(size_t)t * gridDim.x + blockIdx.x];
+        for (uint32_t t = threadIdx.x; t < ntiles; t += NT) {
+            const size_t at = hist_at(t, ntiles, blockIdx.x, gs);
+            sh_cur[t] = off[at];
+            if (SMALL) sh_cur[ntiles + t] = off[(size_t)ntiles * gridDim.x + at];
+        }
     if (!SMALL)
         for (int t = threadIdx.x; t <= 1024; t += NT) K[t] = t < 1024 ? g_ktab[P.kernel][t] : 0;
     __syncthreads();
+    PointIn ahead; // SMALL: the thread's next point, read before this one's arithmetic
+    if constexpr (SMALL) {
+        const unsigned long long e = e_lo + (unsigned long long)blockIdx.x * chunk + threadIdx.x;
+        if (e < total) src_load(src, e, 0u, 0u, ahead.x, ahead.y, ahead.z, ahead.w, ahead.h);
+    }
     for (unsigned long long a = e_lo + (unsigned long long)blockIdx.x * chunk; a < total;
          a += (unsigned long long)gridDim.x * chunk) {
         const unsigned long long b = min(total, a + chunk);
@@ -961,7 +996,12 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
             const unsigned long long e = e0 + threadIdx.x;
             int res = 0;
             Splat s;
-            if (e < b) {
+            if constexpr (SMALL) {
+                const PointIn q = ahead;
+                const unsigned long long en = e0 + NT < b ? e + NT : a + (unsigned long long)gridDim.x * chunk + threadIdx.x;
+                if (en < total) src_load(src, en, 0u, 0u, ahead.x, ahead.y, ahead.z, ahead.w, ahead.h);
+                if (e < b) res = project(P, q.x, q.y, q.z, q.w, q.h, s);
+            } else if (e < b) {
                 float x, y, z, w, h;
                 src_load(src, e, j0, j1, x, y, z, w, h);
                 res = project(P, x, y, z, w, h, s);
@@ -1001,14 +1041,15 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
     if (!SMALL && cstats) count_hits(hits, cstats);
 }
 
-__global__ void k_fill_items_n(uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
+// work items of nruns runs: run t belongs to tile t mod ntiles
+__global__ void k_fill_items_n(uint32_t nruns, uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
                                const uint32_t *item_off, uint32_t per_item, uint4 *items)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ntiles) return;
+    if (t >= nruns) return;
     const uint32_t c = tile_cnt[t], o = tile_off[t];
     uint32_t k = item_off[t];
-    for (uint32_t s = 0; s < c; s += per_item, ++k) items[k] = make_uint4(t, o + s, o + min(c, s + per_item), 0u);
+    for (uint32_t s = 0; s < c; s += per_item, ++k) items[k] = make_uint4(t % ntiles, o + s, o + min(c, s + per_item), 0u);
 }
 
 // Small-box records of one work item (a tile and up to ITEM_SMALL of its records): each warp takes
@@ -1110,15 +1151,15 @@ __global__ void k_tile_items(uint32_t ntiles, const uint32_t *tile_cnt, uint32_t
 }
 
 // also clears the unit counter of the splat launch that follows
-__global__ void k_fill_items(uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
+__global__ void k_fill_items(uint32_t nruns, uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
                              const uint32_t *item_off, uint4 *items, unsigned *next)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) *next = 0u;
-    if (t >= ntiles) return;
+    if (t >= nruns) return;
     const uint32_t c = tile_cnt[t], o = tile_off[t];
     uint32_t k = item_off[t];
-    for (uint32_t s = 0; s < c; s += ITEM, ++k) items[k] = make_uint4(t, o + s, o + min(c, s + ITEM), 0u);
+    for (uint32_t s = 0; s < c; s += ITEM, ++k) items[k] = make_uint4(t % ntiles, o + s, o + min(c, s + ITEM), 0u);
 }
 
 // ------------------------------------------------------------------ R3
@@ -1559,7 +1600,7 @@ template <> constexpr bool unordered_source<SrcFlat>() { return true; }
 // allow -- or through the global tile counters.
 struct Binning {
     bool part;
-    unsigned grid;
+    unsigned grid, groups; // CTAs; groups of grid / groups CTAs
     uint32_t chunk;
     size_t smem;
 };
@@ -1578,6 +1619,16 @@ template <class Src> Binning binning(const Src &src, const Proj &P)
                      : CHUNK;
     b.grid = b.part ? (unsigned)std::max<unsigned long long>(1, std::min<unsigned long long>(full, (src.bound + b.chunk - 1) / b.chunk))
                     : full;
+    // Records go to one place per (CTA, tile).  Of points in no order every CTA writes to all of them all the
+    // time, and stores spread over gigabytes miss the address-translation caches: a group's region is
+    // kept to some 128 MB (24 bytes of records a point).  150M points: scatter 5.37 ms in one region of 3.7 GB,
+    // 3.8 in 8, 3.0 in 19 and in 152; 16.8M: 0.66 in one, 0.57 in 3.  More runs are more work items with fewer records.
+    b.groups = 1;
+    if (b.part && unordered_source<Src>()) {
+        const unsigned want = (unsigned)std::min<unsigned long long>(b.grid / 8, src.bound * 24 >> 27);
+        b.groups = std::max(1u, want);
+        b.grid = b.grid / b.groups * b.groups;
+    }
     return b;
 }
 
@@ -1590,27 +1641,33 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
     const Binning bn = binning(src, P);
     constexpr bool SMALL = unordered_source<Src>();
     const size_t nh = (size_t)ntiles * bn.grid, nall = SMALL ? 2 * nh : nh;
+    const uint32_t nruns = ntiles * bn.groups, gs = bn.grid / bn.groups;
+    r->tile_cnt.ensure(A, nruns, s);
+    r->tile_off.ensure(A, nruns + 1, s);
+    r->item_cnt.ensure(A, nruns, s);
+    r->item_off.ensure(A, nruns + 1, s);
     if (bn.part) {
         r->cta_hist.ensure(A, nall, s);
         r->cta_off.ensure(A, nall + 1, s);
         launch(GBLOD_K_PROJECT_COUNT, k_project_hist<Src, SMALL>, dim3(bn.grid), dim3(PART_THREADS<SMALL>), bn.smem, s, src, P, lo, hi,
-               bn.chunk, r->cta_hist.p, r->status, stats);
+               bn.chunk, gs, r->cta_hist.p, r->status, stats);
         scan_exclusive_u32(A, r->scan, r->cta_hist.p, r->cta_off.p, nall, r->cta_off.p + nall, s);
-        const dim3 tg((ntiles + 255) / 256);
-        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, ntiles, (uint32_t)bn.grid, ITEM,
+        const dim3 tg((nruns + 255) / 256);
+        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, ITEM,
                (const uint32_t *)r->cta_off.p, (const uint32_t *)(r->cta_off.p + nh), r->tile_cnt.p, r->tile_off.p,
                r->item_cnt.p);
         if (SMALL) {
-            r->tile_cnt_s.ensure(A, ntiles, s);
-            r->tile_off_s.ensure(A, ntiles + 1, s);
-            r->item_cnt_s.ensure(A, ntiles, s);
-            r->item_off_s.ensure(A, ntiles + 1, s);
-            launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, ntiles, (uint32_t)bn.grid, ITEM_SMALL,
+            r->tile_cnt_s.ensure(A, nruns, s);
+            r->tile_off_s.ensure(A, nruns + 1, s);
+            r->item_cnt_s.ensure(A, nruns, s);
+            r->item_off_s.ensure(A, nruns + 1, s);
+            launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, ITEM_SMALL,
                    (const uint32_t *)(r->cta_off.p + nh), (const uint32_t *)(r->cta_off.p + 2 * nh), r->tile_cnt_s.p,
                    r->tile_off_s.p, r->item_cnt_s.p);
-            scan_exclusive_u32(A, r->scan, r->item_cnt_s.p, r->item_off_s.p, ntiles, r->item_off_s.p + ntiles, s);
+            scan_exclusive_u32(A, r->scan, r->item_cnt_s.p, r->item_off_s.p, nruns, r->item_off_s.p + nruns, s);
         }
     } else {
+        r->tile_cur.ensure(A, ntiles, s);
         GB_CUDA(cudaMemsetAsync(r->tile_cnt.p, 0, (size_t)ntiles * 4, s));
         launch(GBLOD_K_PROJECT_COUNT, k_project_count<Src>, dim3(bn.grid), dim3(RT), 0, s, src, P, lo, hi, r->tile_cnt.p,
                r->status, stats);
@@ -1618,15 +1675,15 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
         launch(GBLOD_K_RENDER_OTHER, k_tile_items, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
                (const uint32_t *)r->tile_cnt.p, r->item_cnt.p);
     }
-    scan_exclusive_u32(A, r->scan, r->item_cnt.p, r->item_off.p, ntiles, r->item_off.p + ntiles, s);
+    scan_exclusive_u32(A, r->scan, r->item_cnt.p, r->item_off.p, nruns, r->item_off.p + nruns, s);
     unsigned long long *h = static_cast<unsigned long long *>(r->hs.get(40));
     h[2] = h[3] = h[4] = 0;
     GB_CUDA(cudaMemcpyAsync(h, &stats->pairs, 8, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaMemcpyAsync(h + 1, &stats->points, 8, cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(h + 2, r->item_off.p + ntiles, 4, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(h + 2, r->item_off.p + nruns, 4, cudaMemcpyDeviceToHost, s));
     const bool streams = bn.part && SMALL;
     if (streams) {
-        GB_CUDA(cudaMemcpyAsync(h + 3, r->item_off_s.p + ntiles, 4, cudaMemcpyDeviceToHost, s));
+        GB_CUDA(cudaMemcpyAsync(h + 3, r->item_off_s.p + nruns, 4, cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaMemcpyAsync(h + 4, r->cta_off.p + 2 * nh, 4, cudaMemcpyDeviceToHost, s));
     }
     GB_CUDA(cudaStreamSynchronize(s));
@@ -1655,14 +1712,16 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
     const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y);
     const Binning bn = binning(src, P);
     constexpr bool SMALL = unordered_source<Src>();
+    const uint32_t nruns = ntiles * bn.groups;
+    const dim3 tg((nruns + 255) / 256);
     FrameStatsDev *cstats = r->count_updates ? r->stats : (FrameStatsDev *)nullptr;
     r->records.ensure(A, pc.pairs, s);
     r->items.ensure(A, (size_t)pc.items + pc.small_items, s);
     if (bn.part) {
         launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter_part<Src, SMALL>, dim3(bn.grid), dim3(PART_THREADS<SMALL>), bn.smem, s,
-               src, P, lo, hi, bn.chunk, (const uint32_t *)r->cta_off.p, r->records.p, img, cstats);
+               src, P, lo, hi, bn.chunk, bn.grid / bn.groups, (const uint32_t *)r->cta_off.p, r->records.p, img, cstats);
         if (SMALL) {
-            launch(GBLOD_K_RENDER_OTHER, k_fill_items_n, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
+            launch(GBLOD_K_RENDER_OTHER, k_fill_items_n, tg, dim3(256), 0, s, nruns, ntiles,
                    (const uint32_t *)r->tile_cnt_s.p, (const uint32_t *)r->tile_off_s.p,
                    (const uint32_t *)r->item_off_s.p, ITEM_SMALL, r->items.p + pc.items);
             launch(GBLOD_K_SPLAT, r->count_updates ? k_splat_small<true> : k_splat_small<false>, dim3(pc.small_items),
@@ -1673,7 +1732,7 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
         launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter<Src>, dim3(bn.grid), dim3(RT), 0, s, src, P, lo, hi,
                r->tile_cur.p, r->records.p, img, cstats);
     }
-    launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
+    launch(GBLOD_K_RENDER_OTHER, k_fill_items, tg, dim3(256), 0, s, nruns, ntiles,
            (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p, (const uint32_t *)r->item_off.p,
            r->items.p, r->status + 1);
     launch_splat(r->count_updates, r->records.p, r->items.p, pc.items, r->status + 1, P, img, r->stats, s);
@@ -1686,11 +1745,6 @@ void frame_common(gblod_renderer *r, const Src &src, const Proj &P, const gblod_
     const Allocator &A = r->A;
     const uint32_t ntiles = (uint32_t)(P.tiles_x * P.tiles_y);
     r->count_updates = (rp.flags & GBLOD_RENDER_COUNT_UPDATES) != 0;
-    r->tile_cnt.ensure(A, ntiles, s);
-    r->tile_off.ensure(A, ntiles + 1, s);
-    r->tile_cur.ensure(A, ntiles, s);
-    r->item_cnt.ensure(A, ntiles, s);
-    r->item_off.ensure(A, ntiles + 1, s);
     r->pass_stats.ensure(A, 1, s);
     const size_t npix = (size_t)P.W * P.H;
     unsigned long long *img = reinterpret_cast<unsigned long long *>(accum);
@@ -2602,7 +2656,7 @@ gblod_status render_brute_noalloc(const float *xyz, const float *mass, const flo
     launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter<SrcFlat>, dim3(G), dim3(RT), 0, s, src, P, 0ull, ~0ull,
            tile_cur, records, img,
            (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? stats : (FrameStatsDev *)nullptr);
-    launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((nt + 255) / 256), dim3(256), 0, s, nt,
+    launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((nt + 255) / 256), dim3(256), 0, s, nt, nt,
            (const uint32_t *)tile_cnt, (const uint32_t *)tile_off, (const uint32_t *)item_off, items, status + 1);
     launch_splat((rp.flags & GBLOD_RENDER_COUNT_UPDATES) != 0, records, items, nitems, status + 1, P, img, stats, s);
     if (image) {

@@ -41,3 +41,25 @@ def test_binning_equals_the_oracle(n, W, H, tw, th, budget):
     assert st == 0 and r.status() == G.OK and np.array_equal(G.u64(acc), want)
     t.free()
     r.close()
+
+
+@pytest.mark.parametrize("n", [11_200_000, 17_000_001])
+def test_records_in_several_regions(n):
+    """Enough unordered points for two and three groups of blocks: the same image and counts as through the global
+    tile counters."""
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    xyz = torch.rand((n, 3), device="cuda", generator=g)
+    mass = torch.rand(n, device="cuda", generator=g) + 0.5
+    h = torch.rand(n, device="cuda", generator=g) * 0.004 + 1e-4
+    cam = synth.look_at((0.4, 0.6, -0.7), (0.5, 0.5, 0.5), width=1500, height=1200)
+    r = G.Renderer()
+    _, a = r.render_bruteforce(xyz, mass, h, cam, G.make_params(count_updates=True))
+    sa = r.stats()
+    _, b = r.render_bruteforce(xyz, mass, h, cam, G.make_params(tile_w=8, tile_h=4, count_updates=True))
+    sb = r.stats()
+    assert r.status() == G.OK and torch.equal(a, b)
+    for k in ("points", "splats", "amplitude_lo", "amplitude_hi", "pixel_updates"):
+        assert sa[k] == sb[k], k
+    r.close()
