@@ -466,6 +466,46 @@ __device__ __forceinline__ int classify(const gblod_node &g, const Frustum &fr)
     return lhs > rhs ? 2 : 1;
 }
 
+// A node is drawn if the rule emits it and refines all its ancestors.  Trees of up to SELECT_FLAT nodes classify
+// every node and look at the ancestors' classes, in two launches (up to SELECT_ONE nodes: in one block that
+// also does k_sel_prefix's work); larger trees are walked level by level, which reads only the nodes that are
+// reached.  A level costs a launch of 5 to 6 us whatever its size: 64 nodes, 4 levels 29 us with first and
+// prefix launch, now 8 us; 1M particles, 11 levels 63 us, now 12 us.  What bounds the flat form is the FP64
+// of the rule, some 80 operations a node at two a clock and SM: 2^19 nodes take as long as ten levels.
+constexpr uint64_t SELECT_ONE = 256, SELECT_FLAT = 1u << 19;
+
+__global__ void __launch_bounds__(128) k_classify(const gblod_node *__restrict__ nodes, uint32_t nn, Frustum fr,
+                                                  uint8_t *__restrict__ cls)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nn) cls[i] = (uint8_t)classify(nodes[i], fr);
+}
+
+// appends the warp's nodes with `take` set to sel
+template <class T> __device__ __forceinline__ void append_nodes(bool take, T node, T *__restrict__ sel, uint32_t *nsel)
+{
+    const uint32_t em = __ballot_sync(0xffffffffu, take);
+    if (!em) return;
+    const int leader = __ffs(em) - 1;
+    uint32_t b = 0;
+    if ((int)(threadIdx.x & 31) == leader) b = atomicAdd(nsel, (uint32_t)__popc(em));
+    b = __shfl_sync(0xffffffffu, b, leader);
+    if (take) sel[b + __popc(em & gbd::lanemask_lt())] = node;
+}
+
+// Emitted nodes are kept only if they belong to this part of a split frame (node index mod n_parts ==
+// part; n_parts = 1 keeps every one).
+__global__ void __launch_bounds__(RT) k_select_flat(const gblod_node *__restrict__ nodes, uint32_t nn,
+                                                    const uint8_t *__restrict__ cls, uint32_t *__restrict__ sel,
+                                                    uint32_t *nsel, uint32_t part, uint32_t n_parts)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    bool take = i < nn && cls[i] == 1 && (n_parts <= 1 || i % n_parts == part);
+    if (take)
+        for (int p = nodes[i].parent; p >= 0 && take; p = nodes[p].parent) take = cls[p] == 2;
+    append_nodes(take, i, sel, nsel);
+}
+
 __global__ void k_select_init(uint32_t *front, uint32_t *cnt)
 {
     front[0] = 0u;
@@ -481,7 +521,6 @@ __global__ void __launch_bounds__(RT) k_select_level(const gblod_node *__restric
                                                      uint32_t n_parts)
 {
     const uint32_t n = *nin;
-    const uint32_t lt = gbd::lanemask_lt();
     const int lane = threadIdx.x & 31;
     for (uint32_t base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
         const uint32_t i = base + threadIdx.x;
@@ -495,15 +534,7 @@ __global__ void __launch_bounds__(RT) k_select_level(const gblod_node *__restric
             cfirst = g.child_first;
             if (cls == 1 && n_parts > 1 && node % n_parts != part) cls = 0;
         }
-        // warp-aggregated appends
-        const uint32_t em = __ballot_sync(0xffffffffu, cls == 1);
-        if (em) {
-            const int leader = __ffs(em) - 1;
-            uint32_t b = 0;
-            if (lane == leader) b = atomicAdd(nsel, (uint32_t)__popc(em));
-            b = __shfl_sync(0xffffffffu, b, leader);
-            if (cls == 1) sel[b + __popc(em & lt)] = node;
-        }
+        append_nodes(cls == 1, node, sel, nsel);
         uint32_t want = cls == 2 ? ccount : 0u, incl = want;
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
@@ -565,6 +596,79 @@ __global__ void __launch_bounds__(1024) k_sel_prefix(const gblod_node *__restric
     }
 }
 
+// R1 of a tree of at most SELECT_ONE nodes: a node per thread, classes and parents in shared memory
+__global__ void __launch_bounds__(SELECT_ONE) k_select_one(const gblod_node *__restrict__ nodes, uint32_t nn, Frustum fr,
+                                                           uint32_t part, uint32_t n_parts, uint32_t *__restrict__ sel,
+                                                           uint32_t *nsel, uint64_t *__restrict__ pfx,
+                                                           int64_t *__restrict__ base, FrameStatsDev *stats)
+{
+    __shared__ uint8_t cls[SELECT_ONE];
+    __shared__ int16_t parent[SELECT_ONE];
+    __shared__ unsigned long long points[SELECT_ONE / 32];
+    __shared__ uint32_t taken[SELECT_ONE / 32];
+    const uint32_t i = threadIdx.x;
+    const int lane = i & 31, warp = i >> 5;
+    unsigned long long c = 0, pf = 0;
+    if (i < nn) {
+        const gblod_node g = nodes[i];
+        parent[i] = (int16_t)g.parent;
+        cls[i] = (uint8_t)classify(g, fr);
+        c = g.point_count;
+        pf = g.point_first;
+    }
+    __syncthreads();
+    bool take = i < nn && cls[i] == 1 && (n_parts <= 1 || i % n_parts == part);
+    if (take)
+        for (int p = parent[i]; p >= 0 && take; p = parent[p]) take = cls[p] == 2;
+    const uint32_t em = __ballot_sync(0xffffffffu, take);
+    if (!take) c = 0;
+    unsigned long long incl = c;
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long o = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += o;
+    }
+    if (lane == 31) {
+        points[warp] = incl;
+        taken[warp] = (uint32_t)__popc(em);
+    }
+    __syncthreads();
+    unsigned long long ex = incl - c, all = 0;
+    uint32_t at = (uint32_t)__popc(em & gbd::lanemask_lt()), n = 0;
+    for (int w = 0; w < (int)(SELECT_ONE / 32); ++w) {
+        ex += w < warp ? points[w] : 0ull;
+        at += w < warp ? taken[w] : 0u;
+        all += points[w];
+        n += taken[w];
+    }
+    if (take) {
+        sel[at] = i;
+        pfx[at] = ex;
+        base[at] = (int64_t)pf - (int64_t)ex;
+    }
+    if (i == 0) {
+        *nsel = n;
+        pfx[n] = all;
+        stats->points = all;
+        stats->nodes_selected = n;
+    }
+}
+
+// The largest j < n with pfx[j] <= v (pfx[0] = 0), by a whole warp: 33 parts a step, where one thread's
+// bisection waits for log2(n) reads one after another (at the head of every chunk of points).
+__device__ __forceinline__ uint32_t warp_find(const uint64_t *__restrict__ pfx, uint32_t n, unsigned long long v)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t lo = 0, hi = n; // pfx[lo] <= v, and pfx[hi] > v or hi = n
+    while (hi - lo > 1) {
+        const uint32_t step = (hi - lo + 32) / 33, at = lo + step * (lane + 1);
+        const uint32_t m = __ballot_sync(0xffffffffu, at < hi && pfx[at] <= v);
+        const uint32_t k = (uint32_t)__popc(m); // the lanes below the first that is past v
+        hi = min(hi, lo + step * (k + 1));
+        lo += step * k;
+    }
+    return lo;
+}
+
 // ------------------------------------------------------------------ R2
 struct SrcLOD {
     const float4 *pts4;
@@ -597,17 +701,9 @@ __device__ __forceinline__ void src_range(const SrcLOD &s, unsigned long long a,
                                           uint32_t &j1)
 {
     __shared__ uint32_t sj[2];
-    if (threadIdx.x < 2) {
-        const unsigned long long v = threadIdx.x == 0 ? a : b - 1;
-        uint32_t lo = 0, hi = *s.nsel; // largest j with pfx[j] <= v
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (s.pfx[mid] <= v)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        sj[threadIdx.x] = lo;
+    if (threadIdx.x < 64) {
+        const uint32_t j = warp_find(s.pfx, *s.nsel, threadIdx.x < 32 ? a : b - 1);
+        if ((threadIdx.x & 31) == 0) sj[threadIdx.x >> 5] = j;
     }
     __syncthreads();
     j0 = sj[0];
@@ -1828,7 +1924,7 @@ struct ViewDev {
     unsigned long long *accum;
     uint8_t *image;
     unsigned long long pix_base;
-    uint32_t tile_base, n_nodes;
+    uint32_t tile_base, n_nodes, node_base;
     double lo_acc, hi_acc; // fixed tone range in accumulator units (unused when automatic)
 };
 
@@ -1851,6 +1947,44 @@ __global__ void k_bzero(const ViewDev *__restrict__ views)
         V.accum[i] = 0ull;
 }
 
+// The flat form of the selection over all views' nodes (SELECT_FLAT in all)
+__device__ __forceinline__ int view_of_node(const ViewDev *__restrict__ views, int n, uint32_t e)
+{
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (views[mid].node_base <= e) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+__global__ void __launch_bounds__(128) k_bclassify(const ViewDev *__restrict__ views, int n, uint32_t total,
+                                                   uint8_t *__restrict__ cls)
+{
+    const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const ViewDev &V = views[view_of_node(views, n, e)];
+    cls[e] = (uint8_t)classify(V.nodes[e - V.node_base], V.F);
+}
+
+__global__ void __launch_bounds__(RT) k_bselect_flat(const ViewDev *__restrict__ views, int n, uint32_t total,
+                                                     const uint8_t *__restrict__ cls,
+                                                     unsigned long long *__restrict__ sel, uint32_t *nsel)
+{
+    const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
+    int v = 0;
+    uint32_t node = 0;
+    bool take = e < total && cls[e] == 1;
+    if (take) {
+        v = view_of_node(views, n, e);
+        const uint32_t b = views[v].node_base;
+        const gblod_node *nodes = views[v].nodes;
+        node = e - b;
+        for (int p = nodes[node].parent; p >= 0 && take; p = nodes[p].parent) take = cls[b + (uint32_t)p] == 2;
+    }
+    append_nodes(take, (unsigned long long)v << 32 | node, sel, nsel);
+}
+
 __global__ void k_bselect_init(const ViewDev *__restrict__ views, int n, unsigned long long *front, uint32_t *cnt)
 {
     for (int v = threadIdx.x; v < n; v += blockDim.x)
@@ -1863,7 +1997,6 @@ __global__ void __launch_bounds__(RT) k_bselect_level(const ViewDev *__restrict_
                                                       unsigned long long *__restrict__ sel, uint32_t *nsel)
 {
     const uint32_t n = *nin;
-    const uint32_t lt = gbd::lanemask_lt();
     const int lane = threadIdx.x & 31;
     for (uint32_t base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
         const uint32_t i = base + threadIdx.x;
@@ -1878,14 +2011,7 @@ __global__ void __launch_bounds__(RT) k_bselect_level(const ViewDev *__restrict_
             ccount = g.child_count;
             cfirst = g.child_first;
         }
-        const uint32_t em = __ballot_sync(0xffffffffu, cls == 1);
-        if (em) {
-            const int leader = __ffs(em) - 1;
-            uint32_t b = 0;
-            if (lane == leader) b = atomicAdd(nsel, (uint32_t)__popc(em));
-            b = __shfl_sync(0xffffffffu, b, leader);
-            if (cls == 1) sel[b + __popc(em & lt)] = ent;
-        }
+        append_nodes(cls == 1, ent, sel, nsel);
         uint32_t want = cls == 2 ? ccount : 0u, incl = want;
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
@@ -1942,14 +2068,9 @@ __device__ __forceinline__ void bsrc_range(const SrcBatch &s, unsigned long long
                                            uint32_t &j0, uint32_t &j1)
 {
     __shared__ uint32_t sj[2];
-    if (threadIdx.x < 2) {
-        const unsigned long long v = threadIdx.x == 0 ? a : b - 1;
-        uint32_t lo = 0, hi = *s.nsel;
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (s.pfx[mid] <= v) lo = mid; else hi = mid;
-        }
-        sj[threadIdx.x] = lo;
+    if (threadIdx.x < 64) {
+        const uint32_t j = warp_find(reinterpret_cast<const uint64_t *>(s.pfx), *s.nsel, threadIdx.x < 32 ? a : b - 1);
+        if ((threadIdx.x & 31) == 0) sj[threadIdx.x >> 5] = j;
     }
     __syncthreads();
     j0 = sj[0];
@@ -2232,6 +2353,7 @@ BatchPlan plan_batch(const gblod_view *views, int n, const gblod_render_params &
         d.pix_base = b.npix;
         d.tile_base = b.ntiles;
         d.n_nodes = (uint32_t)V.octree->n_nodes;
+        d.node_base = (uint32_t)b.nodes;
         d.lo_acc = std::ldexp(rp.tone_lo, 32);
         d.hi_acc = std::ldexp(rp.tone_hi, 32);
         const unsigned long long tiles = (unsigned long long)d.P.tiles_x * d.P.tiles_y;
@@ -2329,13 +2451,22 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     launch(GBLOD_K_RENDER_OTHER, k_bzero, GV, dim3(256), 0, s, (const ViewDev *)dv);
     // R1 over (view, node) pairs
     uint32_t *nsel = r->lvl_cnt.p + b.max_levels + 1;
-    unsigned long long *fin = r->b_frontA.p, *fout = r->b_frontB.p;
-    launch(GBLOD_K_SELECT_NODES, k_bselect_init, dim3(1), dim3(256), 0, s, (const ViewDev *)dv, n, fin, r->lvl_cnt.p);
-    for (uint32_t d = 0; d < b.max_levels; ++d) {
-        launch(GBLOD_K_SELECT_NODES, k_bselect_level, dim3((unsigned)persistent_blocks(2)), dim3(RT), 0, s,
-               (const ViewDev *)dv, (const unsigned long long *)fin, (const uint32_t *)(r->lvl_cnt.p + d), fout,
-               r->lvl_cnt.p + d + 1, r->b_sel.p, nsel);
-        std::swap(fin, fout);
+    if (b.nodes <= SELECT_FLAT) {
+        uint8_t *cls = reinterpret_cast<uint8_t *>(r->b_frontA.p);
+        const uint32_t total = (uint32_t)b.nodes;
+        launch(GBLOD_K_SELECT_NODES, k_bclassify, dim3((total + 127) / 128), dim3(128), 0, s, (const ViewDev *)dv, n, total,
+               cls);
+        launch(GBLOD_K_SELECT_NODES, k_bselect_flat, dim3((total + RT - 1) / RT), dim3(RT), 0, s, (const ViewDev *)dv, n,
+               total, (const uint8_t *)cls, r->b_sel.p, nsel);
+    } else {
+        unsigned long long *fin = r->b_frontA.p, *fout = r->b_frontB.p;
+        launch(GBLOD_K_SELECT_NODES, k_bselect_init, dim3(1), dim3(256), 0, s, (const ViewDev *)dv, n, fin, r->lvl_cnt.p);
+        for (uint32_t d = 0; d < b.max_levels; ++d) {
+            launch(GBLOD_K_SELECT_NODES, k_bselect_level, dim3((unsigned)persistent_blocks(2)), dim3(RT), 0, s,
+                   (const ViewDev *)dv, (const unsigned long long *)fin, (const uint32_t *)(r->lvl_cnt.p + d), fout,
+                   r->lvl_cnt.p + d + 1, r->b_sel.p, nsel);
+            std::swap(fin, fout);
+        }
     }
     const uint32_t cap = (uint32_t)(b.nodes + 1);
     launch(GBLOD_K_SELECT_NODES, k_bsel_counts, dim3(G), dim3(256), 0, s, (const ViewDev *)dv,
@@ -2452,30 +2583,41 @@ void render_lod(gblod_renderer *r, const gblod_octree *o, const gblod_camera &ca
     GB_CUDA(cudaMemsetAsync(r->stats, 0, offsetof(FrameStatsDev, pixel_updates_total), s));
     const uint64_t nn = o->n_nodes;
     const int levels = o->depth_max + 1;
-    r->frontA.ensure(A, nn + 1, s);
-    r->frontB.ensure(A, nn + 1, s);
     r->sel.ensure(A, nn + 1, s);
     r->lvl_cnt.ensure(A, levels + 2, s);
     r->sel_pfx.ensure(A, nn + 2, s);
     r->sel_base.ensure(A, nn + 1, s);
-    GB_CUDA(cudaMemsetAsync(r->lvl_cnt.p, 0, (size_t)(levels + 2) * 4, s));
     uint32_t *nsel = r->lvl_cnt.p + levels + 1;
     const bool q = rp.point_format == GBLOD_POINTS_BLOCK16;
     const gblod_node *nodes = q ? o->qnodes : o->nodes;
-    if (nn > 0) {
-        const Frustum fr = make_frustum(cam, rp, o);
-        launch(GBLOD_K_SELECT_NODES, k_select_init, dim3(1), dim3(1), 0, s, r->frontA.p, r->lvl_cnt.p);
-        uint32_t *fin = r->frontA.p, *fout = r->frontB.p;
-        const unsigned G = (unsigned)persistent_blocks(2);
-        for (int d = 0; d < levels; ++d) {
-            launch(GBLOD_K_SELECT_NODES, k_select_level, dim3(G), dim3(RT), 0, s, nodes, fr,
-                   (const uint32_t *)fin, (const uint32_t *)(r->lvl_cnt.p + d), fout, r->lvl_cnt.p + d + 1,
-                   r->sel.p, nsel, part, n_parts);
-            std::swap(fin, fout);
+    const Frustum fr = make_frustum(cam, rp, o);
+    if (nn <= SELECT_ONE) {
+        launch(GBLOD_K_SELECT_NODES, k_select_one, dim3(1), dim3((unsigned)SELECT_ONE), 0, s, nodes, (uint32_t)nn, fr, part,
+               n_parts, r->sel.p, nsel, r->sel_pfx.p, r->sel_base.p, r->stats);
+    } else {
+        GB_CUDA(cudaMemsetAsync(r->lvl_cnt.p, 0, (size_t)(levels + 2) * 4, s));
+        r->frontA.ensure(A, nn + 1, s);
+        if (nn <= SELECT_FLAT) {
+            uint8_t *cls = reinterpret_cast<uint8_t *>(r->frontA.p);
+            launch(GBLOD_K_SELECT_NODES, k_classify, dim3((unsigned)((nn + 127) / 128)), dim3(128), 0, s, nodes, (uint32_t)nn,
+                   fr, cls);
+            launch(GBLOD_K_SELECT_NODES, k_select_flat, dim3((unsigned)((nn + RT - 1) / RT)), dim3(RT), 0, s, nodes,
+                   (uint32_t)nn, (const uint8_t *)cls, r->sel.p, nsel, part, n_parts);
+        } else {
+            r->frontB.ensure(A, nn + 1, s);
+            launch(GBLOD_K_SELECT_NODES, k_select_init, dim3(1), dim3(1), 0, s, r->frontA.p, r->lvl_cnt.p);
+            uint32_t *fin = r->frontA.p, *fout = r->frontB.p;
+            const unsigned G = (unsigned)persistent_blocks(2);
+            for (int d = 0; d < levels; ++d) {
+                launch(GBLOD_K_SELECT_NODES, k_select_level, dim3(G), dim3(RT), 0, s, nodes, fr,
+                       (const uint32_t *)fin, (const uint32_t *)(r->lvl_cnt.p + d), fout, r->lvl_cnt.p + d + 1,
+                       r->sel.p, nsel, part, n_parts);
+                std::swap(fin, fout);
+            }
         }
+        launch(GBLOD_K_SELECT_NODES, k_sel_prefix, dim3(1), dim3(1024), 0, s, nodes, (const uint32_t *)r->sel.p,
+               (const uint32_t *)nsel, r->sel_pfx.p, r->sel_base.p, r->stats);
     }
-    launch(GBLOD_K_SELECT_NODES, k_sel_prefix, dim3(1), dim3(1024), 0, s, nodes, (const uint32_t *)r->sel.p,
-           (const uint32_t *)nsel, r->sel_pfx.p, r->sel_base.p, r->stats);
     SrcLOD src{o->pts4, o->hs, r->sel_pfx.p, r->sel_base.p, nsel, &r->stats->points, o->n_points};
     if (q) {
         SrcLODQ sq;
