@@ -126,61 +126,187 @@ __device__ __forceinline__ uint32_t lower_bound_u64(const uint64_t *a, uint32_t 
     return lo;
 }
 
-__global__ void k_child_counts(const uint64_t *__restrict__ skey, const uint64_t *__restrict__ code,
-                               const uint32_t *__restrict__ first, const uint32_t *__restrict__ count, uint64_t L,
-                               uint32_t nd, int d, uint32_t n_max, uint32_t *cc, uint32_t *cf, uint32_t *nz)
-{
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (size_t)nd * 8) return;
-    const uint64_t node = L + (t >> 3);
-    const uint32_t o = (uint32_t)(t & 7);
-    const uint32_t c = count[node];
-    if (c > n_max && d < GBLOD_MAX_DEPTH) {
-        const uint64_t pfx = code[node] ^ (1ull << (3 * d));
-        const uint64_t cp = (pfx << 3) | o;
-        const int sh = 60 - 3 * d;
-        const uint32_t b = first[node], e = b + c;
-        const uint32_t lo = lower_bound_u64(skey, b, e, cp << sh);
-        const uint32_t hi = lower_bound_u64(skey, lo, e, (cp + 1) << sh);
-        cc[t] = hi - lo;
-        cf[t] = lo;
-        nz[t] = hi > lo ? 1u : 0u;
-    } else {
-        cc[t] = 0u;
-        cf[t] = 0u;
-        nz[t] = 0u;
-    }
-}
-
 struct NodeSoA {
     uint64_t *code;
     uint32_t *first, *count, *child_first, *child_count;
     int32_t *depth, *parent;
 };
 
-__global__ void k_emit_children(NodeSoA N, const uint32_t *__restrict__ cc, const uint32_t *__restrict__ cf,
-                                const uint32_t *__restrict__ slot, uint64_t L, uint32_t nd, int d, uint64_t Lnext)
+// The refined nodes of all levels come from one pass over the sorted keys: particle j is the first of a
+// depth-d cell if it shares fewer than d octal digits with particle j - 1, and that cell holds more than
+// n_max particles if j shares d digits or more with particle j + n_max.  Numbered by (depth, j) they are in the
+// order of their nodes; their children (eight searches each, all levels at once) in that order are the
+// nodes in level order.  A level at a time cost two launches, a scan and a wait for its node count: 1M
+// particles, 11 levels 0.65 ms from the sorted particles to the node table, now 0.21.  Bound by the launches and
+// two waits; 150M particles: by the pass over the keys, 0.28 ms.
+constexpr int DEPTHS = GBLOD_MAX_DEPTH; // a refined node's depth is below this
+constexpr uint32_t RB = 4096;           // positions per block
+constexpr int RT_REF = 256;
+
+// octal digits two keys that differ by the bits x share, of 21
+__device__ __forceinline__ int shared_digits(uint64_t x) { return x ? (__clzll((long long)x) - 1) / 3 : 21; }
+
+// depths (lo, hi] at which position j starts a refined node
+__device__ __forceinline__ void refined_depths(const uint64_t *__restrict__ skey, size_t n, uint64_t n_max, size_t j,
+                                               int &lo, int &hi)
+{
+    lo = hi = 0;
+    if (j + n_max >= n) return; // every cell that starts here is small enough
+    const uint64_t k = skey[j];
+    // more digits shared with the later particle than with the one before: the differing bits are a smaller
+    // number (nearly all positions end here)
+    const uint64_t before = j ? k ^ skey[j - 1] : ~0ull, after = k ^ skey[j + n_max];
+    if (after >= before) return;
+    lo = j ? shared_digits(before) : -1;
+    hi = max(lo, min(shared_digits(after), DEPTHS - 1));
+}
+
+// refined nodes by depth and block: hist[d * gridDim.x + block]
+__global__ void __launch_bounds__(RT_REF) k_count_refined(const uint64_t *__restrict__ skey, size_t n, uint64_t n_max,
+                                                          uint32_t *__restrict__ hist)
+{
+    __shared__ uint32_t cnt[DEPTHS];
+    if (threadIdx.x < DEPTHS) cnt[threadIdx.x] = 0u;
+    __syncthreads();
+    const size_t base = (size_t)blockIdx.x * RB;
+#pragma unroll 8
+    for (uint32_t q = threadIdx.x; q < RB; q += RT_REF) {
+        int lo, hi;
+        refined_depths(skey, n, n_max, base + q, lo, hi);
+        for (int d = lo + 1; d <= hi; ++d) atomicAdd(&cnt[d], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < DEPTHS) hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
+}
+
+// first[i] = particle of refined node i; dfirst[d] = the first refined node of depth d (DEPTHS + 1 entries)
+__global__ void __launch_bounds__(RT_REF) k_list_refined(const uint64_t *__restrict__ skey, size_t n, uint64_t n_max,
+                                                         const uint32_t *__restrict__ off, uint32_t *__restrict__ first,
+                                                         uint32_t *__restrict__ dfirst)
+{
+    __shared__ uint32_t bits[DEPTHS][RB / 32];   // positions of the block that start a refined node
+    __shared__ uint16_t before[DEPTHS][RB / 32]; // those in the words before
+    const uint32_t G = gridDim.x, total = off[(size_t)DEPTHS * G];
+    if (blockIdx.x == 0 && threadIdx.x <= DEPTHS)
+        dfirst[threadIdx.x] = threadIdx.x < DEPTHS ? off[(size_t)threadIdx.x * G] : total;
+    uint32_t mine = 0;
+    if (threadIdx.x < DEPTHS) {
+        const size_t at = (size_t)threadIdx.x * G + blockIdx.x;
+        mine = off[at + 1] - off[at];
+    }
+    if (!__syncthreads_or((int)mine)) return;
+    for (int i = threadIdx.x; i < DEPTHS * (int)(RB / 32); i += RT_REF) (&bits[0][0])[i] = 0u;
+    __syncthreads();
+    const size_t base = (size_t)blockIdx.x * RB;
+    for (uint32_t q = threadIdx.x; q < RB; q += RT_REF) {
+        int lo, hi;
+        refined_depths(skey, n, n_max, base + q, lo, hi);
+        for (int d = lo + 1; d <= hi; ++d) atomicOr(&bits[d][q >> 5], 1u << (q & 31));
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int d = threadIdx.x >> 5; d < DEPTHS; d += RT_REF / 32) {
+        uint32_t c[RB / 1024], sum = 0; // a lane's consecutive words
+#pragma unroll
+        for (int k = 0; k < (int)(RB / 1024); ++k) {
+            c[k] = sum;
+            sum += __popc(bits[d][lane * (RB / 1024) + k]);
+        }
+        uint32_t incl = sum;
+        for (int s = 1; s < 32; s <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += o;
+        }
+#pragma unroll
+        for (int k = 0; k < (int)(RB / 1024); ++k) before[d][lane * (RB / 1024) + k] = (uint16_t)(incl - sum + c[k]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < DEPTHS * (int)(RB / 32); i += RT_REF) {
+        const int d = i / (int)(RB / 32), w = i % (int)(RB / 32);
+        uint32_t m = bits[d][w], at = m ? off[(size_t)d * G + blockIdx.x] + before[d][w] : 0u;
+        while (m) {
+            first[at++] = (uint32_t)(base + (size_t)w * 32 + (uint32_t)(__ffs((int)m) - 1));
+            m &= m - 1u;
+        }
+    }
+}
+
+__device__ __forceinline__ int depth_of(const uint32_t *__restrict__ dfirst, uint32_t i)
+{
+    int lo = 0, hi = DEPTHS;
+    while (hi - lo > 1) { // the last depth whose first refined node is at or before i
+        const int mid = (lo + hi) >> 1;
+        if (dfirst[mid] <= i) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// Child t & 7 of refined node t >> 3: its particles [cf, cf + cc), and the flags to be scanned: 1 if there
+// is one, 2^32 if it is refined itself
+__global__ void k_children(uint32_t n_ref, const uint32_t *__restrict__ ref_first, const uint32_t *__restrict__ dfirst,
+                           const uint64_t *__restrict__ skey, uint32_t n, uint32_t n_max, uint32_t *__restrict__ cc,
+                           uint32_t *__restrict__ cf, uint64_t *__restrict__ flag)
 {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (size_t)nd * 8) return;
-    const uint64_t parent = L + (t >> 3);
-    if (cc[t]) {
-        const uint64_t j = Lnext + slot[t];
-        N.code[j] = N.code[parent] * 8 + (t & 7);
-        N.first[j] = cf[t];
-        N.count[j] = cc[t];
-        N.depth[j] = d + 1;
-        N.parent[j] = (int32_t)parent;
-        N.child_first[j] = 0u;
-        N.child_count[j] = 0u;
+    const bool on = t < (size_t)n_ref * 8; // whole groups of eight lanes
+    const uint32_t i = on ? (uint32_t)(t >> 3) : 0u, o = (uint32_t)(t & 7), j = ref_first[i];
+    const int d = depth_of(dfirst, i), sh = 60 - 3 * d;
+    const uint64_t cp = ((skey[j] >> (63 - 3 * d)) << 3) | o;
+    const uint32_t lo = o ? lower_bound_u64(skey, j, n, cp << sh) : j;
+    uint32_t hi = __shfl_down_sync(0xffffffffu, lo, 1);
+    if (o == 7) hi = lower_bound_u64(skey, lo, n, (cp + 1) << sh);
+    if (!on) return;
+    const uint32_t c = hi - lo;
+    cc[t] = c;
+    cf[t] = lo;
+    flag[t] = (c ? 1ull : 0ull) | (c > n_max && d + 1 < DEPTHS ? 1ull << 32 : 0ull);
+}
+
+// Numbers from the scanned flags (pos): the node of child t is 1 + its low word, the refined node (if it is
+// one) 1 + its high word.  node[i] = node of refined node i; level[d] = first node of depth d, level[DEPTHS + 2]
+// entries from depth 0 on.
+__global__ void k_number_nodes(uint32_t n_ref, const uint64_t *__restrict__ flag, const uint64_t *__restrict__ pos,
+                               const uint32_t *__restrict__ dfirst, uint32_t *__restrict__ node,
+                               unsigned long long *__restrict__ level)
+{
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, m = (size_t)n_ref * 8;
+    if (t < m && flag[t] >> 32) node[1 + (uint32_t)(pos[t] >> 32)] = 1u + (uint32_t)pos[t];
+    if (t == 0) node[0] = 0u;
+    if (t <= DEPTHS) { // pos[m] is the total
+        if (t == 0) level[0] = 0ull;
+        level[t + 1] = 1ull + (uint32_t)pos[(size_t)dfirst[t] * 8];
     }
-    if ((t & 7) == 0) {
-        uint32_t k = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) k += cc[t + q] ? 1u : 0u;
-        N.child_first[parent] = k ? (uint32_t)(Lnext + slot[t]) : 0u;
-        N.child_count[parent] = k;
+}
+
+__global__ void k_emit_nodes(NodeSoA N, uint32_t n, uint32_t n_ref, const uint32_t *__restrict__ ref_first,
+                             const uint32_t *__restrict__ dfirst, const uint64_t *__restrict__ skey,
+                             const uint32_t *__restrict__ cc, const uint32_t *__restrict__ cf,
+                             const uint64_t *__restrict__ flag, const uint64_t *__restrict__ pos,
+                             const uint32_t *__restrict__ node)
+{
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, m = (size_t)n_ref * 8;
+    auto children = [&](size_t x, bool refined, uint32_t i) {
+        const uint32_t a = refined ? (uint32_t)pos[(size_t)i * 8] : 0u, b = refined ? (uint32_t)pos[(size_t)i * 8 + 8] : 0u;
+        N.child_first[x] = refined ? 1u + a : 0u;
+        N.child_count[x] = b - a;
+    };
+    if (t == 0) {
+        N.code[0] = 1ull;
+        N.first[0] = 0u;
+        N.count[0] = n;
+        N.depth[0] = 0;
+        N.parent[0] = -1;
+        children(0, n_ref > 0, 0u);
     }
+    if (t >= m || !cc[t]) return;
+    const uint32_t i = (uint32_t)(t >> 3), x = 1u + (uint32_t)pos[t];
+    const int d = depth_of(dfirst, i);
+    N.code[x] = (1ull << (3 * (d + 1))) | ((skey[ref_first[i]] >> (63 - 3 * d)) << 3) | (t & 7);
+    N.first[x] = cf[t];
+    N.count[x] = cc[t];
+    N.depth[x] = d + 1;
+    N.parent[x] = (int32_t)node[i];
+    children(x, flag[t] >> 32 != 0, 1u + (uint32_t)(pos[t] >> 32));
 }
 
 // ------------------------------------------------------------------ node table
@@ -304,28 +430,37 @@ __global__ void k_leaf_nodes(size_t nn, const uint32_t *__restrict__ flags, cons
     }
 }
 
-// One level, deepest first: cull radius and bounds of every node of the level.
-__global__ void k_bottom_up(uint64_t L, uint32_t nd, const uint32_t *flags, const uint32_t *child_first,
-                            const uint32_t *child_count, float *bmin, float *bmax, const unsigned *hmax_bits,
-                            float *hcull)
+// Cull radius and bounds of every node, from the leaves up: a thread per node that is not refined climbs as
+// long as it is the last of a node's children to arrive, and takes that node's.  (A launch per level
+// before: the same 37 us for 11 levels on the device, but the host had 11 launches to make.)  Children are read past L1, where a line may be older
+// than their values.
+__global__ void k_bottom_up(size_t nn, const uint32_t *__restrict__ flags, const uint32_t *__restrict__ child_first,
+                            const uint32_t *__restrict__ child_count, const int32_t *__restrict__ parent, float *bmin,
+                            float *bmax, const unsigned *__restrict__ hmax_bits, float *hcull, uint32_t *arrived)
 {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nd) return;
-    const uint64_t i = L + t;
-    float h = __uint_as_float(hmax_bits[i]);
-    if (flags[i] & FL_INTERNAL) {
-        float mn0 = INFINITY, mn1 = INFINITY, mn2 = INFINITY, mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY;
+    if (t >= nn || (flags[t] & FL_INTERNAL)) return;
+    hcull[t] = __uint_as_float(hmax_bits[t]);
+    for (int i = parent[t], next; i >= 0; i = next) {
         const uint32_t k0 = child_first[i], kc = child_count[i];
-        for (uint32_t k = k0; k < k0 + kc; ++k) {
-            mn0 = fminf(mn0, bmin[3 * k]); mn1 = fminf(mn1, bmin[3 * k + 1]); mn2 = fminf(mn2, bmin[3 * k + 2]);
-            mx0 = fmaxf(mx0, bmax[3 * k]); mx1 = fmaxf(mx1, bmax[3 * k + 1]); mx2 = fmaxf(mx2, bmax[3 * k + 2]);
-            const float hc = hcull[k];
+        next = parent[i];
+        __threadfence();
+        if (atomicAdd(&arrived[i], 1u) + 1u < kc) return;
+        __threadfence();
+        float h = __uint_as_float(hmax_bits[i]);
+        float mn0 = INFINITY, mn1 = INFINITY, mn2 = INFINITY, mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY;
+#pragma unroll
+        for (uint32_t q = 0; q < 8; ++q) { // all children's reads in flight (past the last: the last again)
+            const uint32_t k = k0 + min(q, kc - 1u);
+            mn0 = fminf(mn0, __ldcg(&bmin[3 * k])); mn1 = fminf(mn1, __ldcg(&bmin[3 * k + 1])); mn2 = fminf(mn2, __ldcg(&bmin[3 * k + 2]));
+            mx0 = fmaxf(mx0, __ldcg(&bmax[3 * k])); mx1 = fmaxf(mx1, __ldcg(&bmax[3 * k + 1])); mx2 = fmaxf(mx2, __ldcg(&bmax[3 * k + 2]));
+            const float hc = __ldcg(&hcull[k]);
             h = hc > h ? hc : h;
         }
         bmin[3 * i] = mn0; bmin[3 * i + 1] = mn1; bmin[3 * i + 2] = mn2;
         bmax[3 * i] = mx0; bmax[3 * i + 1] = mx1; bmax[3 * i + 2] = mx2;
+        hcull[i] = h;
     }
-    hcull[i] = h;
 }
 
 struct PackIn {
@@ -365,33 +500,16 @@ __global__ void k_pack_nodes(size_t nn, PackIn P, gblod_node *out)
     out[i] = g;
 }
 
-// growable node arrays (structure of arrays), contents kept on growth
+// node arrays (structure of arrays)
 struct NodeStore {
     DBuf<uint64_t> code;
     DBuf<uint32_t> first, count, child_first, child_count;
     DBuf<int32_t> depth, parent;
-    size_t cap = 0;
 
-    template <class T> static void grow1(const Allocator &A, DBuf<T> &b, size_t used, size_t want, cudaStream_t s)
+    void ensure(const Allocator &A, size_t n, cudaStream_t s)
     {
-        T *np = static_cast<T *>(A.get(want * sizeof(T), s));
-        if (b.p && used) GB_CUDA(cudaMemcpyAsync(np, b.p, used * sizeof(T), cudaMemcpyDeviceToDevice, s));
-        if (b.p) A.put(b.p, b.cap * sizeof(T), s);
-        b.p = np;
-        b.cap = want;
-    }
-    void reserve(const Allocator &A, size_t used, size_t need, cudaStream_t s)
-    {
-        if (need <= cap) return;
-        size_t want = std::max(need, cap * 2);
-        grow1(A, code, used, want, s);
-        grow1(A, first, used, want, s);
-        grow1(A, count, used, want, s);
-        grow1(A, child_first, used, want, s);
-        grow1(A, child_count, used, want, s);
-        grow1(A, depth, used, want, s);
-        grow1(A, parent, used, want, s);
-        cap = want;
+        code.ensure(A, n, s); first.ensure(A, n, s); count.ensure(A, n, s); child_first.ensure(A, n, s);
+        child_count.ensure(A, n, s); depth.ensure(A, n, s); parent.ensure(A, n, s);
     }
     NodeSoA soa() { return NodeSoA{code.p, first.p, count.p, child_first.p, child_count.p, depth.p, parent.p}; }
     void release(const Allocator &A, cudaStream_t s)
@@ -400,17 +518,6 @@ struct NodeStore {
         child_count.release(A, s); depth.release(A, s); parent.release(A, s);
     }
 };
-
-__global__ void k_init_root(NodeSoA N, uint32_t n)
-{
-    N.code[0] = 1ull;
-    N.first[0] = 0u;
-    N.count[0] = n;
-    N.depth[0] = 0;
-    N.parent[0] = -1;
-    N.child_first[0] = 0u;
-    N.child_count[0] = 0u;
-}
 
 template <class T> T read1(const T *d, cudaStream_t s, HostStage &hs)
 {
@@ -446,12 +553,10 @@ struct BuildTemps {
     ScanTmp scan;
     SortTmp sort;
     NodeStore N;
-    DBuf<uint32_t> cc, cf, nz, slot;
     BuildTemps(const Allocator &a, cudaStream_t st) : A(a), s(st) {}
     ~BuildTemps()
     {
         N.release(A, s);
-        cc.release(A, s); cf.release(A, s); nz.release(A, s); slot.release(A, s);
         scan.buf.release(A, s);
         sort.buf.release(A, s);
         sort.scan.buf.release(A, s);
@@ -459,19 +564,23 @@ struct BuildTemps {
 };
 } // namespace
 
-static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const float *mass, const float *h,
+static void build_octree_impl(gblod_octree *o, const float *xyz, const float *mass, const float *h,
                                        const uint32_t *ids, uint64_t n, const gblod_build_params &p,
-                                       const Allocator &A, cudaStream_t s, bool roomy);
+                                       const Allocator &A, cudaStream_t s, HostStage &hs, bool roomy);
 
 gblod_octree *build_octree(const float *xyz, const float *mass, const float *h, const uint32_t *ids, uint64_t n,
                            const gblod_build_params &p, const Allocator &A, cudaStream_t s)
 {
     // A roomy build's work arrays peak at about 94 bytes a particle, a lean one's at 66.  Memory from a
     // caller's allocator is spent leanly; from the library's pool leanly only when roomy does not fit.
+    HostStage hs;
     for (bool roomy = !A.has_hook;; roomy = false) {
         gblod_octree *o = new gblod_octree();
         try {
-            return build_octree_impl(o, xyz, mass, h, ids, n, p, A, s, roomy);
+            // the work arrays are given back, in stream order, under the last kernels
+            build_octree_impl(o, xyz, mass, h, ids, n, p, A, s, hs, roomy);
+            GB_CUDA(cudaStreamSynchronize(s));
+            return o;
         } catch (const Error &e) {
             (void)cudaStreamSynchronize(s);
             free_octree(o);
@@ -484,11 +593,10 @@ gblod_octree *build_octree(const float *xyz, const float *mass, const float *h, 
     }
 }
 
-static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const float *mass, const float *h,
+static void build_octree_impl(gblod_octree *o, const float *xyz, const float *mass, const float *h,
                                        const uint32_t *ids, uint64_t n, const gblod_build_params &p,
-                                       const Allocator &A, cudaStream_t s, bool roomy)
+                                       const Allocator &A, cudaStream_t s, HostStage &hs, bool roomy)
 {
-    HostStage hs;
     BuildTemps tmp(A, s);
     ScanTmp &scan = tmp.scan;
     SortTmp &sort = tmp.sort;
@@ -501,7 +609,7 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
     o->side = p.root_side;
     if (n == 0) {
         o->level_first = {0};
-        return o;
+        return;
     }
     const int T = 256;
     const unsigned G = (unsigned)persistent_blocks(8);
@@ -586,32 +694,45 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
     if (!o->equal_mass) scan_exclusive_u128(A, scan, mpre.p, mpre.p, n, mtot.p, s);
     const uint32_t *sorted_ids = ids ? sid.p : sidx;
 
-    // A3: node table, one level at a time
+    // A3: refined nodes, their children, the nodes in level order
     NodeStore &N = tmp.N;
-    N.reserve(A, 0, 1024, s);
-    launch(GBLOD_K_BUILD_OTHER, k_init_root, dim3(1), dim3(1), 0, s, N.soa(), (uint32_t)n);
-    std::vector<uint64_t> level_first = {0, 1};
-    DBuf<uint32_t> &cc = tmp.cc, &cf = tmp.cf, &nz = tmp.nz, &slot = tmp.slot;
     Scratch<uint32_t> total(A, 1, s);
-    for (int d = 0; d < GBLOD_MAX_DEPTH; ++d) {
-        const uint64_t L = level_first[d];
-        const uint32_t nd = (uint32_t)(level_first[d + 1] - L);
-        if (nd == 0) break;
-        const size_t m = (size_t)nd * 8;
-        cc.ensure(A, m, s); cf.ensure(A, m, s); nz.ensure(A, m, s); slot.ensure(A, m, s);
-        launch(GBLOD_K_BUILD_OTHER, k_child_counts, dim3(blocks_for(m, T)), dim3(T), 0, s, (const uint64_t *)skey,
-               (const uint64_t *)N.code.p, (const uint32_t *)N.first.p, (const uint32_t *)N.count.p, L, nd, d,
-               p.n_max, cc.p, cf.p, nz.p);
-        scan_exclusive_u32(A, scan, nz.p, slot.p, m, total.p, s);
-        const uint32_t nnext = read1(total.p, s, hs);
-        const uint64_t Lnext = level_first[d + 1];
-        N.reserve(A, Lnext, Lnext + nnext, s);
-        launch(GBLOD_K_BUILD_OTHER, k_emit_children, dim3(blocks_for(m, T)), dim3(T), 0, s, N.soa(),
-               (const uint32_t *)cc.p, (const uint32_t *)cf.p, (const uint32_t *)slot.p, L, nd, d, Lnext);
-        if (nnext == 0) break;
-        level_first.push_back(Lnext + nnext);
+    const uint32_t nb = (uint32_t)((n + RB - 1) / RB);
+    uint32_t n_ref = 0;
+    std::vector<uint64_t> level_first = {0, 1};
+    {
+        Scratch<uint32_t> roff(A, (size_t)DEPTHS * nb + 1, s), dfirst(A, DEPTHS + 1, s);
+        if (n > p.n_max) {
+            launch(GBLOD_K_BUILD_OTHER, k_count_refined, dim3(nb), dim3(RT_REF), 0, s, (const uint64_t *)skey, (size_t)n,
+                   (uint64_t)p.n_max, roff.p);
+            scan_exclusive_u32(A, scan, roff.p, roff.p, (size_t)DEPTHS * nb, roff.p + (size_t)DEPTHS * nb, s);
+            n_ref = read1(roff.p + (size_t)DEPTHS * nb, s, hs);
+        }
+        const size_t m = (size_t)n_ref * 8;
+        const unsigned mg = blocks_for(std::max<size_t>(m, DEPTHS + 1), T);
+        Scratch<uint32_t> rfirst(A, n_ref, s), node(A, n_ref, s), cc(A, m, s), cf(A, m, s);
+        Scratch<uint64_t> flag(A, m, s), pos(A, m + 1, s);
+        if (n_ref) {
+            Scratch<unsigned long long> level(A, DEPTHS + 2, s);
+            launch(GBLOD_K_BUILD_OTHER, k_list_refined, dim3(nb), dim3(RT_REF), 0, s, (const uint64_t *)skey, (size_t)n,
+                   (uint64_t)p.n_max, (const uint32_t *)roff.p, rfirst.p, dfirst.p);
+            launch(GBLOD_K_BUILD_OTHER, k_children, dim3(blocks_for(m, T)), dim3(T), 0, s, n_ref,
+                   (const uint32_t *)rfirst.p, (const uint32_t *)dfirst.p, (const uint64_t *)skey, (uint32_t)n, p.n_max,
+                   cc.p, cf.p, flag.p);
+            scan_exclusive_u64(A, scan, flag.p, pos.p, m, pos.p + m, s);
+            launch(GBLOD_K_BUILD_OTHER, k_number_nodes, dim3(mg), dim3(T), 0, s, n_ref, (const uint64_t *)flag.p,
+                   (const uint64_t *)pos.p, (const uint32_t *)dfirst.p, node.p, level.p);
+            auto *hl = static_cast<unsigned long long *>(hs.get((DEPTHS + 2) * sizeof(unsigned long long)));
+            GB_CUDA(cudaMemcpyAsync(hl, level.p, (DEPTHS + 2) * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+            GB_CUDA(cudaStreamSynchronize(s));
+            // level[d + 1] = the first node of depth d + 1, up to the depth with no nodes left
+            for (int d = 2; d < DEPTHS + 2 && hl[d] > level_first.back(); ++d) level_first.push_back(hl[d]);
+        }
+        N.ensure(A, level_first.back(), s);
+        launch(GBLOD_K_BUILD_OTHER, k_emit_nodes, dim3(mg), dim3(T), 0, s, N.soa(), (uint32_t)n, n_ref,
+               (const uint32_t *)rfirst.p, (const uint32_t *)dfirst.p, (const uint64_t *)skey, (const uint32_t *)cc.p,
+               (const uint32_t *)cf.p, (const uint64_t *)flag.p, (const uint64_t *)pos.p, (const uint32_t *)node.p);
     }
-    cc.release(A, s); cf.release(A, s); nz.release(A, s); slot.release(A, s);
     const size_t nn = level_first.back();
     o->n_nodes = nn;
     o->depth_max = (int)level_first.size() - 2;
@@ -621,20 +742,25 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
     Scratch<uint32_t> flags(A, nn, s), isrep(A, nn, s), reppos(A, nn, s);
     Scratch<uint64_t> pcount(A, nn, s), pfirst(A, nn, s), ptotal(A, 1, s), mlo(A, nn, s), mhi(A, nn, s);
     Scratch<float> w(A, nn, s), sc(A, nn, s), hcull(A, nn, s), bmin(A, 3 * nn, s), bmax(A, 3 * nn, s);
-    Scratch<unsigned> hmax(A, nn, s);
+    Scratch<unsigned> hmax(A, 2 * nn, s); // largest h, then k_bottom_up's arrivals
     launch(GBLOD_K_BUILD_OTHER, k_node_classify, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn,
            (const uint32_t *)N.count.p, (const int32_t *)N.depth.p, p.n_max, flags.p, pcount.p, isrep.p);
     scan_exclusive_u64(A, scan, pcount.p, pfirst.p, nn, ptotal.p, s);
     scan_exclusive_u32(A, scan, isrep.p, reppos.p, nn, total.p, s);
-    const uint64_t npts = read1(ptotal.p, s, hs);
-    const uint32_t n_rep = read1(total.p, s, hs);
+    uint64_t *hp = static_cast<uint64_t *>(hs.get(16));
+    uint32_t *hr = reinterpret_cast<uint32_t *>(hp + 1);
+    GB_CUDA(cudaMemcpyAsync(hp, ptotal.p, 8, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(hr, total.p, 4, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaStreamSynchronize(s));
+    const uint64_t npts = *hp;
+    const uint32_t n_rep = *hr;
     o->n_points = npts;
     launch(GBLOD_K_BUILD_OTHER, k_node_mass, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn, (size_t)n,
            (const uint32_t *)N.first.p, (const uint32_t *)N.count.p, (const uint32_t *)flags.p,
            o->equal_mass ? (const U128 *)nullptr : (const U128 *)mpre.p, (const U128 *)mtot.p, m0, p.n_max, mlo.p,
            mhi.p, w.p, sc.p);
     mpre.reset();
-    GB_CUDA(cudaMemsetAsync(hmax.p, 0, nn * sizeof(unsigned), s));
+    GB_CUDA(cudaMemsetAsync(hmax.p, 0, 2 * nn * sizeof(unsigned), s));
 
     o->pts4 = static_cast<float4 *>(A.get(npts * sizeof(float4), s));
     o->hs = static_cast<float *>(A.get(npts * sizeof(float), s));
@@ -658,20 +784,14 @@ static gblod_octree *build_octree_impl(gblod_octree *o, const float *xyz, const 
            (const uint32_t *)flags.p, (const uint32_t *)N.first.p, (const uint32_t *)N.count.p,
            (const uint64_t *)pfirst.p, (const float4 *)s4, o->equal_mass ? (const float *)nullptr : (const float *)sm.p,
            m0, o->pts4, o->hs, o->pt_src, bmin.p, bmax.p, hmax.p);
-    for (int d = o->depth_max; d >= 0; --d) {
-        const uint64_t L = level_first[d];
-        const uint32_t nd = (uint32_t)(level_first[d + 1] - L);
-        launch(GBLOD_K_BUILD_OTHER, k_bottom_up, dim3(blocks_for(nd, T)), dim3(T), 0, s, L, nd,
-               (const uint32_t *)flags.p, (const uint32_t *)N.child_first.p, (const uint32_t *)N.child_count.p,
-               bmin.p, bmax.p, (const unsigned *)hmax.p, hcull.p);
-    }
+    launch(GBLOD_K_BUILD_OTHER, k_bottom_up, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn, (const uint32_t *)flags.p,
+           (const uint32_t *)N.child_first.p, (const uint32_t *)N.child_count.p, (const int32_t *)N.parent.p, bmin.p, bmax.p,
+           (const unsigned *)hmax.p, hcull.p, hmax.p + nn);
     PackIn P{N.code.p, pfirst.p, mlo.p, mhi.p, N.first.p, N.count.p, N.child_first.p, N.child_count.p, flags.p,
              N.depth.p, N.parent.p, hcull.p, w.p, sc.p, bmin.p, bmax.p, p.n_max};
     launch(GBLOD_K_BUILD_OTHER, k_pack_nodes, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn, P, o->nodes);
-    GB_CUDA(cudaStreamSynchronize(s));
     o->bytes = nn * sizeof(gblod_node) + npts * (sizeof(float4) + sizeof(float) + sizeof(uint32_t)) +
                n * (sizeof(uint64_t) + sizeof(uint32_t));
-    return o;
 }
 
 } // namespace gb

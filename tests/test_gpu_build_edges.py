@@ -63,3 +63,23 @@ def test_build_edges_equal_the_oracle(kind, n):
         t.free()
         torch.cuda.synchronize()
         assert b.used == 0
+
+
+@pytest.mark.parametrize("n, n_max", [(2, 1), (4096, 1), (4097, 4096), (8193, 1), (30000, 2), (9000, 8999), (9000, 9000)])
+@pytest.mark.parametrize("kind", KINDS + ["pairs"])
+def test_refined_nodes_equal_the_oracle(kind, n, n_max):
+    """Node tables at the edges of the pass that finds the refined nodes: blocks of 4096 positions full of
+    them, none, chains of single children down to the last level, runs of equal keys that end a block."""
+    from paper_0811_2055_gb300 import gblod
+    torch.cuda.set_device(0)
+    xyz, mass, h, _ = _data("uniform" if kind == "pairs" else kind, n, 4)
+    if kind == "pairs":     # every particle twice: over-full nodes at the last level
+        xyz[1::2] = xyz[: len(xyz[1::2]) * 2: 2]
+    ot = O.build_tree(xyz, mass, h, seed=4, n_max=n_max)
+    t = gblod.build_lod(*to_dev(xyz, mass, h), n_max=n_max, seed=4)
+    compare_trees(t.export(), ot)
+    t.quantize()
+    qn, on = t.export_block16()["qnodes"], O.block_quantize(ot)[2].nodes
+    for f in ("bmin", "bmax", "h_cull", "parent"):
+        assert np.array_equal(qn[f], on[f]), f
+    t.free()
