@@ -58,17 +58,16 @@ static_assert(US_THREADS == 256 && RS_TILE % US_THREADS == 0, "one upsweep threa
 // memory in the tile's digit order, and written out by consecutive threads, so that each digit's run
 // of keys (about 16 per tile and digit) goes to consecutive addresses.
 //
-// Ranking, one round of 32 keys of a warp: every lane sets its bit in its digit's word of the warp's
-// table, and the word then names the lanes with the same digit.  (__match_any_sync does the same by a
-// loop over the distinct values: 260 cycles a round for random digits against 31; it was most of this
-// kernel's time.)  512 threads x 8 keys, two CTAs per SM: 150M pairs 1.84 -> 1.06 ms a pass, 3.6 GB
-// moved (256 x 16 1.16 ms, 1024 x 8 1.17, three CTAs at 42 registers 1.30).
+// Ranking, one round of 32 keys of a warp: eight votes, one per bit, give every lane the lanes with the same
+// digit, and a table of the warp's counts the keys before them.  All rounds' votes come first: they need
+// no memory and run under the loads and the table reads of other warps.  (A mask table in shared memory
+// instead of the votes: 30 cycles a round of the one shared-memory port, and the ranking bound the kernel;
+// __match_any_sync loops over the distinct values, 260 cycles.)  512 threads x 8 keys, two CTAs per SM:
+// 150M pairs, 3.6 GB moved, 1.84 ms a pass with match_any, 1.06 with the mask table, now 0.96 (a copy of the pairs
+// 0.54; without ranking 0.67, three CTAs at 42 registers 1.19).
 struct ScatterSmem {
     uint64_t k[RS_TILE];
-    union {
-        uint32_t v[RS_TILE];
-        uint32_t match[RS_WARPS][256]; // lanes of the current round by digit; zero between rounds
-    };
+    uint32_t v[RS_TILE];
     uint32_t wh[RS_WARPS][256]; // keys of each digit in this warp so far, then in the warps before
     uint32_t to[256];           // global position of a digit's first key, less its tile-local one
     uint32_t tstart[256];       // first tile-local position of each digit
@@ -86,6 +85,7 @@ __global__ void __launch_bounds__(RS_THREADS, RS_CTAS)
     const size_t tile0 = (size_t)blockIdx.x * RS_TILE;
     const size_t base = tile0 + (size_t)warp * (RS_ROUNDS * 32);
     const uint32_t nt = (uint32_t)min((size_t)RS_TILE, n - tile0); // keys in this tile
+    const uint32_t off = threadIdx.x < 256 ? offs[(size_t)threadIdx.x * ntiles + blockIdx.x] : 0u;
     uint64_t k[RS_ROUNDS];
     uint32_t v[RS_ROUNDS];
     uint32_t rk[RS_ROUNDS];
@@ -99,24 +99,28 @@ __global__ void __launch_bounds__(RS_THREADS, RS_CTAS)
         const size_t i = base + (size_t)r * 32 + lane;
         v[r] = i < n ? vin[i] : 0u;
     }
-    for (int i = lane; i < 256; i += 32) {
-        sm.wh[warp][i] = 0u;
-        sm.match[warp][i] = 0u;
-    }
+    for (int i = lane; i < 256; i += 32) sm.wh[warp][i] = 0u;
     __syncwarp();
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+        const uint32_t d = (uint32_t)(k[r] >> shift) & 255u;
+        uint32_t peers = __ballot_sync(0xffffffffu, base + (size_t)r * 32 + lane < n);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const bool bit = (d >> b) & 1u;
+            const uint32_t m = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? m : ~m;
+        }
+        rk[r] = peers;
+    }
 #pragma unroll
     for (int r = 0; r < RS_ROUNDS; ++r) {
         const bool ok = base + (size_t)r * 32 + lane < n;
         const uint32_t d = (uint32_t)(k[r] >> shift) & 255u;
-        if (ok) atomicOr(&sm.match[warp][d], 1u << lane);
-        __syncwarp();
-        const uint32_t peers = sm.match[warp][d], cur = sm.wh[warp][d], before = __popc(peers & lt);
+        const uint32_t peers = rk[r], cur = sm.wh[warp][d], before = __popc(peers & lt);
         rk[r] = cur + before;
         __syncwarp();
-        if (ok && before == 0) {
-            sm.wh[warp][d] = cur + __popc(peers);
-            sm.match[warp][d] = 0u;
-        }
+        if (ok && before == 0) sm.wh[warp][d] = cur + __popc(peers);
         __syncwarp();
     }
     __syncthreads();
@@ -142,7 +146,7 @@ __global__ void __launch_bounds__(RS_THREADS, RS_CTAS)
         uint32_t start = incl - total;
         for (int w = 0; w < warp; ++w) start += sm.wsum[w];
         sm.tstart[threadIdx.x] = start;
-        sm.to[threadIdx.x] = offs[(size_t)threadIdx.x * ntiles + blockIdx.x] - start; // modulo 2^32
+        sm.to[threadIdx.x] = off - start; // modulo 2^32
     }
     __syncthreads();
     // keys and values in tile-local digit order
