@@ -1043,9 +1043,11 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
 // counts, offsets and work items (of per_item records) of the tiles' runs from the scanned (tile, CTA) histogram
 // of CTA groups of G
 __global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, uint32_t per_item, const uint32_t *__restrict__ off,
-                                  const uint32_t *total, uint32_t *tile_cnt, uint32_t *tile_off, uint32_t *item_cnt)
+                                  const uint32_t *total, uint32_t *tile_cnt, uint32_t *tile_off, uint32_t *item_cnt,
+                                  unsigned long long *frame_tiles, uint32_t in_frame)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0 && frame_tiles) *frame_tiles = in_frame;
     if (t >= ntiles) return;
     const uint32_t a = off[(size_t)t * G], b = t + 1 < ntiles ? off[(size_t)(t + 1) * G] : *total;
     tile_off[t] = a;
@@ -1240,18 +1242,21 @@ __global__ void __launch_bounds__(RT, 4) k_splat_small(const uint4 *__restrict__
     if (COUNT) count_hits(hits, stats);
 }
 
-__global__ void k_tile_items(uint32_t ntiles, const uint32_t *tile_cnt, uint32_t *item_cnt)
+__global__ void k_tile_items(uint32_t ntiles, const uint32_t *tile_cnt, uint32_t *item_cnt,
+                             unsigned long long *frame_tiles)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0 && frame_tiles) *frame_tiles = ntiles;
     if (t < ntiles) item_cnt[t] = (tile_cnt[t] + ITEM - 1) / ITEM;
 }
 
-// also clears the unit counter of the splat launch that follows
+// also clears the unit counter of the splat launch that follows and the frame's maximum (may be null)
 __global__ void k_fill_items(uint32_t nruns, uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
-                             const uint32_t *item_off, uint4 *items, unsigned *next)
+                             const uint32_t *item_off, uint4 *items, unsigned *next, unsigned long long *maxv)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) *next = 0u;
+    if (t == 0 && maxv) *maxv = 0ull;
     if (t >= nruns) return;
     const uint32_t c = tile_cnt[t], o = tile_off[t];
     uint32_t k = item_off[t];
@@ -1746,23 +1751,23 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
     r->item_off.ensure(A, nruns + 1, s);
     if (bn.part) {
         r->cta_hist.ensure(A, nall, s);
-        r->cta_off.ensure(A, nall + 1, s);
+        r->cta_off.ensure(A, nall, s);
         launch(GBLOD_K_PROJECT_COUNT, k_project_hist<Src, SMALL>, dim3(bn.grid), dim3(PART_THREADS<SMALL>), bn.smem, s, src, P, lo, hi,
                bn.chunk, gs, r->cta_hist.p, r->status, stats);
-        scan_exclusive_u32(A, r->scan, r->cta_hist.p, r->cta_off.p, nall, r->cta_off.p + nall, s);
+        scan_exclusive_u32(A, r->scan, r->cta_hist.p, r->cta_off.p, nall, &stats->records, s);
         const dim3 tg((nruns + 255) / 256);
         launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, ITEM,
-               (const uint32_t *)r->cta_off.p, (const uint32_t *)(r->cta_off.p + nh), r->tile_cnt.p, r->tile_off.p,
-               r->item_cnt.p);
+               (const uint32_t *)r->cta_off.p, SMALL ? (const uint32_t *)(r->cta_off.p + nh) : &stats->records,
+               r->tile_cnt.p, r->tile_off.p, r->item_cnt.p, &stats->tiles, ntiles);
         if (SMALL) {
             r->tile_cnt_s.ensure(A, nruns, s);
-            r->tile_off_s.ensure(A, nruns + 1, s);
+            r->tile_off_s.ensure(A, nruns, s);
             r->item_cnt_s.ensure(A, nruns, s);
-            r->item_off_s.ensure(A, nruns + 1, s);
+            r->item_off_s.ensure(A, nruns, s);
             launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, ITEM_SMALL,
-                   (const uint32_t *)(r->cta_off.p + nh), (const uint32_t *)(r->cta_off.p + 2 * nh), r->tile_cnt_s.p,
-                   r->tile_off_s.p, r->item_cnt_s.p);
-            scan_exclusive_u32(A, r->scan, r->item_cnt_s.p, r->item_off_s.p, nruns, r->item_off_s.p + nruns, s);
+                   (const uint32_t *)(r->cta_off.p + nh), &stats->records, r->tile_cnt_s.p, r->tile_off_s.p,
+                   r->item_cnt_s.p, (unsigned long long *)nullptr, 0u);
+            scan_exclusive_u32(A, r->scan, r->item_cnt_s.p, r->item_off_s.p, nruns, &stats->small_items, s);
         }
     } else {
         r->tile_cur.ensure(A, ntiles, s);
@@ -1771,22 +1776,15 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
                r->status, stats);
         scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, ntiles, r->tile_off.p + ntiles, s);
         launch(GBLOD_K_RENDER_OTHER, k_tile_items, dim3((ntiles + 255) / 256), dim3(256), 0, s, ntiles,
-               (const uint32_t *)r->tile_cnt.p, r->item_cnt.p);
+               (const uint32_t *)r->tile_cnt.p, r->item_cnt.p, &stats->tiles);
     }
-    scan_exclusive_u32(A, r->scan, r->item_cnt.p, r->item_off.p, nruns, r->item_off.p + nruns, s);
-    unsigned long long *h = static_cast<unsigned long long *>(r->hs.get(40));
-    h[2] = h[3] = h[4] = 0;
-    GB_CUDA(cudaMemcpyAsync(h, &stats->pairs, 8, cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(h + 1, &stats->points, 8, cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(h + 2, r->item_off.p + nruns, 4, cudaMemcpyDeviceToHost, s));
-    const bool streams = bn.part && SMALL;
-    if (streams) {
-        GB_CUDA(cudaMemcpyAsync(h + 3, r->item_off_s.p + nruns, 4, cudaMemcpyDeviceToHost, s));
-        GB_CUDA(cudaMemcpyAsync(h + 4, r->cta_off.p + 2 * nh, 4, cudaMemcpyDeviceToHost, s));
-    }
+    scan_exclusive_u32(A, r->scan, r->item_cnt.p, r->item_off.p, nruns, &stats->items, s);
+    FrameStatsDev *h = static_cast<FrameStatsDev *>(r->hs.get(sizeof(FrameStatsDev)));
+    GB_CUDA(cudaMemcpyAsync(h, stats, sizeof(FrameStatsDev), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
-    return PassCounts{streams ? (h[4] & 0xFFFFFFFFull) : h[0], h[1], (uint32_t)(h[2] & 0xFFFFFFFFull),
-                      (uint32_t)(h[3] & 0xFFFFFFFFull)};
+    const bool streams = bn.part && SMALL;
+    return PassCounts{streams ? (unsigned long long)h->records : h->pairs, h->points, h->items,
+                      streams ? h->small_items : 0u};
 }
 
 // R3 over `items` work items: a persistent grid, no more CTAs than the units need
@@ -1832,7 +1830,7 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
     }
     launch(GBLOD_K_RENDER_OTHER, k_fill_items, tg, dim3(256), 0, s, nruns, ntiles,
            (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p, (const uint32_t *)r->item_off.p,
-           r->items.p, r->status + 1);
+           r->items.p, r->status + 1, r->maxv.p);
     launch_splat(r->count_updates, r->records.p, r->items.p, pc.items, r->status + 1, P, img, r->stats, s);
 }
 
@@ -1850,13 +1848,12 @@ void frame_common(gblod_renderer *r, const Src &src, const Proj &P, const gblod_
         r->accum.ensure(A, npix, s);
         img = r->accum.p;
     }
+    r->maxv.ensure(A, 1, s);
     GB_CUDA(cudaMemsetAsync(img, 0, npix * 8, s));
     const unsigned long long RECORD_BUDGET =
         rp.record_budget ? std::min<unsigned long long>(rp.record_budget, RECORD_BUDGET_MAX) : RECORD_BUDGET_DEFAULT;
     // whole frame first; its counts also give the frame statistics
     const PassCounts all = bin_count(r, src, P, 0ull, ~0ull, r->stats, s);
-    const unsigned long long tl[1] = {ntiles};
-    GB_CUDA(cudaMemcpyAsync(&r->stats->tiles, tl, 8, cudaMemcpyHostToDevice, s));
     if (all.pairs <= RECORD_BUDGET) {
         bin_splat(r, src, P, 0ull, ~0ull, all, img, s);
     } else {
@@ -1885,10 +1882,8 @@ void frame_common(gblod_renderer *r, const Src &src, const Proj &P, const gblod_
         }
     }
     if (image) {
-        r->maxv.ensure(A, 1, s);
         double lo = 0.0, hi = 0.0;
         if (rp.tone_auto) {
-            GB_CUDA(cudaMemsetAsync(r->maxv.p, 0, 8, s));
             launch(GBLOD_K_TONEMAP, k_image_max, dim3(tone_blocks(npix)), dim3(256), 0, s,
                    (const unsigned long long *)img, npix, r->maxv.p);
         } else {
@@ -2490,7 +2485,7 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
         scan_exclusive_u32(A, r->scan, r->b_hist.p, r->b_hist.p, nh, r->b_hist.p + nh, s);
         launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, b.ntiles, (uint32_t)GP, ITEM,
                (const uint32_t *)r->b_hist.p, (const uint32_t *)(r->b_hist.p + nh), r->tile_cnt.p, r->tile_off.p,
-               r->item_cnt.p);
+               r->item_cnt.p, (unsigned long long *)nullptr, 0u);
         launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, true>, dim3(GP), dim3(RT), smem, s, src, r->b_hist.p, b.ntiles, kernel,
                r->records.p, rec_cap, r->status, r->stats, count);
     } else {
@@ -2499,7 +2494,7 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
                (uint4 *)nullptr, 0ull, r->status, r->stats, 0);
         scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, b.ntiles, r->tile_off.p + b.ntiles, s);
         launch(GBLOD_K_RENDER_OTHER, k_tile_items, tg, dim3(256), 0, s, b.ntiles, (const uint32_t *)r->tile_cnt.p,
-               r->item_cnt.p);
+               r->item_cnt.p, (unsigned long long *)nullptr);
         GB_CUDA(cudaMemcpyAsync(r->tile_cur.p, r->tile_off.p, (size_t)b.ntiles * 4, cudaMemcpyDeviceToDevice, s));
         launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, false>, dim3(G), dim3(RT), 0, s, src, r->tile_cur.p, b.ntiles, kernel,
                r->records.p, rec_cap, r->status, r->stats, count);
@@ -2774,7 +2769,7 @@ gblod_status render_brute_noalloc(const float *xyz, const float *mass, const flo
            status, stats);
     scan_exclusive_u32(none, scan, tile_cnt, tile_off, ntiles, tile_off + ntiles, s);
     launch(GBLOD_K_RENDER_OTHER, k_tile_items, dim3((nt + 255) / 256), dim3(256), 0, s, nt,
-           (const uint32_t *)tile_cnt, item_cnt);
+           (const uint32_t *)tile_cnt, item_cnt, (unsigned long long *)nullptr);
     scan_exclusive_u32(none, scan, item_cnt, item_off, ntiles, item_off + ntiles, s);
     if (scan.buf.p != base + NA_OFF_SCAN) fail(GBLOD_ERR_CUDA, "scan temp left the fixed scratch");
 
@@ -2801,7 +2796,8 @@ gblod_status render_brute_noalloc(const float *xyz, const float *mass, const flo
            tile_cur, records, img,
            (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? stats : (FrameStatsDev *)nullptr);
     launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((nt + 255) / 256), dim3(256), 0, s, nt, nt,
-           (const uint32_t *)tile_cnt, (const uint32_t *)tile_off, (const uint32_t *)item_off, items, status + 1);
+           (const uint32_t *)tile_cnt, (const uint32_t *)tile_off, (const uint32_t *)item_off, items, status + 1,
+           (unsigned long long *)nullptr);
     launch_splat((rp.flags & GBLOD_RENDER_COUNT_UPDATES) != 0, records, items, nitems, status + 1, P, img, stats, s);
     if (image) {
         double lo = 0.0, hi = 0.0;
