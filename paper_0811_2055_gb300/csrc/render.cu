@@ -287,13 +287,12 @@ __device__ __forceinline__ unsigned walk_boxes(const BoxWalk &b, uint32_t tag, T
 // pair's point and shuffling its operands; columns and rows a box does not have idle.  Distances in 32
 // bits and Wq < 2^32 (group_box decides; walk_boxes takes the rest).  K has a zero entry 1024.  at(t, x, y) gives,
 // for a box's column x from row y (t: the point's tag if TAGGED, else 0), the function (j, c) that receives every
-// nonzero contribution c < 2^32 to row y + j.  Returns this lane's pixel updates (COUNT).  Every lane of the
-// warp calls it.  Small boxes of 150M particles, the whole box in view (k_splat_small): 7.9 ms walked, 8.1 ms with
-// this alone, 6.6 ms with the smallest boxes in lane_boxes (the shuffles and lookups of idle lanes bind
-// here: the additions alone are 0.8 ms).  LOD scatter of 16.8M particles 0.59 -> 0.43 ms.
+// nonzero contribution c < 2^32 to row y + j.  Returns this lane's pixel updates.  Every lane of the warp calls
+// it.  LOD scatter of 16.8M particles 0.59 -> 0.43 ms; with a box per lane (BoxQueues) 0.51: a row of a
+// group is one transaction of the global additions.
 __device__ __forceinline__ bool group_box(int r, float Wf) { return r <= R_NARROW && Wf < 0x1p32f; }
 
-template <bool COUNT, bool TAGGED = false, class At>
+template <bool TAGGED, class At>
 __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t S, float Wf, int x0, int x1, int y0,
                                                 int y1, const int32_t *K, At at, uint32_t tag = 0u)
 {
@@ -333,7 +332,7 @@ __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t 
                 const uint32_t idx = j0 + j < rows ? min(__umulhi(dx2 + (uint32_t)(d * d), qS) >> 5, 1024u) : 1024u;
                 const uint32_t kv = (uint32_t)K[idx];
                 c[j] = Wh * kv + ((Wl * kv) >> 16);
-                if (COUNT) hits += idx < 1024u ? 1u : 0u;
+                hits += idx < 1024u ? 1u : 0u;
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -343,37 +342,91 @@ __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t 
     return hits;
 }
 
-// The same for boxes of at most LANE_BOX x LANE_BOX pixels, one per lane: nothing is shuffled, and 32
-// different points' table reads and additions go out together.
-constexpr int LANE_BOX = 4;
-template <bool COUNT, class Add>
-__device__ __forceinline__ unsigned lane_boxes(bool on, int U, int V, uint32_t S, float Wf, int x0, int x1, int y0,
-                                               int y1, const int32_t *K, Add add)
+// A warp's queues of small boxes, by size (4, 6 and 8 pixels on a side): a box waits until 32 of its size have
+// come, and those are taken one per lane (lane_boxes) -- no operand is shuffled, every lane has a point,
+// and the 32 points' table reads and additions go out together.  k_splat_small, 150M particles, the whole box
+// in view: 6.6 ms with the smallest boxes one per lane as they came and the rest in groups of eight lanes, 4.7 so
+// (sizes 3, 5, 8: 4.7; 4, 5, 8: 4.8; 5, 6, 8: 4.9); bound by the arithmetic of the padded boxes.
+constexpr int QUEUES = 3;
+struct BoxQueues {
+    uint4 rec[QUEUES][64]; // U, V, S, amplitude
+    uint2 box[QUEUES][64]; // x0 | y0 << 16, width | height << 8
+};
+
+template <int N, bool COUNT, class At>
+__device__ __forceinline__ unsigned lane_boxes(bool on, const uint4 R, const uint2 B, const int32_t *K, At at)
 {
-    const int bw = on ? x1 - x0 + 1 : 0, bh = on ? y1 - y0 + 1 : 0;
+    const int bw = on ? (int)(B.y & 0xFFu) : 0, bh = on ? (int)(B.y >> 8) : 0;
+    const int x0 = (int)(B.x & 0xFFFFu), y0 = (int)(B.x >> 16);
     const int mh = (int)__reduce_max_sync(0xffffffffu, (unsigned)bh);
-    const uint32_t Wq = on ? __float2uint_rn(Wf) : 0u, Wh = Wq >> 16, Wl = Wq & 0xFFFFu;
-    uint32_t dx2[LANE_BOX];
+    const uint32_t Wq = on ? __float2uint_rn(__uint_as_float(R.w)) : 0u, Wh = Wq >> 16, Wl = Wq & 0xFFFFu;
+    const auto add = at(x0, y0);
+    uint32_t dx2[N];
 #pragma unroll
-    for (int c = 0; c < LANE_BOX; ++c) {
-        const int dx = (x0 + c) * 256 + 128 - U;
+    for (int c = 0; c < N; ++c) {
+        const int dx = (x0 + c) * 256 + 128 - (int)R.x;
         dx2[c] = (uint32_t)(dx * dx);
     }
     unsigned hits = 0;
     for (int j = 0; j < mh; ++j) {
-        const int dy = (y0 + j) * 256 + 128 - V;
+        const int dy = (y0 + j) * 256 + 128 - (int)R.y;
         const uint32_t dy2 = (uint32_t)(dy * dy);
-        uint32_t v[LANE_BOX];
+        const int w = j < bh ? bw : 0;
+        uint32_t v[N];
 #pragma unroll
-        for (int c = 0; c < LANE_BOX; ++c) {
-            const uint32_t idx = c < bw && j < bh ? min(__umulhi(dx2[c] + dy2, S) >> 5, 1024u) : 1024u;
+        for (int c = 0; c < N; ++c) {
+            const uint32_t idx = min(__umulhi(dx2[c] + dy2, R.z) >> 5, 1024u);
             const uint32_t kv = (uint32_t)K[idx];
             v[c] = Wh * kv + ((Wl * kv) >> 16);
-            if (COUNT) hits += idx < 1024u ? 1u : 0u;
+            if (COUNT) hits += c < w && idx < 1024u ? 1u : 0u;
         }
 #pragma unroll
-        for (int c = 0; c < LANE_BOX; ++c)
-            if (v[c]) add(x0 + c, y0 + j, v[c]);
+        for (int c = 0; c < N; ++c)
+            if (c < w) add(c, j, v[c]);
+    }
+    return hits;
+}
+
+// Takes queue q's last boxes, 32 of them or (fewer) all n
+template <bool COUNT, class At>
+__device__ __forceinline__ unsigned take_boxes(const BoxQueues &Q, int q, int n, const int32_t *K, At at)
+{
+    const int lane = threadIdx.x & 31, first = max(n - 32, 0);
+    const bool on = first + lane < n;
+    const uint4 R = on ? Q.rec[q][first + lane] : make_uint4(0u, 0u, 0u, 0u);
+    const uint2 B = on ? Q.box[q][first + lane] : make_uint2(0u, 0u);
+    switch (q) {
+    case 0: return lane_boxes<4, COUNT>(on, R, B, K, at);
+    case 1: return lane_boxes<6, COUNT>(on, R, B, K, at);
+    default: return lane_boxes<8, COUNT>(on, R, B, K, at);
+    }
+}
+
+// Adds the lanes' boxes to the queues (on: this lane has one; n: boxes in each queue, the same in all lanes),
+// takes what has become full.  Every lane of the warp calls it.
+template <bool COUNT, class At>
+__device__ __forceinline__ unsigned queue_boxes(BoxQueues &Q, int (&n)[QUEUES], bool on, const uint4 R, int x0, int x1,
+                                                int y0, int y1, const int32_t *K, At at)
+{
+    const int side = on ? max(x1 - x0, y1 - y0) + 1 : 0;
+    const int mine = on ? (side <= 4 ? 0 : (side <= 6 ? 1 : 2)) : -1;
+    unsigned hits = 0;
+#pragma unroll
+    for (int q = 0; q < QUEUES; ++q) {
+        const uint32_t m = __ballot_sync(0xffffffffu, mine == q);
+        if (!m) continue;
+        if (mine == q) {
+            const int to = n[q] + __popc(m & gbd::lanemask_lt());
+            Q.rec[q][to] = R;
+            Q.box[q][to] = make_uint2((uint32_t)x0 | (uint32_t)y0 << 16, (uint32_t)(x1 - x0 + 1) | (uint32_t)(y1 - y0 + 1) << 8);
+        }
+        n[q] += __popc(m);
+        __syncwarp();
+        if (n[q] >= 32) {
+            hits += take_boxes<COUNT>(Q, q, n[q], K, at);
+            n[q] -= 32;
+            __syncwarp();
+        }
     }
     return hits;
 }
@@ -1124,7 +1177,7 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
                 }
             }
             if (!SMALL) {
-                hits += group_boxes<true>(
+                hits += group_boxes<false>(
                     mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K,
                     [&](uint32_t, int x, int y) {
                         unsigned long long *p = img + (size_t)y * P.W + x;
@@ -1151,43 +1204,55 @@ __global__ void k_fill_items_n(uint32_t nruns, uint32_t ntiles, const uint32_t *
 }
 
 // Small-box records of one work item (a tile and up to ITEM_SMALL of its records): each warp takes
-// 32 records at a time and takes their pixel boxes, clipped to the tile, four at a time (group_boxes) or, for
+// 32 records at a time and takes their pixel boxes, clipped to the tile, by size (BoxQueues) or, for
 // wide supports and the largest amplitudes, together (walk_boxes), adding the
 // per-pixel rule's contributions to a shared tile image.  A contribution c < 2^49 is added as three
 // fields, c = lo + mid 2^16 + hi 2^32 with lo, mid < 2^16, to 32-bit words by fire-and-forget
 // 32-bit shared atomics (hi, rarely nonzero, only when it is): a pixel receives at most one
 // contribution per record, so at most ITEM_SMALL = 2^12 per item, and no word can overflow
-// (mid sums < 2^28, lo sums < 2^32, hi sums < 2^29).  The lo and mid words have four copies, one per group
-// of two warps, so that warps adding to the same pixel -- points pile up in dense halo cores --
-// mostly meet only in the final sum; the fields are then recombined in 64 bits and added to the
-// image once per pixel.  A box is small once clipped to the image, so its pixels can lie far from a
+// (mid sums < 2^28, lo sums < 2^32, hi sums < 2^29).  The fields are then recombined in 64 bits and added
+// to the image once per pixel.  One copy of the tile: with four for the warps of a CTA (44 KB more with the
+// queues) two CTAs fit an SM instead of four, and 150M particles take 6.6 ms instead of 4.7.  A box is small once clipped to the image, so its pixels can lie far from a
 // centre outside the image (the visible sliver of a large blob): walk_boxes takes 64-bit distances
 // for those.
 static_assert(ITEM_SMALL <= (1u << 12), "32-bit field sums of the small-box tile image");
+struct SmallSmem {
+    uint32_t lo[1024], mid[1024], hi[1024]; // TW x TH <= 1024 (checked on the host)
+    int32_t K[1025];
+    BoxQueues queue[RT / 32];
+};
+
 template <bool COUNT>
-__global__ void __launch_bounds__(RT, 4) k_splat_small(const uint4 *__restrict__ rec, const uint4 *__restrict__ items,
+__global__ void __launch_bounds__(RT) k_splat_small(const uint4 *__restrict__ rec, const uint4 *__restrict__ items,
                                                       Proj P, unsigned long long *__restrict__ img, FrameStatsDev *stats)
 {
-    __shared__ uint32_t tlo[4][1024], tmid[4][1024], thi[1024]; // TW x TH <= 1024 (checked on the host)
-    __shared__ int32_t K[1025];
-    if (threadIdx.x == 0) K[1024] = 0;
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    SmallSmem &sm = *reinterpret_cast<SmallSmem *>(small_smem);
+    const int32_t *K = sm.K;
+    if (threadIdx.x == 0) sm.K[1024] = 0;
     for (int i = threadIdx.x; i < 1024; i += RT) {
-        K[i] = g_ktab[P.kernel][i];
-        thi[i] = 0u;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            tlo[c][i] = 0u;
-            tmid[c][i] = 0u;
-        }
+        sm.K[i] = g_ktab[P.kernel][i];
+        sm.lo[i] = sm.mid[i] = sm.hi[i] = 0u;
     }
     __syncthreads();
-    uint32_t *lo = tlo[(threadIdx.x >> 6) & 3], *mid = tmid[(threadIdx.x >> 6) & 3];
+    const int warp = threadIdx.x >> 5;
+    uint32_t *lo = sm.lo, *mid = sm.mid;
     const uint4 it = items[blockIdx.x];
     const int tx = (int)(it.x % (uint32_t)P.tiles_x), ty = (int)(it.x / (uint32_t)P.tiles_x);
     const int X0 = tx * P.TW, Y0 = ty * P.TH;
     const int X1 = min(X0 + P.TW, P.W) - 1, Y1 = min(Y0 + P.TH, P.H) - 1;
     const int TW = P.TW;
     unsigned hits = 0;
+    int nq[QUEUES] = {0, 0, 0};
+    // a contribution below 2^32 as 20 low bits and the rest in the middle word (2^12 contributions of less than
+    // 2^20 stay below 2^32)
+    auto at = [&](int x, int y) {
+        const int p = (y - Y0) * TW + (x - X0);
+        return [=](int c, int j, uint32_t v) {
+            atomicAdd(&lo[p + j * TW + c], v & 0xFFFFFu);
+            atomicAdd(&mid[p + j * TW + c], (v >> 20) << 4);
+        };
+    };
     for (uint32_t base = it.y + (threadIdx.x & ~31u); base < it.z; base += RT) { // uniform per warp
         const uint32_t r = base + (threadIdx.x & 31u);
         BoxWalk b;
@@ -1207,36 +1272,25 @@ __global__ void __launch_bounds__(RT, 4) k_splat_small(const uint4 *__restrict__
                 if (!mine) b = box_walk(U, V, R.z, __float2ull_rn(__uint_as_float(R.w)), rad, x0, x1, y0, y1);
             }
         }
-        // a contribution below 2^32 as 20 low bits and, where it has more, the rest in the middle word
-        // (2^12 contributions of less than 2^20 stay below 2^32)
-        auto at = [&](uint32_t, int x, int y) {
-            const int p = (y - Y0) * TW + (x - X0);
-            return [=](int j, uint32_t c) {
-                atomicAdd(&lo[p + j * TW], c & 0xFFFFFu);
-                if (c >> 20) atomicAdd(&mid[p + j * TW], (c >> 20) << 4);
-            };
-        };
-        const bool tiny = mine && x1 - x0 < LANE_BOX && y1 - y0 < LANE_BOX;
-        hits += lane_boxes<COUNT>(tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K,
-                                  [&](int x, int y, uint32_t c) { at(0u, x, y)(0, c); });
-        hits += group_boxes<COUNT>(mine && !tiny, (int)R.x, (int)R.y, R.z, __uint_as_float(R.w), x0, x1, y0, y1, K, at);
+        hits += queue_boxes<COUNT>(sm.queue[warp], nq, mine, R, x0, x1, y0, y1, K, at);
         hits += walk_boxes<false>(b, 0u, [&](uint32_t, uint32_t i) { return K[i]; },
                                   [&](uint32_t, int x, int y, unsigned long long c) {
             const int p = (y - Y0) * TW + (x - X0);
             atomicAdd(&lo[p], (uint32_t)c & 0xFFFFu);
             atomicAdd(&mid[p], ((uint32_t)c >> 16));
             const uint32_t h = (uint32_t)(c >> 32);
-            if (h) atomicAdd(&thi[p], h);
+            if (h) atomicAdd(&sm.hi[p], h);
         });
     }
+#pragma unroll
+    for (int q = 0; q < QUEUES; ++q)
+        if (nq[q]) hits += take_boxes<COUNT>(sm.queue[warp], q, nq[q], K, at);
     __syncthreads();
     const int tw = X1 - X0 + 1, th = Y1 - Y0 + 1;
     for (int i = threadIdx.x; i < tw * th; i += RT) {
         const int y = i / tw, x = i - y * tw, k = y * P.TW + x;
         const unsigned long long v =
-            (unsigned long long)tlo[0][k] + tlo[1][k] + tlo[2][k] + tlo[3][k] +
-            (((unsigned long long)tmid[0][k] + tmid[1][k] + tmid[2][k] + tmid[3][k]) << 16) +
-            ((unsigned long long)thi[k] << 32);
+            sm.lo[k] + ((unsigned long long)sm.mid[k] << 16) + ((unsigned long long)sm.hi[k] << 32);
         if (v) atomicAdd(&img[(size_t)(Y0 + y) * P.W + (X0 + x)], v);
     }
     if (COUNT) count_hits(hits, stats);
@@ -1821,7 +1875,7 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
                    (const uint32_t *)r->tile_cnt_s.p, (const uint32_t *)r->tile_off_s.p,
                    (const uint32_t *)r->item_off_s.p, ITEM_SMALL, r->items.p + pc.items);
             launch(GBLOD_K_SPLAT, r->count_updates ? k_splat_small<true> : k_splat_small<false>, dim3(pc.small_items),
-                   dim3(RT), 0, s, (const uint4 *)r->records.p, (const uint4 *)(r->items.p + pc.items), P, img, r->stats);
+                   dim3(RT), sizeof(SmallSmem), s, (const uint4 *)r->records.p, (const uint4 *)(r->items.p + pc.items), P, img, r->stats);
         }
     } else {
         GB_CUDA(cudaMemcpyAsync(r->tile_cur.p, r->tile_off.p, (size_t)ntiles * 4, cudaMemcpyDeviceToDevice, s));
@@ -2195,7 +2249,7 @@ __global__ void __launch_bounds__(RT, 4) k_bproject(SrcBatch src, uint32_t *__re
                     unsigned long long *p = V.accum + (size_t)y * W + x;
                     return [p, W](int j, unsigned long long c) { atomicAdd(&p[(size_t)j * W], c); };
                 };
-                hits += group_boxes<true, true>(mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at, (uint32_t)v);
+                hits += group_boxes<true>(mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at, (uint32_t)v);
                 hits += walk_boxes<true>(direct, (uint32_t)v, [&](uint32_t, uint32_t i) { return K[i]; },
                                          [&](uint32_t t, int x, int y, unsigned long long c) { at(t, x, y)(0, c); });
             } else if (n) {
@@ -2373,6 +2427,8 @@ void set_splat_smem()
                           (const void *)k_bproject<true, true>};
     for (const void *f : part)
         GB_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PART_MAX_SMEM));
+    GB_CUDA(cudaFuncSetAttribute(k_splat_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem)));
+    GB_CUDA(cudaFuncSetAttribute(k_splat_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem)));
     const int bytes = (int)sizeof(SplatSmem);
     GB_CUDA(cudaFuncSetAttribute(k_splat_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     GB_CUDA(cudaFuncSetAttribute(k_splat_tiles<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));

@@ -63,3 +63,24 @@ def test_records_in_several_regions(n):
     for k in ("points", "splats", "amplitude_lo", "amplitude_hi", "pixel_updates"):
         assert sa[k] == sb[k], k
     r.close()
+
+
+@pytest.mark.parametrize("side", [0.4, 1.1, 1.9, 2.6, 3.3])
+@pytest.mark.parametrize("n", [1, 31, 33, 4095, 4097, 70001])
+def test_small_boxes_by_size_equal_the_oracle(side, n):
+    """Small boxes of each size alone and together (queues of 4, 6 and 8 pixels that fill, overflow by one and end in
+    the middle), all on one pixel and spread out, light and heavy."""
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    rng = np.random.default_rng(n)
+    xyz = rng.uniform(0.0, 1.0, (n, 3)).astype(np.float32)
+    xyz[n // 2:] = xyz[0]
+    mass = np.exp2(rng.uniform(-12.0, 4.0, n)).astype(np.float32)
+    cam = synth.look_at((0.5, 0.5, -1.5), (0.5, 0.5, 0.5), width=130, height=67)
+    h = (side / 3.0 * 2.0 / cam["f_px"] * rng.uniform(0.5, 1.0, n)).astype(np.float32)
+    r = G.Renderer()
+    want, st, nd = O.splat_particles(xyz, mass, h, cam, O.rparams(sigma_min_px=0.25))
+    _, acc = r.render_bruteforce(*to_dev(xyz, mass, h), cam, G.make_params(sigma_min_px=0.25))
+    assert st == 0 and r.status() == G.OK and np.array_equal(G.u64(acc), want)
+    assert r.stats()["splats"] == nd
+    r.close()
