@@ -17,7 +17,8 @@ constexpr uint32_t FL_LEAF = GBLOD_NODE_LEAF, FL_INTERNAL = GBLOD_NODE_INTERNAL,
 inline unsigned blocks_for(size_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 // ------------------------------------------------------------------ A1 and input checks
-__global__ void k_mass_check(const float *mass, size_t n, unsigned *minb, unsigned *maxb, unsigned *bad)
+// out (zeroed before): the complement of the smallest mass's bits, the largest one's bits, 1 if a mass is not allowed
+__global__ void k_mass_check(const float *mass, size_t n, unsigned *out)
 {
     unsigned lo = 0xFFFFFFFFu, hi = 0u, nbad = 0u;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -36,9 +37,9 @@ __global__ void k_mass_check(const float *mass, size_t n, unsigned *minb, unsign
         nbad |= __shfl_xor_sync(0xffffffffu, nbad, d);
     }
     if ((threadIdx.x & 31) == 0) {
-        atomicMin(minb, lo);
-        atomicMax(maxb, hi);
-        if (nbad) atomicOr(bad, 1u);
+        atomicMax(out, ~lo);
+        atomicMax(out + 1, hi);
+        if (nbad) atomicOr(out + 2, 1u);
     }
 }
 
@@ -500,25 +501,6 @@ __global__ void k_pack_nodes(size_t nn, PackIn P, gblod_node *out)
     out[i] = g;
 }
 
-// node arrays (structure of arrays)
-struct NodeStore {
-    DBuf<uint64_t> code;
-    DBuf<uint32_t> first, count, child_first, child_count;
-    DBuf<int32_t> depth, parent;
-
-    void ensure(const Allocator &A, size_t n, cudaStream_t s)
-    {
-        code.ensure(A, n, s); first.ensure(A, n, s); count.ensure(A, n, s); child_first.ensure(A, n, s);
-        child_count.ensure(A, n, s); depth.ensure(A, n, s); parent.ensure(A, n, s);
-    }
-    NodeSoA soa() { return NodeSoA{code.p, first.p, count.p, child_first.p, child_count.p, depth.p, parent.p}; }
-    void release(const Allocator &A, cudaStream_t s)
-    {
-        code.release(A, s); first.release(A, s); count.release(A, s); child_first.release(A, s);
-        child_count.release(A, s); depth.release(A, s); parent.release(A, s);
-    }
-};
-
 template <class T> T read1(const T *d, cudaStream_t s, HostStage &hs)
 {
     T *h = static_cast<T *>(hs.get(sizeof(T)));
@@ -552,11 +534,9 @@ struct BuildTemps {
     cudaStream_t s;
     ScanTmp scan;
     SortTmp sort;
-    NodeStore N;
     BuildTemps(const Allocator &a, cudaStream_t st) : A(a), s(st) {}
     ~BuildTemps()
     {
-        N.release(A, s);
         scan.buf.release(A, s);
         sort.buf.release(A, s);
         sort.scan.buf.release(A, s);
@@ -615,19 +595,15 @@ static void build_octree_impl(gblod_octree *o, const float *xyz, const float *ma
     const unsigned G = (unsigned)persistent_blocks(8);
     float m0 = 0.0f; // the common mass when all are equal
 
-    // masses: range and whether they are all equal
-    {
-        Scratch<unsigned> mm(A, 3, s);
-        const unsigned init[3] = {0xFFFFFFFFu, 0u, 0u};
-        GB_CUDA(cudaMemcpyAsync(mm.p, init, sizeof(init), cudaMemcpyHostToDevice, s));
-        launch(GBLOD_K_BUILD_OTHER, k_mass_check, dim3(G), dim3(T), 0, s, mass, (size_t)n, mm.p, mm.p + 1, mm.p + 2);
-        unsigned *hm = static_cast<unsigned *>(hs.get(3 * sizeof(unsigned)));
-        GB_CUDA(cudaMemcpyAsync(hm, mm.p, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-        GB_CUDA(cudaStreamSynchronize(s));
-        if (hm[2]) fail(GBLOD_ERR_RANGE, "gblod_build_lod: every mass must be finite and in [2^-24, 2^24]");
-        o->equal_mass = hm[0] == hm[1] ? 1 : 0;
-        std::memcpy(&m0, &hm[0], sizeof(float));
-    }
+    // masses: range and whether they are all equal; read with the sort's first counts (the sort's own read
+    // uses the stage's first bytes)
+    unsigned long long *diff;
+    unsigned *mm;
+    const Scratch<unsigned char> checks = carve(A, s, {part(diff, 1), part(mm, 3)});
+    GB_CUDA(cudaMemsetAsync(checks.p, 0, checks.n, s));
+    launch(GBLOD_K_BUILD_OTHER, k_mass_check, dim3(G), dim3(T), 0, s, mass, (size_t)n, mm);
+    const unsigned *hm = static_cast<unsigned *>(hs.get(256)) + 16;
+    GB_CUDA(cudaMemcpyAsync(const_cast<unsigned *>(hm), mm, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
 
     // A1 + A2: keys in (key, id) order.  Roomy builds hold all work arrays of the sort and the sorted
     // particles in one block: the pool then finds the same few sizes free in every build (with an array
@@ -648,21 +624,24 @@ static void build_octree_impl(gblod_octree *o, const float *xyz, const float *ma
     int sexp = 0;
     const int pow2 = p.root_lo[0] == 0.0 && p.root_lo[1] == 0.0 && p.root_lo[2] == 0.0 &&
                      std::frexp(scale, &sexp) == 0.5 && sexp > -120 && sexp < 120 ? 1 : 0;
-    Scratch<unsigned long long> diff(A, 1, s);
-    GB_CUDA(cudaMemsetAsync(diff.p, 0, sizeof(unsigned long long), s));
     if (ids) {
         launch(GBLOD_K_BUILD_OTHER, k_id_keys, dim3(G), dim3(T), 0, s, ids, (size_t)n, keys, vals);
         radix_sort_pairs(A, sort, &keys, &vals, other_key(), other_val(), n, 32, s, hs);
         // vals = input indices in id order; keys in that order
         uint64_t *kdst = other_key();
         launch(GBLOD_K_MORTON, k_morton, dim3(G), dim3(T), 0, s, xyz, h, (const uint32_t *)vals, (size_t)n,
-               p.root_lo[0], p.root_lo[1], p.root_lo[2], scale, kdst, (uint32_t *)nullptr, pack, diff.p, pow2);
+               p.root_lo[0], p.root_lo[1], p.root_lo[2], scale, kdst, (uint32_t *)nullptr, pack, diff, pow2);
         keys = kdst;
     } else {
         launch(GBLOD_K_MORTON, k_morton, dim3(G), dim3(T), 0, s, xyz, h, (const uint32_t *)nullptr, (size_t)n,
-               p.root_lo[0], p.root_lo[1], p.root_lo[2], scale, keys, vals, pack, diff.p, pow2);
+               p.root_lo[0], p.root_lo[1], p.root_lo[2], scale, keys, vals, pack, diff, pow2);
     }
-    radix_sort_pairs(A, sort, &keys, &vals, other_key(), other_val(), n, 63, s, hs, diff.p);
+    radix_sort_pairs(A, sort, &keys, &vals, other_key(), other_val(), n, 63, s, hs, diff);
+    if (n == 1) GB_CUDA(cudaStreamSynchronize(s)); // nothing to sort, no count read
+    if (hm[2]) fail(GBLOD_ERR_RANGE, "gblod_build_lod: every mass must be finite and in [2^-24, 2^24]");
+    const unsigned lightest = ~hm[0];
+    o->equal_mass = lightest == hm[1] ? 1 : 0;
+    std::memcpy(&m0, &lightest, sizeof(float));
     // keep the sorted keys and permutation in the octree
     if (keys == kalt && roomy) {
         GB_CUDA(cudaMemcpyAsync(keyA.p, keys, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
@@ -695,8 +674,12 @@ static void build_octree_impl(gblod_octree *o, const float *xyz, const float *ma
     const uint32_t *sorted_ids = ids ? sid.p : sidx;
 
     // A3: refined nodes, their children, the nodes in level order
-    NodeStore &N = tmp.N;
-    Scratch<uint32_t> total(A, 1, s);
+    NodeSoA N;
+    uint32_t *flags, *isrep, *reppos, *total;
+    uint64_t *pcount, *pfirst, *ptotal, *mlo, *mhi;
+    float *w, *sc, *hcull, *bmin, *bmax;
+    unsigned *hmax; // largest h, then k_bottom_up's arrivals
+    Scratch<unsigned char> node_mem;
     const uint32_t nb = (uint32_t)((n + RB - 1) / RB);
     uint32_t n_ref = 0;
     std::vector<uint64_t> level_first = {0, 1};
@@ -710,28 +693,35 @@ static void build_octree_impl(gblod_octree *o, const float *xyz, const float *ma
         }
         const size_t m = (size_t)n_ref * 8;
         const unsigned mg = blocks_for(std::max<size_t>(m, DEPTHS + 1), T);
-        Scratch<uint32_t> rfirst(A, n_ref, s), node(A, n_ref, s), cc(A, m, s), cf(A, m, s);
-        Scratch<uint64_t> flag(A, m, s), pos(A, m + 1, s);
+        uint32_t *rfirst, *node, *cc, *cf;
+        uint64_t *flag, *pos;
+        unsigned long long *level;
+        const Scratch<unsigned char> ref_mem = carve(A, s, {part(rfirst, n_ref), part(node, n_ref), part(cc, m), part(cf, m),
+                                                            part(flag, m), part(pos, m + 1), part(level, DEPTHS + 2)});
         if (n_ref) {
-            Scratch<unsigned long long> level(A, DEPTHS + 2, s);
             launch(GBLOD_K_BUILD_OTHER, k_list_refined, dim3(nb), dim3(RT_REF), 0, s, (const uint64_t *)skey, (size_t)n,
-                   (uint64_t)p.n_max, (const uint32_t *)roff.p, rfirst.p, dfirst.p);
+                   (uint64_t)p.n_max, (const uint32_t *)roff.p, rfirst, dfirst.p);
             launch(GBLOD_K_BUILD_OTHER, k_children, dim3(blocks_for(m, T)), dim3(T), 0, s, n_ref,
-                   (const uint32_t *)rfirst.p, (const uint32_t *)dfirst.p, (const uint64_t *)skey, (uint32_t)n, p.n_max,
-                   cc.p, cf.p, flag.p);
-            scan_exclusive_u64(A, scan, flag.p, pos.p, m, pos.p + m, s);
-            launch(GBLOD_K_BUILD_OTHER, k_number_nodes, dim3(mg), dim3(T), 0, s, n_ref, (const uint64_t *)flag.p,
-                   (const uint64_t *)pos.p, (const uint32_t *)dfirst.p, node.p, level.p);
+                   (const uint32_t *)rfirst, (const uint32_t *)dfirst.p, (const uint64_t *)skey, (uint32_t)n, p.n_max,
+                   cc, cf, flag);
+            scan_exclusive_u64(A, scan, flag, pos, m, pos + m, s);
+            launch(GBLOD_K_BUILD_OTHER, k_number_nodes, dim3(mg), dim3(T), 0, s, n_ref, (const uint64_t *)flag,
+                   (const uint64_t *)pos, (const uint32_t *)dfirst.p, node, level);
             auto *hl = static_cast<unsigned long long *>(hs.get((DEPTHS + 2) * sizeof(unsigned long long)));
-            GB_CUDA(cudaMemcpyAsync(hl, level.p, (DEPTHS + 2) * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+            GB_CUDA(cudaMemcpyAsync(hl, level, (DEPTHS + 2) * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
             GB_CUDA(cudaStreamSynchronize(s));
             // level[d + 1] = the first node of depth d + 1, up to the depth with no nodes left
             for (int d = 2; d < DEPTHS + 2 && hl[d] > level_first.back(); ++d) level_first.push_back(hl[d]);
         }
-        N.ensure(A, level_first.back(), s);
-        launch(GBLOD_K_BUILD_OTHER, k_emit_nodes, dim3(mg), dim3(T), 0, s, N.soa(), (uint32_t)n, n_ref,
-               (const uint32_t *)rfirst.p, (const uint32_t *)dfirst.p, (const uint64_t *)skey, (const uint32_t *)cc.p,
-               (const uint32_t *)cf.p, (const uint64_t *)flag.p, (const uint64_t *)pos.p, (const uint32_t *)node.p);
+        const size_t nn = level_first.back();
+        node_mem = carve(A, s, {part(N.code, nn), part(N.first, nn), part(N.count, nn), part(N.child_first, nn),
+                                part(N.child_count, nn), part(N.depth, nn), part(N.parent, nn), part(flags, nn),
+                                part(isrep, nn), part(reppos, nn), part(total, 1), part(pcount, nn), part(pfirst, nn),
+                                part(ptotal, 1), part(mlo, nn), part(mhi, nn), part(w, nn), part(sc, nn), part(hcull, nn),
+                                part(bmin, 3 * nn), part(bmax, 3 * nn), part(hmax, 2 * nn)});
+        launch(GBLOD_K_BUILD_OTHER, k_emit_nodes, dim3(mg), dim3(T), 0, s, N, (uint32_t)n, n_ref,
+               (const uint32_t *)rfirst, (const uint32_t *)dfirst.p, (const uint64_t *)skey, (const uint32_t *)cc,
+               (const uint32_t *)cf, (const uint64_t *)flag, (const uint64_t *)pos, (const uint32_t *)node);
     }
     const size_t nn = level_first.back();
     o->n_nodes = nn;
@@ -739,28 +729,24 @@ static void build_octree_impl(gblod_octree *o, const float *xyz, const float *ma
     o->level_first = level_first;
 
     // classify, number the stored points, masses and representative parameters
-    Scratch<uint32_t> flags(A, nn, s), isrep(A, nn, s), reppos(A, nn, s);
-    Scratch<uint64_t> pcount(A, nn, s), pfirst(A, nn, s), ptotal(A, 1, s), mlo(A, nn, s), mhi(A, nn, s);
-    Scratch<float> w(A, nn, s), sc(A, nn, s), hcull(A, nn, s), bmin(A, 3 * nn, s), bmax(A, 3 * nn, s);
-    Scratch<unsigned> hmax(A, 2 * nn, s); // largest h, then k_bottom_up's arrivals
     launch(GBLOD_K_BUILD_OTHER, k_node_classify, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn,
-           (const uint32_t *)N.count.p, (const int32_t *)N.depth.p, p.n_max, flags.p, pcount.p, isrep.p);
-    scan_exclusive_u64(A, scan, pcount.p, pfirst.p, nn, ptotal.p, s);
-    scan_exclusive_u32(A, scan, isrep.p, reppos.p, nn, total.p, s);
+           (const uint32_t *)N.count, (const int32_t *)N.depth, p.n_max, flags, pcount, isrep);
+    scan_exclusive_u64(A, scan, pcount, pfirst, nn, ptotal, s);
+    scan_exclusive_u32(A, scan, isrep, reppos, nn, total, s);
     uint64_t *hp = static_cast<uint64_t *>(hs.get(16));
     uint32_t *hr = reinterpret_cast<uint32_t *>(hp + 1);
-    GB_CUDA(cudaMemcpyAsync(hp, ptotal.p, 8, cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(hr, total.p, 4, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(hp, ptotal, 8, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(hr, total, 4, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
     const uint64_t npts = *hp;
     const uint32_t n_rep = *hr;
     o->n_points = npts;
     launch(GBLOD_K_BUILD_OTHER, k_node_mass, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn, (size_t)n,
-           (const uint32_t *)N.first.p, (const uint32_t *)N.count.p, (const uint32_t *)flags.p,
-           o->equal_mass ? (const U128 *)nullptr : (const U128 *)mpre.p, (const U128 *)mtot.p, m0, p.n_max, mlo.p,
-           mhi.p, w.p, sc.p);
+           (const uint32_t *)N.first, (const uint32_t *)N.count, (const uint32_t *)flags,
+           o->equal_mass ? (const U128 *)nullptr : (const U128 *)mpre.p, (const U128 *)mtot.p, m0, p.n_max, mlo,
+           mhi, w, sc);
     mpre.reset();
-    GB_CUDA(cudaMemsetAsync(hmax.p, 0, 2 * nn * sizeof(unsigned), s));
+    GB_CUDA(cudaMemsetAsync(hmax, 0, 2 * nn * sizeof(unsigned), s));
 
     o->pts4 = static_cast<float4 *>(A.get(npts * sizeof(float4), s));
     o->hs = static_cast<float *>(A.get(npts * sizeof(float), s));
@@ -771,8 +757,8 @@ static void build_octree_impl(gblod_octree *o, const float *xyz, const float *ma
     if (n_rep) {
         Scratch<uint32_t> reps(A, n_rep, s);
         launch(GBLOD_K_BUILD_OTHER, k_compact_reps, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn,
-               (const uint32_t *)isrep.p, (const uint32_t *)reppos.p, reps.p);
-        SelectIn in{s4, sm.p, sorted_ids, N.code.p, N.first.p, N.count.p, pfirst.p, w.p, sc.p, hmax.p,
+               (const uint32_t *)isrep, (const uint32_t *)reppos, reps.p);
+        SelectIn in{s4, sm.p, sorted_ids, N.code, N.first, N.count, pfirst, w, sc, hmax,
                     o->pts4, o->hs, o->pt_src, p.n_max};
         // the packed particles and the sort's buffers are done with: 28 bytes a particle for the codes
         select_representatives(A, s, hs, scan, in, reps.p, n_rep, p.n_max, p.seed, o->equal_mass,
@@ -781,14 +767,14 @@ static void build_octree_impl(gblod_octree *o, const float *xyz, const float *ma
 
     // leaves, bounds, cull radii
     launch(GBLOD_K_BUILD_OTHER, k_leaf_nodes, dim3((unsigned)std::min<size_t>(nn, 65535 * 4)), dim3(T), 0, s, nn,
-           (const uint32_t *)flags.p, (const uint32_t *)N.first.p, (const uint32_t *)N.count.p,
-           (const uint64_t *)pfirst.p, (const float4 *)s4, o->equal_mass ? (const float *)nullptr : (const float *)sm.p,
-           m0, o->pts4, o->hs, o->pt_src, bmin.p, bmax.p, hmax.p);
-    launch(GBLOD_K_BUILD_OTHER, k_bottom_up, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn, (const uint32_t *)flags.p,
-           (const uint32_t *)N.child_first.p, (const uint32_t *)N.child_count.p, (const int32_t *)N.parent.p, bmin.p, bmax.p,
-           (const unsigned *)hmax.p, hcull.p, hmax.p + nn);
-    PackIn P{N.code.p, pfirst.p, mlo.p, mhi.p, N.first.p, N.count.p, N.child_first.p, N.child_count.p, flags.p,
-             N.depth.p, N.parent.p, hcull.p, w.p, sc.p, bmin.p, bmax.p, p.n_max};
+           (const uint32_t *)flags, (const uint32_t *)N.first, (const uint32_t *)N.count,
+           (const uint64_t *)pfirst, (const float4 *)s4, o->equal_mass ? (const float *)nullptr : (const float *)sm.p,
+           m0, o->pts4, o->hs, o->pt_src, bmin, bmax, hmax);
+    launch(GBLOD_K_BUILD_OTHER, k_bottom_up, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn, (const uint32_t *)flags,
+           (const uint32_t *)N.child_first, (const uint32_t *)N.child_count, (const int32_t *)N.parent, bmin, bmax,
+           (const unsigned *)hmax, hcull, hmax + nn);
+    PackIn P{N.code, pfirst, mlo, mhi, N.first, N.count, N.child_first, N.child_count, flags,
+             N.depth, N.parent, hcull, w, sc, bmin, bmax, p.n_max};
     launch(GBLOD_K_BUILD_OTHER, k_pack_nodes, dim3(blocks_for(nn, T)), dim3(T), 0, s, nn, P, o->nodes);
     o->bytes = nn * sizeof(gblod_node) + npts * (sizeof(float4) + sizeof(float) + sizeof(uint32_t)) +
                n * (sizeof(uint64_t) + sizeof(uint32_t));

@@ -445,56 +445,60 @@ void select_representatives(const Allocator &A, cudaStream_t s, HostStage &hs, S
                             const uint32_t *rep_nodes, uint32_t n_rep, uint32_t n_max, uint64_t seed,
                             int equal_mass, void *spare, size_t spare_bytes)
 {
-    Scratch<uint32_t> nchunks(A, n_rep + 1, s), chunk_off(A, n_rep + 1, s), nbins(A, n_rep, s), hoff(A, n_rep, s);
-    Scratch<uint64_t> nwords(A, n_rep, s), woff(A, n_rep, s);
-    Scratch<uint8_t> logb(A, n_rep, s);
-    Scratch<int16_t> bin0(A, n_rep, s);
-    Scratch<float> rmean(A, n_rep, s);
-    Scratch<uint32_t> tot32(A, 2, s);
-    Scratch<uint64_t> tot64(A, 1, s);
+    uint32_t *nchunks, *chunk_off, *nbins, *hoff, *tot32;
+    uint64_t *nwords, *woff, *tot64;
+    uint8_t *logb;
+    int16_t *bin0;
+    float *rmean;
+    const Scratch<unsigned char> per_rep =
+        carve(A, s, {part(nchunks, n_rep), part(chunk_off, n_rep + 1), part(nbins, n_rep), part(hoff, n_rep), part(tot32, 2),
+                     part(nwords, n_rep), part(woff, n_rep), part(tot64, 1), part(logb, n_rep), part(bin0, n_rep),
+                     part(rmean, n_rep)});
     launch(GBLOD_K_BUILD_OTHER, k_sel_setup, dim3((n_rep + 255) / 256), dim3(256), 0, s, n_rep, rep_nodes, in.ncount,
-           in.nw, n_max, equal_mass, nchunks.p, nbins.p, logb.p, bin0.p, rmean.p,
-           nwords.p);
-    scan_exclusive_u32(A, scan, nchunks.p, chunk_off.p, n_rep, chunk_off.p + n_rep, s);
-    scan_exclusive_u32(A, scan, nbins.p, hoff.p, n_rep, tot32.p, s);
-    scan_exclusive_u64(A, scan, nwords.p, woff.p, n_rep, tot64.p, s);
+           in.nw, n_max, equal_mass, nchunks, nbins, logb, bin0, rmean,
+           nwords);
+    scan_exclusive_u32(A, scan, nchunks, chunk_off, n_rep, chunk_off + n_rep, s);
+    scan_exclusive_u32(A, scan, nbins, hoff, n_rep, tot32, s);
+    scan_exclusive_u64(A, scan, nwords, woff, n_rep, tot64, s);
     uint32_t *h32 = static_cast<uint32_t *>(hs.get(16));
     uint64_t *h64 = reinterpret_cast<uint64_t *>(h32 + 2);
-    GB_CUDA(cudaMemcpyAsync(h32, chunk_off.p + n_rep, 4, cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(h32 + 1, tot32.p, 4, cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(h64, tot64.p, 8, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(h32, chunk_off + n_rep, 4, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(h32 + 1, tot32, 4, cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(h64, tot64, 8, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
     const uint32_t n_chunks = h32[0], n_bins = h32[1];
     const uint64_t total_words = *h64;
 
-    RepInfo R{rep_nodes, chunk_off.p, hoff.p, logb.p, bin0.p, rmean.p, woff.p};
-    Scratch<Chunk> chunks(A, n_chunks, s);
+    RepInfo R{rep_nodes, chunk_off, hoff, logb, bin0, rmean, woff};
+    Chunk *chunks;
+    uint32_t *hist, *tb, *cursor, *kept, *bitmap, *chunk_sel, *chunk_pos;
+    uint64_t *ccap, *cand_off;
+    const Scratch<unsigned char> work =
+        carve(A, s, {part(chunks, n_chunks), part(hist, n_bins), part(tb, n_rep), part(cursor, 2 * (size_t)n_rep),
+                     part(ccap, n_rep), part(cand_off, n_rep), part(bitmap, total_words), part(chunk_sel, n_chunks),
+                     part(chunk_pos, n_chunks)});
+    kept = cursor + n_rep;
     launch(GBLOD_K_BUILD_OTHER, k_sel_chunks, dim3((n_chunks + 255) / 256), dim3(256), 0, s, n_chunks, n_rep, in, R,
-           chunks.p);
+           chunks);
     uint16_t *codes = (size_t)n_chunks * CH * sizeof(uint16_t) <= spare_bytes ? static_cast<uint16_t *>(spare) : nullptr;
-    Scratch<uint32_t> hist(A, n_bins, s), tb(A, n_rep, s), counters(A, 2 * (size_t)n_rep, s);
-    Scratch<uint64_t> ccap(A, n_rep, s), cand_off(A, n_rep, s);
-    Scratch<uint32_t> bitmap(A, total_words, s);
-    uint32_t *cursor = counters.p, *kept = counters.p + n_rep;
-    GB_CUDA(cudaMemsetAsync(hist.p, 0, (size_t)n_bins * 4, s));
-    GB_CUDA(cudaMemsetAsync(counters.p, 0, 2 * (size_t)n_rep * 4, s));
-    launch(GBLOD_K_SEL_HIST, k_sel_hist, dim3(n_chunks), dim3(ST), 0, s, in, R, (const Chunk *)chunks.p, seed,
-           equal_mass, hist.p, codes);
-    launch(GBLOD_K_BUILD_OTHER, k_sel_find, dim3(n_rep), dim3(ST), 0, s, R, n_max, equal_mass, (const uint32_t *)hist.p,
-           tb.p, ccap.p);
-    scan_exclusive_u64(A, scan, ccap.p, cand_off.p, n_rep, tot64.p, s);
-    const uint64_t cand_total = readback(tot64.p, s, hs);
+    GB_CUDA(cudaMemsetAsync(hist, 0, (size_t)n_bins * 4, s));
+    GB_CUDA(cudaMemsetAsync(cursor, 0, 2 * (size_t)n_rep * 4, s));
+    launch(GBLOD_K_SEL_HIST, k_sel_hist, dim3(n_chunks), dim3(ST), 0, s, in, R, (const Chunk *)chunks, seed,
+           equal_mass, hist, codes);
+    launch(GBLOD_K_BUILD_OTHER, k_sel_find, dim3(n_rep), dim3(ST), 0, s, R, n_max, equal_mass, (const uint32_t *)hist,
+           tb, ccap);
+    scan_exclusive_u64(A, scan, ccap, cand_off, n_rep, tot64, s);
+    const uint64_t cand_total = readback(tot64, s, hs);
     Scratch<Cand> cand(A, 2 * (size_t)cand_total + 2, s);
-    Scratch<uint32_t> chunk_sel(A, n_chunks, s), chunk_pos(A, n_chunks, s);
     launch(GBLOD_K_SEL_MARK, codes ? k_sel_mark<true> : k_sel_mark<false>, dim3(n_chunks), dim3(ST), 0, s, in,
-           (const Chunk *)chunks.p, seed, equal_mass, (const uint16_t *)codes, (const uint32_t *)tb.p, (const uint64_t *)cand_off.p, cursor, kept,
-           chunk_sel.p, cand.p, bitmap.p);
+           (const Chunk *)chunks, seed, equal_mass, (const uint16_t *)codes, (const uint32_t *)tb, (const uint64_t *)cand_off, cursor, kept,
+           chunk_sel, cand.p, bitmap);
     launch(GBLOD_K_BUILD_OTHER, k_sel_resolve, dim3(n_rep), dim3(ST), 0, s, R, n_max, equal_mass, (const uint32_t *)kept,
-           (const uint32_t *)cursor, (const uint64_t *)cand_off.p, cand_total, cand.p, bitmap.p, chunk_sel.p);
-    scan_exclusive_u32(A, scan, chunk_sel.p, chunk_pos.p, n_chunks, tot32.p, s);
-    launch(GBLOD_K_SEL_WRITE, k_sel_write, dim3(n_chunks), dim3(ST), 0, s, in, (const Chunk *)chunks.p, (const uint32_t *)bitmap.p,
-           (const uint32_t *)chunk_pos.p);
-    const uint32_t n_kept = readback(tot32.p, s, hs); // modulo 2^32, like the positions it sums
+           (const uint32_t *)cursor, (const uint64_t *)cand_off, cand_total, cand.p, bitmap, chunk_sel);
+    scan_exclusive_u32(A, scan, chunk_sel, chunk_pos, n_chunks, tot32, s);
+    launch(GBLOD_K_SEL_WRITE, k_sel_write, dim3(n_chunks), dim3(ST), 0, s, in, (const Chunk *)chunks, (const uint32_t *)bitmap,
+           (const uint32_t *)chunk_pos);
+    const uint32_t n_kept = readback(tot32, s, hs); // modulo 2^32, like the positions it sums
     if (n_kept != (uint32_t)((uint64_t)n_rep * n_max))
         fail(GBLOD_ERR_CUDA, "subselection kept " + std::to_string(n_kept) + " points, expected " +
                                  std::to_string((uint64_t)n_rep * n_max));
