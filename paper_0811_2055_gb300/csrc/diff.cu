@@ -18,7 +18,7 @@ namespace {
 
 constexpr int DRT = 256;          // block size
 constexpr int DTW = 64, DTH = 16; // forward tile: eight strips of 8 x 16 pixels, a warp each
-constexpr uint32_t DITEM = 1024;  // records per work item
+constexpr uint32_t DITEM = 1024;  // records per work item, at most
 constexpr float E45 = 0.011108996538242306f;   // exp(-4.5)
 constexpr float INV_2PI_C = 0.16951204f;       // 1 / (2 pi (1 - 5.5 exp(-4.5)))
 constexpr float LOG2E = 1.4426950408889634f;
@@ -117,9 +117,9 @@ __global__ void __launch_bounds__(DRT) k_dbin(const DCam *__restrict__ cams, int
     }
 }
 
-// One block: work items {tile, first record, end, 0} of at most DITEM records of every (view, tile), from
+// One block: work items {tile, first record, end, 0} of at most per_item records of every (view, tile), from
 // the scanned histogram (total = its end); *nitems gets their number, *next the unit counter's start.
-__global__ void __launch_bounds__(1024) k_ditems(uint32_t nt, uint32_t parts, const uint32_t *__restrict__ off,
+__global__ void __launch_bounds__(1024) k_ditems(uint32_t nt, uint32_t parts, uint32_t per_item, const uint32_t *__restrict__ off,
                                                  const uint32_t *total, uint4 *__restrict__ items, uint32_t *nitems,
                                                  uint32_t *next)
 {
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(1024) k_ditems(uint32_t nt, uint32_t parts, co
             a = off[(size_t)t * parts];
             b = t + 1 < nt ? off[(size_t)(t + 1) * parts] : *total;
         }
-        const uint32_t k = (b - a + DITEM - 1) / DITEM;
+        const uint32_t k = (b - a + per_item - 1) / per_item;
         uint32_t incl = k;
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(1024) k_ditems(uint32_t nt, uint32_t parts, co
             all += wsum[q];
         }
         uint32_t at = run + before + incl - k;
-        for (uint32_t s = a; s < b; s += DITEM, ++at) items[at] = make_uint4(t, s, min(b, s + DITEM), 0u);
+        for (uint32_t s = a; s < b; s += per_item, ++at) items[at] = make_uint4(t, s, min(b, s + per_item), 0u);
         run += all;
         __syncthreads();
     }
@@ -595,8 +595,12 @@ void diff_forward(gblod_renderer *r, const float *xyz, const float *w, const flo
         GB_CUDA(cudaStreamSynchronize(s));
         if (*total == 0) continue;
         r->d_rec.ensure(A, *total, s);
-        r->d_items.ensure(A, (size_t)nt + *total / DITEM, s);
-        launch(GBLOD_K_RENDER_OTHER, k_ditems, dim3(1), dim3(1024), 0, s, nt, parts, (const uint32_t *)r->d_off.p,
+        // DITEM records an item, fewer if that gives less than four units a warp (16,000 points, 8 views of 128 x 128:
+        // 66 us with 1024, 31 with 128; a million points, many items anyway: 1.62 ms, 2.12 with 128)
+        const uint32_t even = (*total / ((uint32_t)persistent_blocks(4) * 4u) + 31u) / 32u * 32u;
+        const uint32_t per_item = std::max(128u, std::min(DITEM, even));
+        r->d_items.ensure(A, (size_t)nt + *total / per_item, s);
+        launch(GBLOD_K_RENDER_OTHER, k_ditems, dim3(1), dim3(1024), 0, s, nt, parts, per_item, (const uint32_t *)r->d_off.p,
                (const uint32_t *)(r->d_off.p + nh), r->d_items.p, r->d_cnt.p, r->d_cnt.p + 1);
         if (shared) {
             launch(GBLOD_K_RENDER_OTHER, k_dbin<true, true>, grid, dim3(DRT), ntiles * 4, s, dc, v0, xyz, w, logh,
@@ -621,9 +625,9 @@ void diff_backward(gblod_renderer *r, const float *xyz, const float *w, const fl
     uint32_t *nbig = r->d_cnt.p + 2;
     GB_CUDA(cudaMemsetAsync(nbig, 0, 4, s));
     // with few points the views are split over blocks: a warp's four points times its views are walked
-    // one after another, so about 128 warps per SM are wanted (16,000 points x 8 views: 154 us unsplit, 82 us split)
+    // one after another, so about 256 warps per SM are wanted (16,000 points x 8 views: 154 us unsplit, 75 us split; 128 warps 82)
     const unsigned gx = (unsigned)((n + DRT / 8 - 1) / (DRT / 8));
-    const int split = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)nv, (uint64_t)persistent_blocks(16) / gx));
+    const int split = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)nv, (uint64_t)persistent_blocks(32) / gx));
     const int views_per = (nv + split - 1) / split;
     const dim3 grid(gx, (unsigned)((nv + views_per - 1) / views_per));
     if (grid.y > 1) {

@@ -1093,10 +1093,22 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
     }
 }
 
-// counts, offsets and work items (of per_item records) of the tiles' runs from the scanned (tile, CTA) histogram
-// of CTA groups of G
-__global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, uint32_t per_item, const uint32_t *__restrict__ off,
-                                  const uint32_t *total, uint32_t *tile_cnt, uint32_t *tile_off, uint32_t *item_cnt,
+// Records per work item of `total` records: ITEM, less if that makes fewer than `want` items, so that a small
+// frame's work spreads over the grid and ends together (a million particles, 640 x 360: 275 -> 125 us; 262k, 512 x
+// 512: 46 -> 13 us, with 256 at least 25).
+constexpr uint32_t ITEM_MIN = 64;
+__host__ __device__ __forceinline__ uint32_t item_size(uint32_t total, uint32_t want)
+{
+    const uint32_t per = (total / want + 31u) / 32u * 32u;
+    return per < ITEM_MIN ? ITEM_MIN : (per < ITEM ? per : ITEM);
+}
+// wanted items: four units a warp of the splat kernel's grid (a unit is a strip of up to eight)
+uint32_t items_wanted() { return (uint32_t)persistent_blocks(4) * 4u; }
+
+// counts, offsets and work items (of per_item records; 0: by item_size) of the tiles' runs from the scanned
+// (tile, CTA) histogram of CTA groups of G
+__global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, uint32_t per_item, uint32_t want,
+                                  const uint32_t *__restrict__ off, const uint32_t *total, uint32_t *tile_cnt, uint32_t *tile_off, uint32_t *item_cnt,
                                   unsigned long long *frame_tiles, uint32_t in_frame)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1105,6 +1117,7 @@ __global__ void k_tiles_from_hist(uint32_t ntiles, uint32_t G, uint32_t per_item
     const uint32_t a = off[(size_t)t * G], b = t + 1 < ntiles ? off[(size_t)(t + 1) * G] : *total;
     tile_off[t] = a;
     tile_cnt[t] = b - a;
+    if (!per_item) per_item = item_size(*total, want);
     item_cnt[t] = (b - a + per_item - 1) / per_item;
 }
 
@@ -1306,7 +1319,8 @@ __global__ void k_tile_items(uint32_t ntiles, const uint32_t *tile_cnt, uint32_t
 
 // also clears the unit counter of the splat launch that follows and the frame's maximum (may be null)
 __global__ void k_fill_items(uint32_t nruns, uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
-                             const uint32_t *item_off, uint4 *items, unsigned *next, unsigned long long *maxv)
+                             const uint32_t *item_off, uint32_t per_item, uint4 *items, unsigned *next,
+                             unsigned long long *maxv)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) *next = 0u;
@@ -1314,7 +1328,7 @@ __global__ void k_fill_items(uint32_t nruns, uint32_t ntiles, const uint32_t *ti
     if (t >= nruns) return;
     const uint32_t c = tile_cnt[t], o = tile_off[t];
     uint32_t k = item_off[t];
-    for (uint32_t s = 0; s < c; s += ITEM, ++k) items[k] = make_uint4(t % ntiles, o + s, o + min(c, s + ITEM), 0u);
+    for (uint32_t s = 0; s < c; s += per_item, ++k) items[k] = make_uint4(t % ntiles, o + s, o + min(c, s + per_item), 0u);
 }
 
 // ------------------------------------------------------------------ R3
@@ -1745,6 +1759,7 @@ constexpr unsigned long long RECORD_BUDGET_MAX = 1ull << 31;     // offsets stay
 
 struct PassCounts {
     unsigned long long pairs, points; // records of the pass (both streams when partitioned), points
+    unsigned long long binned;        // records of the tile stream alone
     uint32_t items, small_items;      // splat work items, small-box work items (partitioned only)
 };
 
@@ -1810,7 +1825,7 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
                bn.chunk, gs, r->cta_hist.p, r->status, stats);
         scan_exclusive_u32(A, r->scan, r->cta_hist.p, r->cta_off.p, nall, &stats->records, s);
         const dim3 tg((nruns + 255) / 256);
-        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, ITEM,
+        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, 0u, items_wanted(),
                (const uint32_t *)r->cta_off.p, SMALL ? (const uint32_t *)(r->cta_off.p + nh) : &stats->records,
                r->tile_cnt.p, r->tile_off.p, r->item_cnt.p, &stats->tiles, ntiles);
         if (SMALL) {
@@ -1818,7 +1833,7 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
             r->tile_off_s.ensure(A, nruns, s);
             r->item_cnt_s.ensure(A, nruns, s);
             r->item_off_s.ensure(A, nruns, s);
-            launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, ITEM_SMALL,
+            launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, nruns, gs, ITEM_SMALL, 0u,
                    (const uint32_t *)(r->cta_off.p + nh), &stats->records, r->tile_cnt_s.p, r->tile_off_s.p,
                    r->item_cnt_s.p, (unsigned long long *)nullptr, 0u);
             scan_exclusive_u32(A, r->scan, r->item_cnt_s.p, r->item_off_s.p, nruns, &stats->small_items, s);
@@ -1837,7 +1852,7 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
     GB_CUDA(cudaMemcpyAsync(h, stats, sizeof(FrameStatsDev), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
     const bool streams = bn.part && SMALL;
-    return PassCounts{streams ? (unsigned long long)h->records : h->pairs, h->points, h->items,
+    return PassCounts{streams ? (unsigned long long)h->records : h->pairs, h->points, h->pairs, h->items,
                       streams ? h->small_items : 0u};
 }
 
@@ -1884,7 +1899,7 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
     }
     launch(GBLOD_K_RENDER_OTHER, k_fill_items, tg, dim3(256), 0, s, nruns, ntiles,
            (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p, (const uint32_t *)r->item_off.p,
-           r->items.p, r->status + 1, r->maxv.p);
+           bn.part ? item_size((uint32_t)pc.binned, items_wanted()) : ITEM, r->items.p, r->status + 1, r->maxv.p);
     launch_splat(r->count_updates, r->records.p, r->items.p, pc.items, r->status + 1, P, img, r->stats, s);
 }
 
@@ -2287,8 +2302,9 @@ __global__ void __launch_bounds__(RT, 4) k_bproject(SrcBatch src, uint32_t *__re
 __global__ void k_bfill_items(uint32_t ntiles, const ViewDev *__restrict__ views, int nviews,
                               const uint32_t *tile_cnt, const uint32_t *tile_off, const uint32_t *item_off,
                               uint4 *items, uint32_t items_cap, unsigned long long rec_cap,
-                              const FrameStatsDev *stats, unsigned *status)
+                              const FrameStatsDev *stats, unsigned *status, uint32_t want)
 {
+    const uint32_t per_item = want ? item_size((uint32_t)stats->pairs, want) : ITEM;
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0 && (stats->pairs > rec_cap || item_off[ntiles] > items_cap)) atomicOr(status, ST_CAPACITY);
     if (t >= ntiles) return;
@@ -2299,8 +2315,8 @@ __global__ void k_bfill_items(uint32_t ntiles, const ViewDev *__restrict__ views
     }
     const uint32_t c = tile_cnt[t], o = tile_off[t], local = t - views[lo].tile_base;
     uint32_t k = item_off[t];
-    for (uint32_t s = 0; s < c && k < items_cap; s += ITEM, ++k) {
-        const uint32_t b = o + s, e = o + min(c, s + ITEM);
+    for (uint32_t s = 0; s < c && k < items_cap; s += per_item, ++k) {
+        const uint32_t b = o + s, e = o + min(c, s + per_item);
         // records beyond the capacity were never written: clip (the batch is flagged)
         const uint32_t bc = (uint32_t)min((unsigned long long)b, rec_cap), ec = (uint32_t)min((unsigned long long)e, rec_cap);
         items[k] = make_uint4(local, bc, ec, (uint32_t)lo);
@@ -2353,6 +2369,9 @@ int batch_part(uint32_t ntiles)
     if (smem > PART_MAX_SMEM) return 0;
     return (int)std::min<size_t>(4, std::max<size_t>(1, 216 * 1024 / (smem + 6 * 1024)));
 }
+
+// work items of a batch, at most (item_size makes no more than are wanted, or than ITEM records each give)
+uint64_t batch_items(uint32_t ntiles, uint64_t records) { return ntiles + std::max<uint64_t>(records / ITEM, items_wanted()) + 1; }
 
 // histogram entries of a batch of up to ntiles tiles
 size_t batch_hist(uint32_t ntiles)
@@ -2460,7 +2479,7 @@ void reserve_batch(gblod_renderer *r, const gblod_view *views, int n, const gblo
     r->item_cnt.ensure(A, b.ntiles, s);
     r->item_off.ensure(A, b.ntiles + 1, s);
     r->records.ensure(A, rec_cap, s);
-    r->items.ensure(A, b.ntiles + rec_cap / ITEM + 1, s);
+    r->items.ensure(A, batch_items(b.ntiles, rec_cap), s);
     r->maxv.ensure(A, n, s);
     r->b_hist.ensure(A, batch_hist(b.ntiles) + 1, s);
     // scan temp for the largest scans of this batch
@@ -2478,7 +2497,7 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     BatchPlan b = plan_batch(views, n, rp);
     const Allocator &A = r->A;
     // scratch must have been reserved (no allocation here, so the call can be graph-captured)
-    const uint64_t items_cap = b.ntiles + r->b_rec_cap / ITEM + 1;
+    const uint64_t items_cap = batch_items(b.ntiles, r->b_rec_cap);
     if (r->b_views.cap < (size_t)n * sizeof(ViewDev) || r->b_frontA.cap < b.nodes + 1 || r->b_sel.cap < b.nodes + 1 ||
         r->b_pfx.cap < b.nodes + 2 || r->lvl_cnt.cap < b.max_levels + 3 || r->tile_cnt.cap < b.ntiles ||
         r->tile_off.cap < b.ntiles + 1 || r->item_off.cap < b.ntiles + 1 || r->records.cap < r->b_rec_cap ||
@@ -2539,7 +2558,7 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
         launch(GBLOD_K_PROJECT_COUNT, k_bproject<false, true>, dim3(GP), dim3(RT), smem, s, src, r->b_hist.p, b.ntiles, kernel,
                (uint4 *)nullptr, 0ull, r->status, r->stats, 0);
         scan_exclusive_u32(A, r->scan, r->b_hist.p, r->b_hist.p, nh, r->b_hist.p + nh, s);
-        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, b.ntiles, (uint32_t)GP, ITEM,
+        launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, b.ntiles, (uint32_t)GP, 0u, items_wanted(),
                (const uint32_t *)r->b_hist.p, (const uint32_t *)(r->b_hist.p + nh), r->tile_cnt.p, r->tile_off.p,
                r->item_cnt.p, (unsigned long long *)nullptr, 0u);
         launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, true>, dim3(GP), dim3(RT), smem, s, src, r->b_hist.p, b.ntiles, kernel,
@@ -2559,7 +2578,7 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     launch(GBLOD_K_RENDER_OTHER, k_bfill_items, dim3((b.ntiles + 255) / 256), dim3(256), 0, s, b.ntiles,
            (const ViewDev *)dv, n, (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p,
            (const uint32_t *)r->item_off.p, r->items.p, (uint32_t)items_cap, (unsigned long long)r->b_rec_cap,
-           (const FrameStatsDev *)r->stats, r->status);
+           (const FrameStatsDev *)r->stats, r->status, per_sm ? items_wanted() : 0u);
     // R3: persistent over the items of all views
     launch(GBLOD_K_SPLAT, (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? k_bsplat<true> : k_bsplat<false>, dim3(G), dim3(RT),
            sizeof(SplatSmem), s, (const uint4 *)r->records.p, (const uint4 *)r->items.p,
@@ -2852,7 +2871,7 @@ gblod_status render_brute_noalloc(const float *xyz, const float *mass, const flo
            tile_cur, records, img,
            (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? stats : (FrameStatsDev *)nullptr);
     launch(GBLOD_K_RENDER_OTHER, k_fill_items, dim3((nt + 255) / 256), dim3(256), 0, s, nt, nt,
-           (const uint32_t *)tile_cnt, (const uint32_t *)tile_off, (const uint32_t *)item_off, items, status + 1,
+           (const uint32_t *)tile_cnt, (const uint32_t *)tile_off, (const uint32_t *)item_off, ITEM, items, status + 1,
            (unsigned long long *)nullptr);
     launch_splat((rp.flags & GBLOD_RENDER_COUNT_UPDATES) != 0, records, items, nitems, status + 1, P, img, stats, s);
     if (image) {

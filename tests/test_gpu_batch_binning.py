@@ -113,3 +113,30 @@ def test_tone_map_edges(n, lo, hi):
     img = r.tonemap(d, G.make_params(**{**kw, "tone_auto": lo is None}))
     assert u8_close(img.cpu().numpy(), O.tonemap(acc.reshape(7 if n > 16384 else 1, -1), O.rparams(**kw))) <= 1
     r.close()
+
+
+@pytest.mark.parametrize("n", [40, 4000, 60_000])
+@pytest.mark.parametrize("size", [(40, 24), (130, 67), (511, 300)])
+def test_small_frames_in_small_items(n, size):
+    """Records few and many against the work items wanted (below, between and above the bounds of an item's
+    size), in one tile and in many, alone and in a batch, against the oracle bit for bit."""
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    p = synth.tiny(n, seed=n)
+    h = p.h * 6.0
+    ot = O.build_tree(p.xyz, p.mass, h, seed=1, n_max=900)
+    t = G.build_lod(*to_dev(p.xyz, p.mass, h), n_max=900, seed=1)
+    views = _views(t, _cams(3, *size))
+    par = G.make_params(lambda_px=5.0)
+    r = G.Renderer()
+    r.reserve_batch(views, par, record_capacity=1 << 24)
+    r.render_batch(views, par)
+    torch.cuda.synchronize()
+    assert r.status() == G.OK
+    for _, cam, img, acc in views:
+        want, st, nd, _ = O.render_lod(ot, cam, O.rparams(lambda_px=5.0))
+        assert st == 0 and np.array_equal(G.u64(acc), want)
+        img1, acc1 = r.render(t, cam, par)
+        assert torch.equal(acc1, acc) and torch.equal(img1, img)
+    t.free()
+    r.close()
