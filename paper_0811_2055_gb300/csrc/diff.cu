@@ -537,20 +537,52 @@ DCam make_dcam(const gblod_camera &c, const gblod_render_params &rp)
     return d;
 }
 
-// the views' constants, on the device
-const DCam *upload_cams(gblod_renderer *r, uint64_t n, const gblod_camera *cams, int nv, const gblod_render_params &rp,
-                        cudaStream_t s)
+// One launch at the head of a pass: the views' constants, from the kernel's parameters (a copy from pageable
+// memory costs the host 11 to 18 us, a launch 5), and everything the pass adds to, zeroed.
+constexpr int CAMS_PER_LAUNCH = 32;
+struct DSetup {
+    int first, n;
+    float *zero[3];
+    unsigned long long count[3];
+    uint32_t *counter; // may be null
+    DCam cam[CAMS_PER_LAUNCH];
+};
+static_assert(sizeof(DSetup) <= 4096, "kernel parameters");
+
+__global__ void k_dsetup(const __grid_constant__ DSetup S, DCam *__restrict__ cams)
+{
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < (size_t)S.n) cams[S.first + t] = S.cam[t];
+    if (t == 0 && S.counter) *S.counter = 0u;
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        for (size_t i = t; i < S.count[q]; i += (size_t)gridDim.x * blockDim.x) S.zero[q][i] = 0.0f;
+}
+
+void check_views(uint64_t n, const gblod_camera *cams, int nv)
 {
     if (n >= 0xFFFFFFFFull) fail(GBLOD_ERR_INVALID_ARG, "too many points");
     for (int v = 0; v < nv; ++v)
         if (cams[v].width != cams[0].width || cams[v].height != cams[0].height)
             fail(GBLOD_ERR_INVALID_ARG, "all views need one resolution");
-    std::vector<DCam> hc(nv);
-    for (int v = 0; v < nv; ++v) hc[v] = make_dcam(cams[v], rp);
+}
+
+// S: what to zero
+const DCam *setup(gblod_renderer *r, const gblod_camera *cams, int nv, const gblod_render_params &rp, DSetup S,
+                  cudaStream_t s)
+{
     r->d_cams.ensure(r->A, (size_t)nv * sizeof(DCam), s);
-    GB_CUDA(cudaMemcpyAsync(r->d_cams.p, hc.data(), (size_t)nv * sizeof(DCam), cudaMemcpyHostToDevice, s));
-    r->d_cnt.ensure(r->A, 4, s); // counters: work items, next unit, listed large records
-    return reinterpret_cast<const DCam *>(r->d_cams.p);
+    DCam *dc = reinterpret_cast<DCam *>(r->d_cams.p);
+    for (S.first = 0; S.first < nv; S.first += CAMS_PER_LAUNCH) {
+        S.n = std::min(CAMS_PER_LAUNCH, nv - S.first);
+        for (int v = 0; v < S.n; ++v) S.cam[v] = make_dcam(cams[S.first + v], rp);
+        const unsigned long long most = std::max({S.count[0], S.count[1], S.count[2]});
+        const unsigned g = (unsigned)std::min<unsigned long long>((unsigned long long)persistent_blocks(8), most / 1024 + 1);
+        launch(GBLOD_K_RENDER_OTHER, k_dsetup, dim3(g), dim3(256), 0, s, S, dc);
+        S.counter = nullptr;
+        for (unsigned long long &c : S.count) c = 0;
+    }
+    return dc;
 }
 
 } // namespace
@@ -558,10 +590,14 @@ const DCam *upload_cams(gblod_renderer *r, uint64_t n, const gblod_camera *cams,
 void diff_forward(gblod_renderer *r, const float *xyz, const float *w, const float *logh, uint64_t n,
                   const gblod_camera *cams, int nv, const gblod_render_params &rp, float *images, cudaStream_t s)
 {
-    const DCam *dc = upload_cams(r, n, cams, nv, rp, s);
+    check_views(n, cams, nv);
     const Allocator &A = r->A;
     const DCam c0 = make_dcam(cams[0], rp);
-    GB_CUDA(cudaMemsetAsync(images, 0, (size_t)nv * c0.W * c0.H * sizeof(float), s));
+    r->d_cnt.ensure(A, 4, s); // counters: work items, next unit, listed large records
+    DSetup S{};
+    S.zero[0] = images;
+    S.count[0] = (unsigned long long)nv * c0.W * c0.H;
+    const DCam *dc = setup(r, cams, nv, rp, S, s);
     if (n == 0) return;
     const uint32_t ntiles = (uint32_t)(c0.tiles_x * c0.tiles_y);
     const bool shared = ntiles <= 12288; // 48 KB of counters
@@ -619,22 +655,27 @@ void diff_backward(gblod_renderer *r, const float *xyz, const float *w, const fl
                    const gblod_camera *cams, int nv, const gblod_render_params &rp, const float *grad_img, float *gxyz,
                    float *gw, float *glogh, cudaStream_t s)
 {
-    const DCam *dc = upload_cams(r, n, cams, nv, rp, s);
+    check_views(n, cams, nv);
     if (n == 0) return;
+    r->d_cnt.ensure(r->A, 4, s);
     r->d_big.ensure(r->A, DBIG_CAP, s);
     uint32_t *nbig = r->d_cnt.p + 2;
-    GB_CUDA(cudaMemsetAsync(nbig, 0, 4, s));
     // with few points the views are split over blocks: a warp's four points times its views are walked
     // one after another, so about 256 warps per SM are wanted (16,000 points x 8 views: 154 us unsplit, 75 us split; 128 warps 82)
     const unsigned gx = (unsigned)((n + DRT / 8 - 1) / (DRT / 8));
     const int split = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)nv, (uint64_t)persistent_blocks(32) / gx));
     const int views_per = (nv + split - 1) / split;
     const dim3 grid(gx, (unsigned)((nv + views_per - 1) / views_per));
-    if (grid.y > 1) {
-        GB_CUDA(cudaMemsetAsync(gxyz, 0, n * 3 * sizeof(float), s));
-        GB_CUDA(cudaMemsetAsync(gw, 0, n * sizeof(float), s));
-        GB_CUDA(cudaMemsetAsync(glogh, 0, n * sizeof(float), s));
+    DSetup S{};
+    S.counter = nbig;
+    if (grid.y > 1) { // blocks add up
+        float *const g[3] = {gxyz, gw, glogh};
+        for (int q = 0; q < 3; ++q) {
+            S.zero[q] = g[q];
+            S.count[q] = q ? n : 3 * n;
+        }
     }
+    const DCam *dc = setup(r, cams, nv, rp, S, s);
     launch(GBLOD_K_SPLAT, grid.y > 1 ? k_dgather<true> : k_dgather<false>, grid, dim3(DRT), 0, s, dc, nv, views_per, xyz,
            w, logh, (uint32_t)n, grad_img, gxyz, gw, glogh, r->d_big.p, nbig);
     launch(GBLOD_K_SPLAT, k_dbig, dim3((unsigned)persistent_blocks(4)), dim3(DRT), 0, s, dc, xyz, w, logh, grad_img, gxyz,
