@@ -95,7 +95,7 @@ __device__ __forceinline__ uint32_t find_slot(const uint32_t *chunk_off, uint32_
 }
 
 // What a block needs to know of its chunk, laid out once (blocks that looked it up through the node arrays,
-// four dependent loads: 150M, mark 0.93 -> 0.72 ms, write 1.52 -> 1.43)
+// four dependent loads: 150M, mark 0.93 -> 0.72 ms, write 1.52 -> 1.43; the warps' lists 1.28)
 struct __align__(16) Chunk {
     uint32_t j0, len, start, r; // first element; elements; the first one's position in the node; rep slot
     uint64_t code, words;       // node code; first bitmap word
@@ -391,6 +391,7 @@ __global__ void __launch_bounds__(ST) k_sel_write(SelectIn in, const Chunk *chun
                                                   const uint32_t *chunk_pos)
 {
     __shared__ uint32_t woff[ST / 32];
+    __shared__ uint16_t kept[ST / 32][ROUNDS * 32];
     const Chunk C = load_chunk(chunks);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nw = (C.len + 31) / 32;
@@ -405,24 +406,29 @@ __global__ void __launch_bounds__(ST) k_sel_write(SelectIn in, const Chunk *chun
     if (!mine) return;
     const uint64_t pf = in.npfirst[C.node];
     const float wr = in.nw[C.node], sr = in.ns[C.node];
+    // the warp's kept elements, in order, so that every lane of the copy has one and its stores are contiguous
     const uint32_t lt = gbd::lanemask_lt();
-    float hm = 0.0f;
-    const uint32_t j0 = C.j0 + w0 * 32 + lane;
-#pragma unroll 4
+    uint16_t *list = kept[warp];
+    uint32_t n = 0;
+#pragma unroll
     for (int q = 0; q < ROUNDS; ++q) {
         const uint32_t W = __shfl_sync(0xffffffffu, mw, q);
-        const uint32_t rank = base + __popc(W & lt);
-        if (((W >> lane) & 1u) && rank < in.n_max) {
-            const uint64_t idx = pf + rank;
-            const uint32_t j = j0 + q * 32;
-            const float4 p = __ldg(&in.s4[j]);
-            const float h = __fmul_rn(p.w, sr);
-            in.pts4[idx] = make_float4(p.x, p.y, p.z, wr);
-            in.hs[idx] = h;
-            in.pt_src[idx] = j;
-            hm = h > hm ? h : hm;
-        }
-        base += __popc(W);
+        if ((W >> lane) & 1u) list[n + __popc(W & lt)] = (uint16_t)(q * 32 + lane);
+        n += __popc(W);
+    }
+    __syncwarp();
+    float hm = 0.0f;
+    const uint32_t j0 = C.j0 + w0 * 32, end = base < in.n_max ? min(mine, in.n_max - base) : 0u;
+#pragma unroll 4
+    for (uint32_t k = lane; k < end; k += 32) {
+        const uint64_t idx = pf + base + k;
+        const uint32_t j = j0 + list[k];
+        const float4 p = __ldg(&in.s4[j]);
+        const float h = __fmul_rn(p.w, sr);
+        in.pts4[idx] = make_float4(p.x, p.y, p.z, wr);
+        in.hs[idx] = h;
+        in.pt_src[idx] = j;
+        hm = h > hm ? h : hm;
     }
     for (int d = 16; d > 0; d >>= 1) {
         const float o = __shfl_xor_sync(0xffffffffu, hm, d);
