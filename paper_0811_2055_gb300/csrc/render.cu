@@ -284,7 +284,8 @@ __device__ __forceinline__ unsigned walk_boxes(const BoxWalk &b, uint32_t tag, T
 // The per-pixel rule over boxes of at most 8 x 8 pixels, four points at a time: a group of eight lanes
 // takes one point of the warp's (on: this lane has one), a column per lane, row by row.  A round of 32
 // (point, pixel) pairs is about 14 instructions, where walk_boxes spends some 66 more on finding each
-// pair's point and shuffling its operands; columns and rows a box does not have idle.  Distances in 32
+// pair's point and shuffling its operands; columns and rows a box does not have idle.  With LANES 4, eight
+// points of boxes of up to four columns at a time (a 512 x 512 frame's scatter 32 -> 26 us).  Distances in 32
 // bits and Wq < 2^32 (group_box decides; walk_boxes takes the rest).  K has a zero entry 1024.  at(t, x, y) gives,
 // for a box's column x from row y (t: the point's tag if TAGGED, else 0), the function (j, c) that receives every
 // nonzero contribution c < 2^32 to row y + j.  Returns this lane's pixel updates.  Every lane of the warp calls
@@ -292,14 +293,14 @@ __device__ __forceinline__ unsigned walk_boxes(const BoxWalk &b, uint32_t tag, T
 // group is one transaction of the global additions.
 __device__ __forceinline__ bool group_box(int r, float Wf) { return r <= R_NARROW && Wf < 0x1p32f; }
 
-template <bool TAGGED, class At>
+template <int LANES, bool TAGGED, class At>
 __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t S, float Wf, int x0, int x1, int y0,
                                                 int y1, const int32_t *K, At at, uint32_t tag = 0u)
 {
-    static_assert(DIRECT_BOX <= 8, "a group's lanes are the columns of a box");
+    static_assert(DIRECT_BOX <= 8 && (LANES == 4 || LANES == 8), "a group's lanes are the columns of a box");
     const uint32_t m = __ballot_sync(0xffffffffu, on);
     if (!m) return 0u;
-    const int lane = threadIdx.x & 31, col = lane & 7;
+    const int lane = threadIdx.x & 31, col = lane & (LANES - 1);
     __shared__ uint8_t nth[32][32]; // lanes that have a point, in order
     uint8_t *own = nth[threadIdx.x >> 5];
     __syncwarp();
@@ -309,8 +310,8 @@ __device__ __forceinline__ unsigned group_boxes(bool on, int U, int V, uint32_t 
     const uint32_t ext = (uint32_t)(x1 - x0) | (uint32_t)(y1 - y0) << 8;
     const int n = __popc(m);
     unsigned hits = 0;
-    for (int r = 0; r < n; r += 4) {
-        const int k = r + (lane >> 3);
+    for (int r = 0; r < n; r += 32 / LANES) {
+        const int k = r + lane / LANES;
         const int src = own[min(k, n - 1)];
         const uint32_t qxy = __shfl_sync(0xffffffffu, xy, src), qext = __shfl_sync(0xffffffffu, ext, src);
         const int qU = __shfl_sync(0xffffffffu, U, src), qV = __shfl_sync(0xffffffffu, V, src);
@@ -1190,12 +1191,13 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
                 }
             }
             if (!SMALL) {
-                hits += group_boxes<false>(
-                    mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K,
-                    [&](uint32_t, int x, int y) {
-                        unsigned long long *p = img + (size_t)y * P.W + x;
-                        return [p, &P](int j, uint32_t c) { atomicAdd(&p[(size_t)j * P.W], (unsigned long long)c); };
-                    });
+                auto at = [&](uint32_t, int x, int y) {
+                    unsigned long long *p = img + (size_t)y * P.W + x;
+                    return [p, &P](int j, uint32_t c) { atomicAdd(&p[(size_t)j * P.W], (unsigned long long)c); };
+                };
+                const bool four = x1 - x0 < 4;
+                hits += group_boxes<4, false>(mine && four, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at);
+                hits += group_boxes<8, false>(mine && !four, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at);
                 hits += walk_boxes<false>(
                     direct, 0u, [&](uint32_t, uint32_t i) { return K[i]; },
                     [&](uint32_t, int x, int y, unsigned long long c) { atomicAdd(&img[(size_t)y * P.W + x], c); });
@@ -2264,7 +2266,9 @@ __global__ void __launch_bounds__(RT, 4) k_bproject(SrcBatch src, uint32_t *__re
                     unsigned long long *p = V.accum + (size_t)y * W + x;
                     return [p, W](int j, unsigned long long c) { atomicAdd(&p[(size_t)j * W], c); };
                 };
-                hits += group_boxes<true>(mine, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at, (uint32_t)v);
+                const bool four = x1 - x0 < 4;
+                hits += group_boxes<4, true>(mine && four, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at, (uint32_t)v);
+                hits += group_boxes<8, true>(mine && !four, s.U, s.V, s.S, s.Wf, x0, x1, y0, y1, K, at, (uint32_t)v);
                 hits += walk_boxes<true>(direct, (uint32_t)v, [&](uint32_t, uint32_t i) { return K[i]; },
                                          [&](uint32_t t, int x, int y, unsigned long long c) { at(t, x, y)(0, c); });
             } else if (n) {
