@@ -2502,11 +2502,14 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     const Allocator &A = r->A;
     // scratch must have been reserved (no allocation here, so the call can be graph-captured)
     const uint64_t items_cap = batch_items(b.ntiles, r->b_rec_cap);
-    if (r->b_views.cap < (size_t)n * sizeof(ViewDev) || r->b_frontA.cap < b.nodes + 1 || r->b_sel.cap < b.nodes + 1 ||
-        r->b_pfx.cap < b.nodes + 2 || r->lvl_cnt.cap < b.max_levels + 3 || r->tile_cnt.cap < b.ntiles ||
-        r->tile_off.cap < b.ntiles + 1 || r->item_off.cap < b.ntiles + 1 || r->records.cap < r->b_rec_cap ||
-        r->items.cap < items_cap || r->maxv.cap < (size_t)n || r->b_hist.cap < batch_hist(b.ntiles) + 1 ||
-        r->b_rec_cap == 0)
+    // Every buffer the call uses is looked at: frames grow some of them too (a frame in groups tile_cnt, tile_off,
+    // item_cnt and item_off, but not tile_cur), so one buffer's size says nothing of another's.
+    if (r->b_views.cap < (size_t)n * sizeof(ViewDev) || r->b_frontA.cap < b.nodes + 1 || r->b_frontB.cap < b.nodes + 1 ||
+        r->b_sel.cap < b.nodes + 1 || r->b_counts.cap < b.nodes + 1 || r->b_pfx.cap < b.nodes + 2 ||
+        r->b_base.cap < b.nodes + 1 || r->lvl_cnt.cap < b.max_levels + 3 || r->tile_cnt.cap < b.ntiles ||
+        r->tile_off.cap < b.ntiles + 1 || r->tile_cur.cap < b.ntiles || r->item_cnt.cap < b.ntiles ||
+        r->item_off.cap < b.ntiles + 1 || r->records.cap < r->b_rec_cap || r->items.cap < items_cap ||
+        r->maxv.cap < (size_t)n || r->b_hist.cap < batch_hist(b.ntiles) + 1 || r->b_rec_cap == 0)
         fail(GBLOD_ERR_INVALID_ARG, "gblod_render_batch: call gblod_renderer_reserve_batch for this batch first");
     r->last_stream = s;
     r->last_was_lod = false;

@@ -1,0 +1,53 @@
+"""What gblod_renderer_reserve_batch promises: a batch that was not reserved for is refused before anything is
+launched, whatever other calls have grown the renderer's buffers to."""
+import pytest
+import torch
+
+from paper_0811_2055_gb300 import synth
+
+from gpu_helpers import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _views(tree, n, W, H):
+    out = []
+    for k in range(n):
+        cam = synth.look_at((0.5, 0.5, -1.0 - 0.1 * k), (0.5, 0.5, 0.5), width=W, height=H)
+        out.append((tree, cam, torch.zeros((H, W), dtype=torch.uint8, device="cuda"),
+                    torch.zeros((H, W), dtype=torch.int64, device="cuda")))
+    return out
+
+
+def test_larger_batch_after_a_large_frame_is_refused():
+    """Eight 1080p views reserved, one 4K frame of 40M particles drawn (its runs of records are counted in groups),
+    then eight 4K views: 64,800 tiles go through the global counters, in scratch of 16,320 tiles."""
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    p = synth.tiny(20000, seed=3)
+    t = G.build_lod(*to_dev(p.xyz, p.mass, p.h), n_max=400, seed=2)
+    small, large = _views(t, 8, 1920, 1080), _views(t, 8, 3840, 2160)
+    par = G.make_params()
+    r = G.Renderer()
+    r.reserve_batch(small, par, record_capacity=1 << 29)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    n = 40_000_000
+    xyz = torch.rand(n, 3, generator=g, device="cuda")
+    one = torch.ones(n, device="cuda")
+    r.render_bruteforce(xyz, one, 1e-4 * one, large[0][1], par)
+    torch.cuda.synchronize()
+    launched = G.launch_count()
+    with pytest.raises(G.GblodError) as e:
+        r.render_batch(large, par)
+    assert e.value.code == G.ERR_INVALID_ARG and G.launch_count() == launched
+    r.render_batch(small, par)  # what was reserved still runs
+    torch.cuda.synchronize()
+    assert r.status() == G.OK
+    alone = G.Renderer()
+    for _, cam, img, acc in small:
+        ia, aa = alone.render(t, cam, par)
+        assert torch.equal(acc, aa) and torch.equal(img, ia)
+    alone.close()
+    r.close()
+    t.free()
