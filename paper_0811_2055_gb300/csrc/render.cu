@@ -1087,10 +1087,18 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
     if (lane == 0 && pairs) atomicAdd(&stats->pairs, pairs);
     amp.flush(stats);
     __syncthreads();
+    unsigned long long smalls = 0;
     for (uint32_t t = threadIdx.x; t < ntiles; t += NT) {
         const size_t at = hist_at(t, ntiles, blockIdx.x, gs);
         hist[at] = sh_cnt[t];
-        if (SMALL) hist[(size_t)ntiles * gridDim.x + at] = sh_cnt[ntiles + t];
+        if (SMALL) {
+            hist[(size_t)ntiles * gridDim.x + at] = sh_cnt[ntiles + t];
+            smalls += sh_cnt[ntiles + t];
+        }
+    }
+    if (SMALL) {
+        for (int d = 16; d > 0; d >>= 1) smalls += __shfl_xor_sync(0xffffffffu, smalls, d);
+        if (lane == 0 && smalls) atomicAdd(&stats->small_pairs, smalls);
     }
 }
 
@@ -1853,9 +1861,9 @@ PassCounts bin_count(gblod_renderer *r, const Src &src, const Proj &P, unsigned 
     FrameStatsDev *h = static_cast<FrameStatsDev *>(r->hs.get(sizeof(FrameStatsDev)));
     GB_CUDA(cudaMemcpyAsync(h, stats, sizeof(FrameStatsDev), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
-    const bool streams = bn.part && SMALL;
-    return PassCounts{streams ? (unsigned long long)h->records : h->pairs, h->points, h->pairs, h->items,
-                      streams ? h->small_items : 0u};
+    // the scanned offsets, and with them the item counts, are modulo 2^32: the pass is sized by the 64-bit counts, and
+    // one whose records do not fit the budget is split before anything is placed
+    return PassCounts{h->pairs + h->small_pairs, h->points, h->pairs, h->items, bn.part && SMALL ? h->small_items : 0u};
 }
 
 // R3 over `items` work items: a persistent grid, no more CTAs than the units need

@@ -6,7 +6,8 @@
 namespace gb {
 struct FrameStatsDev {
     unsigned long long nodes_selected, points, splats, pairs, tiles, amp_lo, amp_hi;
-    uint32_t items, small_items, records, pad; // of the last binning: work items, records of both streams
+    unsigned long long small_pairs;            // records of the small-box stream
+    uint32_t items, small_items, records, pad; // of the last binning: work items, records of both streams modulo 2^32
     unsigned long long pixel_updates;       // (splat, pixel) contributions of the last frame
     unsigned long long pixel_updates_total; // since the renderer was created (never reset)
 };
