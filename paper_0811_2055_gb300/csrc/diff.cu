@@ -76,12 +76,14 @@ __device__ __forceinline__ void dtiles(const DCam &c, const DProj &o, int &tx0, 
 // records {u, v, a = -log2(e) / (2 sigma^2), c = w norm / sigma^2} with shared-memory atomics.  (Counting
 // with warp-aggregated global atomics spent 260 cycles a round in __match_any_sync: 1M points x 16
 // views, count + records 4.7 ms; now 0.4 ms.)  With more tiles than a CTA's shared memory holds (SHARED
-// false) the counters are global, cnt[(view, tile)], and there is one part.
+// false) the counters are global, cnt[(view, tile)], and there is one part.  The scan is modulo 2^32; `pairs` (may
+// be null) gets the number of records in 64 bits from the counting pass.
 template <bool SCATTER, bool SHARED>
 __global__ void __launch_bounds__(DRT) k_dbin(const DCam *__restrict__ cams, int v0, const float *__restrict__ xyz,
                                               const float *__restrict__ w, const float *__restrict__ logh, uint32_t n,
                                               uint32_t per_part, uint32_t *__restrict__ hist,
-                                              const uint32_t *__restrict__ off, float4 *__restrict__ rec)
+                                              const uint32_t *__restrict__ off, float4 *__restrict__ rec,
+                                              unsigned long long *pairs)
 {
     extern __shared__ uint32_t dsh[];
     const DCam c = cams[v0 + blockIdx.y];
@@ -93,12 +95,14 @@ __global__ void __launch_bounds__(DRT) k_dbin(const DCam *__restrict__ cams, int
             dsh[t] = SCATTER ? off[(row0 + t) * parts + blockIdx.x] : 0u;
         __syncthreads();
     }
-    const uint32_t i0 = blockIdx.x * per_part, i1 = min(n, i0 + per_part); // i0 < n
+    const uint32_t i0 = blockIdx.x * per_part, i1 = min(n, i0 + per_part); // i0 < n; n is at most DPOINTS
+    unsigned long long placed = 0;
     for (uint32_t i = i0 + threadIdx.x; i < i1; i += DRT) {
         DProj o;
         if (!dproject(c, xyz, logh, i, o)) continue;
         int tx0, tx1, ty0, ty1;
         dtiles(c, o, tx0, tx1, ty0, ty1);
+        if (!SCATTER && pairs) placed += (unsigned long long)(max(tx1 - tx0 + 1, 0) * (ty1 - ty0 + 1));
         float4 r;
         if (SCATTER) {
             const float s2 = o.s * o.s;
@@ -114,6 +118,10 @@ __global__ void __launch_bounds__(DRT) k_dbin(const DCam *__restrict__ cams, int
     if (SHARED && !SCATTER) {
         __syncthreads();
         for (uint32_t t = threadIdx.x; t < ntiles; t += DRT) hist[(row0 + t) * parts + blockIdx.x] = dsh[t];
+    }
+    if (!SCATTER && pairs) {
+        for (int d = 16; d > 0; d >>= 1) placed += __shfl_xor_sync(0xffffffffu, placed, d);
+        if ((threadIdx.x & 31) == 0 && placed) atomicAdd(pairs, placed);
     }
 }
 
@@ -587,24 +595,44 @@ const DCam *setup(gblod_renderer *r, const gblod_camera *cams, int nv, const gbl
 
 } // namespace
 
-void diff_forward(gblod_renderer *r, const float *xyz, const float *w, const float *logh, uint64_t n,
+// A forward pass goes by pieces: views [v0, v0 + nv), points [lo, hi).  The records of a piece are at most
+// DRECORDS (16 GiB); a piece of more is counted, halved and counted again.  A piece has at most DPOINTS points, so
+// that their numbers and coordinate indices stay below 2^32.
+constexpr unsigned long long DRECORDS = 1ull << 30;
+constexpr uint64_t DPOINTS = 1ull << 30;
+struct DPiece {
+    int v0, nv;
+    uint64_t lo, hi;
+};
+
+void diff_forward(gblod_renderer *r, const float *xyz_all, const float *w_all, const float *logh_all, uint64_t n_all,
                   const gblod_camera *cams, int nv, const gblod_render_params &rp, float *images, cudaStream_t s)
 {
-    check_views(n, cams, nv);
+    check_views(n_all, cams, nv);
     const Allocator &A = r->A;
     const DCam c0 = make_dcam(cams[0], rp);
-    r->d_cnt.ensure(A, 4, s); // counters: work items, next unit, listed large records
+    r->d_cnt.ensure(A, 8, s); // counters: work items, next unit, listed large records, -, records (64 bits)
+    auto *d_pairs = reinterpret_cast<unsigned long long *>(r->d_cnt.p + 4);
     DSetup S{};
     S.zero[0] = images;
     S.count[0] = (unsigned long long)nv * c0.W * c0.H;
     const DCam *dc = setup(r, cams, nv, rp, S, s);
-    if (n == 0) return;
     const uint32_t ntiles = (uint32_t)(c0.tiles_x * c0.tiles_y);
     const bool shared = ntiles <= 12288; // 48 KB of counters
-    // views per chunk: about 2^26 (view, point) pairs, so records stay near a few GB, 2^24 tiles, a grid's y size
-    const int vchunk = (int)std::max<uint64_t>(1, std::min<uint64_t>({(uint64_t)nv, (1ull << 26) / n, 32768ull, (1ull << 24) / ntiles}));
-    for (int v0 = 0; v0 < nv; v0 += vchunk) {
-        const int cnv = std::min(vchunk, nv - v0);
+    std::vector<DPiece> todo;
+    for (uint64_t lo = 0; lo < n_all; lo += DPOINTS) {
+        const uint64_t hi = std::min(n_all, lo + DPOINTS);
+        // views per chunk: about 2^26 (view, point) pairs, so records stay near a few GB, 2^24 tiles, a grid's y size
+        const int vchunk = (int)std::max<uint64_t>(1, std::min<uint64_t>({(uint64_t)nv, (1ull << 26) / (hi - lo), 32768ull, (1ull << 24) / ntiles}));
+        for (int v0 = 0; v0 < nv; v0 += vchunk) todo.push_back(DPiece{v0, std::min(vchunk, nv - v0), lo, hi});
+    }
+    std::reverse(todo.begin(), todo.end()); // taken from the back
+    while (!todo.empty()) {
+        const DPiece pc = todo.back();
+        todo.pop_back();
+        const int v0 = pc.v0, cnv = pc.nv;
+        const uint64_t n = pc.hi - pc.lo;
+        const float *xyz = xyz_all + 3 * pc.lo, *w = w_all + pc.lo, *logh = logh_all + pc.lo;
         const uint32_t nt = ntiles * (uint32_t)cnv;
         // parts of the points per view: at least 512 points each, about eight CTAs per SM in all, and a
         // histogram of at most 2^22 columns
@@ -617,18 +645,32 @@ void diff_forward(gblod_renderer *r, const float *xyz, const float *w, const flo
         r->d_hist.ensure(A, nh, s);
         r->d_off.ensure(A, nh + 1, s);
         const dim3 grid(gx, (unsigned)cnv);
+        // the records are counted in 64 bits where there could be 2^32
+        const bool many = (unsigned long long)cnv * n * ntiles >> 32 != 0; // at most 2^30 pairs, 2^18 tiles each
+        unsigned long long *pairs = many ? d_pairs : nullptr;
+        if (many) GB_CUDA(cudaMemsetAsync(d_pairs, 0, sizeof(*d_pairs), s));
         if (shared) {
             launch(GBLOD_K_RENDER_OTHER, k_dbin<false, true>, grid, dim3(DRT), ntiles * 4, s, dc, v0, xyz, w, logh,
-                   (uint32_t)n, per, r->d_hist.p, (const uint32_t *)nullptr, (float4 *)nullptr);
+                   (uint32_t)n, per, r->d_hist.p, (const uint32_t *)nullptr, (float4 *)nullptr, pairs);
         } else {
             GB_CUDA(cudaMemsetAsync(r->d_hist.p, 0, nh * 4, s));
             launch(GBLOD_K_RENDER_OTHER, k_dbin<false, false>, grid, dim3(DRT), 0, s, dc, v0, xyz, w, logh,
-                   (uint32_t)n, per, r->d_hist.p, (const uint32_t *)nullptr, (float4 *)nullptr);
+                   (uint32_t)n, per, r->d_hist.p, (const uint32_t *)nullptr, (float4 *)nullptr, pairs);
         }
         scan_exclusive_u32(A, r->scan, r->d_hist.p, r->d_off.p, nh, r->d_off.p + nh, s);
-        uint32_t *total = static_cast<uint32_t *>(r->hs.get(16));
+        auto *h64 = static_cast<unsigned long long *>(r->hs.get(16));
+        uint32_t *total = reinterpret_cast<uint32_t *>(h64 + 1);
+        if (many) GB_CUDA(cudaMemcpyAsync(h64, d_pairs, sizeof(*d_pairs), cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaMemcpyAsync(total, r->d_off.p + nh, 4, cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaStreamSynchronize(s));
+        if ((many ? *h64 : *total) > DRECORDS) {
+            const int vm = cnv / 2;
+            const uint64_t mid = pc.lo + n / 2;
+            // one point of one view has at most 2^18 records
+            todo.push_back(cnv > 1 ? DPiece{v0 + vm, cnv - vm, pc.lo, pc.hi} : DPiece{v0, 1, mid, pc.hi});
+            todo.push_back(cnv > 1 ? DPiece{v0, vm, pc.lo, pc.hi} : DPiece{v0, 1, pc.lo, mid});
+            continue;
+        }
         if (*total == 0) continue;
         r->d_rec.ensure(A, *total, s);
         // DITEM records an item, fewer if that gives less than four units a warp (16,000 points, 8 views of 128 x 128:
@@ -640,10 +682,11 @@ void diff_forward(gblod_renderer *r, const float *xyz, const float *w, const flo
                (const uint32_t *)(r->d_off.p + nh), r->d_items.p, r->d_cnt.p, r->d_cnt.p + 1);
         if (shared) {
             launch(GBLOD_K_RENDER_OTHER, k_dbin<true, true>, grid, dim3(DRT), ntiles * 4, s, dc, v0, xyz, w, logh,
-                   (uint32_t)n, per, (uint32_t *)nullptr, (const uint32_t *)r->d_off.p, r->d_rec.p);
+                   (uint32_t)n, per, (uint32_t *)nullptr, (const uint32_t *)r->d_off.p, r->d_rec.p,
+                   (unsigned long long *)nullptr);
         } else { // the offsets themselves are the cursors (k_ditems has read them)
             launch(GBLOD_K_RENDER_OTHER, k_dbin<true, false>, grid, dim3(DRT), 0, s, dc, v0, xyz, w, logh,
-                   (uint32_t)n, per, r->d_off.p, (const uint32_t *)nullptr, r->d_rec.p);
+                   (uint32_t)n, per, r->d_off.p, (const uint32_t *)nullptr, r->d_rec.p, (unsigned long long *)nullptr);
         }
         launch(GBLOD_K_SPLAT, k_dforward, dim3((unsigned)persistent_blocks(4)), dim3(DRT), 0, s, dc, v0,
                (const float4 *)r->d_rec.p, (const uint4 *)r->d_items.p, (const uint32_t *)r->d_cnt.p, r->d_cnt.p + 1,
@@ -657,7 +700,7 @@ void diff_backward(gblod_renderer *r, const float *xyz, const float *w, const fl
 {
     check_views(n, cams, nv);
     if (n == 0) return;
-    r->d_cnt.ensure(r->A, 4, s);
+    r->d_cnt.ensure(r->A, 8, s);
     r->d_big.ensure(r->A, DBIG_CAP, s);
     uint32_t *nbig = r->d_cnt.p + 2;
     // with few points the views are split over blocks: a warp's four points times its views are walked
