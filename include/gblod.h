@@ -324,6 +324,8 @@ gblod_status gblod_renderer_reserve_batch(gblod_renderer *r, const gblod_view *v
 
 /* Renders every view (R1-R4).  Enqueues work on `stream` and returns without waiting: no host
  * synchronisation and no allocation happen inside, so the call can be recorded into a CUDA graph.
+ * Such a graph stays valid until the renderer is reserved for again, autotuned or destroyed, or draws a
+ * frame that takes more (tile, splat) records at a time than record_capacity: those may move the scratch.
  * Requires a prior gblod_renderer_reserve_batch covering this batch (GBLOD_ERR_INVALID_ARG
  * otherwise).  A batch whose (tile, splat) records exceed the reserved capacity sets the sticky
  * capacity status (gblod_renderer_status returns GBLOD_ERR_CAPACITY) and its images are invalid.

@@ -2484,21 +2484,21 @@ void reserve_batch(gblod_renderer *r, const gblod_view *views, int n, const gblo
     r->b_counts.ensure(A, b.nodes + 1, s);
     r->b_pfx.ensure(A, b.nodes + 2, s);
     r->b_base.ensure(A, b.nodes + 1, s);
-    r->lvl_cnt.ensure(A, b.max_levels + 3, s);
-    r->tile_cnt.ensure(A, b.ntiles, s);
-    r->tile_off.ensure(A, b.ntiles + 1, s);
-    r->tile_cur.ensure(A, b.ntiles, s);
-    r->item_cnt.ensure(A, b.ntiles, s);
-    r->item_off.ensure(A, b.ntiles + 1, s);
+    r->b_lvl_cnt.ensure(A, b.max_levels + 3, s);
+    r->b_tile_cnt.ensure(A, b.ntiles, s);
+    r->b_tile_off.ensure(A, b.ntiles + 1, s);
+    r->b_tile_cur.ensure(A, b.ntiles, s);
+    r->b_item_cnt.ensure(A, b.ntiles, s);
+    r->b_item_off.ensure(A, b.ntiles + 1, s);
     r->records.ensure(A, rec_cap, s);
-    r->items.ensure(A, batch_items(b.ntiles, rec_cap), s);
+    r->b_items.ensure(A, batch_items(b.ntiles, rec_cap), s);
     r->maxv.ensure(A, n, s);
     r->b_hist.ensure(A, batch_hist(b.ntiles) + 1, s);
     // scan temp for the largest scans of this batch
-    scan_exclusive_u64(A, r->scan, reinterpret_cast<const uint64_t *>(r->b_counts.p),
+    scan_exclusive_u64(A, r->b_scan, reinterpret_cast<const uint64_t *>(r->b_counts.p),
                        reinterpret_cast<uint64_t *>(r->b_pfx.p), b.nodes + 1, nullptr, s);
-    scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, b.ntiles, nullptr, s);
-    scan_exclusive_u32(A, r->scan, r->b_hist.p, r->b_hist.p, batch_hist(b.ntiles), nullptr, s);
+    scan_exclusive_u32(A, r->b_scan, r->b_tile_cnt.p, r->b_tile_off.p, b.ntiles, nullptr, s);
+    scan_exclusive_u32(A, r->b_scan, r->b_hist.p, r->b_hist.p, batch_hist(b.ntiles), nullptr, s);
     r->b_rec_cap = rec_cap;
     GB_CUDA(cudaStreamSynchronize(s));
 }
@@ -2510,13 +2510,12 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     const Allocator &A = r->A;
     // scratch must have been reserved (no allocation here, so the call can be graph-captured)
     const uint64_t items_cap = batch_items(b.ntiles, r->b_rec_cap);
-    // Every buffer the call uses is looked at: frames grow some of them too (a frame in groups tile_cnt, tile_off,
-    // item_cnt and item_off, but not tile_cur), so one buffer's size says nothing of another's.
+    // every buffer the call uses is looked at: one buffer's size says nothing of another's
     if (r->b_views.cap < (size_t)n * sizeof(ViewDev) || r->b_frontA.cap < b.nodes + 1 || r->b_frontB.cap < b.nodes + 1 ||
         r->b_sel.cap < b.nodes + 1 || r->b_counts.cap < b.nodes + 1 || r->b_pfx.cap < b.nodes + 2 ||
-        r->b_base.cap < b.nodes + 1 || r->lvl_cnt.cap < b.max_levels + 3 || r->tile_cnt.cap < b.ntiles ||
-        r->tile_off.cap < b.ntiles + 1 || r->tile_cur.cap < b.ntiles || r->item_cnt.cap < b.ntiles ||
-        r->item_off.cap < b.ntiles + 1 || r->records.cap < r->b_rec_cap || r->items.cap < items_cap ||
+        r->b_base.cap < b.nodes + 1 || r->b_lvl_cnt.cap < b.max_levels + 3 || r->b_tile_cnt.cap < b.ntiles ||
+        r->b_tile_off.cap < b.ntiles + 1 || r->b_tile_cur.cap < b.ntiles || r->b_item_cnt.cap < b.ntiles ||
+        r->b_item_off.cap < b.ntiles + 1 || r->records.cap < r->b_rec_cap || r->b_items.cap < items_cap ||
         r->maxv.cap < (size_t)n || r->b_hist.cap < batch_hist(b.ntiles) + 1 || r->b_rec_cap == 0)
         fail(GBLOD_ERR_INVALID_ARG, "gblod_render_batch: call gblod_renderer_reserve_batch for this batch first");
     r->last_stream = s;
@@ -2531,11 +2530,11 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
     }
     const unsigned G = (unsigned)persistent_blocks(4);
     GB_CUDA(cudaMemsetAsync(r->stats, 0, offsetof(FrameStatsDev, pixel_updates_total), s));
-    GB_CUDA(cudaMemsetAsync(r->lvl_cnt.p, 0, (size_t)(b.max_levels + 3) * 4, s));
+    GB_CUDA(cudaMemsetAsync(r->b_lvl_cnt.p, 0, (size_t)(b.max_levels + 3) * 4, s));
     const dim3 GV((unsigned)std::max(1, (int)G / n), (unsigned)n); // (blocks per view, views)
     launch(GBLOD_K_RENDER_OTHER, k_bzero, GV, dim3(256), 0, s, (const ViewDev *)dv);
     // R1 over (view, node) pairs
-    uint32_t *nsel = r->lvl_cnt.p + b.max_levels + 1;
+    uint32_t *nsel = r->b_lvl_cnt.p + b.max_levels + 1;
     if (b.nodes <= SELECT_FLAT) {
         uint8_t *cls = reinterpret_cast<uint8_t *>(r->b_frontA.p);
         const uint32_t total = (uint32_t)b.nodes;
@@ -2545,18 +2544,18 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
                total, (const uint8_t *)cls, r->b_sel.p, nsel);
     } else {
         unsigned long long *fin = r->b_frontA.p, *fout = r->b_frontB.p;
-        launch(GBLOD_K_SELECT_NODES, k_bselect_init, dim3(1), dim3(256), 0, s, (const ViewDev *)dv, n, fin, r->lvl_cnt.p);
+        launch(GBLOD_K_SELECT_NODES, k_bselect_init, dim3(1), dim3(256), 0, s, (const ViewDev *)dv, n, fin, r->b_lvl_cnt.p);
         for (uint32_t d = 0; d < b.max_levels; ++d) {
             launch(GBLOD_K_SELECT_NODES, k_bselect_level, dim3((unsigned)persistent_blocks(2)), dim3(RT), 0, s,
-                   (const ViewDev *)dv, (const unsigned long long *)fin, (const uint32_t *)(r->lvl_cnt.p + d), fout,
-                   r->lvl_cnt.p + d + 1, r->b_sel.p, nsel);
+                   (const ViewDev *)dv, (const unsigned long long *)fin, (const uint32_t *)(r->b_lvl_cnt.p + d), fout,
+                   r->b_lvl_cnt.p + d + 1, r->b_sel.p, nsel);
             std::swap(fin, fout);
         }
     }
     const uint32_t cap = (uint32_t)(b.nodes + 1);
     launch(GBLOD_K_SELECT_NODES, k_bsel_counts, dim3(G), dim3(256), 0, s, (const ViewDev *)dv,
            (const unsigned long long *)r->b_sel.p, (const uint32_t *)nsel, cap, r->b_counts.p);
-    scan_exclusive_u64(A, r->scan, reinterpret_cast<const uint64_t *>(r->b_counts.p),
+    scan_exclusive_u64(A, r->b_scan, reinterpret_cast<const uint64_t *>(r->b_counts.p),
                        reinterpret_cast<uint64_t *>(r->b_pfx.p), cap, reinterpret_cast<uint64_t *>(&r->stats->points),
                        s);
     launch(GBLOD_K_SELECT_NODES, k_bsel_base, dim3(G), dim3(256), 0, s, (const ViewDev *)dv,
@@ -2572,34 +2571,34 @@ void render_batch(gblod_renderer *r, const gblod_view *views, int n, const gblod
         const size_t smem = (size_t)b.ntiles * 4, nh = (size_t)b.ntiles * GP;
         launch(GBLOD_K_PROJECT_COUNT, k_bproject<false, true>, dim3(GP), dim3(RT), smem, s, src, r->b_hist.p, b.ntiles, kernel,
                (uint4 *)nullptr, 0ull, r->status, r->stats, 0);
-        scan_exclusive_u32(A, r->scan, r->b_hist.p, r->b_hist.p, nh, r->b_hist.p + nh, s);
+        scan_exclusive_u32(A, r->b_scan, r->b_hist.p, r->b_hist.p, nh, r->b_hist.p + nh, s);
         launch(GBLOD_K_RENDER_OTHER, k_tiles_from_hist, tg, dim3(256), 0, s, b.ntiles, (uint32_t)GP, 0u, items_wanted(),
-               (const uint32_t *)r->b_hist.p, (const uint32_t *)(r->b_hist.p + nh), r->tile_cnt.p, r->tile_off.p,
-               r->item_cnt.p, (unsigned long long *)nullptr, 0u);
+               (const uint32_t *)r->b_hist.p, (const uint32_t *)(r->b_hist.p + nh), r->b_tile_cnt.p, r->b_tile_off.p,
+               r->b_item_cnt.p, (unsigned long long *)nullptr, 0u);
         launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, true>, dim3(GP), dim3(RT), smem, s, src, r->b_hist.p, b.ntiles, kernel,
                r->records.p, rec_cap, r->status, r->stats, count);
     } else {
-        GB_CUDA(cudaMemsetAsync(r->tile_cnt.p, 0, (size_t)b.ntiles * 4, s));
-        launch(GBLOD_K_PROJECT_COUNT, k_bproject<false, false>, dim3(G), dim3(RT), 0, s, src, r->tile_cnt.p, b.ntiles, kernel,
+        GB_CUDA(cudaMemsetAsync(r->b_tile_cnt.p, 0, (size_t)b.ntiles * 4, s));
+        launch(GBLOD_K_PROJECT_COUNT, k_bproject<false, false>, dim3(G), dim3(RT), 0, s, src, r->b_tile_cnt.p, b.ntiles, kernel,
                (uint4 *)nullptr, 0ull, r->status, r->stats, 0);
-        scan_exclusive_u32(A, r->scan, r->tile_cnt.p, r->tile_off.p, b.ntiles, r->tile_off.p + b.ntiles, s);
-        launch(GBLOD_K_RENDER_OTHER, k_tile_items, tg, dim3(256), 0, s, b.ntiles, (const uint32_t *)r->tile_cnt.p,
-               r->item_cnt.p, (unsigned long long *)nullptr);
-        GB_CUDA(cudaMemcpyAsync(r->tile_cur.p, r->tile_off.p, (size_t)b.ntiles * 4, cudaMemcpyDeviceToDevice, s));
-        launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, false>, dim3(G), dim3(RT), 0, s, src, r->tile_cur.p, b.ntiles, kernel,
+        scan_exclusive_u32(A, r->b_scan, r->b_tile_cnt.p, r->b_tile_off.p, b.ntiles, r->b_tile_off.p + b.ntiles, s);
+        launch(GBLOD_K_RENDER_OTHER, k_tile_items, tg, dim3(256), 0, s, b.ntiles, (const uint32_t *)r->b_tile_cnt.p,
+               r->b_item_cnt.p, (unsigned long long *)nullptr);
+        GB_CUDA(cudaMemcpyAsync(r->b_tile_cur.p, r->b_tile_off.p, (size_t)b.ntiles * 4, cudaMemcpyDeviceToDevice, s));
+        launch(GBLOD_K_PROJECT_SCATTER, k_bproject<true, false>, dim3(G), dim3(RT), 0, s, src, r->b_tile_cur.p, b.ntiles, kernel,
                r->records.p, rec_cap, r->status, r->stats, count);
     }
-    scan_exclusive_u32(A, r->scan, r->item_cnt.p, r->item_off.p, b.ntiles, r->item_off.p + b.ntiles, s);
+    scan_exclusive_u32(A, r->b_scan, r->b_item_cnt.p, r->b_item_off.p, b.ntiles, r->b_item_off.p + b.ntiles, s);
     launch(GBLOD_K_RENDER_OTHER, k_bfill_items, dim3((b.ntiles + 255) / 256), dim3(256), 0, s, b.ntiles,
-           (const ViewDev *)dv, n, (const uint32_t *)r->tile_cnt.p, (const uint32_t *)r->tile_off.p,
-           (const uint32_t *)r->item_off.p, r->items.p, (uint32_t)items_cap, (unsigned long long)r->b_rec_cap,
+           (const ViewDev *)dv, n, (const uint32_t *)r->b_tile_cnt.p, (const uint32_t *)r->b_tile_off.p,
+           (const uint32_t *)r->b_item_off.p, r->b_items.p, (uint32_t)items_cap, (unsigned long long)r->b_rec_cap,
            (const FrameStatsDev *)r->stats, r->status, per_sm ? items_wanted() : 0u);
     // R3: persistent over the items of all views
     launch(GBLOD_K_SPLAT, (rp.flags & GBLOD_RENDER_COUNT_UPDATES) ? k_bsplat<true> : k_bsplat<false>, dim3(G), dim3(RT),
-           sizeof(SplatSmem), s, (const uint4 *)r->records.p, (const uint4 *)r->items.p,
-           (const uint32_t *)(r->item_off.p + b.ntiles),
+           sizeof(SplatSmem), s, (const uint4 *)r->records.p, (const uint4 *)r->b_items.p,
+           (const uint32_t *)(r->b_item_off.p + b.ntiles),
            (uint32_t)items_cap, strips_of(b.host[0].P.TW, b.host[0].P.TH), b.host[0].P.kernel, (const ViewDev *)dv,
-           r->lvl_cnt.p + b.max_levels + 2, r->stats);
+           r->b_lvl_cnt.p + b.max_levels + 2, r->stats);
     // R4
     const dim3 GT((tone_blocks(b.npix) + (unsigned)n - 1) / (unsigned)n, (unsigned)n);
     if (rp.tone_auto) {
@@ -2630,13 +2629,16 @@ void renderer_release(gblod_renderer *r)
     r->frontA.release(A, s); r->frontB.release(A, s); r->sel.release(A, s); r->lvl_cnt.release(A, s);
     r->sel_pfx.release(A, s); r->sel_base.release(A, s);
     r->tile_cnt.release(A, s); r->tile_off.release(A, s); r->tile_cur.release(A, s);
-    r->cta_hist.release(A, s); r->cta_off.release(A, s); r->b_hist.release(A, s);
+    r->cta_hist.release(A, s); r->cta_off.release(A, s);
     r->tile_cnt_s.release(A, s); r->tile_off_s.release(A, s); r->item_cnt_s.release(A, s); r->item_off_s.release(A, s);
     r->item_cnt.release(A, s); r->item_off.release(A, s);
     r->records.release(A, s); r->items.release(A, s); r->accum.release(A, s); r->maxv.release(A, s);
     r->pass_stats.release(A, s);
     r->b_views.release(A, s); r->b_frontA.release(A, s); r->b_frontB.release(A, s); r->b_sel.release(A, s);
     r->b_counts.release(A, s); r->b_pfx.release(A, s); r->b_base.release(A, s);
+    r->b_lvl_cnt.release(A, s); r->b_tile_cnt.release(A, s); r->b_tile_off.release(A, s); r->b_tile_cur.release(A, s);
+    r->b_item_cnt.release(A, s); r->b_item_off.release(A, s); r->b_hist.release(A, s); r->b_items.release(A, s);
+    r->b_scan.buf.release(A, s);
     r->d_cams.release(A, s); r->d_rec.release(A, s); r->d_hist.release(A, s); r->d_off.release(A, s);
     r->d_cnt.release(A, s); r->d_items.release(A, s); r->d_big.release(A, s);
     r->scan.buf.release(A, s);

@@ -26,7 +26,6 @@ struct gblod_renderer {
     gb::DBuf<int64_t> sel_base;
     // R2 / R3
     gb::DBuf<uint32_t> tile_cnt, tile_off, tile_cur, item_cnt, item_off;
-    gb::DBuf<uint32_t> b_hist;            // batches: the same, scanned in place
     gb::DBuf<uint32_t> cta_hist, cta_off; // partitioned binning: (tile, CTA) counts and their offsets
     gb::DBuf<uint32_t> tile_cnt_s, tile_off_s, item_cnt_s, item_off_s; // its small-box record stream
     gb::DBuf<uint4> records, items;
@@ -36,6 +35,13 @@ struct gblod_renderer {
     gb::DBuf<unsigned char> b_views; // per-view device constants (projection, frustum, pointers)
     gb::DBuf<unsigned long long> b_frontA, b_frontB, b_sel, b_counts, b_pfx;
     gb::DBuf<long long> b_base;
+    // A captured batch keeps the addresses it was captured with, so batches share with the other calls, which grow
+    // their buffers as they need, only `records` (grown by a frame of more records than b_rec_cap), and
+    // `maxv`, `stats` and `status`, which they do not move.
+    gb::ScanTmp b_scan;
+    gb::DBuf<uint32_t> b_lvl_cnt, b_tile_cnt, b_tile_off, b_tile_cur, b_item_cnt, b_item_off;
+    gb::DBuf<uint32_t> b_hist; // (tile, CTA) counts, scanned in place
+    gb::DBuf<uint4> b_items;
     uint64_t b_rec_cap = 0;
     // differentiable float splat
     gb::DBuf<unsigned char> d_cams;

@@ -51,3 +51,48 @@ def test_larger_batch_after_a_large_frame_is_refused():
     alone.close()
     r.close()
     t.free()
+
+
+def test_a_captured_batch_survives_other_calls_on_the_renderer():
+    """Calls that grow the renderer's own buffers (runs of records in groups, more tiles, deeper trees, fits) between the
+    capture of a batch and its replay; none needs more records than were reserved."""
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    p = synth.tiny(20000, seed=3)
+    t = G.build_lod(*to_dev(p.xyz, p.mass, p.h), n_max=400, seed=2)
+    deep = G.build_lod(*to_dev(p.xyz, p.mass, p.h), n_max=1, seed=2)
+    views = _views(t, 2, 1920, 1080)
+    par = G.make_params(lambda_px=6.0)
+    r = G.Renderer()
+    r.reserve_batch(views, par, record_capacity=1 << 28)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        r.render_batch(views, par)
+    s.synchronize()
+    want = [(img.clone(), acc.clone()) for _, _, img, acc in views]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        r.render_batch(views, par)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    n = 12_000_000
+    xyz = torch.rand(n, 3, generator=gen, device="cuda")
+    one = torch.ones(n, device="cuda")
+    r.render_bruteforce(xyz, one, 2e-3 * one, views[0][1], par)
+    r.render_bruteforce(xyz, one, 1e-4 * one, synth.look_at((0.5, 0.5, -1.0), (0.5, 0.5, 0.5), width=7680, height=4320))
+    r.render(deep, views[0][1], G.make_params(lambda_px=0.0))
+    G.diff_render(r, xyz[:1000], one[:1000], one[:1000] - 6.0, [views[0][1]])
+    torch.cuda.synchronize()
+    for _, _, img, acc in views:
+        img.zero_()
+        acc.zero_()
+    torch.cuda.empty_cache()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert r.status() == G.OK
+    for (_, _, img, acc), (wi, wa) in zip(views, want):
+        assert torch.equal(acc, wa) and torch.equal(img, wi)
+    r.close()
+    t.free()
+    deep.free()
