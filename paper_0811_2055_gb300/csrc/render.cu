@@ -1108,7 +1108,8 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
 constexpr uint32_t ITEM_MIN = 64;
 __host__ __device__ __forceinline__ uint32_t item_size(uint32_t total, uint32_t want)
 {
-    const uint32_t per = (total / want + 31u) / 32u * 32u;
+    const uint32_t each = total / want + (total % want != 0u); // rounded up: no more than `want` full items
+    const uint32_t per = each < ITEM ? (each + 31u) / 32u * 32u : ITEM;
     return per < ITEM_MIN ? ITEM_MIN : (per < ITEM ? per : ITEM);
 }
 // wanted items: four units a warp of the splat kernel's grid (a unit is a strip of up to eight)
@@ -2382,7 +2383,8 @@ int batch_part(uint32_t ntiles)
     return (int)std::min<size_t>(4, std::max<size_t>(1, 216 * 1024 / (smem + 6 * 1024)));
 }
 
-// work items of a batch, at most (item_size makes no more than are wanted, or than ITEM records each give)
+// work items of a batch, at most: one begun item a tile, and full ones, of which there are no more than are
+// wanted, or than ITEM records each give
 uint64_t batch_items(uint32_t ntiles, uint64_t records) { return ntiles + std::max<uint64_t>(records / ITEM, items_wanted()) + 1; }
 
 // histogram entries of a batch of up to ntiles tiles

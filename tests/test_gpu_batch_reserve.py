@@ -96,3 +96,26 @@ def test_a_captured_batch_survives_other_calls_on_the_renderer():
     r.close()
     t.free()
     deep.free()
+
+
+def test_a_batch_whose_records_fit_its_reservation_is_drawn():
+    """As many records as make the most work items for their number: a quotient just above an item size (32 tiles,
+    all reached by each of 2 want + 66 particles: 64 < records / want < 65), reserved with little to spare."""
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    n = 2 * 16 * torch.cuda.get_device_properties(0).multi_processor_count + 66
+    p = synth.tiny(n, seed=5)
+    xyz = (0.5 + 0.01 * (p.xyz - 0.5)).astype("float32")
+    t = G.build_lod(*to_dev(xyz, p.mass, 0.0 * p.h + 0.4), n_max=8000, seed=1)
+    views = _views(t, 1, 256, 128)
+    r = G.Renderer()
+    r.reserve_batch(views, record_capacity=1 << 22)
+    r.render_batch(views)
+    torch.cuda.synchronize()
+    assert r.status() == G.OK and r.stats()["pairs"] == 32 * n
+    alone = G.Renderer()
+    ia, aa = alone.render(t, views[0][1])
+    assert torch.equal(views[0][3], aa) and torch.equal(views[0][2], ia)
+    alone.close()
+    r.close()
+    t.free()
