@@ -322,25 +322,78 @@ struct DSums {
     }
 };
 
+// A record's derivatives with respect to its weight, centre and sigma
+struct DTerms {
+    float w = 0.f, u = 0.f, v = 0.f, s = 0.f;
+};
+
+// from the plain sums over its disc
+__device__ __forceinline__ DTerms dterms(float s, float wi, const DSums &S)
+{
+    const float is = 1.0f / s, is2 = is * is, norm = INV_2PI_C * is2, k = S.ge - E45 * S.g, wn = wi * norm;
+    DTerms T;
+    T.w = norm * k;
+    T.u = wn * (S.gex * is2);
+    T.v = wn * (S.gey * is2);
+    T.s = wn * (is * (S.ger * is2 - 2.0f * k));
+    return T;
+}
+
+// The same pixel by pixel over every step-th row, by a whole warp: each pixel's terms are scaled before they are added,
+// and a pixel without upstream value is left out.  For gradients that the plain sums do not give as finite numbers:
+// a weight that is not finite where nothing comes from upstream is 0, not inf 0; one infinite upstream value is
+// infinite, not inf - inf; and sums that overflow before they are scaled.
+__device__ __forceinline__ DTerms dterms_each(const float *__restrict__ img, int W, int x0, int x1, int y0, int y1,
+                                              int step, float u, float v, float s, float wi)
+{
+    const float s2 = s * s, a = -0.5f * LOG2E / s2, norm = INV_2PI_C / s2, is = 1.0f / s, is2 = is * is;
+    const int lane = threadIdx.x & 31, lw = x1 - x0 >= 16 ? 5 : 3, across = 1 << lw; // 32 columns x 1 row, or 8 x 4
+    DTerms T;
+    for (int y = y0 + (lane >> lw) * step; y <= y1; y += (32 >> lw) * step) {
+#pragma unroll 4
+        for (int x = x0 + (lane & (across - 1)); x <= x1; x += across) {
+            const float g = __ldg(&img[(size_t)y * W + x]), dx = (float)x + 0.5f - u, dy = (float)y + 0.5f - v;
+            const float r2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
+            if (g != 0.0f && r2 < 9.0f * s2) {
+                const float e = ex2(r2 * a) * norm, k = e - E45 * norm, gw = g * wi;
+                T.w += g * k;
+                T.u += gw * e * dx * is2;
+                T.v += gw * e * dy * is2;
+                T.s += gw * ((e * r2 * is2 - 2.0f * k) * is);
+            }
+        }
+        if (isnan(T.w) && isnan(T.u) && isnan(T.v) && isnan(T.s)) break; // nothing changes them any more
+    }
+    for (int d = 16; d > 0; d >>= 1) {
+        T.w += __shfl_xor_sync(0xffffffffu, T.w, d);
+        T.u += __shfl_xor_sync(0xffffffffu, T.u, d);
+        T.v += __shfl_xor_sync(0xffffffffu, T.v, d);
+        T.s += __shfl_xor_sync(0xffffffffu, T.s, d);
+    }
+    return T;
+}
+
 struct DGrad {
     float x = 0.f, y = 0.f, z = 0.f, w = 0.f, l = 0.f;
-    // chains a record's (w, u, v, sigma) derivatives to its position, weight and log smoothing length
-    __device__ __forceinline__ void add(const DCam &c, const DProj &o, float wi, const DSums &S)
+    // chains a record's derivatives to its position, weight and log smoothing length
+    __device__ __forceinline__ void add(const DCam &c, const DProj &o, const DTerms &T)
     {
-        const float is = 1.0f / o.s, is2 = is * is, norm = INV_2PI_C * is2, k = S.ge - E45 * S.g;
-        const float tw = norm * k, wn = wi * norm;
-        const float tu = wn * (S.gex * is2), tv = wn * (S.gey * is2), ts = wn * (is * (S.ger * is2 - 2.0f * k));
-        if (tw == 0.f && tu == 0.f && tv == 0.f && ts == 0.f) return;
+        if (T.w == 0.f && T.u == 0.f && T.v == 0.f && T.s == 0.f) return;
         const float iz = 1.0f / o.zc;
-        const float dxc = tu * c.F * iz;
-        const float dyc = -tv * c.F * iz;
+        const float dxc = T.u * c.F * iz;
+        const float dyc = -T.v * c.F * iz;
         const float ds_dz = o.clamped ? 0.0f : -o.s * iz;
-        const float dzc = tu * (-c.F * o.xc * iz * iz) + tv * (c.F * o.yc * iz * iz) + ts * ds_dz;
+        const float dzc = T.u * (-c.F * o.xc * iz * iz) + T.v * (c.F * o.yc * iz * iz) + T.s * ds_dz;
         x += c.rx * dxc + c.ux * dyc + c.fx * dzc;
         y += c.ry * dxc + c.uy * dyc + c.fy * dzc;
         z += c.rz * dxc + c.uz * dyc + c.fz * dzc;
-        w += tw;
-        if (!o.clamped) l += ts * o.s;
+        w += T.w;
+        if (!o.clamped) l += T.s * o.s;
+    }
+    // false if a term that was added is not finite (or nearly so)
+    __device__ __forceinline__ bool finite() const
+    {
+        return fabsf(x) + fabsf(y) + fabsf(z) + fabsf(w) + fabsf(l) < INFINITY;
     }
     __device__ __forceinline__ void add_to(uint32_t i, float *gxyz, float *gw, float *glogh) const
     {
@@ -385,7 +438,8 @@ __global__ void __launch_bounds__(DRT, 4) k_dgather(const DCam *__restrict__ cam
                                                  const float *__restrict__ xyz, const float *__restrict__ w,
                                                  const float *__restrict__ logh, uint32_t n,
                                                  const float *__restrict__ grad, float *gxyz, float *gw, float *glogh,
-                                                 uint2 *__restrict__ big, uint32_t *nbig)
+                                                 uint2 *__restrict__ big, uint32_t *nbig,
+                                                 uint32_t *__restrict__ oddw, uint32_t *nodd)
 {
     __shared__ float part[DRT / 8][8][41]; // per group and view: eight lanes' sums (41: conflict-free reads)
     const int lane = threadIdx.x & 31, l8 = lane & 7, g0 = lane & 24;
@@ -466,7 +520,12 @@ __global__ void __launch_bounds__(DRT, 4) k_dgather(const DCam *__restrict__ cam
             S.reduce<16>();
             if (lane == src) own = S;
         }
-        if (vis) G.add(cams[vb + l8], o, wi, own);
+        if (vis) G.add(cams[vb + l8], o, dterms(o.s, wi, own));
+    }
+    if (__any_sync(0xffffffffu, !G.finite())) { // left to k_dbig
+        if (lane == 0)
+            oddw[atomicAdd(nodd, 1u)] = (blockIdx.y * gridDim.x + blockIdx.x) * (DRT / 32) + (threadIdx.x >> 5);
+        G = DGrad();
     }
 #pragma unroll
     for (int d = 4; d > 0; d >>= 1) {
@@ -488,16 +547,38 @@ __global__ void __launch_bounds__(DRT, 4) k_dgather(const DCam *__restrict__ cam
     }
 }
 
-// the listed large records: a unit is every DBIG_SLICES-th row of one, a warp a row at a time
+// whether (i, view) is in the list of large records, by a whole warp
+__device__ __forceinline__ bool dlisted(const uint2 *__restrict__ big, uint32_t i, uint32_t view)
+{
+    bool found = false;
+    for (uint32_t k = threadIdx.x & 31; k < DBIG_CAP; k += 32) {
+        const uint2 b = __ldg(&big[k]);
+        found |= b.x == i && b.y == view;
+    }
+    return __any_sync(0xffffffffu, found);
+}
+
+// What k_dgather leaves: the listed large records (a unit is every DBIG_SLICES-th row of one, a warp a row at a
+// time), and the warps whose plain sums did not give finite gradients, term by term.  Both here, after the walks, so
+// that the second costs k_dgather no registers (with dterms_each inside it: 1M points x 16 views 3.19 -> 3.25 ms).
+constexpr uint32_t DBIG_ODD = 2048; // units a block can have
+constexpr unsigned DBIG_BLOCKS = DBIG_CAP * DBIG_SLICES / DBIG_ODD; // at least so many blocks
 __global__ void __launch_bounds__(DRT) k_dbig(const DCam *__restrict__ cams, const float *__restrict__ xyz,
                                               const float *__restrict__ w, const float *__restrict__ logh,
                                               const float *__restrict__ grad, float *gxyz, float *gw, float *glogh,
-                                              const uint2 *__restrict__ big, const uint32_t *nbig)
+                                              const uint2 *__restrict__ big, const uint32_t *nbig, uint32_t n, int nv,
+                                              int views_per, uint32_t gather_x, const uint32_t *__restrict__ oddw,
+                                              const uint32_t *nodd)
 {
     __shared__ DSums part[DRT / 32];
+    __shared__ DTerms each[DRT / 32];
+    __shared__ uint32_t odd[DBIG_ODD / 32]; // units whose gradient is not finite
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t units = min(*nbig, DBIG_CAP) * DBIG_SLICES;
-    for (uint32_t k = blockIdx.x; k < units; k += gridDim.x) {
+    const uint32_t units = min(*nbig, DBIG_CAP) * DBIG_SLICES, nw = *nodd;
+    if (blockIdx.x >= max(units, nw)) return;
+    if (threadIdx.x < DBIG_ODD / 32) odd[threadIdx.x] = 0u;
+    uint32_t nth = 0; // unit of the block
+    for (uint32_t k = blockIdx.x; k < units; k += gridDim.x, ++nth) {
         const uint2 b = big[k / DBIG_SLICES];
         const DCam &c = cams[b.y];
         DProj o;
@@ -522,9 +603,70 @@ __global__ void __launch_bounds__(DRT) k_dbig(const DCam *__restrict__ cams, con
                 S.ger += part[q].ger;
             }
             DGrad G;
-            G.add(c, o, w[b.x], S);
-            G.add_to(b.x, gxyz, gw, glogh);
+            G.add(c, o, dterms(o.s, w[b.x], S));
+            if (G.finite()) G.add_to(b.x, gxyz, gw, glogh);
+            else odd[nth >> 5] |= 1u << (nth & 31);
         }
+    }
+    __syncthreads();
+    // those again, term by term
+    for (uint32_t q = 0; q < (nth + 31) / 32; ++q)
+        for (uint32_t m = odd[q]; m; m &= m - 1u) {
+            const uint32_t k = blockIdx.x + (q * 32 + (uint32_t)__ffs((int)m) - 1u) * gridDim.x;
+            const uint2 b = big[k / DBIG_SLICES];
+            const DCam &c = cams[b.y];
+            DProj o;
+            (void)dproject(c, xyz, logh, b.x, o);
+            int x0, x1, y0, y1;
+            dbox(o.u, o.v, o.s, c.W, c.H, x0, x1, y0, y1);
+            const DTerms T = dterms_each(grad + (size_t)b.y * c.W * c.H, c.W, x0, x1, y0 + (int)(k % DBIG_SLICES) + warp * DBIG_SLICES, y1,
+                                         DBIG_SLICES * (DRT / 32), o.u, o.v, o.s, w[b.x]);
+            if (lane == 0) each[warp] = T;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                DTerms A;
+                for (int v = 0; v < DRT / 32; ++v) {
+                    A.w += each[v].w;
+                    A.u += each[v].u;
+                    A.v += each[v].v;
+                    A.s += each[v].s;
+                }
+                DGrad G;
+                G.add(c, o, A);
+                G.add_to(b.x, gxyz, gw, glogh);
+            }
+            __syncthreads();
+        }
+    // a warp of k_dgather each: four points, their views eight at a time
+    const int l8 = lane & 7, W = cams[0].W, H = cams[0].H;
+    for (uint32_t j = blockIdx.x * (DRT / 32) + warp; j < nw; j += gridDim.x * (DRT / 32)) {
+        const uint32_t id = oddw[j], block = id / (DRT / 32);
+        const unsigned long long i64 = (unsigned long long)(block % gather_x) * (DRT / 8) + id % (DRT / 32) * 4 + (lane >> 3);
+        const bool live = i64 < n;
+        const uint32_t i = live ? (uint32_t)i64 : 0u;
+        const int va = (int)(block / gather_x) * views_per, ve = min(nv, va + views_per);
+        const float wi = w[i];
+        DGrad G;
+        for (int vb = va; vb < ve; vb += 8) {
+            DProj o;
+            o.u = o.v = 0.f;
+            o.s = 1.f;
+            int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
+            if (live && vb + l8 < ve && dproject(cams[vb + l8], xyz, logh, i, o)) dbox(o.u, o.v, o.s, W, H, x0, x1, y0, y1);
+            const bool vis = x0 <= x1 && y0 <= y1, large = vis && (long long)(x1 - x0 + 1) * (y1 - y0 + 1) >= DBIG;
+            for (uint32_t m = __ballot_sync(0xffffffffu, vis && (!large || *nbig > DBIG_CAP)); m; m &= m - 1u) {
+                const int src = __ffs(m) - 1;
+                const uint32_t view = (uint32_t)(vb + (src & 7)), qi = __shfl_sync(0xffffffffu, i, src);
+                if (__shfl_sync(0xffffffffu, large, src) && dlisted(big, qi, view)) continue;
+                const int qx0 = __shfl_sync(0xffffffffu, x0, src), qx1 = __shfl_sync(0xffffffffu, x1, src);
+                const int qy0 = __shfl_sync(0xffffffffu, y0, src), qy1 = __shfl_sync(0xffffffffu, y1, src);
+                const float qu = __shfl_sync(0xffffffffu, o.u, src), qv = __shfl_sync(0xffffffffu, o.v, src);
+                const float qs = __shfl_sync(0xffffffffu, o.s, src), qw = __shfl_sync(0xffffffffu, wi, src);
+                const DTerms T = dterms_each(grad + (size_t)view * W * H, W, qx0, qx1, qy0, qy1, 1, qu, qv, qs, qw);
+                if (lane == src) G.add(cams[view], o, T);
+            }
+        }
+        if (live) G.add_to(i, gxyz, gw, glogh); // zeros so far, or the sums of the point's other views
     }
 }
 
@@ -552,7 +694,7 @@ struct DSetup {
     int first, n;
     float *zero[3];
     unsigned long long count[3];
-    uint32_t *counter; // may be null
+    uint32_t *counter; // two words; may be null
     DCam cam[CAMS_PER_LAUNCH];
 };
 static_assert(sizeof(DSetup) <= 4096, "kernel parameters");
@@ -561,7 +703,7 @@ __global__ void k_dsetup(const __grid_constant__ DSetup S, DCam *__restrict__ ca
 {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < (size_t)S.n) cams[S.first + t] = S.cam[t];
-    if (t == 0 && S.counter) *S.counter = 0u;
+    if (t < 2 && S.counter) S.counter[t] = 0u;
 #pragma unroll
     for (int q = 0; q < 3; ++q)
         for (size_t i = t; i < S.count[q]; i += (size_t)gridDim.x * blockDim.x) S.zero[q][i] = 0.0f;
@@ -611,7 +753,7 @@ void diff_forward(gblod_renderer *r, const float *xyz_all, const float *w_all, c
     check_views(n_all, cams, nv);
     const Allocator &A = r->A;
     const DCam c0 = make_dcam(cams[0], rp);
-    r->d_cnt.ensure(A, 8, s); // counters: work items, next unit, listed large records, -, records (64 bits)
+    r->d_cnt.ensure(A, 8, s); // counters: work items, next unit, listed large records, listed warps, records (64 bits)
     auto *d_pairs = reinterpret_cast<unsigned long long *>(r->d_cnt.p + 4);
     DSetup S{};
     S.zero[0] = images;
@@ -702,7 +844,7 @@ void diff_backward(gblod_renderer *r, const float *xyz, const float *w, const fl
     if (n == 0) return;
     r->d_cnt.ensure(r->A, 8, s);
     r->d_big.ensure(r->A, DBIG_CAP, s);
-    uint32_t *nbig = r->d_cnt.p + 2;
+    uint32_t *nbig = r->d_cnt.p + 2, *nodd = nbig + 1;
     // with few points the views are split over blocks: a warp's four points times its views are walked
     // one after another, so about 256 warps per SM are wanted (16,000 points x 8 views: 154 us unsplit, 75 us split; 128 warps 82)
     const unsigned gx = (unsigned)((n + DRT / 8 - 1) / (DRT / 8));
@@ -718,11 +860,13 @@ void diff_backward(gblod_renderer *r, const float *xyz, const float *w, const fl
             S.count[q] = q ? n : 3 * n;
         }
     }
+    r->d_odd.ensure(r->A, (size_t)grid.x * grid.y * (DRT / 32), s);
     const DCam *dc = setup(r, cams, nv, rp, S, s);
     launch(GBLOD_K_SPLAT, grid.y > 1 ? k_dgather<true> : k_dgather<false>, grid, dim3(DRT), 0, s, dc, nv, views_per, xyz,
-           w, logh, (uint32_t)n, grad_img, gxyz, gw, glogh, r->d_big.p, nbig);
-    launch(GBLOD_K_SPLAT, k_dbig, dim3((unsigned)persistent_blocks(4)), dim3(DRT), 0, s, dc, xyz, w, logh, grad_img, gxyz,
-           gw, glogh, (const uint2 *)r->d_big.p, (const uint32_t *)nbig);
+           w, logh, (uint32_t)n, grad_img, gxyz, gw, glogh, r->d_big.p, nbig, r->d_odd.p, nodd);
+    launch(GBLOD_K_SPLAT, k_dbig, dim3(std::max((unsigned)persistent_blocks(4), DBIG_BLOCKS)), dim3(DRT), 0, s, dc, xyz, w, logh, grad_img, gxyz,
+           gw, glogh, (const uint2 *)r->d_big.p, (const uint32_t *)nbig, (uint32_t)n, nv, views_per, grid.x,
+           (const uint32_t *)r->d_odd.p, (const uint32_t *)nodd);
 }
 
 } // namespace gb

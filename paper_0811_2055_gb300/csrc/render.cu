@@ -2642,7 +2642,7 @@ void renderer_release(gblod_renderer *r)
     r->b_item_cnt.release(A, s); r->b_item_off.release(A, s); r->b_hist.release(A, s); r->b_items.release(A, s);
     r->b_scan.buf.release(A, s);
     r->d_cams.release(A, s); r->d_rec.release(A, s); r->d_hist.release(A, s); r->d_off.release(A, s);
-    r->d_cnt.release(A, s); r->d_items.release(A, s); r->d_big.release(A, s);
+    r->d_cnt.release(A, s); r->d_items.release(A, s); r->d_big.release(A, s); r->d_odd.release(A, s);
     r->scan.buf.release(A, s);
 }
 

@@ -46,7 +46,7 @@ struct gblod_renderer {
     // differentiable float splat
     gb::DBuf<unsigned char> d_cams;
     gb::DBuf<float4> d_rec;
-    gb::DBuf<uint32_t> d_hist, d_off, d_cnt;
+    gb::DBuf<uint32_t> d_hist, d_off, d_cnt, d_odd;
     gb::DBuf<uint4> d_items;
     gb::DBuf<uint2> d_big;
     cudaStream_t last_stream = nullptr;
