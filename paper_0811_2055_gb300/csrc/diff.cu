@@ -73,7 +73,8 @@ __device__ __forceinline__ void dtiles(const DCam &c, const DProj &o, int &tx0, 
 // Forward binning.  blockIdx.y is a view of the chunk, blockIdx.x a part of the points; a CTA counts its
 // (tile, point) pairs per tile in shared memory and writes one histogram column, hist[(view, tile)][part];
 // the exclusive scan of hist gives every part its base in every tile, and the record pass places
-// records {u, v, a = -log2(e) / (2 sigma^2), c = w norm / sigma^2} with shared-memory atomics.  (Counting
+// records {u, v, a = -log2(e) / (2 sigma^2), c = w norm / sigma^2} (c not finite: {u, v, -a, w}) with shared-memory
+// atomics.  (Counting
 // with warp-aggregated global atomics spent 260 cycles a round in __match_any_sync: 1M points x 16
 // views, count + records 4.7 ms; now 0.4 ms.)  With more tiles than a CTA's shared memory holds (SHARED
 // false) the counters are global, cnt[(view, tile)], and there is one part.  The scan is modulo 2^32; `pairs` (may
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(DRT) k_dbin(const DCam *__restrict__ cams, int
         if (SCATTER) {
             const float s2 = o.s * o.s;
             r = make_float4(o.u, o.v, -0.5f * LOG2E / s2, w[i] * (INV_2PI_C / s2));
+            if (!isfinite(r.w)) r = make_float4(o.u, o.v, -r.z, w[i]);
         }
         for (int ty = ty0; ty <= ty1; ++ty)
             for (int tx = tx0; tx <= tx1; ++tx) {
@@ -171,8 +173,8 @@ __global__ void __launch_bounds__(1024) k_ditems(uint32_t nt, uint32_t parts, ui
 // with the sums in registers.  Per (record, pixel): two products, the exponential, and
 // max(e - exp(-4.5), 0) as a saturating addition, which is 0 from the support edge on, so no pixel is
 // tested.  (A thread per pixel of 16 x 16 tiles with two divisions a pair: 1M points x 16 views 5.2 ms;
-// now 1.6 ms.)  Records with a weight that is not finite must not reach pixels outside their disc:
-// they have a list of their own, with the test.
+// now 1.6 ms.)  Records whose weight, or its product with the norm, is not finite must not reach
+// pixels outside their disc, and inside it the kernel's value scales the weight first: they have a list of their own.
 enum { D_BOTH, D_UP, D_LOW, D_ODD, D_LISTS };
 constexpr int DLIST_MIN = 16, DLIST = DLIST_MIN - 1 + 32;
 struct DSmem {
@@ -191,7 +193,7 @@ __device__ __forceinline__ void dwalk(const float4 *__restrict__ list, int n, fl
         for (int k = 0; k < N; ++k) {
             const float d = dy + 4 * k, t = fmaf(d * d, A.z, ta), e = ex2(t);
             if (!TEST) acc[FIRST + k] = fmaf(A.w, __saturatef(e - E45), acc[FIRST + k]);
-            else if (t > -4.5f * LOG2E) acc[FIRST + k] = fmaf(A.w, e - E45, acc[FIRST + k]);
+            else if (t > -4.5f * LOG2E) acc[FIRST + k] += A.w * (e - E45) * (A.z * (-2.0f / LOG2E * INV_2PI_C));
         }
     }
 }
@@ -227,9 +229,11 @@ __global__ void __launch_bounds__(DRT, 4) k_dforward(const DCam *__restrict__ ca
         if (lane < D_LISTS) count[lane] = 0u;
         for (uint32_t base = it.y; base < it.z; base += 32) {
             float4 R = make_float4(0.f, 0.f, -1.f, 0.f);
-            bool up = false, low = false;
+            bool up = false, low = false, odd = false;
             if (base + lane < it.z) {
                 R = __ldg(&rec[base + lane]);
+                odd = R.z > 0.0f;
+                R.z = -fabsf(R.z);
                 const float r9 = __fdividef(-4.5f * LOG2E, R.z) * (1.0f + 0x1p-18f); // 9 sigma^2, rounded up
                 const float ex = fmaxf(fmaxf(cx0 - R.x, R.x - cx1), 0.0f), ex2_ = ex * ex;
                 const float eu = fmaxf(fmaxf(cy0 - R.y, R.y - cy1), 0.0f);
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(DRT, 4) k_dforward(const DCam *__restrict__ ca
             }
             const bool in = up || low;
             __syncwarp(); // the counters and the walks of the round before
-            const int l = !isfinite(R.w) ? D_ODD : (up && low ? D_BOTH : (up ? D_UP : D_LOW));
+            const int l = odd ? D_ODD : (up && low ? D_BOTH : (up ? D_UP : D_LOW));
 #pragma unroll
             for (int q = 0; q < D_LISTS; ++q) {
                 const uint32_t m = __ballot_sync(0xffffffffu, in && l == q);

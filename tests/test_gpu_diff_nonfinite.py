@@ -182,3 +182,33 @@ def test_several_views_of_a_point_in_one_block(n, nv, bad):
         # the same terms of a view, then nv of them, in 32 bits in another order
         assert bool(((got[k].double() - want).abs()[ok] <= (2 * nv * 2.0 ** -24 * size + 1e-30)[ok]).all())
     r.close()
+
+
+@pytest.mark.parametrize("w0", [3e38, -3e38, np.inf])
+def test_the_image_of_a_weight_whose_peak_overflows(w0):
+    """sigma 0.25 px: the norm is 2.7, so the peak of a weight of 3e38 overflows, but not its flank: the kernel value
+    scales the weight first."""
+    from paper_0811_2055_gb300 import gblod as G
+    torch.cuda.set_device(0)
+    cam = synth.look_at((0.5, 0.5, -1.0), (0.5, 0.5, 0.5), width=64, height=48)
+    f = np.float32
+    xyz = np.array([[0.5, 0.5, 0.5], [0.6, 0.55, 0.5]], np.float32)
+    w, sig = np.array([w0, 1.0], np.float32), f(0.25)
+    logh = np.full(2, np.log(0.1 * 1.5 / cam["f_px"]), np.float32)
+    r = G.Renderer()
+    par = G.make_params(sigma_min_px=0.25)
+    img = G.diff_render(r, *to_dev(xyz, w, logh), [cam], par).cpu().numpy()[0]
+    unit = G.diff_render(r, *to_dev(xyz, np.array([1.0, 0.0], np.float32), logh), [cam], par).cpu().numpy()[0]
+    rest = G.diff_render(r, *to_dev(xyz, np.array([0.0, 1.0], np.float32), logh), [cam], par).cpu().numpy()[0]
+    on = unit > 0
+    norm = f(0.16951204) / (sig * sig)
+    with np.errstate(over="ignore"):
+        want = (f(w0) * (unit[on] / norm)) * norm
+    assert on.sum() >= 4
+    if np.isfinite(w0):
+        assert np.isfinite(want).all()  # the centre lies between four pixels
+        assert np.allclose(img[on], want, rtol=1e-4)
+    else:
+        assert (img[on] == np.inf).all()
+    assert np.array_equal(img[~on], rest[~on])
+    r.close()
