@@ -51,9 +51,10 @@ typedef enum {
  * A NULL gblod_allocator* (or NULL alloc) selects, for builds and octrees, the library's own
  * stream-ordered memory pool of the current device (cudaMallocFromPoolAsync / cudaFreeAsync), and,
  * for renderers (grow-only buffers), cudaMallocAsync / cudaFreeAsync on the device's default pool.
- * The library's pool keeps the memory freed into it mapped, for the next builds (a build frees its
- * sort buffers before it allocates the sorted arrays; an octree's arrays return to it when freed):
- * it holds at most the builds' peak footprint.  gblod_trim_cache returns it. */
+ * The library's pool keeps the memory freed into it mapped, for the next builds (an octree's arrays
+ * return to it when freed): it holds at most the builds' peak footprint, some 94 bytes a particle
+ * with the octree, or 66 for builds of more than 2^28 particles and where 94 do not fit.
+ * gblod_trim_cache returns it. */
 typedef void *(*gblod_alloc_fn)(size_t bytes, void *stream, void *ctx);
 typedef void (*gblod_free_fn)(void *ptr, size_t bytes, void *stream, void *ctx);
 typedef struct {
