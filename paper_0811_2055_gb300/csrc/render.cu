@@ -1238,17 +1238,6 @@ __global__ void __launch_bounds__(PART_THREADS<SMALL>, 1024 / PART_THREADS<SMALL
     if (!SMALL && cstats) count_hits(hits, cstats);
 }
 
-// work items of nruns runs: run t belongs to tile t mod ntiles
-__global__ void k_fill_items_n(uint32_t nruns, uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
-                               const uint32_t *item_off, uint32_t per_item, uint4 *items)
-{
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nruns) return;
-    const uint32_t c = tile_cnt[t], o = tile_off[t];
-    uint32_t k = item_off[t];
-    for (uint32_t s = 0; s < c; s += per_item, ++k) items[k] = make_uint4(t % ntiles, o + s, o + min(c, s + per_item), 0u);
-}
-
 // Small-box records of one work item (a tile and up to ITEM_SMALL of its records): each warp takes
 // 32 records at a time and takes their pixel boxes, clipped to the tile, by size (BoxQueues) or, for
 // wide supports and the largest amplitudes, together (walk_boxes), adding the
@@ -1350,13 +1339,14 @@ __global__ void k_tile_items(uint32_t ntiles, const uint32_t *tile_cnt, uint32_t
     if (t < ntiles) item_cnt[t] = (tile_cnt[t] + ITEM - 1) / ITEM;
 }
 
-// also clears the unit counter of the splat launch that follows and the frame's maximum (may be null)
+// Work items of nruns runs: run t belongs to tile t mod ntiles.  Also clears the unit counter of the splat launch that
+// follows and the frame's maximum (either may be null)
 __global__ void k_fill_items(uint32_t nruns, uint32_t ntiles, const uint32_t *tile_cnt, const uint32_t *tile_off,
                              const uint32_t *item_off, uint32_t per_item, uint4 *items, unsigned *next,
                              unsigned long long *maxv)
 {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t == 0) *next = 0u;
+    if (t == 0 && next) *next = 0u;
     if (t == 0 && maxv) *maxv = 0ull;
     if (t >= nruns) return;
     const uint32_t c = tile_cnt[t], o = tile_off[t];
@@ -1919,9 +1909,10 @@ void bin_splat(gblod_renderer *r, const Src &src, const Proj &P, unsigned long l
         launch(GBLOD_K_PROJECT_SCATTER, k_project_scatter_part<Src, SMALL>, dim3(bn.grid), dim3(PART_THREADS<SMALL>), bn.smem, s,
                src, P, lo, hi, bn.chunk, bn.grid / bn.groups, (const uint32_t *)r->cta_off.p, r->records.p, img, cstats);
         if (SMALL) {
-            launch(GBLOD_K_RENDER_OTHER, k_fill_items_n, tg, dim3(256), 0, s, nruns, ntiles,
+            launch(GBLOD_K_RENDER_OTHER, k_fill_items, tg, dim3(256), 0, s, nruns, ntiles,
                    (const uint32_t *)r->tile_cnt_s.p, (const uint32_t *)r->tile_off_s.p,
-                   (const uint32_t *)r->item_off_s.p, ITEM_SMALL, r->items.p + pc.items);
+                   (const uint32_t *)r->item_off_s.p, ITEM_SMALL, r->items.p + pc.items, (unsigned *)nullptr,
+                   (unsigned long long *)nullptr);
             launch(GBLOD_K_SPLAT, r->count_updates ? k_splat_small<true> : k_splat_small<false>, dim3(pc.small_items),
                    dim3(RT), sizeof(SmallSmem), s, (const uint4 *)r->records.p, (const uint4 *)(r->items.p + pc.items), P, img, r->stats);
         }
