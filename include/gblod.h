@@ -356,14 +356,16 @@ void gblod_autotune_cache_clear(void);
  * indistinguishable from a full rendering): sigma = clamp(f exp(l)/z_c, sigma_min, sigma_max),
  * kernel (exp(-r^2/2 sigma^2) - e^-4.5) / (2 pi sigma^2 (1 - 5.5 e^-4.5)) for r < 3 sigma,
  * fp32 accumulation (sum order not fixed: results agree to rounding, not bit for bit).  Waits for
- * `stream` once per chunk of views to size its scratch. */
+ * `stream` once per chunk of views (or part of one, where its records are very many) to size its
+ * scratch. */
 gblod_status gblod_diff_render(gblod_renderer *r, const float *d_xyz, const float *d_w, const float *d_logh,
                                uint64_t n, const gblod_camera *cams, int32_t n_views,
                                const gblod_render_params *params, float *d_images, void *stream);
 
 /* Adjoint of gblod_diff_render: given dL/dI (d_grad_images, same layout as d_images), writes
  * dL/dxyz (n x 3), dL/dw (n) and dL/dlog h (n) (overwritten; zero through a sigma clamp).  Every
- * per-pixel term is recomputed tile by tile; nothing per pixel is stored between the calls. */
+ * per-pixel term is recomputed, point by point over the points' own discs; nothing per pixel is
+ * stored between the calls.  A pixel whose dL/dI is zero adds nothing, whatever the weight. */
 gblod_status gblod_diff_backward(gblod_renderer *r, const float *d_xyz, const float *d_w, const float *d_logh,
                                  uint64_t n, const gblod_camera *cams, int32_t n_views,
                                  const gblod_render_params *params, const float *d_grad_images, float *d_grad_xyz,

@@ -1,6 +1,6 @@
 // Octree build on the device (octree paragraph of the paper): A1 Morton keys, A2 radix sort,
-// A3 per-node counting level by level, then the node table, exact node masses, leaf blocks and
-// the bottom-up cull data.  The subselection (A4/A5) lives in select.cu.
+// A3 the nodes of all levels from one pass over the sorted keys, exact node masses, leaf blocks and
+// the cull data, from the leaves up.  The subselection (A4/A5) lives in select.cu.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

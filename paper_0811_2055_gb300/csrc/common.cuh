@@ -112,7 +112,6 @@ template <class T> struct Scratch {
     }
 };
 
-// Pinned host staging for small read-backs.
 // Several arrays in one allocation (an allocation and its return cost the host about 3 us), each on a 256-byte
 // boundary: carve(A, s, {part(a, n), part(b, m)}) sets the pointers.
 struct Part {
@@ -133,6 +132,7 @@ inline Scratch<unsigned char> carve(const Allocator &A, cudaStream_t s, std::ini
     return mem;
 }
 
+// Pinned host staging for small read-backs.
 struct HostStage {
     void *p = nullptr;
     size_t bytes = 0;

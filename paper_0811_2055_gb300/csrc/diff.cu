@@ -6,7 +6,8 @@
 // sigma = clamp(F exp(l) / zc, sigma_min, sigma_max), kernel
 //   K(r) = (exp(-r^2 / 2 sigma^2) - exp(-4.5)) / (2 pi sigma^2 C'),  r < 3 sigma,  C' = 1 - 5.5 e^-4.5
 // (unit integral, continuous at the support edge), I = sum_i w_i K_i, fp32 accumulation.
-// The adjoint recomputes every per-pixel term tile by tile; nothing is stored per pixel.
+// The forward pass goes by screen tiles, the adjoint point by point over the points' own discs; it recomputes every
+// per-pixel term, nothing is stored per pixel.
 #include <algorithm>
 #include <cmath>
 #include <vector>

@@ -1,8 +1,8 @@
 // 16-bit block codes of the stored points (storage paragraph): positions in 2 bytes per
 // coordinate spanning the node's cell, weight and smoothing length coded linearly over the
-// node's range.  One block per node codes its points and reduces the decoded bounds; a
-// level-by-level pass (deepest first) then folds the children into each node's subtree bounds
-// and writes the quantised node table.
+// node's range.  One block per node codes its points and reduces the decoded bounds; one launch
+// then climbs from the leaves, folds the children into each node's subtree bounds and writes the
+// quantised node table.
 #include <cmath>
 
 #include "octree.cuh"

@@ -15,9 +15,8 @@ const char *get_error() { return t_err.c_str(); }
 
 // The library's own stream-ordered memory pool of the current device.  Its release threshold is
 // unbounded: memory freed by the library stays mapped in the pool for its next allocations, so a
-// build that frees its sort buffers and then allocates the sorted particle arrays (and a later build
-// of the same size) reuses mapped memory.  Pools with the default threshold of zero unmap freed
-// memory at every stream synchronisation, and the build synchronises once per octree level.
+// later build of the same size reuses mapped memory.  Pools with the default threshold of zero unmap
+// freed memory at every stream synchronisation, and a build has several.
 // gblod_trim_cache returns the cached memory to the device.
 static cudaMemPool_t lib_pool()
 {
