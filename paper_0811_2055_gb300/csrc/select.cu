@@ -95,7 +95,7 @@ __device__ __forceinline__ uint32_t find_slot(const uint32_t *chunk_off, uint32_
 }
 
 // What a block needs to know of its chunk, laid out once (blocks that looked it up through the node arrays,
-// four dependent loads: 150M, mark 0.93 -> 0.72 ms, write 1.52 -> 1.43; the warps' lists 1.28)
+// four dependent loads: 150M, mark 0.93 -> 0.72 ms, write 1.52 -> 1.43, and 1.28 with the warps' lists)
 struct __align__(16) Chunk {
     uint32_t j0, len, start, r; // first element; elements; the first one's position in the node; rep slot
     uint64_t code, words;       // node code; first bitmap word

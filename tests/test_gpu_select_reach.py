@@ -13,14 +13,14 @@ pytestmark = pytest.mark.gpu
 
 
 # deep trees: 65,000 nodes (flat form), and above 2^19 (level by level unless the view is far)
-@pytest.mark.parametrize("n, n_max, lo, side", [(30_000, 1, (0.0, 0.0, 0.0), 1.0), (30_000, 3, (-37.0, 11.5, 1000.0), 0.37),
-                                                (400_003, 1, (0.0, 0.0, 0.0), 1.0)])
-@pytest.mark.parametrize("block16", [False, True])
+@pytest.mark.parametrize("n, n_max, lo, side, block16", [(30_000, 1, (0.0, 0.0, 0.0), 1.0, False),
+                                                         (30_000, 1, (0.0, 0.0, 0.0), 1.0, True),
+                                                         (30_000, 3, (-37.0, 11.5, 1000.0), 0.37, False),
+                                                         (30_000, 3, (-37.0, 11.5, 1000.0), 0.37, True),
+                                                         (400_003, 1, (0.0, 0.0, 0.0), 1.0, False)])
 def test_selection_from_far_and_near(n, n_max, lo, side, block16):
     from paper_0811_2055_gb300 import gblod as G
     torch.cuda.set_device(0)
-    if block16 and n > 100_000:
-        pytest.skip("the form of the points does not matter to the size of the tree")
     p = synth.tiny(n, seed=n_max)
     xyz = (np.asarray(lo) + side * p.xyz.astype(np.float64)).astype(np.float32)
     h = (side * p.h).astype(np.float32)
