@@ -542,7 +542,7 @@ __device__ __forceinline__ int classify(const gblod_node &g, const Frustum &fr)
     return lhs > rhs ? 2 : 1;
 }
 
-// A node is drawn if the rule emits it and refines all its ancestors.  Trees of up to SELECT_FLAT nodes classify
+// A node is drawn if the rule emits it and refines all its ancestors.  Up to SELECT_FLAT reached nodes: classify
 // every node and look at the ancestors' classes, in two launches (up to SELECT_ONE nodes: in one block that
 // also does k_sel_prefix's work); larger trees are walked level by level, which reads only the nodes that are
 // reached.  A level costs a launch of 5 to 6 us whatever its size: 64 nodes, 4 levels 29 us with first and
@@ -2035,7 +2035,7 @@ __global__ void k_bzero(const ViewDev *__restrict__ views)
         V.accum[i] = 0ull;
 }
 
-// The flat form of the selection over all views' nodes (SELECT_FLAT in all)
+// The flat form of the selection over the nodes that the views can reach (up to SELECT_FLAT in all)
 __device__ __forceinline__ int view_of_node(const ViewDev *__restrict__ views, int n, uint32_t e)
 {
     int lo = 0, hi = n;
